@@ -193,12 +193,28 @@ static void layer_scale(Portfolio& pf, LayerConst& lc) {
   to_u128(lc.agg_lim * lc.scale, lc.agg_lim_lo, lc.agg_lim_hi);
 }
 
+// Per ELT the layers that hold it, as bit masks (up to 255 layers), and which layers list their
+// ELTs in strictly ascending order.
+static std::vector<uint64_t> layer_members(Portfolio& pf) {
+  std::vector<uint64_t> mem;
+  pf.layer_asc.assign((size_t)pf.n_layers, 1);
+  if (pf.n_layers < 1 || pf.n_layers > 255) return mem;
+  mem.assign((size_t)std::max(pf.n_elts, 1) * RW_MASK, 0ull);
+  for (int32_t l = 0; l < pf.n_layers; ++l)
+    for (int32_t k = pf.layer_off[(size_t)l]; k < pf.layer_off[(size_t)l + 1]; ++k) {
+      const int32_t j = pf.layer_elts[(size_t)k];
+      if (k > pf.layer_off[(size_t)l] && j <= pf.layer_elts[(size_t)k - 1]) pf.layer_asc[(size_t)l] = 0;
+      mem[(size_t)j * RW_MASK + (size_t)(l >> 6)] |= 1ull << (l & 63);
+    }
+  return mem;
+}
+
 static void free_portfolio(ara_portfolio* p) {
   if (!p) return;
   if (p->borrowed_elts) {
     // a layer set: its own buffers came from the stream-ordered allocator; the ELT tables
     // belong to the pool
-    void* own[] = {p->d_layer_elts, p->d_layers, p->d_q, p->d_bits, p->d_cbits, p->d_err};
+    void* own[] = {p->d_layer_elts, p->d_mem, p->d_layers, p->d_q, p->d_bits, p->d_cbits, p->d_err};
     for (void* q : own)
       if (q) cudaFreeAsync(q, p->owner_stream);
     void* staged[] = {p->d_stage_ids[0], p->d_stage_ids[1], p->d_stage_off[0], p->d_stage_off[1],
@@ -207,7 +223,7 @@ static void free_portfolio(ara_portfolio* p) {
       if (q) cudaFree(q);
   } else {
     void* ptrs[] = {p->d_rec_off, p->d_rec_ids, p->d_rec_orig, p->d_rec_loss, p->d_rec_loss32,
-                    p->d_elt_ret, p->d_elt_lim, p->d_tile_rec, p->d_layer_elts, p->d_layers, p->d_dense, p->d_q,
+                    p->d_elt_ret, p->d_elt_lim, p->d_tile_rec, p->d_ev_ptr, p->d_layer_elts, p->d_mem, p->d_layers, p->d_dense, p->d_q,
                     p->d_bits, p->d_cbits, p->d_err, p->d_stage_ids[0], p->d_stage_ids[1],
                     p->d_stage_off[0], p->d_stage_off[1], p->d_ylt_full};
     for (void* q : ptrs)
@@ -453,6 +469,11 @@ ara_status ara_create_portfolio(int64_t C, int32_t n_elts, const int64_t* rec_of
   if ((st = upload(&p->d_layer_elts, p->layer_elts.data(), p->layer_elts.size())) != ARA_OK)
     return fail(st);
   if ((st = upload(&p->d_layers, p->layers.data(), p->layers.size())) != ARA_OK) return fail(st);
+  {
+    const std::vector<uint64_t> mem = layer_members(*p);
+    if ((st = upload(&p->d_mem, mem.data(), mem.size())) != ARA_OK) return fail(st);
+  }
+  if ((st = build_event_index(*p, 0)) != ARA_OK) return fail(st);
   p->bm_words = ((C + 31) / 32 + 3) / 4 * 4;
   p->cbits_stride = (((C + 1) / 2 + 31) / 32 + 3) / 4 * 4;   // coarsest needed: 1 bit per 2 events
   if (n_layers > 0) {
@@ -535,6 +556,9 @@ ara_status ara_create_layer_set(ara_portfolio* pool, int32_t n_layers, const int
   p->n_tiles = pool->n_tiles;
   p->d_tile_rec = pool->d_tile_rec;
   p->d_dense = pool->d_dense;
+  p->d_ev_ptr = pool->d_ev_ptr;
+  p->d_ev_elt = pool->d_ev_elt;
+  p->d_ev_loss = pool->d_ev_loss;
   p->layer_off.assign(layer_off, layer_off + n_layers + 1);
   p->layer_elts.assign(layer_elts, layer_elts + layer_off[n_layers]);
   p->layers.resize((size_t)n_layers);
@@ -549,6 +573,7 @@ ara_status ara_create_layer_set(ara_portfolio* pool, int32_t n_layers, const int
     lc.elt_end = layer_off[l + 1];
     layer_scale(*p, lc);
   }
+  const std::vector<uint64_t> mem = layer_members(*p);
   DeviceGuard g(p->device);
   const int64_t C = p->catalogue;
   p->bm_words = pool->bm_words;
@@ -559,6 +584,7 @@ ara_status ara_create_layer_set(ara_portfolio* pool, int32_t n_layers, const int
   };
   auto amalloc = [&](void** ptr, size_t n) { return dmalloc_async(ptr, std::max<size_t>(n, 8), s) == cudaSuccess; };
   if (!amalloc((void**)&p->d_layer_elts, 4 * p->layer_elts.size()) ||
+      (!mem.empty() && !amalloc((void**)&p->d_mem, 8 * mem.size())) ||
       !amalloc((void**)&p->d_layers, sizeof(LayerConst) * (size_t)n_layers) ||
       !amalloc((void**)&p->d_q, 8 * (size_t)n_layers * C) ||
       !amalloc((void**)&p->d_bits, 4 * (size_t)n_layers * p->bm_words) ||
@@ -568,6 +594,7 @@ ara_status ara_create_layer_set(ara_portfolio* pool, int32_t n_layers, const int
   if ((!p->layer_elts.empty() &&
        cudaMemcpyAsync(p->d_layer_elts, p->layer_elts.data(), 4 * p->layer_elts.size(),
                        cudaMemcpyHostToDevice, s) != cudaSuccess) ||
+      (!mem.empty() && cudaMemcpyAsync(p->d_mem, mem.data(), 8 * mem.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) ||
       cudaMemcpyAsync(p->d_layers, p->layers.data(), sizeof(LayerConst) * (size_t)n_layers,
                       cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemsetAsync(p->d_bits, 0, 4 * (size_t)n_layers * p->bm_words, s) != cudaSuccess ||

@@ -1,25 +1,24 @@
 // Batched portfolio: every selected layer of a portfolio in one pass over the YET (the program
 // and layer loops of Algorithm 1 folded into one launch).
 //
-// Preparation, per run (all on the stream, captured in the plan's CUDA graph):
+// Preparation, per run (all on the stream, captured in the plan's CUDA graph): the event-major rows
+// of the selected layers, (slot, q) per non-zero occurrence loss (ara_rows.cu, which also holds the
+// stream over them).  Layers that list their ELTs in ascending order, which is what a portfolio
+// usually has, get their rows from the portfolio's event-major records in one kernel.  Any other
+// selection takes the general way, which keeps the layer's own order of the ELT sum:
 //   1. q_i(e) = round(C(sum_j C(x_j(e); R_j, L_j); OccR_i, OccL_i) * 2^f_i) and the hit bitmap
 //      of every selected layer i, in one launch of the single-layer fold kernel (slot i of the
-//      fold workspace; only the non-zero q are stored).  The batched and the single-layer paths
-//      thus share the folded table bit for bit.
-//   2. per-event counts of non-zero q, read from the bitmaps, and their exclusive scan -> CSR
-//      row pointers.
-//   3. event-major CSR rows: for event e, its (layer slot, q) pairs in layer order, packed as
-//      slot << 56 | q (q < 2^55); q is read only where the bitmap bit is set.  The event's row
+//      fold workspace; only the non-zero q are stored).
+//   2. per-event counts of non-zero q, read from the bitmaps, and the exclusive scan of their
+//      16-byte pairs.
+//   3. the rows, end to end: slot << 56 | q in slot order (q < 2^55; q is read only where the bitmap
+//      bit is set), padded to whole pairs with an entry of the spare slot.  The event's row
 //      descriptor holds its first entry and, per request of a merged serving pass (slots are
 //      grouped by request), the number of its entries in one byte each (a row has at most 255
 //      entries, one per slot), so that a trial covered by some of the requests walks only
 //      their part of the row.
-// Stream (persistent, atomic trial queue for uneven trial lengths): a warp takes trials from the
-// queue; for every 32 occurrences it joins their events' CSR rows into one list, walks it 32
-// entries at a time and adds each q to the warp's per-layer accumulator in shared memory (exact
-// 128-bit: 64-bit atomic add with carry); at the end of a trial its lanes apply every layer's
-// aggregate terms to the exact sums and write the YLT entries.  Integer sums make the result independent of the order of the additions and
-// bitwise equal to the single-layer path.
+// Both ways give the same q bit for bit, and the sums are exact integers, so the results equal
+// those of the single-layer path bit for bit.
 
 #include <algorithm>
 #include <vector>
@@ -30,11 +29,6 @@ namespace ara {
 
 constexpr int BT_MAX_LAYERS = 255;          // slot fits in 8 bits (255 = no slot)
 constexpr int BT_SCAN_BLOCK = 1024;
-
-struct BtLayers {
-  int32_t n_sel;
-  int32_t layer[BT_MAX_LAYERS];
-};
 
 // ------------------------------------------------------------------------------------------
 // 2. per-event counts and their exclusive scan (two levels: block sums, then their scan)
@@ -80,9 +74,15 @@ __device__ __forceinline__ uint32_t bt_count(const uint32_t* __restrict__ bits, 
 
 __global__ void __launch_bounds__(BT_SCAN_BLOCK)
 k_bt_scan_blocks(const uint32_t* __restrict__ bits, int64_t bits_stride, int32_t n_sel, int64_t n,
-                 uint32_t* __restrict__ ptr, uint32_t* __restrict__ block_sums) {
+                 uint32_t* __restrict__ ptr, uint32_t* __restrict__ block_sums,
+                 uint32_t* __restrict__ entries) {
   const int64_t e = (int64_t)blockIdx.x * BT_SCAN_BLOCK + threadIdx.x;
-  const uint32_t v = e < n ? bt_count(bits, bits_stride, n_sel, e) : 0u;
+  uint32_t v = e < n ? bt_count(bits, bits_stride, n_sel, e) : 0u;
+  if (entries) {   // rows in pairs of entries: the scan counts pairs, *entries gets the entries
+    const uint32_t c = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(entries, c);
+    v = (v + 1u) >> 1;
+  }
   uint32_t tot;
   const uint32_t ex = block_excl_scan(v, &tot);
   if (e < n) ptr[e] = ex;
@@ -118,7 +118,7 @@ ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t 
                              uint32_t* ptr, uint32_t* block_sums, uint32_t* total, cudaStream_t s) {
   const int64_t n_blocks = (n + BT_SCAN_BLOCK - 1) / BT_SCAN_BLOCK;
   k_bt_scan_blocks<<<(unsigned)n_blocks, BT_SCAN_BLOCK, 0, s>>>(bits, bits_stride, n_sel, n, ptr,
-                                                              block_sums);
+                                                              block_sums, nullptr);
   k_bt_scan_sums<<<1, BT_SCAN_BLOCK, 0, s>>>(block_sums, n_blocks, total);
   k_bt_scan_add<<<(unsigned)((n + 1 + 255) / 256), 256, 0, s>>>(ptr, n, block_sums, total);
   ARA_TRY(cudaGetLastError());
@@ -126,8 +126,7 @@ ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t 
 }
 
 // ------------------------------------------------------------------------------------------
-// 3. CSR rows: one thread per event, layers in slot order (deterministic layout), and the
-//    event's row descriptor (first entry | length << 32)
+// 3. rows: one thread per event, layers in slot order, and the event's row descriptor
 // ------------------------------------------------------------------------------------------
 // Request boundaries of a merged pass, in slots: request r owns [first[r], first[r + 1]); unused
 // requests start at BT_MAX_LAYERS + 1 (past every slot).
@@ -142,13 +141,12 @@ __device__ __forceinline__ uint32_t bt_req_of_slot(const BtReqSlots& rs, int i) 
 __global__ void __launch_bounds__(256)
 k_bt_fill(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restrict__ bits,
           int64_t bits_stride, int64_t catalogue, const uint32_t* __restrict__ ptr,
-          uint64_t* __restrict__ entries, uint64_t* __restrict__ rows, BtReqSlots rs) {
+          uint64_t* __restrict__ entries, uint64_t* __restrict__ rows, BtReqSlots rs, int first_shift) {
   constexpr int U = 8;   // slots per step: their bitmap words and table entries load together
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= catalogue) return;
-  const uint32_t pos0 = ptr[e];
-  uint32_t pos = pos0;
-  const uint32_t end = ptr[e + 1];
+  uint64_t pos = 2ull * ptr[e];
+  const uint64_t end = 2ull * ptr[e + 1];
   uint32_t lens = 0;   // entries of request r in byte r (one 8-byte descriptor per occurrence)
   const uint32_t* b = bits + (e >> 5);
   const int sh = (int)(e & 31);
@@ -170,178 +168,8 @@ k_bt_fill(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restr
         ++pos;
       }
   }
-  rows[e] = (uint64_t)pos0 | ((uint64_t)lens << 32);
-}
-
-// ------------------------------------------------------------------------------------------
-// Stream
-// ------------------------------------------------------------------------------------------
-struct BtStream {
-  int64_t n_trials;
-  const int64_t* offsets;
-  int64_t n_events;
-  const int32_t* ids;
-  uint32_t catalogue;
-  const uint64_t* rows;        // [catalogue]: first entry | length << 32
-  const uint64_t* entries;
-  int32_t n_sel;
-  const LayerConst* layers;    // device, indexed by layer id
-  BtLayers sel;                // slot -> layer id
-  // Requests of the pass (one outside serving): request r owns the slots [rs.first[r],
-  // rs.first[r + 1]) and the trials [t0[r], t1[r]); row i of its YLT (its slot first + i) is
-  // ylt[r] + i * (t1[r] - t0[r]), indexed by t - t0[r]; regimes likewise (or nullptr).
-  int32_t n_req;
-  BtReqSlots rs;
-  int64_t t0[BT_MAX_REQ], t1[BT_MAX_REQ];
-  double* ylt[BT_MAX_REQ];
-  uint8_t* regimes[BT_MAX_REQ];
-  unsigned long long* queue;   // trial counter (zeroed before the launch)
-  int32_t trials_per_grab;
-  int32_t copies;              // accumulator copies per warp: 1, 2 or 4
-  uint32_t* err;
-};
-
-// Non-returning 64-bit shared-memory add.  A segment of at most BT_SEG occurrences adds at most
-// one value below 2^55 per occurrence to a slot's word (a row holds each slot once), so the word
-// cannot wrap: BT_SEG * 2^55 <= 2^64.
-constexpr int BT_SEG = 512;
-__device__ __forceinline__ void smem_red_u64(unsigned long long* a, uint64_t q) {
-  asm volatile("red.shared.add.u64 [%0], %1;" :: "r"((uint32_t)__cvta_generic_to_shared(a)), "l"(q) : "memory");
-}
-
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
-k_bt_stream(BtStream p) {
-  // [WARPS][copies + 2][n_sel]: per copy the 64-bit sums of the current segment, then the
-  // trial's exact 128-bit totals (low and high words) of the finished segments
-  extern __shared__ __align__(16) unsigned long long bt_acc[];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ns = p.n_sel;
-  // Each group of 32 / copies lanes has its own copy of the warp's accumulators, so that lanes
-  // of different groups never add to the same word; the copies are summed exactly at the end of
-  // a trial.
-  const int nc = p.copies;
-  unsigned long long* const acc0 = bt_acc + (int64_t)wid * (nc + 2) * ns;
-  unsigned long long* const lo = acc0 + (int64_t)(lane / (32 / nc)) * ns;
-  unsigned long long* const tot = acc0 + (int64_t)nc * ns;   // [2][n_sel]
-  for (int i = lane; i < (nc + 2) * ns; i += 32) acc0[i] = 0ull;
-  __syncwarp();
-  bool bad_id = false, bad_off = false;
-  while (true) {
-    unsigned long long t0 = 0;
-    if (lane == 0) t0 = atomicAdd(p.queue, (unsigned long long)p.trials_per_grab);
-    t0 = __shfl_sync(0xffffffffu, t0, 0);
-    if (t0 >= (unsigned long long)p.n_trials) break;
-    const int64_t t1 = min((int64_t)t0 + p.trials_per_grab, p.n_trials);
-    for (int64_t t = (int64_t)t0; t < t1; ++t) {
-      // The requests covering trial t (warp-uniform): each occurrence walks the part of its row
-      // from the first to the last of them, [fa, la]; a request inside that range that does not
-      // cover t (at most the two middle ones of four, always adjacent) owns the slots
-      // [skip_lo, skip_hi), whose entries are skipped.
-      uint32_t amask = 0;
-      for (int r = 0; r < p.n_req; ++r)
-        if (t >= p.t0[r] && t < p.t1[r]) amask |= 1u << r;
-      if (amask == 0) continue;
-      const int fa = __ffs(amask) - 1, la = 31 - __clz(amask);
-      const uint32_t sh_lo = 8u * (uint32_t)fa, sh_hi = 8u * (uint32_t)la;
-      const uint32_t inner = ((2u << la) - (1u << fa)) & ~amask;   // uncovered, between fa and la
-      const uint32_t skip_lo = inner ? (uint32_t)p.rs.first[__ffs(inner) - 1] : 0u;
-      const uint32_t skip_n =
-          inner ? (uint32_t)p.rs.first[32 - __clz(inner)] - skip_lo : 0u;
-      int64_t beg = __ldg(p.offsets + t), end = __ldg(p.offsets + t + 1);
-      if (!(0 <= beg && beg <= end && end <= p.n_events)) { bad_off = true; beg = end = 0; }
-      // 32 occurrences at a time.  Their rows are laid end to end (a warp scan of the lengths)
-      // and the warp walks the joined list 32 entries per step: every lane has an entry, and
-      // the lanes of one row read consecutive words.  The lane owning item x is the first lane
-      // whose inclusive length sum exceeds x (a 5-step search over the lanes' sums).
-      // Software pipeline over the rounds: the row descriptors of round k + 1 and the event IDs
-      // of round k + 2 are in flight while round k's entries are walked.
-      auto load_id = [&](int64_t i) -> int64_t {   // -1 past the trial's end
-        return i < end ? (int64_t)(uint32_t)__ldcs(p.ids + i) : (int64_t)-1;
-      };
-      auto load_row = [&](int64_t e) -> uint64_t {
-        if (e < 0) return 0ull;
-        if (e >= (int64_t)p.catalogue) { bad_id = true; return 0ull; }
-        return __ldg(p.rows + e);
-      };
-      uint64_t ri_cur = load_row(load_id(beg + lane));
-      int64_t e_nxt = load_id(beg + 32 + lane);
-      // Adds the segment sums of every copy into the trial's totals and clears them.
-      auto flush = [&]() {
-        __syncwarp();
-        for (int i = lane; i < ns; i += 32) {
-          U128 S{tot[i], tot[ns + i]};
-          for (int c = 0; c < nc; ++c) {
-            add_u64(S, acc0[(int64_t)c * ns + i]);
-            acc0[(int64_t)c * ns + i] = 0ull;
-          }
-          tot[i] = S.lo;
-          tot[ns + i] = S.hi;
-        }
-        __syncwarp();
-      };
-      int rounds = 0;
-      for (int64_t i0 = beg; i0 < end; i0 += 32) {
-        const uint64_t ri_nxt = load_row(e_nxt);
-        e_nxt = load_id(i0 + 64 + lane);
-        // byte r of lens * 0x01010101 is the number of entries of requests 0..r (< 256)
-        const uint32_t incl_b = (uint32_t)(ri_cur >> 32) * 0x01010101u;
-        const uint32_t skip_b = ((incl_b << 8) >> sh_lo) & 0xffu;   // entries before request fa
-        const uint32_t rb = (uint32_t)ri_cur + skip_b;
-        const uint32_t len = ((incl_b >> sh_hi) & 0xffu) - skip_b;
-        ri_cur = ri_nxt;
-        uint32_t incl = len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += v;
-        }
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        const uint32_t base = rb - (incl - len);   // entry of item x (in this lane's row): base + x
-        for (uint32_t w0 = 0; w0 < total; w0 += 32) {
-          const uint32_t x = w0 + (uint32_t)lane;
-          int own = 0;
-#pragma unroll
-          for (int step = 16; step >= 1; step >>= 1) {
-            const uint32_t v = __shfl_sync(0xffffffffu, incl, own + step - 1);
-            if (v <= x) own += step;
-          }
-          const uint32_t b = __shfl_sync(0xffffffffu, base, own);
-          if (x < total) {
-            const uint64_t v = __ldg(p.entries + (uint32_t)(b + x));
-            const int s = (int)(v >> 56);
-            if ((uint32_t)s - skip_lo >= skip_n) smem_red_u64(&lo[s], v & ((1ull << 56) - 1));
-          }
-        }
-        if (++rounds == BT_SEG / 32) {
-          flush();
-          rounds = 0;
-        }
-      }
-      __syncwarp();
-      // aggregate terms of every layer on the exact sums; reset the accumulators
-      for (int i = lane; i < ns; i += 32) {
-        U128 S{tot[i], tot[ns + i]};
-        tot[i] = 0ull;
-        tot[ns + i] = 0ull;
-        for (int c = 0; c < nc; ++c) {
-          add_u64(S, acc0[(int64_t)c * ns + i]);
-          acc0[(int64_t)c * ns + i] = 0ull;
-        }
-        const uint32_t r = bt_req_of_slot(p.rs, i);
-        if (!((amask >> r) & 1u)) continue;
-        const LayerConst lc = p.layers[p.sel.layer[i]];
-        uint8_t reg;
-        const double y = AccOps<U128>::finish(S, lc, reg);
-        const int64_t at = (int64_t)(i - p.rs.first[r]) * (p.t1[r] - p.t0[r]) + (t - p.t0[r]);
-        p.ylt[r][at] = y;
-        if (p.regimes[r]) p.regimes[r][at] = reg;
-      }
-      __syncwarp();
-    }
-  }
-  if (bad_id) atomicOr(p.err, DERR_EVENT_RANGE);
-  if (bad_off) atomicOr(p.err, DERR_OFFSETS);
+  if (pos < end) entries[pos] = (uint64_t)n_sel << 56;   // padding: adds 0 to the spare slot
+  rows[e] = (uint64_t)(ptr[e] << first_shift) | ((uint64_t)lens << 32);
 }
 
 }  // namespace ara
@@ -365,14 +193,17 @@ struct ara_plan {
   int64_t req_t0[BT_MAX_REQ] = {0, 0, 0, 0}, req_t1[BT_MAX_REQ] = {0, 0, 0, 0};
   double* req_ylt[BT_MAX_REQ] = {nullptr, nullptr, nullptr, nullptr};
   uint8_t* req_reg[BT_MAX_REQ] = {nullptr, nullptr, nullptr, nullptr};
-  uint32_t* d_ptr = nullptr;
-  uint64_t* d_rows = nullptr;
+  // The rows (d_rows: their descriptors), from the event-major records (by_event) or the folds.
+  bool by_event = false;
+  RowTable rt;
+  RowSchedule sched;
+  ulonglong2* part = nullptr;        // sums between passes (sched.passes > 1)
+  uint32_t* d_ptr = nullptr;         // general way: scan scratch
   uint32_t* d_bsum = nullptr;
-  uint32_t* d_total = nullptr;
-  uint64_t* d_entries = nullptr;
+  uint64_t* d_rows = nullptr;
+  uint32_t* d_total = nullptr;       // [2] pairs of entries taken, entries
   unsigned long long* d_queue = nullptr;
   int64_t n_blocks = 0;
-  int warps = 16, ctas_per_sm = 2, tpg = 2, copies = 2;
   double tuned_ms = 0.0;
   int n_kernels = 0;
   cudaGraph_t graph = nullptr;
@@ -392,6 +223,10 @@ void single_request(ara_plan& P) {
 
 ara_status bt_prep(ara_plan& P, cudaStream_t s, bool fill, int* n_kernels) {
   Portfolio& pf = *P.pf;
+  if (P.by_event) {
+    if (n_kernels) *n_kernels = 1;
+    return launch_rows_build(pf, P.sel, P.rt, P.rs.first, s);
+  }
   const int n_sel = (int)P.sel.size();
   const int64_t C = pf.catalogue;
   FoldOutHost fo;
@@ -403,14 +238,16 @@ ara_status bt_prep(ara_plan& P, cudaStream_t s, bool fill, int* n_kernels) {
   fo.nonzero_only = 1;
   ara_status st = launch_fold_to(pf, n_sel, P.sel.data(), fo, s, false);
   if (st != ARA_OK) return st;
+  ARA_TRY(cudaMemsetAsync(P.d_total, 0, 2 * sizeof(uint32_t), s));
   k_bt_scan_blocks<<<(unsigned)P.n_blocks, BT_SCAN_BLOCK, 0, s>>>(pf.d_bits, pf.bm_words, n_sel, C,
-                                                                  P.d_ptr, P.d_bsum);
+                                                                  P.d_ptr, P.d_bsum, P.d_total + 1);
   k_bt_scan_sums<<<1, BT_SCAN_BLOCK, 0, s>>>(P.d_bsum, P.n_blocks, P.d_total);
   k_bt_scan_add<<<(unsigned)((C + 1 + 255) / 256), 256, 0, s>>>(P.d_ptr, C, P.d_bsum, P.d_total);
   int k = 4;
   if (fill) {
     k_bt_fill<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(n_sel, pf.d_q, pf.d_bits, pf.bm_words, C,
-                                                          P.d_ptr, P.d_entries, P.d_rows, P.rs);
+                                                          P.d_ptr, P.rt.ovf, P.d_rows, P.rs,
+                                                          P.rt.first_shift);
     ++k;
   }
   ARA_TRY(cudaGetLastError());
@@ -418,56 +255,40 @@ ara_status bt_prep(ara_plan& P, cudaStream_t s, bool fill, int* n_kernels) {
   return ARA_OK;
 }
 
-template <int W>
-ara_status bt_launch_w(ara_plan& P, const BtStream& bs, cudaStream_t s) {
-  const int smem = W * (P.copies + 2) * (int)P.sel.size() * 8;
-  const auto fn = k_bt_stream<W>;
-  if (smem > 48 * 1024)
-    ARA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  fn<<<P.pf->n_sms * P.ctas_per_sm, W * 32, smem, s>>>(bs);
-  ARA_TRY(cudaGetLastError());
-  return ARA_OK;
-}
-
 ara_status bt_stream(ara_plan& P, cudaStream_t s) {
-  BtStream bs{};
-  bs.n_trials = P.n_trials;
-  bs.offsets = P.d_off;
-  bs.n_events = P.n_events;
-  bs.ids = P.d_ids;
-  bs.catalogue = (uint32_t)P.pf->catalogue;
-  bs.rows = P.d_rows;
-  bs.entries = P.d_entries;
-  bs.n_sel = (int32_t)P.sel.size();
-  bs.layers = P.pf->d_layers;
-  bs.sel.n_sel = bs.n_sel;
-  for (int i = 0; i < bs.n_sel; ++i) bs.sel.layer[i] = P.sel[i];
-  bs.n_req = P.n_req;
-  bs.rs = P.rs;
-  for (int r = 0; r < BT_MAX_REQ; ++r) {
-    bs.t0[r] = P.req_t0[r];
-    bs.t1[r] = P.req_t1[r];
-    bs.ylt[r] = P.req_ylt[r];
-    bs.regimes[r] = P.req_reg[r];
+  RowsStream r{};
+  r.n_trials = P.n_trials;
+  r.offsets = P.d_off;
+  r.n_events = P.n_events;
+  r.ids = P.d_ids;
+  r.catalogue = (uint32_t)P.pf->catalogue;
+  r.table = P.rt.table;
+  r.ovf = P.rt.ovf;
+  r.desc = P.d_rows;
+  r.first_shift = P.rt.first_shift;
+  r.part = P.part;
+  r.ns = (int32_t)P.sel.size();
+  r.n_req = P.n_req;
+  r.layers = P.pf->d_layers;
+  r.queue = P.d_queue;
+  r.err = P.pf->d_err;
+  for (int q = 0; q < BT_MAX_REQ; ++q) {
+    r.t0[q] = P.req_t0[q];
+    r.t1[q] = P.req_t1[q];
+    r.ylt[q] = P.req_ylt[q];
+    r.regimes[q] = P.req_reg[q];
   }
-  if (!bs.ylt[0]) return ARA_EINVAL;
-  bs.queue = P.d_queue;
-  bs.trials_per_grab = P.tpg;
-  bs.copies = P.copies;
-  bs.err = P.pf->d_err;
-  ARA_TRY(cudaMemsetAsync(P.d_queue, 0, sizeof(unsigned long long), s));
-  switch (P.warps) {
-    case 8: return bt_launch_w<8>(P, bs, s);
-    case 32: return bt_launch_w<32>(P, bs, s);
-    default: return bt_launch_w<16>(P, bs, s);
-  }
+  for (int q = 0; q <= BT_MAX_REQ; ++q) r.first[q] = P.rs.first[q];
+  for (int i = 0; i < r.ns; ++i) r.layer_of[i] = P.sel[(size_t)i];
+  if (!r.ylt[0]) return ARA_EINVAL;
+  return launch_rows_stream(*P.pf, r, P.rt.K, P.sched, s);
 }
 
 void bt_free(ara_plan* P) {
   if (!P) return;
   if (P->exec) cudaGraphExecDestroy(P->exec);
   if (P->graph) cudaGraphDestroy(P->graph);
-  void* ptrs[] = {P->d_ptr, P->d_rows, P->d_bsum, P->d_total, P->d_entries, P->d_queue};
+  void* ptrs[] = {P->d_ptr, P->d_rows, P->d_bsum, P->d_total, P->d_queue, P->rt.table, P->rt.ovf, P->part};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete P;
@@ -527,46 +348,58 @@ ara_status run_batched_group_async(Portfolio& pf, const GroupArgs& g, cudaStream
 }
 
 namespace {
+// Rows of the plan sized by host-known bounds (every non-zero entry of layer i is an event of one
+// of its ELTs), its scratch from the stream-ordered allocator; nothing waits on the host.
 ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
   Portfolio& pf = *P.pf;
   if ((int)P.sel.size() > BT_MAX_LAYERS || (int)P.sel.size() > pf.n_layers ||
       (int64_t)P.sel.size() * pf.catalogue >= ((int64_t)1 << 32))
     return ARA_ERANGE;
-  int64_t bound = 0;
-  for (int32_t l : P.sel) {
-    const LayerConst& lc = pf.layers[l];
-    for (int k = lc.elt_begin; k < lc.elt_end; ++k) {
-      const int j = pf.layer_elts[k];
-      bound += pf.rec_off[j + 1] - pf.rec_off[j];
-    }
-  }
   const int64_t C = pf.catalogue;
-  P.n_blocks = (C + BT_SCAN_BLOCK - 1) / BT_SCAN_BLOCK;
-  size_t off = 0;
-  auto take = [&](size_t n) { size_t o = (off + 255) / 256 * 256; off = o + n; return o; };
-  const size_t o_ptr = take(4 * (size_t)(C + 1)), o_rows = take(8 * (size_t)C);
-  const size_t o_bsum = take(4 * (size_t)P.n_blocks), o_tot = take(4), o_q = take(8);
-  const size_t o_ent = take(8 * (size_t)std::max<int64_t>(bound, 1));
-  char* buf = nullptr;
-  ARA_TRY(dmalloc_async((void**)&buf, off, s));
-  P.d_ptr = (uint32_t*)(buf + o_ptr);
-  P.d_rows = (uint64_t*)(buf + o_rows);
-  P.d_bsum = (uint32_t*)(buf + o_bsum);
-  P.d_total = (uint32_t*)(buf + o_tot);
-  P.d_queue = (unsigned long long*)(buf + o_q);
-  P.d_entries = (uint64_t*)(buf + o_ent);
-  ara_status st = ARA_OK;
-  {
-    LaunchScope ls(ARA_K_BATCHED, s, 6);
-    st = bt_prep(P, s, true, nullptr);
-    if (st == ARA_OK) st = bt_stream(P, s);
+  for (P.by_event = rows_usable(pf, P.sel);; P.by_event = false) {
+    P.rt = RowTable{};
+    P.rt.K = P.by_event && P.n_req == 1 ? rows_k(pf, P.sel) : 0;
+    const RowSizes z = rows_sizes(pf, P.sel, P.rt.K, P.n_trials);
+    P.rt.first_shift = z.first_shift;
+    P.sched = rows_schedule(pf, (int)P.sel.size(), P.rt.K, z.likely_bytes, z.likely_entries,
+                            P.n_trials, P.n_events);
+    P.n_blocks = (C + BT_SCAN_BLOCK - 1) / BT_SCAN_BLOCK;
+    size_t off = 0;
+    auto take = [&](size_t n) { size_t o = (off + 255) / 256 * 256; off = o + n; return o; };
+    const size_t o_rows = P.rt.K == 0 ? take(8 * (size_t)C) : 0;
+    const size_t o_tab = P.rt.K > 0 ? take(8 * (size_t)P.rt.K * (size_t)C) : 0;
+    const size_t o_tot = take(8), o_q = take(8), o_ovf = take(16 * (size_t)z.pairs);
+    const size_t o_ptr = P.by_event ? 0 : take(4 * (size_t)(C + 1));
+    const size_t o_bsum = P.by_event ? 0 : take(4 * (size_t)P.n_blocks);
+    const size_t o_part = P.sched.passes > 1 ? take(16 * (size_t)P.n_trials * P.sel.size()) : 0;
+    char* buf = nullptr;
+    if (dmalloc_async((void**)&buf, off, s) != cudaSuccess) {
+      cudaGetLastError();
+      if (P.by_event) continue;      // the general way needs less
+      return ARA_ENOMEM;
+    }
+    if (P.rt.K == 0) P.d_rows = (uint64_t*)(buf + o_rows);
+    else P.rt.table = (uint64_t*)(buf + o_tab);
+    P.d_total = (uint32_t*)(buf + o_tot);
+    P.d_queue = (unsigned long long*)(buf + o_q);
+    P.rt.ovf = (uint64_t*)(buf + o_ovf);
+    P.rt.ovf_pairs = (uint32_t)std::min<int64_t>(z.pairs, UINT32_MAX);
+    P.rt.counters = P.d_total;
+    P.rt.desc = P.d_rows;
+    if (!P.by_event) {
+      P.d_ptr = (uint32_t*)(buf + o_ptr);
+      P.d_bsum = (uint32_t*)(buf + o_bsum);
+    }
+    if (P.sched.passes > 1) P.part = (ulonglong2*)(buf + o_part);
+    ara_status st = ARA_OK;
+    {
+      LaunchScope ls(ARA_K_BATCHED, s, (P.by_event ? 1 : 5) + P.sched.passes);
+      st = bt_prep(P, s, true, nullptr);
+      if (st == ARA_OK) st = bt_stream(P, s);
+    }
+    cudaFreeAsync(buf, s);
+    return st;
   }
-  cudaFreeAsync(buf, s);
-  P.d_ptr = P.d_bsum = P.d_total = nullptr;
-  P.d_rows = nullptr;
-  P.d_entries = nullptr;
-  P.d_queue = nullptr;
-  return st;
 }
 }  // namespace
 }  // namespace ara
@@ -619,64 +452,78 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
     bt_free(P);
     return st;
   };
-  if (cudaMalloc(&P->d_ptr, 4 * (size_t)(C + 1)) != cudaSuccess ||
-      cudaMalloc(&P->d_rows, 8 * (size_t)std::max<int64_t>(C, 1)) != cudaSuccess ||
-      cudaMalloc(&P->d_bsum, 4 * (size_t)P->n_blocks) != cudaSuccess ||
-      cudaMalloc(&P->d_total, 4) != cudaSuccess ||
-      cudaMalloc(&P->d_queue, sizeof(unsigned long long)) != cudaSuccess)
+  P->by_event = rows_usable(*pf, P->sel);
+  P->rt.K = P->by_event ? rows_k(*pf, P->sel) : 0;
+  const RowSizes z = rows_sizes(*pf, P->sel, P->rt.K, n_trials);
+  P->rt.first_shift = z.first_shift;
+  if ((P->rt.K > 0 && cudaMalloc(&P->rt.table, 8 * (size_t)P->rt.K * (size_t)C) != cudaSuccess) ||
+      cudaMalloc(&P->d_rows, 8 * (size_t)C) != cudaSuccess || cudaMalloc(&P->d_total, 8) != cudaSuccess ||
+      cudaMalloc(&P->d_queue, sizeof(unsigned long long)) != cudaSuccess ||
+      (!P->by_event && (cudaMalloc(&P->d_ptr, 4 * (size_t)(C + 1)) != cudaSuccess ||
+                        cudaMalloc(&P->d_bsum, 4 * (size_t)P->n_blocks) != cudaSuccess)))
     return fail(ARA_ENOMEM);
-  // size the table once: the counts depend on the portfolio only
+  P->rt.counters = P->d_total;
+  P->rt.desc = P->d_rows;
+  // size the table once (a first build has no room and only counts): the counts depend on the
+  // portfolio only
   ara_status st = bt_prep(*P, s, false, nullptr);
   if (st != ARA_OK) return fail(st);
-  uint32_t total = 0;
-  if (cudaMemcpyAsync(&total, P->d_total, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  uint32_t total[2] = {0, 0};
+  if (cudaMemcpyAsync(total, P->d_total, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return fail(ARA_ECUDA);
-  if (cudaMalloc(&P->d_entries, 8 * (size_t)std::max<uint32_t>(total, 1)) != cudaSuccess)
-    return fail(ARA_ENOMEM);
+  if (cudaMalloc(&P->rt.ovf, 16 * (size_t)std::max<uint32_t>(total[0], 1)) != cudaSuccess) return fail(ARA_ENOMEM);
+  P->rt.ovf_pairs = total[0];
   if ((st = bt_prep(*P, s, true, nullptr)) != ARA_OK) return fail(st);
-  // schedule: the fastest of the candidates on these inputs, or a fixed default
-  if (flags & ARA_PLAN_AUTOTUNE) {
+  const int64_t table_bytes = 8 * C * std::max(P->rt.K, 1) + 16 * (int64_t)total[0];
+  P->sched = rows_schedule(*pf, (int)P->sel.size(), P->rt.K, table_bytes, (double)total[1] / (double)C,
+                           n_trials, n_events);
+  const size_t part_bytes = 16 * (size_t)n_trials * P->sel.size();
+  const bool tune = (flags & ARA_PLAN_AUTOTUNE) != 0;
+  // room for the sums between passes: where the rule takes several, or where they are tried
+  const bool try_passes = tune && P->rt.K == 0 && table_bytes > RW_PASS_BYTES / 2;
+  if ((P->sched.passes > 1 || try_passes) && cudaMalloc(&P->part, part_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    P->part = nullptr;
+    P->sched.passes = 1;
+  }
+  // schedule: the fastest of the candidates on these inputs, or the rule's
+  if (tune) {
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return fail(ARA_ECUDA);
-    const int cand_w[] = {8, 16, 32};
-    const int cand_c[] = {1, 2, 4};
-    const int cand_t[] = {1, 4};
-    const int cand_k[] = {1, 2, 4};
-    float best = 1e30f;
-    int bw = P->warps, bc = P->ctas_per_sm, bt = P->tpg, bk = P->copies;
-    for (int w : cand_w)
-      for (int c : cand_c)
-        for (int t : cand_t)
-          for (int k : cand_k) {
-          const int64_t smem = (int64_t)w * (k + 2) * (int64_t)P->sel.size() * 8;
-          if (smem * c > (int64_t)pf->max_smem_block || w * 32 * c > 2048) continue;
-          P->warps = w;
-          P->ctas_per_sm = c;
-          P->tpg = t;
-          P->copies = k;
-          float ms = 0.f, tot = 0.f;
-          for (int rep = 0; rep < 3; ++rep) {
-            cudaEventRecord(a, s);
-            if ((st = bt_stream(*P, s)) != ARA_OK) {
-              cudaEventDestroy(a);
-              cudaEventDestroy(b);
-              return fail(st);
-            }
-            cudaEventRecord(b, s);
-            if (cudaEventSynchronize(b) != cudaSuccess) return fail(ARA_ECUDA);
-            cudaEventElapsedTime(&ms, a, b);
-            if (rep > 0) tot += ms;
-          }
-          if (tot / 2 < best) { best = tot / 2; bw = w; bc = c; bt = t; bk = k; }
+    const RowSchedule rule = P->sched;
+    RowSchedule best = rule;
+    float best_ms = 1e30f;
+    for (int nc : {4, 8, 16, 32})
+      for (int passes : {1, 2, 3}) {
+        if (nc > 2 * rule.nc || 2 * nc < rule.nc) continue;
+        if (passes > 1 && !(try_passes && P->part)) continue;
+        P->sched = RowSchedule{nc, passes, 0};
+        float ms = 0.f, tot = 0.f;
+        for (int rep = 0; rep < 3 && st == ARA_OK; ++rep) {
+          cudaEventRecord(a, s);
+          st = bt_stream(*P, s);
+          cudaEventRecord(b, s);
+          if (st == ARA_OK && cudaEventSynchronize(b) != cudaSuccess) st = ARA_ECUDA;
+          cudaEventElapsedTime(&ms, a, b);
+          if (rep > 0) tot += ms;
         }
+        if (st == ARA_ERANGE) { st = ARA_OK; continue; }   // too wide for a block's shared memory
+        if (st != ARA_OK) {
+          cudaEventDestroy(a);
+          cudaEventDestroy(b);
+          return fail(st);
+        }
+        if (tot / 2 < best_ms) { best_ms = tot / 2; best = P->sched; }
+      }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
-    P->warps = bw;
-    P->ctas_per_sm = bc;
-    P->tpg = bt;
-    P->copies = bk;
-    P->tuned_ms = best;
+    P->sched = best;
+    P->tuned_ms = best_ms;
+  }
+  if (P->sched.passes == 1 && P->part) {
+    cudaFree(P->part);
+    P->part = nullptr;
   }
   // capture the whole run into a graph on a private stream
   cudaStream_t cs;
@@ -696,7 +543,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
     return fail(ARA_ECUDA);
   }
   P->graph = graph;
-  P->n_kernels = nk + 1;
+  P->n_kernels = nk + P->sched.passes;
   if (cudaGraphInstantiate(&P->exec, graph, 0) != cudaSuccess) return fail(ARA_ECUDA);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(ARA_ECUDA);
   *out = P;
@@ -749,11 +596,11 @@ ara_status ara_plan_launch(ara_plan* P, void* stream) {
 ara_status ara_plan_info(ara_plan* P, int32_t* warps, int32_t* bpsm, int32_t* tpg, double* ms,
                          int32_t* copies) {
   if (!P) return ARA_EINVAL;
-  if (warps) *warps = P->warps;
-  if (bpsm) *bpsm = P->ctas_per_sm;
-  if (tpg) *tpg = P->tpg;
+  if (warps) *warps = RW_WARPS;
+  if (bpsm) *bpsm = P->sched.blocks;
+  if (tpg) *tpg = 1;
   if (ms) *ms = P->tuned_ms;
-  if (copies) *copies = P->copies;
+  if (copies) *copies = std::min(P->sched.nc, 4);
   return ARA_OK;
 }
 
@@ -764,7 +611,7 @@ ara_status ara_plan_table(ara_plan* P, const uint64_t** d_rows, int64_t* n_entri
   if (n_entries) {
     uint32_t total = 0;
     ARA_TRY(cudaDeviceSynchronize());
-    ARA_TRY(cudaMemcpy(&total, P->d_total, 4, cudaMemcpyDeviceToHost));
+    ARA_TRY(cudaMemcpy(&total, P->d_total + 1, 4, cudaMemcpyDeviceToHost));
     *n_entries = total;
   }
   return ARA_OK;

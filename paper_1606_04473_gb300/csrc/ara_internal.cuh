@@ -82,6 +82,8 @@ struct LayerConst {
 // of every tile so that the fold reads each tile's record range instead of searching for it.
 constexpr int FOLD_TILE = 2048;
 
+constexpr int RW_MASK = 4;             // 64-bit words of a layer mask (ara_rows.cu)
+
 struct Portfolio {
   bool borrowed_elts = false;       // a layer set: ELT tables belong to a resident pool
   cudaStream_t owner_stream = nullptr;  // layer sets: stream their buffers were allocated on
@@ -108,6 +110,14 @@ struct Portfolio {
   int64_t* d_tile_rec = nullptr;    // [n_elts][n_tiles + 1]: first record of each ELT per tile
   int32_t* d_layer_elts = nullptr;  // [layer_off[n_layers]]
   LayerConst* d_layers = nullptr;   // [n_layers]
+  // the records again, event by event (ELTs ascending within an event), or null: [C + 1] first
+  // record of every event, and per record its ELT and loss (float or double as stored above)
+  uint32_t* d_ev_ptr = nullptr;
+  int32_t* d_ev_elt = nullptr;
+  void* d_ev_loss = nullptr;
+  // the layers that hold each ELT: [n_elts][RW_MASK] bits, bit l = layer l (up to 255 layers; null)
+  uint64_t* d_mem = nullptr;
+  std::vector<uint8_t> layer_asc;   // per layer: its ELTs are listed in strictly ascending order
   void* d_dense = nullptr;          // [n_elts][catalogue] float or double (ARA_DENSE_TABLES)
   // per-layer fold workspace
   uint64_t* d_q = nullptr;          // [n_layers][catalogue]: q(e) (or o(e) bits for F64_SUM)
@@ -210,6 +220,69 @@ ara_status run_batched_group_async(Portfolio& pf, const GroupArgs& g, cudaStream
 // event-major table): ptr [n + 1], block_sums [ceil(n / 1024)], total [1].
 ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t n_sel, int64_t n,
                              uint32_t* ptr, uint32_t* block_sums, uint32_t* total, cudaStream_t s);
+// Event-major rows and their stream (ara_rows.cu).
+constexpr int RW_MAX_LAYERS = 255;
+constexpr int RW_BUILD_THREADS = 128;
+constexpr int RW_BUILD_SUMS = 2560;            // sums a block of the build holds at a time (20 KB)
+constexpr int64_t RW_MAX_CATALOGUE = (int64_t)1 << 27;
+constexpr int RW_WARPS = 8;                    // warps per block of the streams
+constexpr int RW_MIN_BLOCKS = 4;               // blocks per SM their registers allow
+constexpr int64_t RW_PASS_BYTES = 72ll << 20;  // table bytes per pass (see rows_schedule)
+struct RowTable {
+  int K = 0;                        // entries per row
+  uint64_t* table = nullptr;        // [catalogue][K]
+  uint64_t* ovf = nullptr;          // [2 * ovf_pairs]
+  uint32_t ovf_pairs = 0;
+  uint32_t* counters = nullptr;     // [2]: overflow pairs taken, entries
+  uint64_t* desc = nullptr;         // [catalogue] (optional when K > 0)
+  int first_shift = 1;              // descriptors name the first entry (1) or the first pair (0)
+};
+// How the stream runs: columns of sums per warp, passes over the YET.
+struct RowSchedule {
+  int nc = 8, passes = 1;
+  int blocks = 0;                   // blocks per SM of the last launch
+};
+struct RowSizes {
+  int64_t pairs = 1;                // upper bound of the overflow list (K = 0: of all rows), in pairs
+  int first_shift = 1;
+  double likely_entries = 0.0;      // entries per event, roughly
+  int64_t likely_bytes = 0;         // table and descriptors, roughly
+};
+struct RowsStream {
+  int64_t n_trials;
+  const int64_t* offsets;
+  int64_t n_events;
+  const int32_t* ids;
+  uint32_t catalogue;
+  const uint64_t* table;
+  const uint64_t* ovf;
+  const uint64_t* desc;             // K = 0: [catalogue] first entry | entries per request << 32
+  ulonglong2* part;                 // n_pass > 1: [n_trials][ns] sums so far
+  int32_t pass, n_pass;
+  int32_t first_shift;              // as RowTable
+  uint32_t e_lo, e_n;               // events of this pass
+  int32_t ns;
+  int32_t n_req;
+  const LayerConst* layers;
+  unsigned long long* queue;
+  uint32_t* err;
+  int64_t t0[4], t1[4];             // requests as in GroupArgs (one: all trials)
+  double* ylt[4];
+  uint8_t* regimes[4];
+  int32_t first[5];                 // first slot of each request; unused ones past every slot
+  int32_t layer_of[RW_MAX_LAYERS];  // slot -> layer
+};
+ara_status build_event_index(Portfolio& pf, cudaStream_t s);
+bool rows_usable(const Portfolio& pf, const std::vector<int32_t>& sel);
+int64_t rows_bound(const Portfolio& pf, const std::vector<int32_t>& sel);
+int rows_k(const Portfolio& pf, const std::vector<int32_t>& sel);
+RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K, int64_t n_trials);
+RowSchedule rows_schedule(const Portfolio& pf, int ns, int K, int64_t table_bytes, double entries,
+                          int64_t n_trials, int64_t n_events);
+ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, const RowTable& rt, const int32_t* first,
+                             cudaStream_t s);
+ara_status launch_rows_stream(Portfolio& pf, const RowsStream& p, int K, RowSchedule& sched, cudaStream_t s);
+
 ara_status build_dense(Portfolio& pf, cudaStream_t s);
 // Compiled shapes (warps per block, ring stages) of the bulk-staged YET stream kernel.
 int32_t n_bulk_shapes();

@@ -100,7 +100,11 @@ int64_t estimate_bytes(const Portfolio& pool, const Request& r) {
   {   // batched table (every request may run in a merged batched pass)
     int64_t bound = 0;
     for (int32_t j : r.layer_elts) bound += pool.rec_off[j + 1] - pool.rec_off[j];
-    b += 12 * C + 8 * bound;
+    // its rows: end to end with descriptors and scan scratch, or in place with an overflow list
+    // (ara_rows.cu), and the sums between passes of a large table
+    const int64_t packed = 12 * C + 8 * (bound + std::min(bound, C));
+    b += std::max(packed, 32 * C + 12 * bound);
+    if (packed > RW_PASS_BYTES) b += 16 * nl * n;
   }
   if (r.want_adjoint) {
     int64_t recs = 0;

@@ -1,0 +1,137 @@
+"""Several layers in one pass over event-major rows: every form of the rows (kept in place 1, 2 or
+4 entries to an event, or end to end; one pass or several; 4 to 32 columns of sums) against the
+single-layer path, bit for bit (both paths sum the same integers exactly, so no tolerance)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_1606_04473_gb300 as ara
+
+
+def make(seed, C, n_elts, nnz, layers, f32, trials, events, mult=1.0):
+    """A portfolio of `layers` (lists of ELTs) and a ragged YET with empty and one-event trials; layer
+    terms at multiples of typical losses so that all clamp regimes occur."""
+    g = np.random.default_rng(seed)
+    ids = [g.choice(C, size=min(nnz, C), replace=False).astype(np.int32) for _ in range(n_elts)]
+    loss = [np.exp(11.0 + 2.0 * g.standard_normal(i.size)) for i in ids]
+    if f32:
+        loss = [x.astype(np.float32).astype(np.float64) for x in loss]
+    ret = np.array([np.percentile(x, 20) for x in loss])
+    lim = np.array([np.percentile(x, 95) for x in loss])
+    lim[::7] = np.inf
+    n = len(layers)
+    occ_r = g.uniform(0.0, 2e5, n)
+    occ_r[::5] = 0.0
+    pf = ara.Portfolio(C, ids, loss, ret, lim, layers, occ_r, g.uniform(1e5, 3e6, n),
+                       g.uniform(0.0, 1e6, n) * mult, g.uniform(1e6, 5e7, n) * mult, losses_f32=f32)
+    counts = g.poisson(events, trials)
+    counts[:6] = [0, 1, 0, 31, 32, 33]
+    counts[-1] = 0
+    off = np.zeros(trials + 1, np.int64)
+    np.cumsum(counts, out=off[1:])
+    yet = g.integers(0, C, off[-1], dtype=np.int32)
+    return pf, torch.from_numpy(off).cuda(), torch.from_numpy(yet).cuda()
+
+
+def singles(pf, off, ids, sel):
+    n = off.numel() - 1
+    reg = torch.empty((len(sel), n), dtype=torch.uint8, device="cuda")
+    ys = []
+    for i, l in enumerate(sel):
+        r = torch.empty((1, n), dtype=torch.uint8, device="cuda")
+        ys.append(pf.run_ylt(off, ids, layers=[l], regimes=r)[0])
+        reg[i] = r[0]
+    pf.check()
+    return torch.stack(ys), reg
+
+
+def own(g, n_layers, n_elts, lo, hi):
+    return [sorted(g.choice(n_elts, size=int(g.integers(lo, hi + 1)), replace=False).tolist())
+            for _ in range(n_layers)]
+
+
+# (catalogue, ELTs, records per ELT, layers, ELTs per layer, f32, trials, events per trial): the
+# number of entries per event decides the form (in place 1, 2, 4; end to end), the number of
+# layers the columns (up to 18: 32, 37-40: 16, 74: 8, else 4)
+FORMS = [
+    (5_003, 6, 200, 2, (1, 2), False, 700, 90.0),        # 1 in place, overflow rare
+    (20_011, 12, 1_500, 9, (1, 3), True, 900, 120.0),    # 2 in place
+    (4_096, 24, 300, 16, (2, 4), True, 501, 700.0),      # 4 in place, catalogue of whole tiles
+    (3_000, 30, 1_400, 24, (5, 25), False, 400, 1200.0), # end to end, long rows, several drains
+    (2_049, 40, 500, 64, (3, 30), True, 300, 300.0),     # end to end, 8 columns
+    (1_000, 20, 700, 130, (1, 20), False, 200, 150.0),   # 4 columns, 130 layers, dense
+    (777, 8, 777, 255, (1, 8), True, 65, 40.0),          # every event in every ELT, 255 layers
+    (40, 3, 40, 3, (1, 3), True, 2_000, 3.0),            # a catalogue of one warp, short trials
+]
+
+
+@pytest.mark.parametrize("form", range(len(FORMS)))
+def test_rows_equal_single_layer_runs(form):
+    C, n_elts, nnz, n_layers, (lo, hi), f32, trials, events = FORMS[form]
+    layers = own(np.random.default_rng(form), n_layers, n_elts, lo, hi)
+    pf, off, ids = make(form, C, n_elts, nnz, layers, f32, trials, events)
+    every = list(range(n_layers))
+    ref, reg_ref = singles(pf, off, ids, every)
+    assert 0 < int((reg_ref == 1).sum())
+    some = every[::-1][: max(2, n_layers // 2)]          # a selection that is not in order
+    for sel, autotune in ((every, False), (every, True), (some, False)):
+        reg = torch.full((len(sel), trials), 9, dtype=torch.uint8, device="cuda")
+        plan = ara.BatchedPlan(pf, off, ids, layers=sel, regimes=reg, autotune=autotune)
+        y = plan.launch()
+        pf.check()
+        idx = torch.tensor(sel, device="cuda")
+        assert torch.equal(y, ref[idx]) and torch.equal(reg, reg_ref[idx])
+        rows, n_entries = plan.table()
+        assert int(((rows >> 32) & 0xff).sum()) == n_entries
+        plan.close()
+        a = pf.run_ylt(off, ids, layers=sel, flags=ara.ARA_RUN_BATCHED)
+        pf.check()
+        assert torch.equal(a, ref[idx])
+    pf.close()
+
+
+def test_layers_in_any_elt_order_take_the_general_way():
+    """Layers that do not list their ELTs in ascending order (or twice) keep their own order of the
+    FP64 ELT sum: rows from the per-layer folds, equal to the single-layer runs."""
+    g = np.random.default_rng(3)
+    layers = [g.permutation(12)[:7].tolist() for _ in range(11)] + [[4, 4, 1], []]
+    pf, off, ids = make(5, 4_000, 12, 900, layers, True, 333, 400.0)
+    sel = list(range(len(layers)))
+    ref, reg_ref = singles(pf, off, ids, sel)
+    reg = torch.empty_like(reg_ref)
+    plan = ara.BatchedPlan(pf, off, ids, regimes=reg, autotune=False)
+    assert torch.equal(plan.launch(), ref) and torch.equal(reg, reg_ref)
+    rows, n_entries = plan.table()
+    assert int(((rows >> 32) & 0xff).sum()) == n_entries
+    plan.close()
+    pf.close()
+
+
+@pytest.mark.parametrize("shape", [(2_000_000, 60, 20_000, 70, 4, 18), (1_500_000, 80, 30_000, 120, 3, 20)])
+def test_tables_beyond_l2_run_in_several_passes(shape):
+    """Tables large enough for several passes over the YET (8 and 4 columns): sums carried from
+    pass to pass, equal to the single-layer runs; IDs outside the catalogue are still reported."""
+    C, n_elts, nnz, n_layers, lo, hi = shape
+    layers = own(np.random.default_rng(1), n_layers, n_elts, lo, hi)
+    pf, off, ids = make(2, C, n_elts, nnz, layers, True, 1_500, 900.0, mult=3.0)
+    sel = [0, n_layers // 2, n_layers - 1]
+    ref, reg_ref = singles(pf, off, ids, sel)
+    for autotune in (False, True):
+        reg = torch.empty((n_layers, off.numel() - 1), dtype=torch.uint8, device="cuda")
+        plan = ara.BatchedPlan(pf, off, ids, regimes=reg, autotune=autotune)
+        y = plan.launch()
+        pf.check()
+        assert torch.equal(y[sel], ref) and torch.equal(reg[sel], reg_ref)
+        plan.close()
+    bad = ids.clone()
+    bad[12_345] = C
+    plan = ara.BatchedPlan(pf, off, bad, autotune=False)
+    plan.launch()
+    with pytest.raises(ara.AraError) as ei:
+        pf.check()
+    assert ei.value.status == ara.ARA_EDATA
+    plan.close()
+    pf.close()
