@@ -173,6 +173,9 @@ ARA_API ara_status ara_create_layer_set(ara_portfolio* pool, int32_t n_layers,
  *                    2: S > AggR + AggL), recorded for ara_adjoint
  *   flags            ARA_RUN_* (one of FOLDED / PER_ELT, optionally NO_FILTER, F64_SUM; PREPARED
  *                    and SLOT1 to stream against a fold queued by ara_prepare_ylt)
+ * With flags 0, several layers may run in one pass over event-major rows (as ARA_RUN_BATCHED) where
+ * that is expected to be faster: the same results, with scratch in stream order from the library's
+ * memory pool (without room for it, and while `stream` is being captured, layer by layer).
  * Errors: ARA_EINVAL (also: ARA_RUN_SLOT1 before slot 1 was ever prepared), ARA_ECUDA; data
  * errors via ara_check().
  */

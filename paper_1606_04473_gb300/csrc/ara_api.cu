@@ -672,11 +672,35 @@ ara_status ara_prepare_ylt(ara_portfolio* pf, int32_t n_sel, const int32_t* laye
   return launch_coarsen(*pf, (int32_t)sel.size(), sel.data(), flags, s, slot);
 }
 
-ara_status ara_run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets,
-                       int64_t n_events, const int32_t* d_ids, const float* d_timestamps,
-                       int32_t n_sel, const int32_t* layer_sel, double* d_ylt, uint8_t* d_regimes,
-                       int32_t flags, void* stream) {
-  (void)d_timestamps;
+// Whether an ordinary run of several layers is faster over event-major rows (one pass for all
+// layers, the same results) than layer by layer.  Both costs in microseconds, fitted to runs of
+// 2-250 layers over 1e4-2.5e6 events, 5e4-1e9 occurrences: the per-layer stream takes 1.0 ps per
+// occurrence, 0.17 ns per trial and 8 us per layer, its folds 6 ps per event and layer and 20 ps
+// per record; the rows 20 ps per event and 18 ps per record to build, then 5.5 ps per occurrence and
+// 0.7 (rows in place) or 2.2 (rows end to end) per entry of its event, and 0.035 ns per trial and
+// layer.  At 2e8 occurrences of 2 M events the line lies at 4-5 layers (4 layers: 1.07 ms layer by
+// layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
+static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, int64_t n_trials, int64_t events) {
+  if (sel.size() < 2 || !rows_usable(pf, sel)) return false;
+  const int K = rows_k(pf, sel);
+  const RowSizes z = rows_sizes(pf, sel, K, n_trials);
+  const double C = (double)pf.catalogue, L = (double)sel.size(), ev = (double)events, tr = (double)n_trials;
+  double rec = 0.0;
+  for (int32_t l : sel)
+    for (int k = pf.layer_off[(size_t)l]; k < pf.layer_off[(size_t)l + 1]; ++k) {
+      const size_t j = (size_t)pf.layer_elts[(size_t)k];
+      rec += (double)(pf.rec_off[j + 1] - pf.rec_off[j]);
+    }
+  const double layers = L * (8.0 + 1e-6 * ev + 0.17e-3 * tr + 6e-6 * C) + 20e-6 * rec;
+  const double rows = 16.0 + 20e-6 * C + 18e-6 * rec + 1e-6 * ev * (5.5 + (K ? 0.7 : 2.2) * z.likely_entries) +
+                      0.035e-3 * tr * L;
+  return rows < 0.92 * layers;
+}
+
+static ara_status run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets,
+                          int64_t n_events, const int32_t* d_ids, int32_t n_sel,
+                          const int32_t* layer_sel, double* d_ylt, uint8_t* d_regimes, int32_t flags,
+                          bool rows_ok, void* stream) {
   if (!pf || n_trials < 0 || n_events < 0 || n_trials > ((int64_t)1 << 40)) return ARA_EINVAL;
   std::vector<int32_t> sel;
   ara_status st = check_selection(*pf, n_sel, layer_sel, sel);
@@ -691,8 +715,12 @@ ara_status ara_run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_off
   const bool prepared = (flags & ARA_RUN_PREPARED) != 0;
   const int slot = (flags & ARA_RUN_SLOT1) ? 1 : 0;
   if (slot == 1 && !pf->d_q_alt) return ARA_EINVAL;   // slot 1 never prepared
-  if (!prepared && !(flags & (ARA_RUN_PER_ELT | ARA_RUN_BATCHED))) {
-    if ((st = launch_fold(*pf, (int32_t)sel.size(), sel.data(), flags, s)) != ARA_OK) return st;
+  // An ordinary run of several layers may take the event-major rows.  They need scratch, so a run
+  // that is being captured stays with the per-layer kernels.
+  bool rows = false;
+  if (rows_ok && flags == 0 && rows_faster(*pf, sel, n_trials, n_events)) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    rows = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
   }
   YltArgs a{};
   a.slot = slot;
@@ -709,7 +737,36 @@ ara_status ara_run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_off
   a.row_stride = n_trials;
   a.flags = flags;
   if (flags & ARA_RUN_BATCHED) return run_batched_async(*pf, a, s);
+  if (rows) {
+    st = run_batched_async(*pf, a, s);
+    if (st == ARA_OK) {
+      pf->fold0_missing.resize((size_t)pf->n_layers, 0);
+      for (int32_t l : sel) pf->fold0_missing[(size_t)l] = 1;
+    }
+    if (st != ARA_ENOMEM) return st;   // no room for the rows: layer by layer
+  }
+  if (!prepared && !(flags & ARA_RUN_PER_ELT)) {
+    if ((st = launch_fold(*pf, (int32_t)sel.size(), sel.data(), flags, s)) != ARA_OK) return st;
+  }
+  if (prepared && slot == 0 && !pf->fold0_missing.empty()) {
+    std::vector<int32_t> miss;
+    for (int32_t l : sel)
+      if (pf->fold0_missing[(size_t)l] && std::find(miss.begin(), miss.end(), l) == miss.end()) miss.push_back(l);
+    const int32_t f = flags & ~(ARA_RUN_PREPARED | ARA_RUN_F64_SUM);   // as the unprepared run folded
+    if (!miss.empty() &&
+        ((st = launch_fold(*pf, (int32_t)miss.size(), miss.data(), f, s)) != ARA_OK ||
+         (st = launch_coarsen(*pf, (int32_t)miss.size(), miss.data(), f, s, 0)) != ARA_OK))
+      return st;
+  }
   return launch_ylt(*pf, a, s);
+}
+
+ara_status ara_run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets,
+                       int64_t n_events, const int32_t* d_ids, const float* d_timestamps,
+                       int32_t n_sel, const int32_t* layer_sel, double* d_ylt, uint8_t* d_regimes,
+                       int32_t flags, void* stream) {
+  (void)d_timestamps;
+  return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, n_sel, layer_sel, d_ylt, d_regimes, flags, true, stream);
 }
 
 ara_status ara_check(ara_portfolio* pf, void* stream) {
@@ -954,3 +1011,10 @@ ara_status ara_run_ylt_host(ara_portfolio* pf, int64_t n_trials, const int64_t* 
 }
 
 }  // extern "C"
+
+namespace ara {
+ara_status run_ylt_per_layer(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets, int64_t n_events,
+                             const int32_t* d_ids, double* d_ylt, uint8_t* d_regimes, int32_t flags, void* stream) {
+  return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, 0, nullptr, d_ylt, d_regimes, flags, false, stream);
+}
+}  // namespace ara

@@ -130,6 +130,9 @@ struct Portfolio {
   uint64_t* d_q_alt = nullptr;
   uint32_t* d_bits_alt = nullptr;
   uint32_t* d_cbits_alt = nullptr;
+  // layers whose slot 0 lacks the fold of the last unprepared run (that run took the event-major
+  // rows instead): a prepared run of slot 0 folds them first
+  std::vector<uint8_t> fold0_missing;
   uint32_t* d_err = nullptr;        // device error word
   // host-input pipeline resources (grown on demand)
   cudaStream_t copy_stream = nullptr;
@@ -356,6 +359,13 @@ struct YetIndex {
 // The opaque handle of the C ABI is the portfolio itself.
 struct ara_portfolio : public ara::Portfolio {};
 struct ara_yet_index : public ara::YetIndex {};
+
+namespace ara {
+// ara_run_ylt of every layer that stays with the per-layer kernels (the server: its workers' short
+// kernels share the device better between the passes of others).
+ara_status run_ylt_per_layer(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets, int64_t n_events,
+                             const int32_t* d_ids, double* d_ylt, uint8_t* d_regimes, int32_t flags, void* stream);
+}  // namespace ara
 
 namespace ara {
 

@@ -211,8 +211,7 @@ void run_request(ara_server& S, Request& r, cudaStream_t s) {
     st = ARA_ENOMEM;
   if (st == ARA_OK)
     st = chained_pass(S, s, [&] {
-      return ara_run_ylt(ls, n, S.d_off + r.t0, S.n_events, S.d_ids, nullptr, 0, nullptr, ylt, reg,
-                         r.flags, s);
+      return run_ylt_per_layer(ls, n, S.d_off + r.t0, S.n_events, S.d_ids, ylt, reg, r.flags, s);
     });
   if (st == ARA_OK) st = finish_request(S, r, ls, 0, ylt, reg, s);
   if (st == ARA_OK) st = ara_check(ls, s);

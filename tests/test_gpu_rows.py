@@ -135,3 +135,36 @@ def test_tables_beyond_l2_run_in_several_passes(shape):
     assert ei.value.status == ara.ARA_EDATA
     plan.close()
     pf.close()
+
+
+def test_run_of_several_layers_takes_the_rows_and_keeps_prepared_runs():
+    """An ordinary run of many layers goes through the rows (two kernels, whatever the number of
+    layers) and equals the single-layer runs; a prepared run right after it, without a prepare of
+    its own, still streams against the folds of those layers; a run being captured stays with the
+    per-layer kernels and replays the same values."""
+    g = np.random.default_rng(8)
+    pf, off, ids = make(9, 50_000, 40, 3_000, own(g, 20, 40, 5, 20), True, 2_000, 500.0)
+    sel = list(range(20))
+    ref, reg_ref = singles(pf, off, ids, sel)
+    reg = torch.empty_like(reg_ref)
+    n0 = ara.launch_count()
+    y = pf.run_ylt(off, ids, regimes=reg)
+    assert ara.launch_count() - n0 <= 3
+    assert torch.equal(y, ref) and torch.equal(reg, reg_ref)
+    for layers in ([7, 3], sel):
+        z = pf.run_ylt(off, ids, layers=layers, flags=ara.ARA_RUN_PREPARED)
+        assert torch.equal(z, ref[layers])
+    pf.check()
+    s = torch.cuda.Stream()
+    out = torch.zeros_like(ref)
+    graph = torch.cuda.CUDAGraph()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=s):
+        pf.run_ylt(off, ids, out=out, stream=s)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+    pf.check()
+    pf.close()
