@@ -304,6 +304,8 @@ int32_t adjoint_per_layer();
 // Host check of risk-metric arguments (ranks within [1, n]); ARA_OK or ARA_EINVAL.
 ara_status validate_metrics(int64_t n, int32_t n_rp, const double* rps, int32_t n_tvar,
                             const double* levels);
+// Scratch of a selection of n_t targets in each of n_layers rows of n values.
+size_t select_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_t, int n_sms);
 // m = ceil(N (1 - p)) with the library's integer snapping; -1 when p is outside [0, 1).
 int64_t tail_count_snap(int64_t n, double p);
 // The m-th largest value of each of n_layers device rows: its order key (device, stride
@@ -326,10 +328,12 @@ ara_status risk_metrics_queue(const double* d_ylt, int64_t n_trials, int32_t n_l
                               double* d_pml, double* d_tvar, double* d_mean, uint32_t* d_status,
                               void* scratch, size_t scratch_bytes, size_t* need, cudaStream_t s);
 // PML / TVaR of n_layers device YLT rows into host arrays (synchronises s); scratch from the
-// stream-ordered allocator.
+// stream-ordered allocator.  beside: blocks that run beside other streams' kernels, no cooperative
+// launch (the server).
 ara_status risk_metrics_device(const double* d_ylt, int64_t n, int32_t n_layers, int32_t n_rp,
                                const double* rps, int32_t n_tvar, const double* levels,
-                               double* h_pml, double* h_tvar, double* h_mean, cudaStream_t s);
+                               double* h_pml, double* h_tvar, double* h_mean, cudaStream_t s,
+                               bool beside);
 
 // Event-major index of a device YET (ara_yet_index_create).  The trials are cut into blocks of
 // `block` trials and the catalogue into groups of 32 events.  For block h and group g, the

@@ -1,27 +1,52 @@
 // PML and TVaR (Section IV-A names both as metrics derived from the YLT) as empirical order
 // statistics: PML(RP) is the ceil(N/RP)-th largest year loss, TVaR(p) the mean of the
-// ceil(N(1-p)) largest.  Both come from an exact radix select on order-preserving 64-bit keys
-// of the FP64 year losses (up to 8 passes of 8 bits), followed by one pass summing the tail
-// above the selected key.  One cooperative launch runs every pass: each block adds its
-// shared-memory digit histogram into the pass's global histogram, the layer's blocks meet at a
-// grid barrier (a bounded wait), and every block then reads the histogram and advances the
-// selection itself.
+// ceil(N(1-p)) largest.  Exact selection on order-preserving 64-bit keys of the FP64 year losses,
+// by sampled splitters:
+//   1. every block sorts the same sampled keys of its row (one random position in each of 256 or
+//      1,024 equal parts) and keeps as splitters those near the targets' expected places; then it
+//      classes its slice of the row: above, equal to or between splitters (ties have classes of
+//      their own).  Also the row sum.
+//   2. from the class totals, each target's class; the keys of classes that are open intervals (2 N
+//      per sampled key, on average) go to a list
+//   3. one block per target finds its key in its list
+//   4. TVaR targets: the sums of the values above the selected keys
+// Few rows take one cooperative launch over every SM (k_sel_grid, bounded grid barriers between the
+// steps); many rows a thread-block cluster each (k_sel_cluster, hardware barriers, and blocks that
+// need half an SM, so that they run beside other streams' kernels); rows of at most 4,096 values
+// one block each that sorts them whole (k_sel_small).
 // Results are bit-exact copies of YLT entries (PML) and deterministic FP64 sums (TVaR, mean):
 // fixed per-thread order, fixed warp and block trees, block partials combined in a fixed order.
+//
+// What it replaces: a cooperative radix select of 8-bit digits (4 to 8 passes over the row with a grid
+// barrier each).  Kernel time of one call, 3 targets / 6 targets and the mean, us:
+//   rows x values   1 x 1e3    1 x 3e4    1 x 1.5e5  1 x 1e6    1 x 5e6    8 x 1e5    16 x 2e5   64 x 2e5
+//   radix select    23 / 30    31 / 39    36 / 48    60 / 82    161 / 225  44 / 68    89 / 145   394 / 557
+//   this            19 / 25    31 / 39    33 / 46    47 / 57    122 / 148  38 / 47    62 / 79    119 / 175
+// Few rows are bound by the steps' latencies (sorting the sample 3-9 us, a barrier 1.5 us, a pick 3 us,
+// each pass over the row one L2 round trip), many rows by reading them three times.
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "ara_internal.cuh"
 
 namespace ara {
 
-constexpr int SEL_BITS = 8;
-constexpr int SEL_BINS = 1 << SEL_BITS;
-constexpr int SEL_PASSES = 64 / SEL_BITS;
 constexpr int SEL_MAX_T = 16;
-constexpr int SEL_THREADS = 1024;
+constexpr int SEL_THREADS = 512;
+constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr int SEL_SAMPLE = 1024;                 // sampled keys per row
+constexpr int SEL_CLASSES = 2 * SEL_SAMPLE + 1;
+constexpr int SEL_SMALL = 4096;                  // rows up to this length are sorted whole
+constexpr int SEL_PICK = 4096;                   // list keys the pick keeps in shared memory
+// Rows of one request up to which the cooperative launch is the faster (16 rows of 200,000 values, 3
+// targets: 60 us against 95 us in clusters; 64 rows: 177 and 119).
+constexpr int SEL_GRID_ROWS = 32;
+constexpr unsigned SFULL = 0xffffffffu;
 
 struct SelTargets {
   int32_t n_t;                 // targets per layer
@@ -30,86 +55,123 @@ struct SelTargets {
 };
 
 struct SelState {
-  uint64_t prefix;             // written at the end: the selected key
-  int64_t k;                   // rank still to find among keys matching the prefix
+  uint64_t key;                // the selected key (known at once when its class is a tie)
+  uint64_t lo, hi;             // the open interval it lies in otherwise (0 and ~0 at the ends: closed)
+  int32_t tie;                 // 1: the class is a splitter's own
+  int32_t list;                // the target whose list holds the interval (the first with that class)
+  int64_t before;              // keys above the class
+  int64_t in_class;            // keys in the class
 };
+__device__ __forceinline__ bool in_interval(uint64_t k, uint64_t lo, uint64_t hi) {
+  return (k > lo || (lo == 0ull && k == 0ull)) && (k < hi || (hi == ~0ull && k == ~0ull));
+}
 
-// Scratch layout (one allocation, zero-filled before the launch):
-//   hist   [n_layers][SEL_PASSES][n_t][SEL_BINS]  uint32
-//   bar    [n_layers]                             uint32 grid-barrier counter of the layer
-//   err    [1]                                    uint32: a grid barrier timed out
-//   state  [n_layers][n_t]                        SelState
-//   psum   [n_layers][n_t][blocks]                double   block partial: sum of y > key
-//   pgt    [n_layers][n_t][blocks]                uint64   block partial: #{y > key}
-//   peq    [n_layers][n_t][blocks]                uint64   block partial: #{y == key}
-//   out    [n_layers][n_t]                        double   PML / TVaR
-//   gt, eq [n_layers][n_t]                        uint64   totals
-//   pmean  [n_layers][blocks]                     double   block partial of the row sum
-//   mean   [n_layers]                             double
+// Scratch (one allocation; the first part, up to state, is zero-filled before the launch):
 struct SelScratch {
-  uint32_t* hist;
-  uint32_t* bar;
-  uint32_t* err;
-  SelState* state;
-  double* psum;
-  unsigned long long* pgt;
-  unsigned long long* peq;
-  double* out;
-  unsigned long long* gt;
-  unsigned long long* eq;
-  double* pmean;
-  double* mean;
-  uint32_t* ext_err;     // optional (nullptr): also gets DERR_TIMEOUT when a barrier times out
+  uint32_t* count;             // [n_layers][SEL_CLASSES] class totals
+  uint32_t* n_list;            // [n_layers][n_t] keys in each list
+  uint32_t* bar;               // [n_layers] grid-barrier counters
+  uint32_t* err;               // [1]
+  uint32_t* count2;            // second round: [n_layers][n_t][SEL_CLASSES], else null
+  uint32_t* n_list2;           // second round: [n_layers][n_t]
+  SelState* state;             // [n_layers][n_t]
+  uint64_t* list;              // [n_layers][n_t][cap]
+  double* psum;                  // [n_layers][n_t][blocks] block partials of the tail sums
+  double* pmean;                 // [n_layers][blocks] block partials of the row sum
+  // results, contiguous: out, mean
+  double* out;                 // [n_layers][n_t] PML / TVaR
+  double* mean;                // [n_layers]
+  unsigned long long* gt;      // [n_layers][n_t] #{y > key}
+  unsigned long long* eq;      // [n_layers][n_t] #{y == key}
+  int64_t cap;
+  int32_t sample;              // sampled keys per row
+  uint32_t* ext_err;           // optional (nullptr): also gets DERR_TIMEOUT
   // optional caller outputs, written directly (nullptr: results stay in out / mean only)
-  double* user_pml;      // [n_layers][n_rp]
-  double* user_tvar;     // [n_layers][n_t - n_rp]
-  double* user_mean;     // [n_layers]
+  double* user_pml;            // [n_layers][n_rp]
+  double* user_tvar;           // [n_layers][n_t - n_rp]
+  double* user_mean;           // [n_layers]
 };
 
-template <typename F>
-static size_t layout(int32_t n_layers, int32_t n_t, int32_t blocks, F&& take) {
-  const size_t lt = (size_t)n_layers * n_t, ltb = lt * blocks;
+// Sampled keys of a row: sorting them costs every block 2 us for 256 and 9 us for 1,024, and the
+// intervals they leave are picked from in about 4 us per 4,096 keys.
+__host__ __device__ inline int32_t sel_sample(int64_t n) { return n <= (1 << 19) ? 256 : SEL_SAMPLE; }
+
+// Room for the keys of one open interval between neighbouring samples: the interval that holds a
+// given rank has 2 / sample of the keys on average and more than 16 / sample with probability 2e-6 (a
+// list that would overflow is not used: its target is picked from the row itself).
+static int64_t list_cap(int64_t n) { return std::min<int64_t>(n, 16 * (n / sel_sample(n)) + 4096); }
+
+// A request's launch plan and scratch.  cap: keys per list; rounds: 2 when cap is short of list_cap
+// (the allocation-free call on long rows): overfull intervals are split again before the pick.
+struct SelPlan {
+  int64_t n = 0, cap = 0;
+  int32_t n_layers = 0, n_t = 0, blocks = 1, rounds = 1;
+  bool cluster = false;             // one cluster of `blocks` blocks per row
+  bool small = false;               // one block per row, sorted whole
+  int n_sms = 1;
+  size_t off[13];
+  size_t zero_bytes = 0, bytes = 0;
+};
+// beside: the caller's kernels share the device with other streams' (the server)
+static SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int64_t cap, bool beside = false) {
+  SelPlan y;
+  y.n = n;
+  y.cap = cap;
+  y.n_layers = n_layers;
+  y.n_t = n_t;
+  y.small = n <= SEL_SMALL;
+  y.n_sms = std::max(1, n_sms);
+  y.rounds = !y.small && cap < list_cap(n) ? 2 : 1;
+  const int64_t slots = 2ll * std::max(1, n_sms);           // blocks that run at once
+  y.cluster = !y.small && y.rounds == 1 && n <= (4 << 20) && (beside || n_layers > SEL_GRID_ROWS);
+  if (y.cluster) {                                          // all rows' clusters at once, if they can be
+    y.blocks = 16;
+    while (y.blocks > 1 && ((int64_t)n_layers * y.blocks > slots || n < 2048ll * y.blocks)) y.blocks /= 2;
+  } else if (!y.small) {
+    y.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, std::max<int64_t>(1, n_sms / n_layers)));
+  }
+  const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1), two = y.rounds > 1 ? lt : 0;
+  const size_t grid = y.small || y.cluster ? 0 : 1, lists = y.small ? 0 : 1;
   size_t b = 0;
-  auto t = [&](size_t n) { b = (b + 255) / 256 * 256; take(b); b += n; };
-  t(sizeof(uint32_t) * SEL_PASSES * lt * SEL_BINS);
-  t(sizeof(uint32_t) * n_layers);
-  t(sizeof(uint32_t));
-  t(sizeof(SelState) * lt);
-  t(sizeof(double) * ltb);
-  t(sizeof(uint64_t) * ltb);
-  t(sizeof(uint64_t) * ltb);
-  t(sizeof(double) * lt);
-  t(sizeof(uint64_t) * lt);
-  t(sizeof(uint64_t) * lt);
-  t(sizeof(double) * (size_t)n_layers * blocks);
-  t(sizeof(double) * n_layers);
-  return (b + 255) / 256 * 256;
-}
-
-size_t select_scratch_bytes(int32_t n_layers, int32_t n_t, int32_t blocks) {
-  return layout(n_layers, n_t, blocks, [](size_t) {});
-}
-
-static SelScratch carve(void* base, int32_t n_layers, int32_t n_t, int32_t blocks) {
-  size_t off[12];
   int i = 0;
-  layout(n_layers, n_t, blocks, [&](size_t o) { off[i++] = o; });
+  auto t = [&](size_t k) { b = (b + 15) / 16 * 16; y.off[i++] = b; b += k; };
+  t(4 * grid * L * SEL_CLASSES);
+  t(4 * grid * lt);
+  t(4 * grid * L);
+  t(4);
+  t(4 * two * SEL_CLASSES);
+  t(4 * two);
+  y.zero_bytes = (b + 15) / 16 * 16;
+  t(sizeof(SelState) * lt);
+  t(8 * lists * lt * (size_t)cap);
+  t(8 * grid * lt * (size_t)y.blocks);
+  t(8 * grid * L * (size_t)y.blocks);
+  t(8 * (lt + L));
+  t(8 * lt);
+  t(8 * lt);
+  y.bytes = (b + 255) / 256 * 256;
+  return y;
+}
+
+static SelScratch carve(void* base, const SelPlan& y) {
   char* p = (char*)base;
-  SelScratch s;
-  s.hist = (uint32_t*)(p + off[0]);
-  s.bar = (uint32_t*)(p + off[1]);
-  s.err = (uint32_t*)(p + off[2]);
-  s.state = (SelState*)(p + off[3]);
-  s.psum = (double*)(p + off[4]);
-  s.pgt = (unsigned long long*)(p + off[5]);
-  s.peq = (unsigned long long*)(p + off[6]);
-  s.out = (double*)(p + off[7]);
-  s.gt = (unsigned long long*)(p + off[8]);
-  s.eq = (unsigned long long*)(p + off[9]);
-  s.pmean = (double*)(p + off[10]);
-  s.mean = (double*)(p + off[11]);
-  s.ext_err = nullptr;
-  s.user_pml = s.user_tvar = s.user_mean = nullptr;
+  SelScratch s{};
+  s.count = (uint32_t*)(p + y.off[0]);
+  s.n_list = (uint32_t*)(p + y.off[1]);
+  s.bar = (uint32_t*)(p + y.off[2]);
+  s.err = (uint32_t*)(p + y.off[3]);
+  s.count2 = y.rounds > 1 ? (uint32_t*)(p + y.off[4]) : nullptr;
+  s.n_list2 = (uint32_t*)(p + y.off[5]);
+  s.state = (SelState*)(p + y.off[6]);
+  s.list = (uint64_t*)(p + y.off[7]);
+  s.psum = (double*)(p + y.off[8]);
+  s.pmean = (double*)(p + y.off[9]);
+  s.out = (double*)(p + y.off[10]);
+  s.mean = s.out + (size_t)y.n_layers * y.n_t;
+  s.gt = (unsigned long long*)(p + y.off[11]);
+  s.eq = (unsigned long long*)(p + y.off[12]);
+  s.cap = y.cap;
+  s.sample = sel_sample(y.n);
   return s;
 }
 
@@ -123,6 +185,691 @@ __device__ __forceinline__ double value_of(uint64_t k) {
   return __longlong_as_double((long long)b);
 }
 
+// Bitonic sort of N (a power of two, at least 64) shared-memory keys, descending, by the whole
+// block.  A warp's 32 pairs of a step with stride at most 32 lie in its own 64 keys, so those steps
+// need no block barrier.
+__device__ __forceinline__ void sort_descending(uint64_t* a, int N) {
+  for (int k = 2; k <= N; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int t = threadIdx.x; t < N / 2; t += SEL_THREADS) {
+        const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
+        const uint64_t x = a[i], y = a[i + j];
+        if ((x < y) == ((i & k) == 0)) {
+          a[i] = y;
+          a[i + j] = x;
+        }
+      }
+      if (j > 32 || (j == 1 && k >= 64)) __syncthreads();
+      else __syncwarp();
+    }
+  }
+  __syncthreads();
+}
+
+// The same for the m sampled keys (a power of two, 64 to SEL_SAMPLE), two per thread in registers: thread l of warp w holds keys
+// 64 w + l and 64 w + 32 + l, so steps of stride below 64 are shuffles (or within the thread) and only
+// the ten wider ones go through shared memory.  (All steps through shared memory: 8 us a row; this:
+// 2 us.)
+__device__ __forceinline__ void sort_sample(uint64_t* a, int m) {
+  static_assert(SEL_SAMPLE == 2 * SEL_THREADS, "two keys per thread");
+  const int lane = threadIdx.x & 31, i0 = 64 * (int)(threadIdx.x >> 5) + lane, i1 = i0 + 32;
+  const bool has = i0 < m;   // m is a multiple of 64: whole warps
+  uint64_t x0 = has ? a[i0] : 0ull, x1 = has ? a[i1] : 0ull;
+  auto take = [](uint64_t mine, uint64_t other, bool larger) { return (mine > other) == larger ? mine : other; };
+#pragma unroll 1
+  for (int k = 2; k <= m; k <<= 1) {
+#pragma unroll 1
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      if (!has && j < 64) continue;
+      // key i keeps the larger of the pair (i, i ^ j) when i is its lower place in a descending run
+      const bool l0 = ((i0 & j) == 0) == ((i0 & k) == 0), l1 = ((i1 & j) == 0) == ((i1 & k) == 0);
+      uint64_t y0, y1;
+      if (j >= 64) {
+        __syncthreads();
+        if (has) {
+          a[i0] = x0;
+          a[i1] = x1;
+        }
+        __syncthreads();
+        y0 = has ? a[i0 ^ j] : 0ull;
+        y1 = has ? a[i1 ^ j] : 0ull;
+      } else if (j == 32) {
+        y0 = x1;
+        y1 = x0;
+      } else {
+        y0 = __shfl_xor_sync(SFULL, x0, j);
+        y1 = __shfl_xor_sync(SFULL, x1, j);
+      }
+      x0 = take(x0, y0, l0);
+      x1 = take(x1, y1, l1);
+    }
+  }
+  __syncthreads();
+  if (has) {
+    a[i0] = x0;
+    a[i1] = x1;
+  }
+  __syncthreads();
+}
+
+// Sum over the block by fixed trees; the result is valid in thread 0.  (Carrying the rounding errors
+// along, in the trees alone, made a call of one short row 60 % slower: an FP64 operation has a long
+// latency here.)
+__device__ __forceinline__ double warp_add(double a, int from) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+    if (o <= from) a = __dadd_rn(a, __shfl_down_sync(SFULL, a, o));
+  return a;
+}
+__device__ __forceinline__ double block_sum(double a, double* wsum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  a = warp_add(a, 16);
+  if (lane == 0) wsum[warp] = a;
+  __syncthreads();
+  if (warp == 0) a = warp_add(lane < SEL_WARPS ? wsum[lane] : 0.0, SEL_WARPS / 2);
+  __syncthreads();
+  return a;
+}
+
+// TVaR of m values: the sum of the gt values above the key v, and (m - gt) times v.
+__device__ __forceinline__ double tvar_of(double above, int64_t m, unsigned long long gt, double v) {
+  return (above + (double)(m - (int64_t)gt) * v) / (double)m;
+}
+
+__device__ __forceinline__ void put_result(const SelScratch& sc, const SelTargets& tg, int layer, int t, double r) {
+  const int nt = tg.n_t;
+  sc.out[(int64_t)layer * nt + t] = r;
+  if (t < tg.n_rp) {
+    if (sc.user_pml) sc.user_pml[(int64_t)layer * tg.n_rp + t] = r;
+  } else if (sc.user_tvar) {
+    sc.user_tvar[(int64_t)layer * (nt - tg.n_rp) + (t - tg.n_rp)] = r;
+  }
+}
+
+__device__ __forceinline__ void put_mean(const SelScratch& sc, int layer, double r) {
+  sc.mean[layer] = r;
+  if (sc.user_mean) sc.user_mean[layer] = r;
+}
+
+__device__ __forceinline__ void sel_timeout(const SelScratch& sc) {
+  atomicOr(sc.err, 1u);
+  if (sc.ext_err) atomicOr(sc.ext_err, DERR_TIMEOUT);
+}
+
+// Rows of at most SEL_SMALL values, one block each: the sorted row gives every result directly.
+__global__ void __launch_bounds__(SEL_THREADS)
+k_sel_small(const double* __restrict__ ylt, int32_t n, int32_t n_pad, SelTargets tg, SelScratch sc, int want_mean) {
+  extern __shared__ uint64_t sk[];
+  __shared__ double wsum[SEL_WARPS];
+  __shared__ int32_t cut[2];
+  const int layer = blockIdx.x, nt = tg.n_t;
+  const double* src = ylt + (int64_t)layer * n;
+  for (int i = threadIdx.x; i < n_pad; i += SEL_THREADS) sk[i] = i < n ? key_of(__ldcg(src + i)) : 0ull;
+  __syncthreads();
+  // keys are never 0 for the row's values except the NaN of all ones, which sorts with the padding
+  sort_descending(sk, n_pad);
+  if (want_mean) {
+    double a = 0.0;
+    for (int i = threadIdx.x; i < n; i += SEL_THREADS) a = __dadd_rn(a, value_of(sk[i]));
+    const double s = block_sum(a, wsum);
+    if (threadIdx.x == 0) put_mean(sc, layer, s / (double)n);
+  }
+  for (int t = 0; t < nt; ++t) {
+    const uint64_t key = sk[tg.rank[t] - 1];
+    if (threadIdx.x < 2) {   // keys above (thread 0) and at or above (thread 1) the selected key
+      int lo = 0, hi = n;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (threadIdx.x == 0 ? sk[mid] > key : sk[mid] >= key) lo = mid + 1;
+        else hi = mid;
+      }
+      cut[threadIdx.x] = lo;
+    }
+    __syncthreads();
+    const int gt = cut[0], ge = cut[1];
+    double r = value_of(key);
+    if (t >= tg.n_rp) {
+      double a = 0.0;
+      for (int i = threadIdx.x; i < gt; i += SEL_THREADS) a = __dadd_rn(a, value_of(sk[i]));
+      r = tvar_of(block_sum(a, wsum), tg.rank[t], (unsigned long long)gt, r);
+    }
+    if (threadIdx.x == 0) {
+      put_result(sc, tg, layer, t, r);
+      sc.gt[(int64_t)layer * nt + t] = (unsigned long long)gt;
+      sc.eq[(int64_t)layer * nt + t] = (unsigned long long)(ge - gt);
+      sc.state[(int64_t)layer * nt + t].key = key;
+    }
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// The steps, for one block's slice of one row
+// ------------------------------------------------------------------------------------------
+constexpr int SEL_U = 4;                      // values per thread and step; the next ones are in flight
+constexpr int SEL_QUEUE = 32 + 32 * SEL_U;    // keys a warp's queue can hold
+struct SelShared {                            // shared memory of a block (dynamic: SEL_SMEM bytes)
+  uint64_t key[SEL_SAMPLE];                   // the sorted sample, then the splitters
+  uint64_t queue[SEL_WARPS][SEL_QUEUE];       // per warp: keys waiting for a full warp
+  uint64_t keep[SEL_PICK];                    // the pick's list
+  uint32_t hist[SEL_CLASSES];                 // class counts of the slice (the pick: digit counts)
+  uint32_t cnt[SEL_CLASSES];                  // inclusive prefix of the row's class totals
+  uint64_t ext[2 * SEL_WARPS];
+  double wsum[SEL_WARPS];
+  uint32_t wcnt[SEL_WARPS];
+  SelState st[SEL_MAX_T];
+  int32_t cls[SEL_MAX_T];
+  uint64_t lo[SEL_MAX_T], width[SEL_MAX_T];   // the intervals to collect: keys lo .. lo + width
+  int32_t own[SEL_MAX_T], n_own;
+  uint32_t got[SEL_MAX_T], base[SEL_MAX_T];
+  uint64_t found, prefix;
+  int64_t k, gt, eq;
+  // a cluster's row: its own partial results, and (rank 0) the row's lists and picked targets
+  double pmean, psum[SEL_MAX_T];
+  uint32_t reported, n_list[SEL_MAX_T];
+  uint64_t pick_key[SEL_MAX_T];
+  int64_t pick_gt[SEL_MAX_T];
+};
+constexpr int SEL_SMEM = (int)sizeof(SelShared);
+
+// Calls f(key, valid) for every key >= floor_key of the values [i0, i1) of the row: such keys wait in
+// the warp's queue until 32 are there, so f runs on full warps however few they are (all lanes
+// call it; the last call may have invalid lanes).  all(y, u) sees every value in order (0 past the
+// slice's end; u: 0 .. 3 in turn).  The order of the calls depends on the row alone.  f appears once:
+// the code runs once or twice per launch, and fetching it costs more than running it.  Returns
+// the number of keys >= floor_key (per warp).
+template <typename F, typename G>
+__device__ __forceinline__ uint32_t for_keys_from(const double* __restrict__ row, int64_t i0, int64_t i1,
+                                                  uint64_t floor_key, uint64_t* q, F&& f, G&& all) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  int qn = 0;
+  uint32_t total = 0;
+  double next[SEL_U];
+  const double* at = row + i0 + threadIdx.x;
+  int64_t left = i1 - i0 - (int64_t)threadIdx.x;   // values from this thread's place to the end
+#pragma unroll
+  for (int u = 0; u < SEL_U; ++u) next[u] = left > u * SEL_THREADS ? __ldcg(at + u * SEL_THREADS) : 0.0;
+  bool more = true;
+  while (more) {
+    double y[SEL_U];
+    const int64_t here = left;
+    at += SEL_U * SEL_THREADS;
+    left -= SEL_U * SEL_THREADS;
+    more = left + lane > 0;                        // uniform over the warp
+#pragma unroll
+    for (int u = 0; u < SEL_U; ++u) {
+      y[u] = next[u];
+      next[u] = left > u * SEL_THREADS ? __ldcg(at + u * SEL_THREADS) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < SEL_U; ++u) {
+      if (here + lane <= u * SEL_THREADS) break;   // uniform: the warp is past the end
+      all(y[u], u);
+      const uint64_t k = key_of(y[u]);
+      const bool c = here > u * SEL_THREADS && k >= floor_key;
+      const unsigned m = __ballot_sync(SFULL, c);
+      if (c) q[qn + __popc(m & lt)] = k;
+      qn += __popc(m);
+    }
+    __syncwarp();
+#pragma unroll 1
+    while (qn >= 32 || (!more && qn > 0)) {
+      const int n = min(qn, 32);
+      qn -= n;
+      total += (uint32_t)n;
+      f(lane < n ? q[qn + lane] : 0ull, lane < n);
+    }
+    __syncwarp();
+  }
+  return total;
+}
+
+// The row's splitters into S.key (descending); returns their number.  With a list (of cap keys):
+// SEL_SAMPLE keys of it, all of them.
+__device__ __forceinline__ int row_splitters(SelShared& S, const double* __restrict__ row, int64_t n, int sample,
+                                             const SelTargets& tg, const uint64_t* list = nullptr, int64_t cap = 0) {
+  const int nt = tg.n_t, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (list) sample = SEL_SAMPLE;
+  const int lg = 31 - __clz(sample);   // a power of two
+  for (int j = threadIdx.x; j < sample; j += SEL_THREADS) {
+    const int64_t a = ((int64_t)j * n) >> lg, b = ((int64_t)(j + 1) * n) >> lg;
+    uint64_t z = (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull;   // SplitMix64 of the part's number
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z ^= z >> 31;
+    S.key[j] = list ? __ldcg(list + (((int64_t)j * cap) >> lg))
+                    : key_of(__ldcg(row + a + (int64_t)__umul64hi(z, (uint64_t)(b - a))));
+  }
+  __syncthreads();
+  sort_sample(S.key, sample);
+  if (list) return sample;
+  // Splitters: sample places within 6 standard deviations (and 4 places) of a target's expected
+  // place.  Kept places move to the front in order.
+  bool keep[SEL_SAMPLE / SEL_THREADS];
+  uint64_t mine[SEL_SAMPLE / SEL_THREADS];
+#pragma unroll
+  for (int u = 0; u < SEL_SAMPLE / SEL_THREADS; ++u) {
+    const int i = u * SEL_THREADS + (int)threadIdx.x;
+    mine[u] = S.key[i];
+    keep[u] = false;
+    for (int t = 0; t < nt && i < sample; ++t) {
+      const float r = (float)tg.rank[t] * ((float)sample / (float)n);
+      const float w = 6.0f * sqrtf(fmaxf(r * (1.0f - r / (float)sample), 1.0f)) + 4.0f;
+      keep[u] = keep[u] || fabsf((float)i - r) <= w;
+    }
+  }
+  __syncthreads();
+  int np = 0;
+#pragma unroll
+  for (int u = 0; u < SEL_SAMPLE / SEL_THREADS; ++u) {
+    const unsigned m = __ballot_sync(SFULL, keep[u]);
+    if (lane == 0) S.wcnt[warp] = (uint32_t)__popc(m);
+    __syncthreads();
+    int at = np, all = np;
+    for (int w = 0; w < SEL_WARPS; ++w) {
+      if (w < warp) at += (int)S.wcnt[w];
+      all += (int)S.wcnt[w];
+    }
+    if (keep[u]) S.key[at + __popc(m & ((1u << lane) - 1u))] = mine[u];
+    np = all;
+    __syncthreads();
+  }
+  return np;
+}
+
+// Class counts of the slice into S.hist.  Class 2 i: between splitters i - 1 and i; class 2 i + 1:
+// equal to splitter i (its first place).  Only keys within [lo, hi] count (the whole range, or an
+// interval that is split again).  Returns the slice's sum (thread 0) when want_mean.
+__device__ __forceinline__ double count_slice(SelShared& S, const double* __restrict__ row, int64_t i0, int64_t i1,
+                                              int np, uint64_t lo, uint64_t hi, int want_mean) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i <= 2 * np; i += SEL_THREADS) S.hist[i] = 0u;
+  __syncthreads();
+  double sum[2] = {0.0, 0.0};
+  const int top = np > 0 ? 1 << (31 - __clz(np)) : 0;
+  const bool part = lo != 0ull || hi != ~0ull;
+  // keys below every splitter are counted, not searched
+  const uint64_t floor_key = np == 0 ? ~0ull : part ? lo : S.key[np - 1];
+  const uint32_t near = for_keys_from(row, i0, i1, floor_key, S.queue[warp], [&](uint64_t k, bool valid) {
+    if (part) valid = valid && in_interval(k, lo, hi);
+    int c = 0;               // splitters above k
+    for (int step = top; step; step >>= 1)
+      if (c + step <= np && S.key[c + step - 1] > k) c += step;
+    const uint32_t cls = valid ? 2u * (uint32_t)c + (np > 0 && S.key[min(c, np - 1)] == k ? 1u : 0u) : 0xffffffffu;
+    const unsigned peers = __match_any_sync(SFULL, cls);
+    if (valid && lane == __ffs(peers) - 1) atomicAdd(&S.hist[cls], (uint32_t)__popc(peers));
+  }, [&](double y, int u) {
+    if (want_mean) sum[u & 1] = __dadd_rn(sum[u & 1], y);
+  });
+  if (lane == 0) S.wcnt[warp] = near;
+  __syncthreads();
+  if (warp == 0 && np > 0 && !part) {
+    const uint32_t counted = __reduce_add_sync(SFULL, lane < SEL_WARPS ? S.wcnt[lane] : 0u);
+    if (lane == 0) S.hist[2 * np] += (uint32_t)(i1 - i0) - counted;
+  }
+  __syncthreads();
+  return want_mean ? block_sum(__dadd_rn(sum[0], sum[1]), S.wsum) : 0.0;
+}
+
+// The classes of the targets [first, last) from the row's class totals (S.cnt, i <= 2 np; a barrier
+// after they were written), into S.st, and the intervals to collect (S.own, S.lo, S.width; one per distinct class).  old: the
+// interval that was split (the whole range at first), with the keys before it.
+__device__ __forceinline__ void target_classes(SelShared& S, const SelTargets& tg, int first, int last, int np,
+                                               uint64_t old_lo, uint64_t old_hi, int64_t old_before) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (2 * np + SEL_THREADS) / SEL_THREADS;   // classes per thread
+  uint32_t s = 0;
+  for (int u = 0; u < per; ++u) {
+    const int i = (int)threadIdx.x * per + u;
+    s += i <= 2 * np ? S.cnt[i] : 0u;
+  }
+  uint32_t incl = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(SFULL, incl, o);
+    if (lane >= o) incl += x;
+  }
+  if (lane == 31) S.wcnt[warp] = incl;
+  __syncthreads();
+  uint32_t run = incl - s;
+  for (int w = 0; w < warp; ++w) run += S.wcnt[w];
+  for (int u = 0; u < per; ++u) {
+    const int i = (int)threadIdx.x * per + u;
+    if (i <= 2 * np) {
+      run += S.cnt[i];
+      S.cnt[i] = run;
+    }
+  }
+  __syncthreads();
+  const int q = first + (int)threadIdx.x;
+  if (q < last) {            // the first class whose prefix reaches the rank
+    const int64_t k = tg.rank[q] - old_before;
+    int a = 0, b = 2 * np;
+    while (a < b) {
+      const int mid = (a + b) >> 1;
+      if ((int64_t)S.cnt[mid] >= k) b = mid;
+      else a = mid + 1;
+    }
+    const int64_t before = a ? (int64_t)S.cnt[a - 1] : 0;
+    const int i = a >> 1;    // class 2 i: above splitter i (if any) and below splitter i - 1 (if any)
+    S.st[q] = SelState{a & 1 ? S.key[i] : 0ull, i < np ? S.key[i] : old_lo, i > 0 ? S.key[i - 1] : old_hi,
+                       a & 1, q, old_before + before, (int64_t)S.cnt[a] - before};
+    S.cls[q] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int m = 0;
+    for (int t = first; t < last; ++t) {
+      int f = first;
+      while (S.cls[f] != S.cls[t]) ++f;
+      S.st[t].list = f;
+      if (f == t && !S.st[t].tie) {
+        const uint64_t l = S.st[t].lo, h = S.st[t].hi;
+        S.own[m] = t;
+        S.lo[m] = l == 0ull ? 0ull : l + 1;
+        S.width[m] = (h == ~0ull ? h : h - 1) - S.lo[m];
+        ++m;
+      }
+    }
+    S.n_own = m;
+  }
+  __syncthreads();
+}
+
+// The slice's keys of the intervals, appended to the targets' lists (of at most cap keys); counter(t)
+// is the address of target t's list length.
+template <typename C>
+__device__ __forceinline__ void collect_slice(SelShared& S, const double* __restrict__ row, int64_t i0, int64_t i1,
+                                              uint64_t* list, int64_t cap, C&& counter) {
+  const int m = S.n_own, warp = threadIdx.x >> 5;
+  if (m == 0) return;
+  uint64_t floor_key = ~0ull;
+  for (int q = 0; q < m; ++q) floor_key = min(floor_key, S.lo[q]);
+  // First into the block's own part of S.keep, then to the list with one reservation per interval; what
+  // the part does not hold goes there directly.
+  const int part = SEL_PICK / m;
+  if (threadIdx.x < SEL_MAX_T) S.got[threadIdx.x] = 0u;
+  __syncthreads();
+  for_keys_from(row, i0, i1, floor_key, S.queue[warp], [&](uint64_t k, bool valid) {
+    int mine = -1;           // the intervals are disjoint
+    for (int q = 0; q < m; ++q)
+      if (valid && k - S.lo[q] <= S.width[q]) mine = q;
+    if (mine < 0) return;
+    const uint32_t at = atomicAdd(&S.got[mine], 1u);
+    if (at < (uint32_t)part) {
+      S.keep[mine * part + (int)at] = k;
+    } else {
+      const int t = S.own[mine];
+      const uint32_t p = atomicAdd(counter(t), 1u);
+      if ((int64_t)p < cap) list[(int64_t)t * cap + p] = k;
+    }
+  }, [](double, int) {});
+  __syncthreads();
+  if (threadIdx.x < m) {
+    const uint32_t c = min(S.got[threadIdx.x], (uint32_t)part);
+    S.got[threadIdx.x] = c;
+    S.base[threadIdx.x] = c ? atomicAdd(counter(S.own[threadIdx.x]), c) : 0u;
+  }
+  __syncthreads();
+  for (int q = 0; q < m; ++q)
+    for (uint32_t i = threadIdx.x; i < S.got[q]; i += SEL_THREADS) {
+      const int64_t at = (int64_t)S.base[q] + i;
+      if (at < cap) list[(int64_t)S.own[q] * cap + at] = S.keep[q * part + (int)i];
+    }
+  __syncthreads();
+}
+
+// The key of rank `rank` of a target with state st, by the whole block; *gt and *eq: keys above and
+// equal to it.  list: the list of its interval; one that did not fit is replaced by the row's keys.
+__device__ __forceinline__ uint64_t pick_key(SelShared& S, const double* __restrict__ row, int64_t n, const SelState& st,
+                                             int64_t rank, const uint64_t* list, int64_t cap, int64_t* gt, int64_t* eq) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (st.tie) {
+    *gt = st.before;
+    *eq = st.in_class;
+    return st.key;
+  }
+  const bool listed = st.in_class <= cap;
+  const int64_t N = listed ? st.in_class : n;
+  const bool near = listed && N <= SEL_PICK;
+  auto get = [&](int64_t i, bool& in) -> uint64_t {
+    in = true;
+    if (near) return S.keep[i];
+    if (listed) return __ldcg(list + i);
+    const uint64_t k = key_of(__ldcg(row + i));
+    in = in_interval(k, st.lo, st.hi);
+    return k;
+  };
+  if (listed && N <= 192) {   // short lists (the counting grows with their square): every thread counts the keys above its own
+    const int c = (int)N;
+    const uint64_t x = (int)threadIdx.x < c ? __ldcg(list + threadIdx.x) : 0ull;
+    if ((int)threadIdx.x < c) S.keep[threadIdx.x] = x;
+    __syncthreads();
+    if ((int)threadIdx.x < c) {
+      int above = 0, same = 0;
+#pragma unroll 2
+      for (int i = 0; i < c; ++i) {
+        const uint64_t o = S.keep[i];
+        above += o > x ? 1 : 0;
+        same += o == x ? 1 : 0;
+      }
+      const int64_t k = rank - st.before;
+      if (above < k && k <= above + same) {   // the threads of equal keys write the same values
+        S.found = x;
+        S.gt = above;
+        S.eq = same;
+      }
+    }
+    __syncthreads();
+    const uint64_t key = S.found;
+    *gt = st.before + S.gt;
+    *eq = S.eq;
+    __syncthreads();
+    return key;
+  }
+  // the highest bit in which the keys differ
+  uint64_t mn = ~0ull, mx = 0ull;
+  for (int64_t i = threadIdx.x; i < N; i += SEL_THREADS) {
+    bool in = true;
+    uint64_t k;
+    if (near) S.keep[i] = k = __ldcg(list + i);
+    else k = get(i, in);
+    if (in) { mn = min(mn, k); mx = max(mx, k); }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    mn = min(mn, (uint64_t)__shfl_xor_sync(SFULL, mn, o));
+    mx = max(mx, (uint64_t)__shfl_xor_sync(SFULL, mx, o));
+  }
+  if (lane == 0) { S.ext[warp] = mn; S.ext[SEL_WARPS + warp] = mx; }
+  __syncthreads();
+  for (int w = 0; w < SEL_WARPS; ++w) {
+    mn = min(mn, S.ext[w]);
+    mx = max(mx, S.ext[SEL_WARPS + w]);
+  }
+  // radix select on 8-bit digits, from the first digit that differs until one key is left
+  const uint64_t diff = mn ^ mx;
+  int shift = diff ? (63 - __clzll((long long)diff)) / 8 * 8 : 0;
+  uint64_t prefix = mx >> shift >> 8;                // the bits above the digit
+  int64_t k = rank - st.before, above = 0, count = 0;
+  while (true) {
+    for (int i = threadIdx.x; i < 256; i += SEL_THREADS) S.hist[i] = 0u;
+    __syncthreads();
+    for (int64_t i = threadIdx.x; i < N; i += SEL_THREADS) {
+      bool in;
+      const uint64_t x = get(i, in);
+      if (in && (x >> shift >> 8) == prefix) atomicAdd(&S.hist[(x >> shift) & 255u], 1u);
+    }
+    __syncthreads();
+    if (warp == 0) {         // lane l owns bins [256 - 8 (l + 1), 256 - 8 l), from the top down
+      uint32_t h[8], mine = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        h[u] = S.hist[255 - (8 * lane + u)];
+        mine += h[u];
+      }
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(SFULL, incl, o);
+        if (lane >= o) incl += x;
+      }
+      const int64_t excl = (int64_t)(incl - mine);
+      if (excl < k && k <= (int64_t)incl) {
+        int64_t b4 = excl;
+        int u = 0;
+        for (; u < 7; ++u) {
+          if (b4 + h[u] >= k) break;
+          b4 += h[u];
+        }
+        S.prefix = (prefix << 8) | (uint64_t)(255 - (8 * lane + u));
+        S.k = k - b4;
+        S.gt = above + b4;
+        S.eq = h[u];
+      }
+    }
+    __syncthreads();
+    prefix = S.prefix;       // down to and including this digit
+    k = S.k;
+    above = S.gt;
+    count = S.eq;
+    __syncthreads();
+    if (count == 1 || shift == 0) break;
+    shift -= 8;
+  }
+  uint64_t key = prefix;
+  if (shift > 0) {           // one key has this prefix
+    for (int64_t i = threadIdx.x; i < N; i += SEL_THREADS) {
+      bool in;
+      const uint64_t x = get(i, in);
+      if (in && (x >> shift) == prefix) S.found = x;
+    }
+    __syncthreads();
+    key = S.found;
+    __syncthreads();
+  }
+  *gt = st.before + above;
+  *eq = count;
+  return key;
+}
+
+// The slice's sums of the values above thr[q], q < m <= 4; out(q, sum) is called by thread 0.
+template <typename O>
+__device__ __forceinline__ void tail_slice(SelShared& S, const double* __restrict__ row, int64_t i0, int64_t i1, int m,
+                                           const uint64_t (&thr)[4], O&& out) {
+  uint64_t least = ~0ull;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) least = q < m ? min(least, thr[q]) : least;
+  for_keys_from(row, i0, i1, least, S.queue[threadIdx.x >> 5], [&](uint64_t k, bool valid) {
+    const double y = value_of(k);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < m && valid && k > thr[q]) a[q] = __dadd_rn(a[q], y);
+  }, [](double, int) {});
+#pragma unroll 1
+  for (int q = 0; q < m; ++q) {
+    const double s = block_sum(q == 0 ? a[0] : q == 1 ? a[1] : q == 2 ? a[2] : a[3], S.wsum);
+    if (threadIdx.x == 0) out(q, s);
+  }
+}
+
+// Block b of B's part of a row of n values.
+__device__ __forceinline__ int64_t slice_begin(int64_t n, unsigned b, unsigned B) { return (int64_t)b * n / B; }
+
+// ------------------------------------------------------------------------------------------
+// One kernel per row in a thread-block cluster: the steps with cluster barriers between them.
+// ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(SEL_THREADS, 2)
+k_sel_cluster(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets tg, SelScratch sc, int want_mean,
+              int skip_report) {
+  extern __shared__ __align__(16) unsigned char sel_smem[];
+  SelShared& S = *reinterpret_cast<SelShared*>(sel_smem);
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const unsigned B = gridDim.x, rank = blockIdx.x;     // a cluster spans the grid's x
+  const int layer = l0 + (int)blockIdx.y, nt = tg.n_t;
+  const double* row = ylt + (int64_t)layer * n;
+  const int64_t i0 = slice_begin(n, rank, B), i1 = slice_begin(n, rank + 1, B);
+  if (threadIdx.x < SEL_MAX_T) S.n_list[threadIdx.x] = 0u;
+  const int np = nt > 0 ? row_splitters(S, row, n, sc.sample, tg) : 0;
+  const double part = count_slice(S, row, i0, i1, np, 0ull, ~0ull, want_mean);
+  if (threadIdx.x == 0) {
+    S.pmean = part;
+    S.reported = skip_report ? 0u : 1u;
+  }
+  cluster.sync();
+  // (remote words are read by different threads at once: one after the other costs 300 cycles each)
+  const unsigned lane = threadIdx.x & 31;
+  const bool ok = __all_sync(SFULL, lane >= B || cluster.map_shared_rank(&S, lane < B ? lane : 0u)->reported != 0u);
+  if (ok && nt > 0) {
+    for (int i = threadIdx.x; i <= 2 * np; i += SEL_THREADS) S.cnt[i] = 0u;
+    __syncthreads();
+    const unsigned shift = 31u - (unsigned)__clz((int)B);   // B is a power of two
+    for (unsigned i = threadIdx.x; i < (unsigned)(2 * np + 1) << shift; i += SEL_THREADS) {
+      const uint32_t v = cluster.map_shared_rank(&S, i & (B - 1u))->hist[i >> shift];
+      if (v) atomicAdd(&S.cnt[i >> shift], v);
+    }
+    __syncthreads();
+    target_classes(S, tg, 0, nt, np, 0ull, ~0ull, 0);
+    SelShared* const head = cluster.map_shared_rank(&S, 0);
+    collect_slice(S, row, i0, i1, sc.list + (int64_t)layer * nt * sc.cap, sc.cap,
+                  [&](int t) -> uint32_t* { return &head->n_list[t]; });
+  }
+  cluster.sync();                                      // lists complete, class counts read
+  if (ok) {
+    SelShared* const head = cluster.map_shared_rank(&S, 0);
+    for (int t = (int)rank; t < nt; t += (int)B) {
+      const SelState st = S.st[t];
+      int64_t gt, eq;
+      const uint64_t key = pick_key(S, row, n, st, tg.rank[t], sc.list + ((int64_t)layer * nt + st.list) * sc.cap,
+                                    sc.cap, &gt, &eq);
+      if (threadIdx.x == 0) {
+        const int64_t lt = (int64_t)layer * nt + t;
+        head->pick_key[t] = key;
+        head->pick_gt[t] = gt;
+        sc.state[lt].key = key;
+        sc.gt[lt] = (unsigned long long)gt;
+        sc.eq[lt] = (unsigned long long)eq;
+        if (t < tg.n_rp) put_result(sc, tg, layer, t, value_of(key));
+      }
+    }
+  }
+  cluster.sync();                                      // every target's key is in rank 0
+  if (ok)
+    for (int t0 = tg.n_rp; t0 < nt; t0 += 4) {
+      uint64_t thr[4];
+      const int m = min(4, nt - t0);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) thr[q] = q < m ? cluster.map_shared_rank(&S, 0)->pick_key[t0 + q] : ~0ull;
+      tail_slice(S, row, i0, i1, m, thr, [&](int q, double s) { S.psum[t0 + q] = s; });
+    }
+  cluster.sync();                                      // partial sums complete
+  if (rank == 0) {
+    // warp w: result w of the mean (if wanted) and the TVaR targets; lane b holds block b's partial,
+    // added by a fixed tree
+    if (!ok && threadIdx.x == 0) sel_timeout(sc);
+    for (int w = (int)(threadIdx.x >> 5); ok && w < 1 + nt - tg.n_rp; w += SEL_WARPS) {
+      if (w == 0 && !want_mean) continue;
+      const int t = tg.n_rp + w - 1;
+      const SelShared* const o = cluster.map_shared_rank(&S, lane < B ? lane : 0u);
+      const double a = warp_add(lane < B ? (w == 0 ? o->pmean : o->psum[t]) : 0.0, 8);
+      if (lane != 0) continue;
+      if (w == 0) {
+        put_mean(sc, layer, a / (double)n);
+      } else {
+        put_result(sc, tg, layer, t, tvar_of(a, tg.rank[t], (unsigned long long)S.pick_gt[t], value_of(S.pick_key[t])));
+      }
+    }
+  }
+  cluster.sync();                                      // no block leaves while rank 0 reads it
+}
+
+// ------------------------------------------------------------------------------------------
+// Few rows: the steps in one cooperative launch over every SM, the blocks of a row meeting at grid
+// barriers (bounded waits).
+// ------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -134,13 +881,11 @@ __device__ __forceinline__ uint64_t sel_globaltimer() {
   return t;
 }
 
-// Grid barrier of a cooperative launch: every block adds one to *bar, then waits until it
-// reaches `target` (the number of blocks times the barrier's ordinal).  The wait is bounded by
-// limit_ns; on timeout the block sets *err (and DERR_TIMEOUT in *ext_err) and the whole block
-// returns false.
-__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, uint64_t limit_ns,
-                                             uint32_t* err, uint32_t* ext_err, int skip_arrival,
-                                             int* ok_s) {
+// Every block adds one to *bar, then waits until it reaches `target` (the number of blocks times the
+// barrier's ordinal).  The wait is bounded by limit_ns; on timeout the block records it and the
+// whole block returns false.
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, uint64_t limit_ns, const SelScratch& sc,
+                                             int skip_arrival, int* ok_s) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -151,11 +896,10 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, uin
       while (ld_acquire_gpu(bar) < target) {
         if (sel_globaltimer() - t0 > limit_ns) {
           ok = 0;
-          atomicOr(err, 1u);
-          if (ext_err) atomicOr(ext_err, DERR_TIMEOUT);
+          sel_timeout(sc);
           break;
         }
-        __nanosleep(100);
+        __nanosleep(64);
       }
     }
     __threadfence();
@@ -165,247 +909,81 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, uin
   return *ok_s != 0;
 }
 
-constexpr int SEL_WARPS = SEL_THREADS / 32;
-// Values of a block's slice kept in shared memory across the passes (when the slice fits).
-constexpr int SEL_SMEM_VALUES = 24000;
-
-// Sub-histograms per block: S = SEL_SUBH / ng copies of each group's histogram, warp w adding
-// into copy w mod S, so warps whose keys share a digit (in the first passes, nearly all) do not
-// contend for one shared-memory word.
-constexpr int SEL_SUBH = 32;
-
-// The whole selection of the layers [l0, l0 + gridDim.y): up to 8 radix passes and the tail pass.
-// Block b of a layer owns the contiguous slice [b n / B, (b + 1) n / B) of the layer's row;
-// when it fits, the slice is read once into shared memory and every pass reads it there.
-//
-// Pass: the digit histogram of the keys that match each target's prefix.  Targets whose
-// prefixes are equal share one histogram (in pass 0 all of them do), counted once and stored
-// under the group's first target.  Equal digits within a warp are added with one
-// shared-memory atomic (lanes grouped by __match_any_sync).  After the grid barrier every
-// block picks each target's digit from the global histogram (one warp per target, bins
-// scanned from the top) and keeps the selection state in shared memory.  The counts of the
-// bins above the chosen one add up, over the passes, to #{key > selected key}; the chosen
-// bin's count in the last pass is #{key == selected key}.  The passes stop early once every
-// target's chosen bin holds a single key (distinct values near the targets, the usual case);
-// one scan of the slice then finds those keys.
-//
-// Tail (TVaR targets and the row sum only): the sum of the values above the selected key.
-// Every thread sums its own values in index order, warps and blocks combine with fixed trees,
-// and after a last grid barrier block 0 of each layer combines the block partials in a fixed
-// order: the sums are deterministic.
-__global__ void __launch_bounds__(SEL_THREADS, 1)
-k_select(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets tg, SelScratch sc,
-         int want_mean, uint64_t limit_ns, int64_t smem_values, int skip_arrival) {
-  extern __shared__ double vals[];
-  __shared__ uint32_t h[SEL_SUBH * SEL_BINS];
-  __shared__ uint64_t pre[SEL_MAX_T];
-  __shared__ int64_t kk[SEL_MAX_T];
-  __shared__ unsigned long long cgt[SEL_MAX_T], ceq[SEL_MAX_T];
-  __shared__ uint64_t gpre[SEL_MAX_T];      // prefix of each group
-  __shared__ int32_t gldr[SEL_MAX_T];       // first target of each group
-  __shared__ int32_t tgrp[SEL_MAX_T];       // group of each target
-  __shared__ int32_t ngrp;
-  __shared__ int bar_ok;
-  __shared__ double wsum[SEL_WARPS];
-  const int layer = l0 + blockIdx.y, nt = tg.n_t;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // The blocks of a layer depend only on one another: each layer has its own barrier counter.
-  const uint32_t nblk = gridDim.x;
-  uint32_t* bar = sc.bar + layer;
-  const int64_t i0 = (int64_t)blockIdx.x * n / gridDim.x;
-  const int64_t cnt = ((int64_t)blockIdx.x + 1) * n / gridDim.x - i0;
-  const double* src = ylt + (int64_t)layer * n + i0;
-  const bool resident = cnt <= smem_values;   // smem_values: doubles of dynamic shared memory
-  if (resident) {
-    constexpr int U = 8;   // independent loads in flight per thread
-    for (int64_t j = 0; j < cnt; j += (int64_t)U * SEL_THREADS) {
-      double y[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t i = j + u * SEL_THREADS + threadIdx.x;
-        y[u] = i < cnt ? __ldcg(src + i) : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t i = j + u * SEL_THREADS + threadIdx.x;
-        if (i < cnt) vals[i] = y[u];
-      }
-    }
-  }
-  if (threadIdx.x < nt) {
-    pre[threadIdx.x] = 0ull;
-    kk[threadIdx.x] = tg.rank[threadIdx.x];
-    cgt[threadIdx.x] = 0ull;
-    ceq[threadIdx.x] = 0ull;
-  }
-  __syncthreads();
-  auto value = [&](int64_t i) -> double { return resident ? vals[i] : __ldcg(src + i); };
-
-  const int passes = nt > 0 ? SEL_PASSES : 0;
-  int done = passes;            // passes run
-  for (int pass = 0; pass < passes; ++pass) {
-    if (threadIdx.x == 0) {
-      int ng = 0;
-      for (int t = 0; t < nt; ++t) {
-        int g = 0;
-        while (g < ng && gpre[g] != pre[t]) ++g;
-        if (g == ng) {
-          gpre[g] = pre[t];
-          gldr[g] = t;
-          ++ng;
-        }
-        tgrp[t] = g;
-      }
-      ngrp = ng;
-    }
-    __syncthreads();
-    const int ng = ngrp;
-    int S = SEL_SUBH / ng;                 // sub-histograms per group (a power of two)
-    S = 1 << (31 - __clz(S));
-    for (int i = threadIdx.x; i < ng * S * SEL_BINS; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    const int shift = 64 - SEL_BITS * (pass + 1);
-    uint32_t* hw = h + (warp & (S - 1)) * SEL_BINS;   // this warp's copy (group g: + g S BINS)
-    for (int64_t j = 0; j < cnt; j += SEL_THREADS) {   // bound uniform over the block
-      const int64_t i = j + threadIdx.x;
-      const bool ok = i < cnt;
-      const uint64_t key = key_of(ok ? value(i) : 0.0);
-      const uint32_t d = (uint32_t)(key >> shift) & (SEL_BINS - 1);
-      for (int g = 0; g < ng; ++g) {
-        const bool m = ok && (pass == 0 || (key >> (shift + SEL_BITS)) == (gpre[g] >> (shift + SEL_BITS)));
-        if (!__any_sync(0xffffffffu, m)) continue;
-        const uint32_t peers = __match_any_sync(0xffffffffu, m ? d : 0xffffffffu);
-        if (m && lane == __ffs(peers) - 1) atomicAdd(&hw[g * S * SEL_BINS + d], (uint32_t)__popc(peers));
-      }
-    }
-    __syncthreads();
-    uint32_t* gh = sc.hist + ((int64_t)layer * SEL_PASSES + pass) * nt * SEL_BINS;
-    for (int i = threadIdx.x; i < ng * SEL_BINS; i += blockDim.x) {
-      const int g = i / SEL_BINS, d = i % SEL_BINS;
-      uint32_t c = 0;
-      for (int k = 0; k < S; ++k) c += h[(g * S + k) * SEL_BINS + d];
-      if (c) atomicAdd(&gh[gldr[g] * SEL_BINS + d], c);
-    }
-    if (!grid_barrier(bar, (uint32_t)(pass + 1) * nblk, limit_ns, sc.err, sc.ext_err, skip_arrival, &bar_ok)) return;
-    for (int t = warp; t < nt; t += SEL_WARPS) {
-      const int64_t k = kk[t];
-      const uint32_t* th = gh + gldr[tgrp[t]] * SEL_BINS;
-      // lane l owns bins [SEL_BINS - 8(l+1), SEL_BINS - 8l) (descending order overall)
-      uint32_t c[SEL_BINS / 32];
-      uint32_t mine = 0;
-#pragma unroll
-      for (int u = 0; u < SEL_BINS / 32; ++u) {
-        c[u] = __ldcg(&th[SEL_BINS - 1 - (lane * (SEL_BINS / 32) + u)]);
-        mine += c[u];
-      }
-      uint32_t incl = mine;  // inclusive prefix over lanes (from the top bins down)
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const uint32_t excl = incl - mine;
-      if ((int64_t)excl < k && k <= (int64_t)incl) {
-        int64_t before = excl;
-        int u = 0;
-        for (; u < SEL_BINS / 32; ++u) {
-          if (before + c[u] >= k) break;
-          before += c[u];
-        }
-        const uint32_t bin = SEL_BINS - 1 - (lane * (SEL_BINS / 32) + u);
-        kk[t] = k - before;
-        pre[t] |= (uint64_t)bin << shift;
-        cgt[t] += (unsigned long long)before;           // keys above, with this prefix
-        ceq[t] = c[u];                                  // keys with the new prefix
-      }
-    }
-    __syncthreads();
-    // When every target's prefix matches exactly one key, that key is the selected one and
-    // the remaining passes would change no count: stop.  Every block of the layer read the
-    // same histogram, so all of them stop after the same pass.
-    bool unique = true;
-    for (int t = 0; t < nt; ++t) unique = unique && ceq[t] == 1ull;
-    if (unique) {
-      done = pass + 1;
-      break;
-    }
-  }
-  // Key bits fixed by the passes run: [sh, 64).  Keys above the selected key are the keys whose
-  // fixed bits are above its prefix (after a full selection sh = 0, the plain comparison).
-  const int sh = done > 0 ? 64 - SEL_BITS * done : 0;
-  auto above = [&](uint64_t key, uint64_t prefix) -> bool {
-    return sh == 0 ? key > prefix : (key >> sh) > (prefix >> sh);
-  };
-  if (sh > 0) {   // stopped early: the one key under each target's prefix is its selected key
-    for (int64_t i = threadIdx.x; i < cnt; i += SEL_THREADS) {
-      const uint64_t key = key_of(value(i));
-      for (int t = 0; t < nt; ++t)
-        if ((key >> sh) == (pre[t] >> sh)) sc.state[(int64_t)layer * nt + t].prefix = key;
-    }
-  }
-
-  // ---- tail pass: sums above the selected key (TVaR targets) and the row sum ----
-  for (int t = tg.n_rp; t <= nt; ++t) {
-    if (t == nt && !want_mean) break;
-    const uint64_t thr = t < nt ? pre[t] : 0ull;
-    double a = 0.0;
-    for (int64_t i = threadIdx.x; i < cnt; i += SEL_THREADS) {
-      const double y = value(i);
-      if (t == nt || above(key_of(y), thr)) a = __dadd_rn(a, y);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) a = __dadd_rn(a, __shfl_down_sync(0xffffffffu, a, o));
-    if (lane == 0) wsum[warp] = a;
-    __syncthreads();
-    if (warp == 0) {   // the warps' sums, combined by a fixed tree
-      double s = wsum[lane];
-#pragma unroll
-      for (int o = 16; o; o >>= 1) s = __dadd_rn(s, __shfl_down_sync(0xffffffffu, s, o));
-      if (lane == 0) {
-        if (t < nt) sc.psum[((int64_t)layer * nt + t) * gridDim.x + blockIdx.x] = s;
-        else sc.pmean[(int64_t)layer * gridDim.x + blockIdx.x] = s;
-      }
-    }
-    __syncthreads();
-  }
-  if (!grid_barrier(bar, (uint32_t)(done + 1) * nblk, limit_ns, sc.err, sc.ext_err, skip_arrival, &bar_ok)) return;
-  if (blockIdx.x != 0) return;
-  // Block 0 of the layer: one warp per target (and one for the mean) combines the block
-  // partials: lane l adds blocks l, l + 32, ... in order, then a fixed shuffle tree.
+__global__ void __launch_bounds__(SEL_THREADS, 2)
+k_sel_grid(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets tg, SelScratch sc, int want_mean,
+           uint64_t limit_ns, int skip_arrival) {
+  extern __shared__ __align__(16) unsigned char sel_smem[];
+  SelShared& S = *reinterpret_cast<SelShared*>(sel_smem);
+  __shared__ int ok_s;
   const unsigned B = gridDim.x;
-  for (int t = warp; t <= nt; t += SEL_WARPS) {
-    if (t == nt && !want_mean) continue;
+  const int layer = l0 + (int)blockIdx.y, nt = tg.n_t;
+  const int64_t lt0 = (int64_t)layer * nt;
+  const double* row = ylt + (int64_t)layer * n;
+  const int64_t i0 = slice_begin(n, blockIdx.x, B), i1 = slice_begin(n, blockIdx.x + 1, B);
+  uint32_t met = 0;
+  auto meet = [&]() { return grid_barrier(sc.bar + layer, ++met * B, limit_ns, sc, skip_arrival, &ok_s); };
+  auto block_sums = [&](const double* p) {
     double a = 0.0;
-    if (t == nt) {
-      for (unsigned b = lane; b < B; b += 32) a = __dadd_rn(a, __ldcg(&sc.pmean[(int64_t)layer * B + b]));
-    } else if (t >= tg.n_rp) {
-      const int64_t base = ((int64_t)layer * nt + t) * B;
-      for (unsigned b = lane; b < B; b += 32) a = __dadd_rn(a, __ldcg(&sc.psum[base + b]));
+    for (unsigned b = threadIdx.x; b < B; b += SEL_THREADS) a = __dadd_rn(a, __ldcg(p + b));
+    return block_sum(a, S.wsum);
+  };
+  // Round t = nt: all targets.  Then, where lists may overflow (sc.count2), a round for each target
+  // whose list did: its interval is split again by keys that made it into the list.  Every block
+  // knows the same states.  A list is its first target's: the others sharing it go first.
+#pragma unroll 1
+  for (int t = nt; t >= 0; --t) {
+    SelState old{0ull, 0ull, ~0ull, 0, 0, 0, 0};
+    int np = 0;
+    uint32_t *g = sc.count + (int64_t)layer * SEL_CLASSES, *n_list = sc.n_list + lt0;
+    if (t < nt) {
+      if (!sc.count2) break;
+      old = S.st[t];
+      if (old.tie || old.in_class <= sc.cap) continue;
+      g = sc.count2 + (lt0 + t) * SEL_CLASSES;
+      n_list = sc.n_list2 + lt0;
     }
+    if (nt > 0) np = row_splitters(S, row, n, sc.sample, tg, t < nt ? sc.list + (lt0 + old.list) * sc.cap : nullptr, sc.cap);
+    const double part = count_slice(S, row, i0, i1, np, old.lo, old.hi, t == nt ? want_mean : 0);
+    if (t == nt && want_mean && threadIdx.x == 0) sc.pmean[(int64_t)layer * B + blockIdx.x] = part;
+    for (int i = threadIdx.x; np > 0 && i <= 2 * np; i += SEL_THREADS)
+      if (S.hist[i]) atomicAdd(g + i, S.hist[i]);
+    if (!meet()) return;
+    if (t == nt && want_mean && blockIdx.x == B - 1) {
+      const double s = block_sums(sc.pmean + (int64_t)layer * B);
+      if (threadIdx.x == 0) put_mean(sc, layer, s / (double)n);
+    }
+    if (nt == 0) return;
+    for (int i = threadIdx.x; i <= 2 * np; i += SEL_THREADS) S.cnt[i] = __ldcg(g + i);
+    __syncthreads();
+    target_classes(S, tg, t < nt ? t : 0, t < nt ? t + 1 : nt, np, old.lo, old.hi, old.before);
+    collect_slice(S, row, i0, i1, sc.list + lt0 * sc.cap, sc.cap, [&](int q) { return n_list + q; });
+    if (!meet()) return;
+  }
+  for (int t = (int)blockIdx.x; t < nt; t += (int)B) {
+    const SelState st = S.st[t];
+    int64_t gt, eq;
+    const uint64_t key = pick_key(S, row, n, st, tg.rank[t], sc.list + (lt0 + st.list) * sc.cap, sc.cap, &gt, &eq);
+    if (threadIdx.x == 0) {
+      sc.state[lt0 + t].key = key;
+      sc.gt[lt0 + t] = (unsigned long long)gt;
+      sc.eq[lt0 + t] = (unsigned long long)eq;
+      if (t < tg.n_rp) put_result(sc, tg, layer, t, value_of(key));
+    }
+  }
+  if (nt == tg.n_rp) return;
+  if (!meet()) return;
+  for (int t0 = tg.n_rp; t0 < nt; t0 += 4) {
+    uint64_t thr[4];
+    const int m = min(4, nt - t0);
 #pragma unroll
-    for (int o = 16; o; o >>= 1) a = __dadd_rn(a, __shfl_down_sync(0xffffffffu, a, o));
-    if (lane != 0) continue;
-    if (t == nt) {
-      sc.mean[layer] = a / (double)n;
-      if (sc.user_mean) sc.user_mean[layer] = a / (double)n;
-      continue;
-    }
-    const uint64_t key = sh > 0 ? __ldcg(&sc.state[(int64_t)layer * nt + t].prefix) : pre[t];
-    const double v = value_of(key);
-    double r = v;
-    if (t >= tg.n_rp) {
-      const int64_t m = tg.rank[t];
-      r = (a + (double)(m - (int64_t)cgt[t]) * v) / (double)m;
-    }
-    sc.out[layer * nt + t] = r;
-    if (t < tg.n_rp) {
-      if (sc.user_pml) sc.user_pml[(int64_t)layer * tg.n_rp + t] = r;
-    } else if (sc.user_tvar) {
-      sc.user_tvar[(int64_t)layer * (nt - tg.n_rp) + (t - tg.n_rp)] = r;
-    }
-    sc.gt[layer * nt + t] = cgt[t];
-    sc.eq[layer * nt + t] = ceq[t];
-    sc.state[layer * nt + t] = SelState{key, kk[t]};
+    for (int q = 0; q < 4; ++q) thr[q] = q < m ? __ldcg(&sc.state[lt0 + t0 + q].key) : ~0ull;
+    tail_slice(S, row, i0, i1, m, thr, [&](int q, double s) { sc.psum[(lt0 + t0 + q) * B + blockIdx.x] = s; });
+  }
+  if (!meet()) return;
+  for (int t = tg.n_rp + (int)blockIdx.x; t < nt; t += (int)B) {
+    const double s = block_sums(sc.psum + (lt0 + t) * B);
+    if (threadIdx.x == 0)
+      put_result(sc, tg, layer, t, tvar_of(s, tg.rank[t], __ldcg(sc.gt + lt0 + t), value_of(__ldcg(&sc.state[lt0 + t].key))));
   }
 }
 
@@ -449,67 +1027,81 @@ ara_status validate_metrics(int64_t n, int32_t n_rp, const double* rps, int32_t 
   return select_targets(n, n_rp, rps, n_tvar, levels, tg);
 }
 
-constexpr int SEL_DYN_SMEM = SEL_SMEM_VALUES * (int)sizeof(double);
-
-// Co-resident blocks of k_select on this device (cached per device); 0 on failure.
-static int select_resident_blocks() {
+// Shared-memory and cluster attributes of the kernels, set once per device.
+static ara_status sel_prepare_kernels() {
   static std::mutex mu;
-  static int cached[64] = {0};
+  static bool done[64] = {false};
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  ARA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return ARA_ECUDA;
   std::lock_guard<std::mutex> lk(mu);
-  if (!cached[dev]) {
-    int per_sm = 0, sms = 0;
-    if (cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_DYN_SMEM) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_select, SEL_THREADS, SEL_DYN_SMEM) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm < 1)
-      return 0;
-    cached[dev] = per_sm * sms;
-  }
-  return cached[dev];
+  if (done[dev]) return ARA_OK;
+  for (const void* f : {(const void*)k_sel_cluster, (const void*)k_sel_grid})
+    ARA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
+  ARA_TRY(cudaFuncSetAttribute((const void*)k_sel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  done[dev] = true;
+  return ARA_OK;
 }
 
-// Blocks per layer: one per SM for a single layer, fewer per layer when several share a
-// launch, and never more than one per SEL_THREADS values.
-int32_t select_blocks(int64_t n, int n_sms, int32_t n_layers) {
-  const int64_t b = (n + SEL_THREADS - 1) / SEL_THREADS;
-  const int64_t cap = std::max<int64_t>(1, (int64_t)n_sms / std::max(1, n_layers));
-  return (int32_t)std::max<int64_t>(1, std::min(b, cap));
+size_t select_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_t, int n_sms) {
+  return sel_plan(n, n_layers, n_t, n_sms, list_cap(n), true).bytes;
 }
 
-// Launch the whole selection into `scratch` (zero-filled here); results land in scratch.out.
-// Layers are split into cooperative launches whose blocks are all co-resident.
-ara_status launch_select(const double* d_ylt, int64_t n, int32_t n_layers, const SelTargets& tg,
-                         void* scratch, size_t scratch_bytes, int32_t blocks, int want_mean,
-                         cudaStream_t s, SelScratch* out, uint32_t* ext_err = nullptr,
+// Launch the whole selection into `scratch` (laid out by `y`, its first part zero-filled here);
+// results land in scratch.out / mean.
+ara_status launch_select(const double* d_ylt, const SelPlan& y, const SelTargets& tg, void* scratch,
+                         int want_mean, cudaStream_t s, SelScratch* out, uint32_t* ext_err = nullptr,
                          double* user_pml = nullptr, double* user_tvar = nullptr,
                          double* user_mean = nullptr) {
-  SelScratch sc = carve(scratch, n_layers, tg.n_t, blocks);
+  SelScratch sc = carve(scratch, y);
   sc.ext_err = ext_err;
   sc.user_pml = user_pml;
   sc.user_tvar = user_tvar;
   sc.user_mean = user_mean;
-  ARA_TRY(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
-  const int resident = select_resident_blocks();
-  if (resident < blocks) return ARA_ECUDA;
-  const int32_t per_launch = std::max(1, resident / blocks);
-  const uint64_t limit = wait_limit_ns();
-  const int64_t slice = (n + blocks - 1) / blocks;
-  const int dyn = slice <= SEL_SMEM_VALUES ? (int)(slice * sizeof(double)) : 0;
-  for (int32_t l0 = 0; l0 < n_layers; l0 += per_launch) {
-    const int32_t nl = std::min(per_launch, n_layers - l0);
+  const int64_t n = y.n;
+  const ara_status ready = sel_prepare_kernels();
+  if (ready != ARA_OK) return ready;
+  ARA_TRY(cudaMemsetAsync(scratch, 0, y.zero_bytes, s));
+  if (y.small) {
+    int pad = 64;
+    while (pad < n) pad <<= 1;
     LaunchScope ls(ARA_K_SELECT, s);
+    k_sel_small<<<(unsigned)y.n_layers, SEL_THREADS, (size_t)pad * 8, s>>>(d_ylt, (int32_t)n, pad, tg, sc, want_mean);
+    ARA_TRY(cudaGetLastError());
+    *out = sc;
+    return ARA_OK;
+  }
+  const int skip = debug_skip_arrival();
+  if (y.cluster) {
+    for (int32_t l0 = 0; l0 < y.n_layers; l0 += 32768) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)y.blocks, (unsigned)std::min<int32_t>(32768, y.n_layers - l0));
+      cfg.blockDim = dim3(SEL_THREADS);
+      cfg.dynamicSmemBytes = SEL_SMEM;
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)y.blocks;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      LaunchScope ls(ARA_K_SELECT, s);
+      ARA_TRY(cudaLaunchKernelEx(&cfg, k_sel_cluster, d_ylt, n, l0, tg, sc, want_mean, skip));
+    }
+    *out = sc;
+    return ARA_OK;
+  }
+  const int32_t per = std::max(1, y.n_sms / y.blocks);      // rows whose blocks run at once
+  for (int32_t l0 = 0; l0 < y.n_layers; l0 += per) {
+    const dim3 grid((unsigned)y.blocks, (unsigned)std::min(per, y.n_layers - l0));
+    uint64_t limit = wait_limit_ns();
     int64_t nn = n;
-    int32_t ll0 = l0;
     SelTargets t2 = tg;
-    SelScratch s2 = sc;
-    int wm = want_mean;
-    uint64_t lim = limit;
-    int64_t cap = dyn / (int)sizeof(double);
-    int skip = debug_skip_arrival();
-    void* args[] = {(void*)&d_ylt, &nn, &ll0, &t2, &s2, &wm, &lim, &cap, &skip};
-    ARA_TRY(cudaLaunchCooperativeKernel((const void*)k_select, dim3(blocks, nl), dim3(SEL_THREADS),
-                                        args, (size_t)dyn, s));
+    int wm = want_mean, sk = skip;
+    void* args[] = {(void*)&d_ylt, &nn, &l0, &t2, &sc, &wm, &limit, &sk};
+    LaunchScope ls(ARA_K_SELECT, s);
+    ARA_TRY(cudaLaunchCooperativeKernel((const void*)k_sel_grid, grid, dim3(SEL_THREADS), args, (size_t)SEL_SMEM, s));
   }
   *out = sc;
   return ARA_OK;
@@ -525,20 +1117,19 @@ ara_status select_one_rank(const double* d_ylt, int64_t n, int32_t n_layers, int
                            cudaStream_t s, SelectResult* out, uint32_t* err) {
   SelTargets tg;
   tg.n_t = 1;
-  tg.n_rp = 0;
+  tg.n_rp = 1;               // the key and its counts, no tail sum
   tg.rank[0] = m;
-  const int32_t blocks = select_blocks(n, n_sms, n_layers);
-  const size_t bytes = select_scratch_bytes(n_layers, 1, blocks);
+  const SelPlan y = sel_plan(n, n_layers, 1, n_sms, list_cap(n));
   void* scratch = nullptr;
-  ARA_TRY(dmalloc_async(&scratch, bytes, s));
+  ARA_TRY(dmalloc_async(&scratch, y.bytes, s));
   SelScratch sc;
-  ara_status st = launch_select(d_ylt, n, n_layers, tg, scratch, bytes, blocks, 0, s, &sc, err);
+  ara_status st = launch_select(d_ylt, y, tg, scratch, 0, s, &sc, err);
   if (st != ARA_OK) {
     cudaFreeAsync(scratch, s);
     return st;
   }
   out->scratch = scratch;
-  out->thr_key = &sc.state[0].prefix;
+  out->thr_key = &sc.state[0].key;
   out->thr_stride = sizeof(SelState) / sizeof(uint64_t);
   out->gt = sc.gt;
   out->eq = sc.eq;
@@ -553,7 +1144,7 @@ void free_select_result(SelectResult& r, cudaStream_t s) {
 ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_layers,
                                int32_t n_rp, const double* rps, int32_t n_tvar,
                                const double* levels, double* h_pml, double* h_tvar,
-                               double* h_mean, cudaStream_t s) {
+                               double* h_mean, cudaStream_t s, bool beside) {
   SelTargets tg;
   if (!d_ylt || n_layers < 1) return ARA_EINVAL;
   if ((n_rp > 0 && !h_pml) || (n_tvar > 0 && !h_tvar)) return ARA_EINVAL;
@@ -564,12 +1155,11 @@ ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int32_t blocks = select_blocks(n_trials, sms, n_layers);
-  const size_t bytes = select_scratch_bytes(n_layers, tg.n_t, blocks);
+  const SelPlan y = sel_plan(n_trials, n_layers, tg.n_t, sms, list_cap(n_trials), beside);
   void* scratch = nullptr;
-  ARA_TRY(dmalloc_async(&scratch, bytes, s));
+  ARA_TRY(dmalloc_async(&scratch, y.bytes, s));
   SelScratch sc;
-  st = launch_select(d_ylt, n_trials, n_layers, tg, scratch, bytes, blocks, h_mean != nullptr, s, &sc);
+  st = launch_select(d_ylt, y, tg, scratch, h_mean != nullptr, s, &sc);
   std::vector<double> out((size_t)n_layers * tg.n_t);
   uint32_t timed_out = 0;
   if (st == ARA_OK) {
@@ -611,14 +1201,13 @@ ara_status risk_metrics_queue(const double* d_ylt, int64_t n_trials, int32_t n_l
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int32_t blocks = select_blocks(n_trials, sms, n_layers);
-  *need = select_scratch_bytes(n_layers, tg.n_t, blocks);
+  const SelPlan y = sel_plan(n_trials, n_layers, tg.n_t, sms, list_cap(n_trials));
+  *need = y.bytes;
   if (!scratch || scratch_bytes < *need) return ARA_ERANGE;
   SelScratch sc;
   ARA_TRY(cudaMemsetAsync(d_status, 0, sizeof(uint32_t), s));
-  return launch_select(d_ylt, n_trials, n_layers, tg, scratch, *need, blocks, d_mean != nullptr, s,
-                       &sc, d_status, n_rp > 0 ? d_pml : nullptr, n_tvar > 0 ? d_tvar : nullptr,
-                       d_mean);
+  return launch_select(d_ylt, y, tg, scratch, d_mean != nullptr, s, &sc, d_status,
+                       n_rp > 0 ? d_pml : nullptr, n_tvar > 0 ? d_tvar : nullptr, d_mean);
 }
 }  // namespace ara
 
@@ -639,17 +1228,15 @@ extern "C" ara_status ara_risk_metrics_async(const double* d_ylt, int64_t n_tria
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int32_t blocks = select_blocks(n_trials, sms, n_layers);
-  const size_t bytes = select_scratch_bytes(n_layers, tg.n_t, blocks);
+  const SelPlan y = sel_plan(n_trials, n_layers, tg.n_t, sms, list_cap(n_trials));
   void* scratch = nullptr;
-  if (dmalloc_async(&scratch, bytes, s) != cudaSuccess) return ARA_ENOMEM;
+  if (dmalloc_async(&scratch, y.bytes, s) != cudaSuccess) return ARA_ENOMEM;
   ara_status r = ARA_OK;
   SelScratch sc;
   if (cudaMemsetAsync(d_status, 0, sizeof(uint32_t), s) != cudaSuccess) r = ARA_ECUDA;
   if (r == ARA_OK)   // the kernel writes the results straight into d_pml / d_tvar / d_mean
-    r = launch_select(d_ylt, n_trials, n_layers, tg, scratch, bytes, blocks, d_mean != nullptr, s,
-                      &sc, d_status, n_rp > 0 ? d_pml : nullptr, n_tvar > 0 ? d_tvar : nullptr,
-                      d_mean);
+    r = launch_select(d_ylt, y, tg, scratch, d_mean != nullptr, s, &sc, d_status,
+                      n_rp > 0 ? d_pml : nullptr, n_tvar > 0 ? d_tvar : nullptr, d_mean);
   cudaFreeAsync(scratch, s);
   return r;
 }
@@ -659,7 +1246,7 @@ extern "C" ara_status ara_risk_metrics(const double* d_ylt, int64_t n_trials, in
                                        const double* levels, double* h_pml, double* h_tvar,
                                        double* h_mean, void* stream) {
   return risk_metrics_device(d_ylt, n_trials, n_layers, n_rp, rps, n_tvar, levels, h_pml, h_tvar,
-                             h_mean, (cudaStream_t)stream);
+                             h_mean, (cudaStream_t)stream, false);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -696,41 +1283,58 @@ extern "C" ara_status ara_risk_metrics_static(const double* d_ylt, int64_t n_tri
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  // Fewer blocks shrink the per-block partials; if even one block does not fit, refuse.
-  int32_t blocks = select_blocks(n_trials, sms, n_layers);
-  while (blocks > 1 && select_scratch_bytes(n_layers, tg.n_t, blocks) > ARA_STATIC_SELECT_BYTES)
-    blocks = blocks / 2;
-  const size_t bytes = select_scratch_bytes(n_layers, tg.n_t, blocks);
-  if (bytes > ARA_STATIC_SELECT_BYTES) return ARA_ERANGE;
+  // The request's size is bounded as documented (about 8 KiB per layer and level).
+  const size_t lt = (size_t)n_layers * (size_t)tg.n_t;
+  size_t need = 0;
+  for (size_t part : {8192 * lt, 4 * (size_t)n_layers, (size_t)4, 16 * lt, 8 * lt, 8 * lt, 8 * lt, 8 * lt, 8 * lt,
+                      8 * lt, 8 * (size_t)n_layers, 8 * (size_t)n_layers})
+    need = (need + 255) / 256 * 256 + part;
+  if ((need + 255) / 256 * 256 > ARA_STATIC_SELECT_BYTES) return ARA_ERANGE;
+  // As many layers at a time as the array holds; where even one layer's lists do not fit, shorter
+  // lists and a second round.
+  const int64_t cap = list_cap(n_trials);
+  int32_t per = n_layers;
+  auto plan = [&](int64_t c) {
+    return sel_plan(n_trials, per, tg.n_t, sms, c);
+  };
+  while (per > 1 && plan(cap).bytes > ARA_STATIC_SELECT_BYTES) per = (per + 1) / 2;
+  SelPlan y = plan(cap);
+  for (int64_t c = cap / 2; y.bytes > ARA_STATIC_SELECT_BYTES && c >= SEL_SAMPLE; c /= 2) y = plan(c);
+  if (y.bytes > ARA_STATIC_SELECT_BYTES) return ARA_ERANGE;
   void* scratch = nullptr;
   if ((st = static_scratch(&scratch)) != ARA_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  SelScratch sc;
-  // launch_select clears the used part of the scratch before its first kernel
-  if ((st = launch_select(d_ylt, n_trials, n_layers, tg, scratch, bytes, blocks, h_mean != nullptr,
-                          s, &sc)) != ARA_OK)
-    return st;
-  // Keep the first failing copy's status, but always wait for the stream before returning, so
-  // that no copy queued here can land in the caller's buffers after the call has returned.
   cudaError_t e = cudaSuccess;
-  const size_t row = sizeof(double) * (size_t)tg.n_t;
-  if (e == cudaSuccess && n_rp > 0)
-    e = cudaMemcpy2DAsync(h_pml, sizeof(double) * n_rp, sc.out, row, sizeof(double) * n_rp,
-                          (size_t)n_layers, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && n_tvar > 0)
-    e = cudaMemcpy2DAsync(h_tvar, sizeof(double) * n_tvar, sc.out + n_rp, row,
-                          sizeof(double) * n_tvar, (size_t)n_layers, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && h_mean)
-    e = cudaMemcpyAsync(h_mean, sc.mean, sizeof(double) * n_layers, cudaMemcpyDeviceToHost, s);
   uint32_t timed_out = 0;
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&timed_out, sc.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+  const size_t row = sizeof(double) * (size_t)tg.n_t;
+  for (int32_t l0 = 0; l0 < n_layers && st == ARA_OK && e == cudaSuccess && !timed_out; l0 += per) {
+    const int32_t nl = std::min(per, n_layers - l0);
+    if (nl < per) y = sel_plan(n_trials, nl, tg.n_t, sms, y.cap);
+    SelScratch sc;
+    st = launch_select(d_ylt + (int64_t)l0 * n_trials, y, tg, scratch, h_mean != nullptr, s, &sc);
+    if (st != ARA_OK) break;
+    if (n_rp > 0)
+      e = cudaMemcpy2DAsync(h_pml + (size_t)l0 * n_rp, sizeof(double) * n_rp, sc.out, row, sizeof(double) * n_rp,
+                            (size_t)nl, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && n_tvar > 0)
+      e = cudaMemcpy2DAsync(h_tvar + (size_t)l0 * n_tvar, sizeof(double) * n_tvar, sc.out + n_rp, row,
+                            sizeof(double) * n_tvar, (size_t)nl, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && h_mean)
+      e = cudaMemcpyAsync(h_mean + l0, sc.mean, sizeof(double) * nl, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&timed_out, sc.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    // the next layers reuse the array, and the status decides whether they run
+    if (l0 + nl < n_layers && e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
+  // Always wait for the stream before returning, so that no copy queued here can land in the
+  // caller's buffers after the call has returned.
   if (e != cudaSuccess) note_cuda_error(e, "static risk metrics: result copy", __FILE__, __LINE__);
   const cudaError_t es = cudaStreamSynchronize(s);
   if (e == cudaSuccess && es != cudaSuccess) {
     note_cuda_error(es, "cudaStreamSynchronize", __FILE__, __LINE__);
     e = es;
   }
+  if (st != ARA_OK) return st;
   if (e != cudaSuccess) return ARA_ECUDA;
   return timed_out ? ARA_ETIMEOUT : ARA_OK;
 }

@@ -96,7 +96,8 @@ int64_t estimate_bytes(const Portfolio& pool, const Request& r) {
   const int64_t nl = (int64_t)r.layer_off.size() - 1, n = r.t1 - r.t0, C = pool.catalogue;
   int64_t b = nl * (8 * C + 4 * (pool.bm_words + pool.cbits_stride)) + 4096 * nl;   // layer set
   b += nl * n * 9;                                                                  // YLT + regimes
-  b += 8192 * (int64_t)(r.rps.size() + r.levels.size() + 2) * nl + (1 << 20);       // selection
+  b += (int64_t)select_scratch_bytes(n, (int32_t)nl, (int32_t)(r.rps.size() + r.levels.size()) + 1,
+                                     pool.n_sms) + (1 << 20);                         // selections
   {   // batched table (every request may run in a merged batched pass)
     int64_t bound = 0;
     for (int32_t j : r.layer_elts) bound += pool.rec_off[j + 1] - pool.rec_off[j];
@@ -137,7 +138,7 @@ ara_status finish_request(ara_server& S, Request& r, ara_portfolio* ls, int32_t 
     r.mean.assign(r.want_mean ? (size_t)nl : 0, 0.0);
     st = risk_metrics_device(ylt, n, nl, (int32_t)r.rps.size(), r.rps.data(), (int32_t)r.levels.size(),
                              r.levels.data(), r.pml.data(), r.tvar.data(),
-                             r.want_mean ? r.mean.data() : nullptr, s);
+                             r.want_mean ? r.mean.data() : nullptr, s, true);
   }
   if (st == ARA_OK && r.want_adjoint) {
     int64_t K = 0, M = 0;

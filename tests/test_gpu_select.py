@@ -1,0 +1,74 @@
+"""The selection behind PML and TVaR at the edges of its forms (rows sorted whole, one cooperative
+launch, a cluster per row, lists split a second time), against sorted rows.  PML is a copy of a YLT
+entry, so it is equal; TVaR and the mean are FP64 sums of up to 3e6 values of one sign in trees of
+pairwise depth, 1e-13 relative (about 500 rounding units; the trees are a few tens deep)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_1606_04473_gb300 as ara
+
+RPS = [1.0, 2.0, 10.0, 100.0, 250.0]
+LEVELS = [0.0, 0.5, 0.99]
+
+
+def count(x):
+    r = np.rint(x)
+    return int(r if abs(x - r) <= 1e-9 * max(1.0, abs(x)) else np.ceil(x))
+
+
+def check(y, rps=RPS, levels=LEVELS, call=None):
+    d = torch.from_numpy(y).cuda()
+    call = call or ara.risk_metrics
+    pml, tvar, mean = call(d, rps, levels, want_mean=True)
+    s = np.sort(y, axis=1)[:, ::-1]
+    n = y.shape[1]
+    for i, r in enumerate(rps):
+        assert np.array_equal(pml[:, i], s[:, count(n / r) - 1]), r
+    for i, p in enumerate(levels):
+        m = count(n * (1.0 - p))
+        np.testing.assert_allclose(tvar[:, i], s[:, :m].astype(np.longdouble).mean(1).astype(float), rtol=1e-13)
+    np.testing.assert_allclose(mean, y.astype(np.longdouble).mean(1).astype(float), rtol=1e-13)
+
+
+def rows(seed, n_rows, n):
+    """Shapes a YLT can take: lognormal years, zeros below a retention with ties at a limit, sorted
+    years, few distinct values, one large value in a constant row, near-equal neighbours."""
+    g = np.random.default_rng(seed)
+    out = np.empty((n_rows, n))
+    for i in range(n_rows):
+        x = np.exp(g.normal(14.0, 2.0, n))
+        k = i % 6
+        if k == 1:
+            x = np.clip(x - np.median(x), 0.0, np.quantile(x, 0.97))
+        elif k == 2:
+            x = np.sort(x)
+        elif k == 3:
+            x = g.integers(0, 7, n) * 1e6
+        elif k == 4:
+            x[:] = 3.5
+            x[n // 3] = 1e9
+        elif k == 5:
+            x = 1e6 + np.arange(n) % 5000 * np.spacing(1e6)
+        out[i] = x
+    return out
+
+
+@pytest.mark.parametrize("n_rows,n", [(6, 1), (6, 2), (6, 63), (6, 65), (7, 1000), (6, 4096), (6, 4097), (6, 30_011),
+                                      (32, 5_000), (33, 5_000), (1, 400_003), (40, 70_001), (160, 4_100), (6, 600_000)])
+def test_rows_of_every_form(n_rows, n):
+    levels = [p for p in LEVELS if count(n * (1.0 - p)) >= 1]
+    check(rows(n, n_rows, n), levels=levels)
+
+
+def test_allocation_free_call_splits_overfull_lists():
+    """Sixteen targets on a long row: the fixed array holds lists of a few thousand keys only, so the
+    intervals are split a second time (for several targets that share one, too)."""
+    g = np.random.default_rng(4)
+    y = np.exp(g.normal(14.0, 1.0, (2, 3_000_017)))
+    y[1, : 1_000_000] = 0.0
+    rps = [1.0, 1.5, 2.0, 2.0000001, 2.0000002, 3.0, 10.0, 100.0, 250.0, 1000.0, 2000.0]
+    check(y, rps, [0.0, 0.3, 0.5, 0.9, 0.99], ara.risk_metrics_static)
