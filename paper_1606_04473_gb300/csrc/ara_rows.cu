@@ -202,20 +202,6 @@ struct RowsBuild {
   uint8_t slot_of[256];        // layer -> slot
 };
 
-// round-to-nearest-even of o * 2^fb as an integer, o >= 0 finite, o * 2^fb < 2^55: the value of
-// __double2ull_rn(o * 2^fb) (the product is exact) without the FP64 pipe.
-__device__ __forceinline__ uint64_t fixed_rn(double o, int fb) {
-  const uint64_t b = (uint64_t)__double_as_longlong(o) & 0x7fffffffffffffffull;
-  const int ex = (int)(b >> 52);
-  const uint64_t m = (b & ((1ull << 52) - 1)) | (ex ? 1ull << 52 : 0ull);
-  const int sh = (ex ? ex : 1) - 1075 + fb;
-  if (sh >= 0) return m << min(sh, 63);
-  const int r = -sh;
-  if (r > 54) return 0ull;
-  const uint64_t q = m >> r, rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
-  return q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull);
-}
-
 struct RowsLayer {             // staged per block
   double occ_ret, occ_lim;
   int32_t frac_bits, slot;

@@ -168,3 +168,44 @@ def test_run_of_several_layers_takes_the_rows_and_keeps_prepared_runs():
         assert torch.equal(out, ref)
     pf.check()
     pf.close()
+
+
+@pytest.mark.parametrize("C,n_elts,nnz,f32", [(31, 3, 20, True), (257, 5, 200, False), (70_001, 9, 4_000, True),
+                                              (200_000, 12, 9_000, False), (1_000_003, 8, 60_000, True)])
+def test_fold_by_event_equals_fold_by_tiles(C, n_elts, nnz, f32):
+    """The fold from the event-major records against the fold by tiles, which a layer with its ELTs in
+    another order takes: two ELTs per event at most make the order of the sum irrelevant, so the
+    YLTs, the maxima and the adjoints (occurrence regimes) are equal."""
+    g = np.random.default_rng(C)
+    ids = [np.sort(g.choice(C, size=nnz, replace=False)).astype(np.int32) for _ in range(n_elts)]
+    seen = np.zeros(C, np.int32)
+    keep = []
+    for i in ids:                       # at most two ELTs per event
+        k = seen[i] < 2
+        seen[i[k]] += 1
+        keep.append(i[k])
+    loss = [np.exp(11.0 + 2.0 * g.standard_normal(i.size)) for i in keep]
+    if f32:
+        loss = [x.astype(np.float32).astype(np.float64) for x in loss]
+    ret, lim = np.full(n_elts, 1e4), np.full(n_elts, 1e6)
+    up = list(range(n_elts))
+    part = up[: max(2, n_elts - 2)]     # a layer that does not hold every ELT
+    for layer in (up, part):
+        pf = ara.Portfolio(C, keep, loss, ret, lim, [layer, layer[::-1]], [2e4] * 2, [9e5] * 2, [1e5] * 2, [1e7] * 2,
+                           losses_f32=f32)
+        counts = g.poisson(60.0, 400)
+        off = np.zeros(401, np.int64)
+        np.cumsum(counts, out=off[1:])
+        off, yet = torch.from_numpy(off).cuda(), torch.from_numpy(g.integers(0, C, off[-1], dtype=np.int32)).cuda()
+        reg = torch.empty((2, 400), dtype=torch.uint8, device="cuda")
+        ys = [pf.run_ylt(off, yet, layers=[l], regimes=reg[l:l + 1]) for l in (0, 1)]
+        assert torch.equal(ys[0], ys[1]) and torch.equal(reg[0], reg[1])
+        f64 = [pf.run_ylt(off, yet, layers=[l], flags=ara.ARA_RUN_F64_SUM) for l in (0, 1)]
+        oep = [pf.run_ylt(off, yet, layers=[l], flags=ara.ARA_RUN_OEP) for l in (0, 1)]
+        assert torch.equal(f64[0], f64[1]) and torch.equal(oep[0], oep[1])
+        a, b = (pf.adjoint(off, yet, ys[l], reg[l:l + 1], 0.9, layers=[l]) for l in (0, 1))
+        assert torch.equal(a["layer"], b["layer"])
+        k = len(layer)
+        assert torch.equal(a["elt"], b["elt"].flip(1)) and k == a["elt"].shape[1]
+        pf.check()
+        pf.close()
