@@ -334,9 +334,10 @@ class Portfolio:
         K = sum(len(self.layer_elts[l]) for l in lay)
         M = sum(self.elt_nnz[j] for l in lay for j in self.layer_elts[l])
         dev = ylt.device
-        ge = torch.zeros((2, max(K, 1), 2), dtype=torch.float64, device=dev)
-        gl = torch.zeros((2, n_out, 4), dtype=torch.float64, device=dev)
-        gx = torch.zeros((2, max(M, 1)), dtype=torch.float64, device=dev)
+        # every element that is returned is written by the call
+        ge = torch.empty((2, max(K, 1), 2), dtype=torch.float64, device=dev)
+        gl = torch.empty((2, n_out, 4), dtype=torch.float64, device=dev)
+        gx = torch.empty((2, max(M, 1)), dtype=torch.float64, device=dev)
         ties = np.zeros(n_out, dtype=np.int32)
         if index is not None:
             st = lib().ara_adjoint_indexed(self._h, index._handle(), int(first_trial),

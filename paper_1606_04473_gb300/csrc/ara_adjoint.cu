@@ -1025,6 +1025,34 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
 
 using namespace ara;
 
+// The end of an adjoint call: ties and the device error word in one wait (through pinned memory where
+// a slot is free), then the selection's scratch is released.
+static ara_status adjoint_end(Portfolio& pf, ara_status st, SelectResult& sr, int32_t n_sel, int64_t m,
+                              int32_t* h_ties, cudaStream_t s) {
+  const size_t words = (size_t)(sr.eq - sr.gt) + (size_t)n_sel;     // gt and eq lie in one block
+  PinnedSlot slot;
+  std::vector<unsigned long long> local;
+  unsigned long long* r = (unsigned long long*)slot.p;
+  if (!r || (words + 1) * 8 > PinnedSlot::kBytes) {
+    local.resize(words + 1);
+    r = local.data();
+  }
+  r[words] = 0;
+  if (st == ARA_OK && h_ties &&
+      cudaMemcpyAsync(r, sr.gt, 8 * words, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    st = ARA_ECUDA;
+  if (st == ARA_OK &&
+      cudaMemcpyAsync(&r[words], pf.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    st = ARA_ECUDA;
+  const size_t eq0 = (size_t)(sr.eq - sr.gt);
+  free_select_result(sr, s);
+  if (cudaStreamSynchronize(s) != cudaSuccess && st == ARA_OK) st = ARA_ECUDA;
+  if (st != ARA_OK) return st;
+  if (h_ties)
+    for (int32_t i = 0; i < n_sel; ++i) h_ties[i] = (int64_t)(r[i] + r[eq0 + (size_t)i]) > m ? 1 : 0;
+  return report_device_errors(pf, (uint32_t)r[words], s);
+}
+
 // ara_adjoint over the trial-major YET (yx null) or over its event-major index (yx set: the
 // trials [first_trial, first_trial + n_trials) of the indexed YET; the YET pointers are unused).
 static ara_status adjoint_common(ara_portfolio* pf_, const YetIndex* yx, int64_t first_trial,
@@ -1079,18 +1107,7 @@ static ara_status adjoint_common(ara_portfolio* pf_, const YetIndex* yx, int64_t
     st = adjoint_multi(*pf, sel, n_trials, d_offsets, n_events, d_ids, yx, first_trial, d_ylt, d_regimes, m, sr,
                        d_grad_elt, d_grad_layer, d_grad_loss, total_slots, total_loss, s);
     if (st != ARA_ERANGE || yx) {
-      std::vector<unsigned long long> gt(n_sel), eq(n_sel);
-      if (st == ARA_OK && h_ties) {
-        if (cudaMemcpyAsync(gt.data(), sr.gt, 8 * n_sel, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(eq.data(), sr.eq, 8 * n_sel, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-          st = ARA_ECUDA;
-      }
-      free_select_result(sr, s);
-      if (cudaStreamSynchronize(s) != cudaSuccess && st == ARA_OK) st = ARA_ECUDA;
-      if (st == ARA_OK && h_ties)
-        for (int32_t i = 0; i < n_sel; ++i) h_ties[i] = (int64_t)(gt[i] + eq[i]) > m ? 1 : 0;
-      if (st != ARA_OK) return st;
-      return ara_check(pf_, stream);
+      return adjoint_end(*pf, st, sr, n_sel, m, h_ties, s);
     }
     st = ARA_OK;
   }
@@ -1211,19 +1228,8 @@ static ara_status adjoint_common(ara_portfolio* pf_, const YetIndex* yx, int64_t
       elt_slot0 += n_le;
     }
   }
-  std::vector<unsigned long long> gt(n_sel), eq(n_sel);
-  if (out_st == ARA_OK && h_ties) {
-    if (cudaMemcpyAsync(gt.data(), sr.gt, 8 * n_sel, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(eq.data(), sr.eq, 8 * n_sel, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-      out_st = ARA_ECUDA;
-  }
   cudaFreeAsync(scratch, s);
-  free_select_result(sr, s);
-  if (cudaStreamSynchronize(s) != cudaSuccess && out_st == ARA_OK) out_st = ARA_ECUDA;
-  if (out_st == ARA_OK && h_ties)
-    for (int32_t i = 0; i < n_sel; ++i) h_ties[i] = (int64_t)(gt[i] + eq[i]) > m ? 1 : 0;
-  if (out_st != ARA_OK) return out_st;
-  return ara_check(pf_, stream);
+  return adjoint_end(*pf, out_st, sr, n_sel, m, h_ties, s);
 }
 
 extern "C" ara_status ara_adjoint(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets,

@@ -123,6 +123,38 @@ cudaError_t dmalloc_async(void** ptr, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(ptr, bytes, mp, s);
 }
 
+namespace {
+constexpr int kMaxPinnedSlots = 64;
+std::mutex g_pin_mu;
+std::vector<void*> g_pin_idle;
+int g_pin_total = 0;
+}  // namespace
+
+PinnedSlot::PinnedSlot() : p(nullptr) {
+  {
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    if (!g_pin_idle.empty()) {
+      p = g_pin_idle.back();
+      g_pin_idle.pop_back();
+      return;
+    }
+    if (g_pin_total >= kMaxPinnedSlots) return;
+    ++g_pin_total;
+  }
+  if (cudaHostAlloc(&p, kBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    --g_pin_total;
+  }
+}
+
+PinnedSlot::~PinnedSlot() {
+  if (!p) return;
+  std::lock_guard<std::mutex> lk(g_pin_mu);
+  g_pin_idle.push_back(p);
+}
+
 int64_t pool_idle_bytes(int dev) {
   if (dev < 0 || dev >= kMaxPoolDevices) return 0;
   cudaMemPool_t mp;
@@ -309,6 +341,12 @@ ara_status ara_set_stream_shape(int32_t index) {
 }
 
 ara_status ara_release_memory(void) {
+  {
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    for (void* q : g_pin_idle) cudaFreeHost(q);
+    g_pin_total -= (int)g_pin_idle.size();
+    g_pin_idle.clear();
+  }
   std::lock_guard<std::mutex> lk(g_pool_mu);
   ara_status st = ARA_OK;
   for (int d = 0; d < kMaxPoolDevices; ++d)
@@ -769,19 +807,29 @@ ara_status ara_run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_off
   return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, n_sel, layer_sel, d_ylt, d_regimes, flags, true, stream);
 }
 
+}  // extern "C"
+
+namespace ara {
+ara_status report_device_errors(Portfolio& pf, uint32_t err, cudaStream_t s) {
+  if (!err) return ARA_OK;
+  ARA_TRY(cudaMemsetAsync(pf.d_err, 0, sizeof(uint32_t), s));
+  ARA_TRY(cudaStreamSynchronize(s));
+  return (err & DERR_TIMEOUT) ? ARA_ETIMEOUT : ARA_EDATA;
+}
+}  // namespace ara
+
+extern "C" {
+
 ara_status ara_check(ara_portfolio* pf, void* stream) {
   if (!pf) return ARA_EINVAL;
   DeviceGuard g(pf->device);
   cudaStream_t s = (cudaStream_t)stream;
-  uint32_t err = 0;
-  ARA_TRY(cudaMemcpyAsync(&err, pf->d_err, sizeof(err), cudaMemcpyDeviceToHost, s));
+  uint32_t local = 0;
+  PinnedSlot slot;
+  uint32_t* const err = slot.p ? (uint32_t*)slot.p : &local;
+  ARA_TRY(cudaMemcpyAsync(err, pf->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   ARA_TRY(cudaStreamSynchronize(s));
-  if (err) {
-    ARA_TRY(cudaMemsetAsync(pf->d_err, 0, sizeof(uint32_t), s));
-    ARA_TRY(cudaStreamSynchronize(s));
-    return (err & DERR_TIMEOUT) ? ARA_ETIMEOUT : ARA_EDATA;
-  }
-  return ARA_OK;
+  return report_device_errors(*pf, *err, s);
 }
 
 static ara_status ensure_stage(Portfolio& pf, int64_t events, int64_t trials, int64_t ylt_elems) {

@@ -30,6 +30,18 @@ void note_cuda_error(cudaError_t e, const char* what, const char* file, int line
 // pool's behaviour, which made every synchronous call map its scratch again).  Free with
 // cudaFreeAsync.  ara_release_memory() returns the idle part to the system.
 cudaError_t dmalloc_async(void** ptr, size_t bytes, cudaStream_t s);
+// A small block of pinned host memory, mapped into the device's address space, for the results of a
+// synchronous call: kernels write into it or one copy fills it without staging, where a copy to
+// pageable memory costs the call about 10 us each.  From a bounded list shared by all threads (p is
+// null when it is exhausted: use pageable memory); ara_release_memory() frees the idle ones.
+struct PinnedSlot {
+  static constexpr size_t kBytes = 16384;
+  void* p;
+  PinnedSlot();
+  ~PinnedSlot();
+  PinnedSlot(const PinnedSlot&) = delete;
+  PinnedSlot& operator=(const PinnedSlot&) = delete;
+};
 // Bytes the library's pool on `dev` holds without using them (reusable by the library).
 int64_t pool_idle_bytes(int dev);
 
@@ -223,6 +235,8 @@ ara_status run_batched_group_async(Portfolio& pf, const GroupArgs& g, cudaStream
 // event-major table): ptr [n + 1], block_sums [ceil(n / 1024)], total [1].
 ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t n_sel, int64_t n,
                              uint32_t* ptr, uint32_t* block_sums, uint32_t* total, cudaStream_t s);
+// Status of a device error word read by the host; a set word is cleared.
+ara_status report_device_errors(Portfolio& pf, uint32_t err, cudaStream_t s);
 // Event-major rows and their stream (ara_rows.cu).
 constexpr int RW_MAX_LAYERS = 255;
 constexpr int RW_BUILD_THREADS = 128;

@@ -292,7 +292,7 @@ __device__ __forceinline__ void put_mean(const SelScratch& sc, int layer, double
 }
 
 __device__ __forceinline__ void sel_timeout(const SelScratch& sc) {
-  atomicOr(sc.err, 1u);
+  *(volatile uint32_t*)sc.err = 1u;   // device or mapped host memory
   if (sc.ext_err) atomicOr(sc.ext_err, DERR_TIMEOUT);
 }
 
@@ -1052,8 +1052,9 @@ size_t select_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_t, int n_sms)
 ara_status launch_select(const double* d_ylt, const SelPlan& y, const SelTargets& tg, void* scratch,
                          int want_mean, cudaStream_t s, SelScratch* out, uint32_t* ext_err = nullptr,
                          double* user_pml = nullptr, double* user_tvar = nullptr,
-                         double* user_mean = nullptr) {
+                         double* user_mean = nullptr, uint32_t* host_err = nullptr) {
   SelScratch sc = carve(scratch, y);
+  if (host_err) sc.err = host_err;
   sc.ext_err = ext_err;
   sc.user_pml = user_pml;
   sc.user_tvar = user_tvar;
@@ -1061,7 +1062,8 @@ ara_status launch_select(const double* d_ylt, const SelPlan& y, const SelTargets
   const int64_t n = y.n;
   const ara_status ready = sel_prepare_kernels();
   if (ready != ARA_OK) return ready;
-  ARA_TRY(cudaMemsetAsync(scratch, 0, y.zero_bytes, s));
+  // (without counts in global memory only the error word needs clearing, and the host's is clear)
+  if (!host_err || !(y.small || y.cluster)) ARA_TRY(cudaMemsetAsync(scratch, 0, y.zero_bytes, s));
   if (y.small) {
     int pad = 64;
     while (pad < n) pad <<= 1;
@@ -1159,14 +1161,30 @@ ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_
   void* scratch = nullptr;
   ARA_TRY(dmalloc_async(&scratch, y.bytes, s));
   SelScratch sc;
+  const size_t L = (size_t)n_layers, n_pml = L * n_rp, n_tv = L * n_tvar;
+  PinnedSlot slot;
+  if (slot.p && (n_pml + n_tv + L + 1) * sizeof(double) <= PinnedSlot::kBytes) {
+    // the kernel writes the results straight into the pinned block: no copies, one wait
+    double* const r = (double*)slot.p;
+    volatile uint32_t* const err = (volatile uint32_t*)(r + n_pml + n_tv + L);
+    *err = 0u;
+    st = launch_select(d_ylt, y, tg, scratch, h_mean != nullptr, s, &sc, nullptr, n_rp > 0 ? r : nullptr,
+                       n_tvar > 0 ? r + n_pml : nullptr, h_mean ? r + n_pml + n_tv : nullptr, (uint32_t*)err);
+    cudaFreeAsync(scratch, s);
+    if (cudaStreamSynchronize(s) != cudaSuccess && st == ARA_OK) st = ARA_ECUDA;
+    if (st != ARA_OK) return st;
+    if (*err) return ARA_ETIMEOUT;
+    std::copy(r, r + n_pml, h_pml);
+    std::copy(r + n_pml, r + n_pml + n_tv, h_tvar);
+    if (h_mean) std::copy(r + n_pml + n_tv, r + n_pml + n_tv + L, h_mean);
+    return ARA_OK;
+  }
   st = launch_select(d_ylt, y, tg, scratch, h_mean != nullptr, s, &sc);
-  std::vector<double> out((size_t)n_layers * tg.n_t);
+  std::vector<double> out(L * tg.n_t + L);
   uint32_t timed_out = 0;
   if (st == ARA_OK) {
-    cudaError_t e = cudaMemcpyAsync(out.data(), sc.out, sizeof(double) * out.size(),
+    cudaError_t e = cudaMemcpyAsync(out.data(), sc.out, sizeof(double) * out.size(),   // and the means
                                     cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && h_mean)
-      e = cudaMemcpyAsync(h_mean, sc.mean, sizeof(double) * n_layers, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(&timed_out, sc.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) st = ARA_ECUDA;
@@ -1178,6 +1196,7 @@ ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_
   for (int32_t l = 0; l < n_layers; ++l) {
     for (int i = 0; i < n_rp; ++i) h_pml[(size_t)l * n_rp + i] = out[(size_t)l * tg.n_t + i];
     for (int i = 0; i < n_tvar; ++i) h_tvar[(size_t)l * n_tvar + i] = out[(size_t)l * tg.n_t + n_rp + i];
+    if (h_mean) h_mean[l] = out[L * tg.n_t + l];
   }
   return ARA_OK;
 }
