@@ -375,35 +375,51 @@ __global__ void __launch_bounds__(256) k_adj_scatter(AdjScatterParams p) {
 constexpr int ADJB_WARPS = 32;
 constexpr int ADJB_MAX_SEL = 255;   // slots fit in one byte
 
+// Slots within a row descriptor.
+struct AdjbSlots {
+  uint32_t width, n, mask;          // bits per slot, slots held, the width's mask
+};
+
+static AdjbSlots adjb_slots(int32_t n_sel) {
+  const uint32_t w = n_sel <= 16 ? 4u : n_sel <= 64 ? 6u : 8u;
+  return AdjbSlots{w, 24u / w, (1u << w) - 1u};
+}
+
+__device__ __forceinline__ uint32_t adjb_slot(const AdjbSlots& q, uint64_t rw, uint32_t k) {
+  return (uint32_t)(rw >> (40u + q.width * k)) & q.mask;
+}
+
 // Row descriptor and the slot of every entry.  The descriptor holds the first entry (bits 0-31),
-// the length (bits 32-39) and the slots of the first three entries (bits 40-47, 48-55, 56-63),
-// so that most rows (1.4 entries on average on the adjoint workload) need no entry loads in the
-// histogram pass.  Entries at or beyond cap are not written (cap bounds the allocation; a larger
-// table is reported as a data error).
+// the length (bits 32-39) and, from bit 40, the slots of as many first entries as 24 bits hold at the
+// selection's slot width (6 of 4 bits up to 16 slots, 4 of 6 bits up to 64, else 3 of 8 bits), so
+// that most rows need no entry loads in the histogram pass.  Entries at or beyond cap are not written (cap bounds the allocation; a larger
+// table is reported as a data error).  pair: ptr counts pairs of entries, and every row begins at
+// an even entry (the histogram pass adds to two entries at a time).
 __global__ void __launch_bounds__(256)
 k_adjb_fill(int32_t n_sel, const uint32_t* __restrict__ bits, int64_t bits_stride, int64_t C,
-            const uint32_t* __restrict__ ptr, uint32_t cap, uint8_t* __restrict__ ent,
+            const uint32_t* __restrict__ ptr, int pair, AdjbSlots q, uint32_t cap,
+            uint8_t* __restrict__ ent,
             uint64_t* __restrict__ rows, uint32_t* __restrict__ err) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= C) return;
-  uint32_t pos = ptr[e];
-  uint32_t end = ptr[e + 1];
+  uint32_t pos = ptr[e] << pair;
+  uint32_t end = ptr[e + 1] << pair;
   if (end > cap) {
     atomicOr(err, DERR_EVENT_RANGE);
     end = cap;
     pos = min(pos, cap);
   }
-  uint64_t desc = (uint64_t)pos | ((uint64_t)(end - pos) << 32);
+  uint64_t desc = pos;
   const uint32_t* b = bits + (e >> 5);
   const int sh = (int)(e & 31);
-  int k = 0;
+  uint32_t k = 0;
   for (int i = 0; i < n_sel && pos < end; ++i)
     if ((__ldg(b + (int64_t)i * bits_stride) >> sh) & 1u) {
       ent[pos++] = (uint8_t)i;
-      if (k < 3) desc |= (uint64_t)i << (40 + 8 * k);
+      if (k < q.n) desc |= (uint64_t)i << (40u + q.width * k);
       ++k;
     }
-  rows[e] = desc;
+  rows[e] = desc | ((uint64_t)k << 32);
 }
 
 // Class of every (trial, slot), trial-major [n_trials][n_sel]: 0 outside the slot's aggregate
@@ -443,6 +459,7 @@ struct AdjbHistParams {
   const int32_t* ids;
   int64_t catalogue;
   int32_t n_sel;
+  AdjbSlots q;
   uint32_t cap;               // entries allocated
   const uint8_t* cls;         // [n_trials][n_sel]
   const uint64_t* rows;       // [catalogue]
@@ -456,6 +473,13 @@ struct AdjbHistParams {
 // One warp per trial, dealt round-robin over the grid.  The trial's class row goes to the warp's
 // shared memory; a trial interior for no slot is skipped without reading its events.  Eight IDs
 // per lane are loaded at once, then their row descriptors, then the row entries are walked.
+//
+// L2 bounds it: one random 8-byte gather per occurrence (294 G/s) and one add per counted entry
+// (206 G/s, the same for 4, 8 and 16 bytes).  With PAIR two neighbouring counts take one 64-bit add
+// (the low count cannot carry: an event has fewer than 2^32 occurrences), and the descriptor's
+// narrower slots spare most loads of ent: 16 layers over 2e8 occurrences (1.4 entries per event)
+// 1.69 -> 1.43 ms.  One 32-bit add per entry is for YETs of 2^32 occurrences and more.
+template <bool PAIR>
 __global__ void __launch_bounds__(ADJB_WARPS * 32) k_adjb_hist(AdjbHistParams p) {
   __shared__ uint8_t cls_s[ADJB_WARPS][ADJB_MAX_SEL + 1];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
@@ -496,15 +520,30 @@ __global__ void __launch_bounds__(ADJB_WARPS * 32) k_adjb_hist(AdjbHistParams p)
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const uint32_t first = (uint32_t)rw[u], len = (uint32_t)(rw[u] >> 32) & 0xffu;
-        for (uint32_t k = 0; k < len; ++k) {
-          const uint32_t x = first + k;
-          if (x >= p.cap) break;
-          const uint32_t sl = k < 3 ? (uint32_t)(rw[u] >> (40 + 8 * k)) & 0xffu : p.ent[x];
-          const uint8_t c = cs[sl];
-          if (c) {
-            atomicAdd(p.h_mean + x, 1u);
-            if (c == 2) atomicAdd(p.h_gt + x, 1u);
-            else if (c == 3) atomicAdd(p.h_eq + x, 1u);
+        if constexpr (PAIR) {
+          for (uint32_t k = 0; k < len; k += 2) {
+            const uint32_t x = first + k;
+            if (x + 1 >= p.cap) break;
+            const uint8_t c0 = cs[k < p.q.n ? adjb_slot(p.q, rw[u], k) : (uint32_t)p.ent[x]];
+            uint8_t c1 = 0;
+            if (k + 1 < len) c1 = cs[k + 1 < p.q.n ? adjb_slot(p.q, rw[u], k + 1) : (uint32_t)p.ent[x + 1]];
+            const unsigned long long add = (c0 ? 1ull : 0ull) | (c1 ? 1ull << 32 : 0ull);
+            if (add) atomicAdd(reinterpret_cast<unsigned long long*>(p.h_mean + x), add);
+            if ((c0 | c1) & 2) {
+              if (c0 & 2) atomicAdd((c0 == 2 ? p.h_gt : p.h_eq) + x, 1u);
+              if (c1 & 2) atomicAdd((c1 == 2 ? p.h_gt : p.h_eq) + x + 1, 1u);
+            }
+          }
+        } else {
+          for (uint32_t k = 0; k < len; ++k) {
+            const uint32_t x = first + k;
+            if (x >= p.cap) break;
+            const uint8_t c = cs[k < p.q.n ? adjb_slot(p.q, rw[u], k) : (uint32_t)p.ent[x]];
+            if (c) {
+              atomicAdd(p.h_mean + x, 1u);
+              if (c == 2) atomicAdd(p.h_gt + x, 1u);
+              else if (c == 3) atomicAdd(p.h_eq + x, 1u);
+            }
           }
         }
       }
@@ -565,6 +604,7 @@ struct AdjxHistParams {
   const uint32_t* words;      // [n_trials] class words of slots [q0, q0 + nq)
   const uint8_t* cls;         // [n_trials][n_sel] classes, for the flagged trials
   int32_t n_sel, q0, nq;
+  AdjbSlots q;
   const uint64_t* rows;       // [catalogue] row descriptors (k_adjb_fill)
   const uint8_t* ent;         // [cap] slot of every row entry
   uint32_t cap;
@@ -573,9 +613,9 @@ struct AdjxHistParams {
   uint32_t* h_eq;
 };
 
-__device__ __forceinline__ uint32_t adjx_slot(uint64_t rw, uint32_t first, uint32_t j, uint32_t cap,
-                                              const uint8_t* __restrict__ ent) {
-  if (j < 3) return (uint32_t)(rw >> (40 + 8 * j)) & 0xffu;
+__device__ __forceinline__ uint32_t adjx_slot(const AdjbSlots& q, uint64_t rw, uint32_t first, uint32_t j,
+                                              uint32_t cap, const uint8_t* __restrict__ ent) {
+  if (j < q.n) return adjb_slot(q, rw, j);
   const uint32_t x = first + j;
   return x < cap ? (uint32_t)ent[x] : 0xffu;
 }
@@ -597,7 +637,7 @@ __global__ void __launch_bounds__(1024, 1) k_adjx_hist(AdjxHistParams p) {
     const uint32_t first = (uint32_t)rw, rl = (uint32_t)(rw >> 32) & 0xffu;
     uint32_t j0 = 0, j1 = 0;                                // entries with slot < qlo, < qhi
     for (uint32_t j = 0; j < rl; ++j) {
-      const uint32_t sl = adjx_slot(rw, first, j, p.cap, p.ent);
+      const uint32_t sl = adjx_slot(p.q, rw, first, j, p.cap, p.ent);
       if (first + j >= p.cap) break;
       j0 += sl < qlo ? 1u : 0u;
       j1 += sl < qhi ? 1u : 0u;
@@ -613,7 +653,7 @@ __global__ void __launch_bounds__(1024, 1) k_adjx_hist(AdjxHistParams p) {
       uint32_t sh[ADJX_K], m3[ADJX_K], ca[ADJX_K], cb[ADJX_K];
 #pragma unroll
       for (int k = 0; k < ADJX_K; ++k) {
-        sh[k] = k < have ? 2u * (adjx_slot(rw, first, (uint32_t)(jb + k), p.cap, p.ent) - qlo) : 0u;
+        sh[k] = k < have ? 2u * (adjx_slot(p.q, rw, first, (uint32_t)(jb + k), p.cap, p.ent) - qlo) : 0u;
         m3[k] = k < have ? 3u : 0u;                         // nothing for unused entries
         ca[k] = cb[k] = 0u;
       }
@@ -839,7 +879,10 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
       bound += pf.rec_off[j + 1] - pf.rec_off[j];
     }
   if (bound >= (int64_t)UINT32_MAX || n_sel > ADJB_MAX_SEL) return ARA_ERANGE;
+  // rows of whole pairs of entries, where a count cannot carry into its neighbour's
+  const int pair = !yx && n_events < ((int64_t)1 << 32) && bound + std::min(bound, C) + 2 < (int64_t)UINT32_MAX;
   bound = std::max<int64_t>(bound, 1);
+  if (pair) bound = (bound + std::min(bound, C) + 1) / 2 * 2;
   const int64_t n_blocks = (C + 1023) / 1024;
   size_t off = 0;
   auto take = [&](size_t n) { size_t o = (off + 255) / 256 * 256; off = o + n; return o; };
@@ -850,6 +893,7 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
   const size_t o_hm = take(4 * (size_t)bound), o_hg = take(4 * (size_t)bound), o_he = take(4 * (size_t)bound);
   const size_t o_acc = take(sizeof(AdjCounts) * (size_t)n_sel);
   const size_t o_slots = take(sizeof(SlotCounts) * (size_t)std::max<int64_t>(total_slots, 1));
+  const size_t o_ents = take(4);
   const size_t o_words = yx ? take(sizeof(uint32_t) * (size_t)n_trials) : 0;
   char* scratch = nullptr;
   ARA_TRY(dmalloc_async((void**)&scratch, off, s));
@@ -889,9 +933,9 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
     LaunchScope ls(ARA_K_ADJOINT, s, 6 + n_hist_launches + n_rec_launches);
     // 2. event-major rows of the slots with a non-zero occurrence regime
     st = launch_event_scan(bits, bmw, n_sel, C, ptr, (uint32_t*)(scratch + o_bsum),
-                           (uint32_t*)(scratch + o_tot), s);
+                           (uint32_t*)(scratch + o_tot), pair ? (uint32_t*)(scratch + o_ents) : nullptr, s);
     if (st == ARA_OK) {
-      k_adjb_fill<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(n_sel, bits, bmw, C, ptr, cap, ent,
+      k_adjb_fill<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(n_sel, bits, bmw, C, ptr, pair, adjb_slots(n_sel), cap, ent,
                                                              rows, pf.d_err);
       // 3. the class of every (trial, slot) and the trial counts
       const unsigned cb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_trials + 255) / 256, 64));
@@ -908,6 +952,7 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
         xp.words = words;
         xp.cls = cls;
         xp.n_sel = n_sel;
+        xp.q = adjb_slots(n_sel);
         xp.rows = rows;
         xp.ent = ent;
         xp.cap = cap;
@@ -938,6 +983,7 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
       hp.ids = d_ids ? d_ids : reinterpret_cast<const int32_t*>(d_offsets);
       hp.catalogue = C;
       hp.n_sel = n_sel;
+      hp.q = adjb_slots(n_sel);
       hp.cap = cap;
       hp.cls = cls;
       hp.rows = rows;
@@ -946,7 +992,10 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
       hp.h_gt = hg;
       hp.h_eq = he;
       hp.err = pf.d_err;
-      if (!yx) k_adjb_hist<<<(unsigned)(pf.n_sms * 2), ADJB_WARPS * 32, 0, s>>>(hp);
+      if (!yx) {
+        const auto hist = pair ? k_adjb_hist<true> : k_adjb_hist<false>;
+        hist<<<(unsigned)(pf.n_sms * 2), ADJB_WARPS * 32, 0, s>>>(hp);
+      }
       // 5. per-slot sums of the histograms by occurrence regime
       k_adjb_events<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((C + 255) / 256, 4 * pf.n_sms)),
                       256, (size_t)6 * n_sel * sizeof(unsigned long long), s>>>(C, n_sel, cap, rows, ent,

@@ -234,7 +234,8 @@ ara_status run_batched_group_async(Portfolio& pf, const GroupArgs& g, cudaStream
 // Exclusive scan of the per-event count of set bits over n_sel bitmaps (the rows of an
 // event-major table): ptr [n + 1], block_sums [ceil(n / 1024)], total [1].
 ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t n_sel, int64_t n,
-                             uint32_t* ptr, uint32_t* block_sums, uint32_t* total, cudaStream_t s);
+                             uint32_t* ptr, uint32_t* block_sums, uint32_t* total, uint32_t* entries,
+                             cudaStream_t s);
 // Status of a device error word read by the host; a set word is cleared.
 ara_status report_device_errors(Portfolio& pf, uint32_t err, cudaStream_t s);
 // Event-major rows and their stream (ara_rows.cu).

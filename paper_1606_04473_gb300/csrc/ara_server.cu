@@ -110,7 +110,7 @@ int64_t estimate_bytes(const Portfolio& pool, const Request& r) {
   if (r.want_adjoint) {
     int64_t recs = 0;
     for (int32_t j : r.layer_elts) recs += pool.rec_off[j + 1] - pool.rec_off[j];
-    b += 14 * C + 4 * pool.bm_words + 16 * recs + 64 * (int64_t)r.layer_elts.size() + 64 * nl;
+    b += 14 * C + 4 * pool.bm_words + 16 * recs + 13 * std::min(recs, C) + 64 * (int64_t)r.layer_elts.size() + 64 * nl;
   }
   return b;
 }

@@ -1,0 +1,45 @@
+"""The adjoint of several layers in one pass, whose histogram adds to two entries of an event's row at
+once: equal, bit for bit, to the pass over the event-major index and to one pass per layer.  The counts
+are integers, so no tolerance."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_1606_04473_gb300 as ara
+
+
+# layers at the edges of the slot widths of a row descriptor; rows from mostly empty to one entry per layer
+@pytest.mark.parametrize("n_layers", [2, 3, 16, 17, 64, 65, 255])
+@pytest.mark.parametrize("nnz", [60, 2_000, 4_999])
+def test_pairs_equal_the_other_passes(n_layers, nnz):
+    g = np.random.default_rng(1000 * n_layers + nnz)
+    C, n_elts, trials = 5_000, 12, 700
+    ids = [g.choice(C, size=nnz, replace=False).astype(np.int32) for _ in range(n_elts)]
+    loss = [np.exp(11.0 + 2.0 * g.standard_normal(nnz)) for _ in ids]
+    layers = [sorted(g.choice(n_elts, size=int(g.integers(1, 4)), replace=False).tolist()) for _ in range(n_layers)]
+    z = np.zeros(n_layers)
+    pf = ara.Portfolio(C, ids, loss, np.full(n_elts, 1e4), np.full(n_elts, 1.5e6), layers, z + 1e4, z + 2e6,
+                       g.uniform(0.0, 1e6, n_layers), z + 1e13)
+    counts = g.poisson(300, trials)
+    counts[[0, 5, trials - 1]] = 0
+    off = np.zeros(trials + 1, np.int64)
+    np.cumsum(counts, out=off[1:])
+    off, ev = torch.from_numpy(off).cuda(), torch.from_numpy(g.integers(0, C, off[-1], dtype=np.int32)).cuda()
+    reg = torch.empty((n_layers, trials), dtype=torch.uint8, device="cuda")
+    ylt = pf.run_ylt(off, ev, regimes=reg)
+    pf.check()
+    a = pf.adjoint(off, ev, ylt, reg, 0.98)
+    assert float(a["loss"].abs().sum()) > 0
+    others = [pf.adjoint(None, None, ylt, reg, 0.98, index=pf.yet_index(off, ev))]
+    if n_layers <= 17:
+        ara.debug_set(ara.ARA_DBG_ADJOINT_PER_LAYER, 1)
+        try:
+            others.append(pf.adjoint(off, ev, ylt, reg, 0.98))
+        finally:
+            ara.debug_set(ara.ARA_DBG_ADJOINT_PER_LAYER, 0)
+    for b in others:
+        assert all(torch.equal(a[k], b[k]) for k in ("elt", "layer", "loss")) and np.array_equal(a["ties"], b["ties"])
+    pf.close()
