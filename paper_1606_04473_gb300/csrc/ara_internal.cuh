@@ -297,6 +297,12 @@ int rows_k(const Portfolio& pf, const std::vector<int32_t>& sel);
 RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K, int64_t n_trials);
 RowSchedule rows_schedule(const Portfolio& pf, int ns, int K, int64_t table_bytes, double entries,
                           int64_t n_trials, int64_t n_events);
+// Slots within an adjoint row descriptor (ara_adjoint.cu).
+struct AdjbSlots {
+  uint32_t width, n, mask;          // bits per slot, slots held, the width's mask
+};
+ara_status launch_adjoint_rows(const Portfolio& pf, const std::vector<int32_t>& sel, const AdjbSlots& q, uint32_t cap,
+                               uint8_t* ent, uint64_t* desc, uint8_t* regime, uint32_t* counters, cudaStream_t s);
 ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, const RowTable& rt, const int32_t* first,
                              cudaStream_t s);
 ara_status launch_rows_stream(Portfolio& pf, const RowsStream& p, int K, RowSchedule& sched, cudaStream_t s);

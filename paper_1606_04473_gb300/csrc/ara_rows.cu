@@ -196,6 +196,11 @@ struct RowsBuild {
   uint32_t ovf_pairs;          // capacity of ovf in 16-byte pairs (0: only count)
   uint32_t* counters;          // [0] overflow pairs taken, [1] entries in all rows
   uint64_t* desc;              // [catalogue]: first entry | number of entries << 32 (optional, K > 0)
+  // ADJ only: entries are slots (one byte) of the layers whose occurrence regime is not 0, K = 0, and a
+  // descriptor holds the first slots too (ara_adjoint.cu)
+  uint8_t* ent;
+  uint8_t* regime;             // [ns][catalogue], zeroed
+  AdjbSlots q;
   int32_t first_shift;
   int32_t first[5];            // first slot of each request (as RowsStream)
   uint64_t sel[RW_MASK];       // the selected layers
@@ -236,7 +241,7 @@ __device__ __forceinline__ uint32_t rb_scan(uint32_t v, uint32_t* part, uint32_t
 // is a chain of dependent loads.  A first term is stored, not added (0 + x = x): FP64 instructions
 // issue at 2 lanes per clock and SM here, whatever the number of active lanes.  Events whose sums
 // do not fit take another turn.
-template <typename LossT, int MW>
+template <typename LossT, int MW, bool ADJ>
 __global__ void __launch_bounds__(RW_BUILD_THREADS)
 k_rows_build(RowsBuild p) {
   __shared__ double acc[RW_BUILD_SUMS];
@@ -305,7 +310,14 @@ k_rows_build(RowsBuild p) {
           const uint64_t bit = m & (0ull - m);
           const RowsLayer& l = lay[64 * w + __ffsll((long long)m) - 1];
           double* const s = x + before[w] + __popcll(reach[w] & (bit - 1));
-          const uint64_t q = fixed_rn(clamp_terms_bits(*s, l.occ_ret, l.occ_lim), l.frac_bits);
+          uint64_t q;
+          if (ADJ) {   // the regime: inside the cover or above it
+            const long long ex = __double_as_longlong(__dsub_rn(*s, l.occ_ret));
+            const long long lim = __double_as_longlong(l.occ_lim);
+            q = ex > 0 ? (ex < lim ? 1ull : ex > lim ? 2ull : 0ull) : 0ull;
+          } else {
+            q = fixed_rn(clamp_terms_bits(*s, l.occ_ret, l.occ_lim), l.frac_bits);
+          }
           if (q) {
             *s = __longlong_as_double((long long)q);
             ++n;
@@ -326,7 +338,23 @@ k_rows_build(RowsBuild p) {
     }
     __syncthreads();
     at += base_s;                                 // first pair of this row's part of ovf
-    if (mine && !(need && at + need > p.ovf_pairs)) {   // else a counting run
+    if (ADJ && mine && at + need <= p.ovf_pairs) {
+      uint64_t desc = 2ull * at | ((uint64_t)n << 32);
+      uint32_t k = 0;
+#pragma unroll
+      for (int w = 0; w < MW; ++w)
+        for (uint64_t m = begun[w]; m; m &= m - 1) {
+          const uint64_t bit = m & (0ull - m);
+          const int s = lay[64 * w + __ffsll((long long)m) - 1].slot;
+          const double r = x[before[w] + __popcll(reach[w] & (bit - 1))];
+          p.regime[(int64_t)s * p.catalogue + e] = (uint8_t)__double_as_longlong(r);
+          p.ent[2 * (int64_t)at + k] = (uint8_t)s;
+          if (k < p.q.n) desc |= (uint64_t)s << (40u + p.q.width * k);
+          ++k;
+        }
+      p.desc[e] = desc;
+    }
+    if (!ADJ && mine && !(need && at + need > p.ovf_pairs)) {   // else a counting run
       const uint64_t spare = (uint64_t)p.ns << 56;
       uint64_t* const ov = p.ovf + 2 * (int64_t)at;
       uint64_t* const row = p.table + (int64_t)p.K * e;
@@ -904,10 +932,8 @@ RowSchedule rows_schedule(const Portfolio& pf, int ns, int K, int64_t table_byte
   return r;
 }
 
-ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, const RowTable& rt, const int32_t* first,
-                             cudaStream_t s) {
+static RowsBuild rows_build_params(const Portfolio& pf, const std::vector<int32_t>& sel) {
   RowsBuild p{};
-  for (int i = 0; i < 5; ++i) p.first[i] = first[i];
   p.catalogue = pf.catalogue;
   p.ptr = pf.d_ev_ptr;
   p.elt = pf.d_ev_elt;
@@ -918,6 +944,30 @@ ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, con
   p.n_layers = pf.n_layers;
   p.layers = pf.d_layers;
   p.ns = (int32_t)sel.size();
+  for (int i = 0; i < p.ns; ++i) {
+    const int32_t l = sel[(size_t)i];
+    p.slot_of[l] = (uint8_t)i;
+    p.sel[l >> 6] |= 1ull << (l & 63);
+  }
+  return p;
+}
+
+template <bool ADJ>
+static ara_status launch_build(const Portfolio& pf, const RowsBuild& p, cudaStream_t s) {
+  ARA_TRY(cudaMemsetAsync(p.counters, 0, 2 * sizeof(uint32_t), s));
+  const int smem = pf.n_layers * (int)sizeof(RowsLayer);
+  const bool f32 = pf.d_rec_loss32 != nullptr;
+  const auto fn = pf.n_layers <= 64 ? (f32 ? k_rows_build<float, 1, ADJ> : k_rows_build<double, 1, ADJ>)
+                             : (f32 ? k_rows_build<float, 4, ADJ> : k_rows_build<double, 4, ADJ>);
+  fn<<<(unsigned)((pf.catalogue + RW_BUILD_THREADS - 1) / RW_BUILD_THREADS), RW_BUILD_THREADS, smem, s>>>(p);
+  ARA_TRY(cudaGetLastError());
+  return ARA_OK;
+}
+
+ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, const RowTable& rt, const int32_t* first,
+                             cudaStream_t s) {
+  RowsBuild p = rows_build_params(pf, sel);
+  for (int i = 0; i < 5; ++i) p.first[i] = first[i];
   p.K = rt.K;
   p.table = rt.table;
   p.ovf = rt.ovf;
@@ -925,19 +975,20 @@ ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, con
   p.counters = rt.counters;
   p.desc = rt.desc;
   p.first_shift = rt.first_shift;
-  for (int i = 0; i < p.ns; ++i) {
-    const int32_t l = sel[(size_t)i];
-    p.slot_of[l] = (uint8_t)i;
-    p.sel[l >> 6] |= 1ull << (l & 63);
-  }
-  ARA_TRY(cudaMemsetAsync(rt.counters, 0, 2 * sizeof(uint32_t), s));
-  const int smem = pf.n_layers * (int)sizeof(RowsLayer);
-  const bool f32 = pf.d_rec_loss32 != nullptr;
-  const auto fn = pf.n_layers <= 64 ? (f32 ? k_rows_build<float, 1> : k_rows_build<double, 1>)
-                             : (f32 ? k_rows_build<float, 4> : k_rows_build<double, 4>);
-  fn<<<(unsigned)((pf.catalogue + RW_BUILD_THREADS - 1) / RW_BUILD_THREADS), RW_BUILD_THREADS, smem, s>>>(p);
-  ARA_TRY(cudaGetLastError());
-  return ARA_OK;
+  return launch_build<false>(pf, p, s);
+}
+
+// Rows of the adjoint: cap entries at ent (in pairs), regimes zeroed by the caller, two counter words.
+ara_status launch_adjoint_rows(const Portfolio& pf, const std::vector<int32_t>& sel, const AdjbSlots& q, uint32_t cap,
+                               uint8_t* ent, uint64_t* desc, uint8_t* regime, uint32_t* counters, cudaStream_t s) {
+  RowsBuild p = rows_build_params(pf, sel);
+  p.ent = ent;
+  p.desc = desc;
+  p.regime = regime;
+  p.q = q;
+  p.ovf_pairs = cap / 2;
+  p.counters = counters;
+  return launch_build<true>(pf, p, s);
 }
 
 // Blocks per SM of a stream kernel with this much shared memory; ARA_ERANGE when it does not fit.

@@ -1,6 +1,7 @@
 """The adjoint of several layers in one pass, whose histogram adds to two entries of an event's row at
-once: equal, bit for bit, to the pass over the event-major index and to one pass per layer.  The counts
-are integers, so no tolerance."""
+once and whose rows come from the event-major records (ELTs listed in ascending order) or from the
+layers' folds (any other order): equal, bit for bit, to the pass over the event-major index and to one
+pass per layer.  The counts are integers, so no tolerance."""
 import numpy as np
 import pytest
 
@@ -14,12 +15,14 @@ if torch.cuda.is_available():
 # layers at the edges of the slot widths of a row descriptor; rows from mostly empty to one entry per layer
 @pytest.mark.parametrize("n_layers", [2, 3, 16, 17, 64, 65, 255])
 @pytest.mark.parametrize("nnz", [60, 2_000, 4_999])
-def test_pairs_equal_the_other_passes(n_layers, nnz):
+@pytest.mark.parametrize("ascending", [True, False])
+def test_pairs_equal_the_other_passes(n_layers, nnz, ascending):
     g = np.random.default_rng(1000 * n_layers + nnz)
     C, n_elts, trials = 5_000, 12, 700
     ids = [g.choice(C, size=nnz, replace=False).astype(np.int32) for _ in range(n_elts)]
     loss = [np.exp(11.0 + 2.0 * g.standard_normal(nnz)) for _ in ids]
-    layers = [sorted(g.choice(n_elts, size=int(g.integers(1, 4)), replace=False).tolist()) for _ in range(n_layers)]
+    layers = [sorted(g.choice(n_elts, size=int(g.integers(2, 5)), replace=False).tolist(), reverse=not ascending)
+              for _ in range(n_layers)]
     z = np.zeros(n_layers)
     pf = ara.Portfolio(C, ids, loss, np.full(n_elts, 1e4), np.full(n_elts, 1.5e6), layers, z + 1e4, z + 2e6,
                        g.uniform(0.0, 1e6, n_layers), z + 1e13)
