@@ -185,70 +185,59 @@ __device__ __forceinline__ double value_of(uint64_t k) {
   return __longlong_as_double((long long)b);
 }
 
-// Bitonic sort of N (a power of two, at least 64) shared-memory keys, descending, by the whole
-// block.  A warp's 32 pairs of a step with stride at most 32 lie in its own 64 keys, so those steps
-// need no block barrier.
-__device__ __forceinline__ void sort_descending(uint64_t* a, int N) {
-  for (int k = 2; k <= N; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < N / 2; t += SEL_THREADS) {
-        const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-        const uint64_t x = a[i], y = a[i + j];
-        if ((x < y) == ((i & k) == 0)) {
-          a[i] = y;
-          a[i + j] = x;
-        }
-      }
-      if (j > 32 || (j == 1 && k >= 64)) __syncthreads();
-      else __syncwarp();
-    }
-  }
-  __syncthreads();
-}
-
-// The same for the m sampled keys (a power of two, 64 to SEL_SAMPLE), two per thread in registers: thread l of warp w holds keys
-// 64 w + l and 64 w + 32 + l, so steps of stride below 64 are shuffles (or within the thread) and only
-// the ten wider ones go through shared memory.  (All steps through shared memory: 8 us a row; this:
-// 2 us.)
-__device__ __forceinline__ void sort_sample(uint64_t* a, int m) {
-  static_assert(SEL_SAMPLE == 2 * SEL_THREADS, "two keys per thread");
-  const int lane = threadIdx.x & 31, i0 = 64 * (int)(threadIdx.x >> 5) + lane, i1 = i0 + 32;
-  const bool has = i0 < m;   // m is a multiple of 64: whole warps
-  uint64_t x0 = has ? a[i0] : 0ull, x1 = has ? a[i1] : 0ull;
+// Bitonic sort of m shared-memory keys (a power of two: 512 E, or for E = 2 any from 64), descending,
+// by the whole block, E per thread in registers: thread l of warp w holds the keys 32 E w + 32 u + l,
+// so steps of stride below 32 are shuffles, those below 32 E stay within the thread and only the wider
+// ones go through shared memory.  (1,024 keys with all steps through shared memory: 8 us; this: 2 us.
+// The loops are not unrolled: the code runs once per launch, and fetching it costs more than running it.)
+template <int E>
+__device__ __forceinline__ void sort_keys(uint64_t* a, int m) {
+  const int lane = threadIdx.x & 31, i0 = 32 * E * (int)(threadIdx.x >> 5) + lane;
+  const bool has = i0 < m;   // m is a multiple of 32 E: whole warps
+  uint64_t x[E];
+#pragma unroll
+  for (int u = 0; u < E; ++u) x[u] = has ? a[i0 + 32 * u] : 0ull;
   auto take = [](uint64_t mine, uint64_t other, bool larger) { return (mine > other) == larger ? mine : other; };
+  // key i keeps the larger of the pair (i, i ^ j) when i is its lower place in a descending run
+  auto larger = [](int i, int j, int k) { return ((i & j) == 0) == ((i & k) == 0); };
 #pragma unroll 1
   for (int k = 2; k <= m; k <<= 1) {
 #pragma unroll 1
     for (int j = k >> 1; j > 0; j >>= 1) {
-      if (!has && j < 64) continue;
-      // key i keeps the larger of the pair (i, i ^ j) when i is its lower place in a descending run
-      const bool l0 = ((i0 & j) == 0) == ((i0 & k) == 0), l1 = ((i1 & j) == 0) == ((i1 & k) == 0);
-      uint64_t y0, y1;
-      if (j >= 64) {
+      if (!has && j < 32 * E) continue;
+      if (j >= 32 * E) {
         __syncthreads();
-        if (has) {
-          a[i0] = x0;
-          a[i1] = x1;
-        }
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+          if (has) a[i0 + 32 * u] = x[u];
         __syncthreads();
-        y0 = has ? a[i0 ^ j] : 0ull;
-        y1 = has ? a[i1 ^ j] : 0ull;
-      } else if (j == 32) {
-        y0 = x1;
-        y1 = x0;
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+          if (has) x[u] = take(x[u], a[(i0 + 32 * u) ^ j], larger(i0 + 32 * u, j, k));
+      } else if (j >= 32) {
+#pragma unroll
+        for (int d = 1; d < E; d <<= 1)
+          if (j == 32 * d) {
+#pragma unroll
+            for (int u = 0; u < E; ++u)
+              if (!(u & d)) {
+                const uint64_t p = x[u], q = x[u | d];
+                const bool swap = (p < q) == (((i0 + 32 * u) & k) == 0);
+                x[u] = swap ? q : p;
+                x[u | d] = swap ? p : q;
+              }
+          }
       } else {
-        y0 = __shfl_xor_sync(SFULL, x0, j);
-        y1 = __shfl_xor_sync(SFULL, x1, j);
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+          x[u] = take(x[u], __shfl_xor_sync(SFULL, x[u], j), larger(i0 + 32 * u, j, k));
       }
-      x0 = take(x0, y0, l0);
-      x1 = take(x1, y1, l1);
     }
   }
   __syncthreads();
-  if (has) {
-    a[i0] = x0;
-    a[i1] = x1;
-  }
+#pragma unroll
+  for (int u = 0; u < E; ++u)
+    if (has) a[i0 + 32 * u] = x[u];
   __syncthreads();
 }
 
@@ -296,50 +285,62 @@ __device__ __forceinline__ void sel_timeout(const SelScratch& sc) {
   if (sc.ext_err) atomicOr(sc.ext_err, DERR_TIMEOUT);
 }
 
-// Rows of at most SEL_SMALL values, one block each: the sorted row gives every result directly.
+// Sum of the values of the first n keys, by a fixed tree per 256 keys; valid in lane 0 of the warp.
+__device__ __forceinline__ double warp_sum_keys(const uint64_t* sk, int n) {
+  const int lane = threadIdx.x & 31;
+  double a = 0.0;
+  for (int i0 = lane; i0 < n; i0 += 256) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i0 + 32 * u < n ? value_of(sk[i0 + 32 * u]) : 0.0;
+#pragma unroll
+    for (int d = 4; d; d >>= 1)
+#pragma unroll
+      for (int u = 0; u < d; ++u) v[u] = __dadd_rn(v[u], v[u + d]);
+    a = __dadd_rn(a, v[0]);
+  }
+  return warp_add(a, 16);
+}
+
+// Rows of at most SEL_SMALL values, one block each: the sorted row gives every result directly, a warp
+// to a target (they are chains of dependent shared loads).  Latency bounds it: six rows of
+// 1,600 to 3,300 values in four calls take 92 us, 133 with every step of the sort in shared memory and
+// the targets one after another over the block.
+template <int E>
 __global__ void __launch_bounds__(SEL_THREADS)
 k_sel_small(const double* __restrict__ ylt, int32_t n, int32_t n_pad, SelTargets tg, SelScratch sc, int want_mean) {
   extern __shared__ uint64_t sk[];
   __shared__ double wsum[SEL_WARPS];
-  __shared__ int32_t cut[2];
-  const int layer = blockIdx.x, nt = tg.n_t;
+  const int layer = blockIdx.x, nt = tg.n_t, lane = threadIdx.x & 31;
   const double* src = ylt + (int64_t)layer * n;
   for (int i = threadIdx.x; i < n_pad; i += SEL_THREADS) sk[i] = i < n ? key_of(__ldcg(src + i)) : 0ull;
   __syncthreads();
   // keys are never 0 for the row's values except the NaN of all ones, which sorts with the padding
-  sort_descending(sk, n_pad);
+  sort_keys<E>(sk, n_pad);
   if (want_mean) {
     double a = 0.0;
     for (int i = threadIdx.x; i < n; i += SEL_THREADS) a = __dadd_rn(a, value_of(sk[i]));
     const double s = block_sum(a, wsum);
     if (threadIdx.x == 0) put_mean(sc, layer, s / (double)n);
   }
-  for (int t = 0; t < nt; ++t) {
+  for (int t = threadIdx.x >> 5; t < nt; t += SEL_WARPS) {
     const uint64_t key = sk[tg.rank[t] - 1];
-    if (threadIdx.x < 2) {   // keys above (thread 0) and at or above (thread 1) the selected key
-      int lo = 0, hi = n;
+    int lo = 0, hi = n;
+    if (lane < 2)            // keys above (lane 0) and at or above (lane 1) the selected key
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if (threadIdx.x == 0 ? sk[mid] > key : sk[mid] >= key) lo = mid + 1;
+        if (lane == 0 ? sk[mid] > key : sk[mid] >= key) lo = mid + 1;
         else hi = mid;
       }
-      cut[threadIdx.x] = lo;
-    }
-    __syncthreads();
-    const int gt = cut[0], ge = cut[1];
+    const int gt = __shfl_sync(SFULL, lo, 0), ge = __shfl_sync(SFULL, lo, 1);
     double r = value_of(key);
-    if (t >= tg.n_rp) {
-      double a = 0.0;
-      for (int i = threadIdx.x; i < gt; i += SEL_THREADS) a = __dadd_rn(a, value_of(sk[i]));
-      r = tvar_of(block_sum(a, wsum), tg.rank[t], (unsigned long long)gt, r);
-    }
-    if (threadIdx.x == 0) {
+    if (t >= tg.n_rp) r = tvar_of(warp_sum_keys(sk, gt), tg.rank[t], (unsigned long long)gt, r);
+    if (lane == 0) {
       put_result(sc, tg, layer, t, r);
       sc.gt[(int64_t)layer * nt + t] = (unsigned long long)gt;
       sc.eq[(int64_t)layer * nt + t] = (unsigned long long)(ge - gt);
       sc.state[(int64_t)layer * nt + t].key = key;
     }
-    __syncthreads();
   }
 }
 
@@ -442,7 +443,7 @@ __device__ __forceinline__ int row_splitters(SelShared& S, const double* __restr
                     : key_of(__ldcg(row + a + (int64_t)__umul64hi(z, (uint64_t)(b - a))));
   }
   __syncthreads();
-  sort_sample(S.key, sample);
+  sort_keys<2>(S.key, sample);
   if (list) return sample;
   // Splitters: sample places within 6 standard deviations (and 4 places) of a target's expected
   // place.  Kept places move to the front in order.
@@ -1068,7 +1069,8 @@ ara_status launch_select(const double* d_ylt, const SelPlan& y, const SelTargets
     int pad = 64;
     while (pad < n) pad <<= 1;
     LaunchScope ls(ARA_K_SELECT, s);
-    k_sel_small<<<(unsigned)y.n_layers, SEL_THREADS, (size_t)pad * 8, s>>>(d_ylt, (int32_t)n, pad, tg, sc, want_mean);
+    const auto fn = pad <= 1024 ? k_sel_small<2> : pad <= 2048 ? k_sel_small<4> : k_sel_small<8>;
+    fn<<<(unsigned)y.n_layers, SEL_THREADS, (size_t)pad * 8, s>>>(d_ylt, (int32_t)n, pad, tg, sc, want_mean);
     ARA_TRY(cudaGetLastError());
     *out = sc;
     return ARA_OK;

@@ -72,3 +72,9 @@ def test_allocation_free_call_splits_overfull_lists():
     y[1, : 1_000_000] = 0.0
     rps = [1.0, 1.5, 2.0, 2.0000001, 2.0000002, 3.0, 10.0, 100.0, 250.0, 1000.0, 2000.0]
     check(y, rps, [0.0, 0.3, 0.5, 0.9, 0.99], ara.risk_metrics_static)
+
+
+@pytest.mark.parametrize("n", [64, 1023, 1024, 1025, 2047, 2048, 2049, 4095])
+def test_short_rows_at_the_widths_of_the_sort(n):
+    levels = [p for p in LEVELS if count(n * (1.0 - p)) >= 1]
+    check(rows(n + 1, 5, n), levels=levels)
