@@ -21,7 +21,7 @@
 // barrier each).  Kernel time of one call, 3 targets / 6 targets and the mean, us:
 //   rows x values   1 x 1e3    1 x 3e4    1 x 1.5e5  1 x 1e6    1 x 5e6    8 x 1e5    16 x 2e5   64 x 2e5
 //   radix select    23 / 30    31 / 39    36 / 48    60 / 82    161 / 225  44 / 68    89 / 145   394 / 557
-//   this            19 / 25    31 / 39    33 / 46    47 / 57    122 / 148  38 / 47    62 / 79    119 / 175
+//   this            14 / 17    33 / 40    33 / 40    46 / 57    97 / 121   39 / 46    66 / 85    120 / 166
 // Few rows are bound by the steps' latencies (sorting the sample 3-9 us, a barrier 1.5 us, a pick 3 us,
 // each pass over the row one L2 round trip), many rows by reading them three times.
 
@@ -1039,6 +1039,12 @@ static ara_status sel_prepare_kernels() {
   if (done[dev]) return ARA_OK;
   for (const void* f : {(const void*)k_sel_cluster, (const void*)k_sel_grid})
     ARA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
+  // k_sel_grid has at most one block per SM.  100 KB of shared memory (44 % of 228) keeps two from
+  // sharing one while others stand empty, and a stream kernel queued behind it on another stream from
+  // being given all 228 KB, which leaves its gathers little L1: the paper-scale step, selection on a
+  // second stream, 1.167 -> 1.067 ms (selection 72 -> 61 us, stream 1.09 -> 1.00).
+  ARA_TRY(cudaFuncSetAttribute((const void*)k_sel_grid, cudaFuncAttributePreferredSharedMemoryCarveout, 44));
+  static_assert(SEL_SMEM <= 99 * 1024 && 2 * SEL_SMEM > 99 * 1024, "one block in 100 KB");
   ARA_TRY(cudaFuncSetAttribute((const void*)k_sel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   done[dev] = true;
   return ARA_OK;
