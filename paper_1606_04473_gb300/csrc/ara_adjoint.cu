@@ -876,30 +876,39 @@ static ara_status adjoint_multi(Portfolio& pf, const std::vector<int32_t>& sel, 
   if (bound >= (int64_t)UINT32_MAX || n_sel > ADJB_MAX_SEL) return ARA_ERANGE;
   // rows of whole pairs of entries, where a count cannot carry into its neighbour's
   const bool fits = bound + std::min(bound, C) + 2 < (int64_t)UINT32_MAX;
-  const int pair = !yx && n_events < ((int64_t)1 << 32) && fits;
+  int pair = !yx && n_events < ((int64_t)1 << 32) && fits;
   // Rows straight from the event-major records (in pairs, slots ascending with the layers): one walk
   // of the portfolio's records in place of a fold per layer, a scan and a fill (16 layers over 2 M
   // events: 124 us against 290).  The walk reads every record: a call with 2 layers that hold an eighth
   // of 240 ELTs' records takes 305 us against 295, 4 layers with a quarter 339 against 355, 8 with a
   // half 418 against 474, 64 layers 2.02 ms against 2.64.
-  const bool by_event = fits && rows_usable(pf, sel) && std::is_sorted(sel.begin(), sel.end()) &&
+  bool by_event = fits && rows_usable(pf, sel) && std::is_sorted(sel.begin(), sel.end()) &&
                         4 * bound >= pf.n_records;
-  bound = std::max<int64_t>(bound, 1);
-  if (pair || by_event) bound = (bound + std::min(bound, C) + 1) / 2 * 2;
-  const int64_t n_blocks = (C + 1023) / 1024;
-  size_t off = 0;
-  auto take = [&](size_t n) { size_t o = (off + 255) / 256 * 256; off = o + n; return o; };
-  const size_t o_reg = take((size_t)n_sel * C), o_bits = take(4 * (size_t)n_sel * bmw);
-  const size_t o_ptr = take(4 * (size_t)(C + 1)), o_bsum = take(4 * (size_t)n_blocks), o_tot = take(4);
-  const size_t o_rows = take(8 * (size_t)C), o_ent = take((size_t)bound);
-  const size_t o_cls = take((size_t)n_trials * n_sel);
-  const size_t o_hm = take(4 * (size_t)bound), o_hg = take(4 * (size_t)bound), o_he = take(4 * (size_t)bound);
-  const size_t o_acc = take(sizeof(AdjCounts) * (size_t)n_sel);
-  const size_t o_slots = take(sizeof(SlotCounts) * (size_t)std::max<int64_t>(total_slots, 1));
-  const size_t o_ents = take(8);
-  const size_t o_words = yx ? take(sizeof(uint32_t) * (size_t)n_trials) : 0;
+  const int64_t n_blocks = (C + 1023) / 1024, least = std::max<int64_t>(bound, 1);
+  size_t off, o_reg, o_bits, o_ptr, o_bsum, o_tot, o_rows, o_ent, o_cls, o_hm, o_hg, o_he, o_acc, o_slots, o_ents, o_words;
+  auto lay_out = [&]() {
+    off = 0;
+    auto take = [&](size_t n) { size_t o = (off + 255) / 256 * 256; off = o + n; return o; };
+    bound = pair || by_event ? (least + std::min(least, C) + 1) / 2 * 2 : least;
+    o_reg = take((size_t)n_sel * C), o_bits = take(4 * (size_t)n_sel * bmw);
+    o_ptr = take(4 * (size_t)(C + 1)), o_bsum = take(4 * (size_t)n_blocks), o_tot = take(4);
+    o_rows = take(8 * (size_t)C), o_ent = take((size_t)bound);
+    o_cls = take((size_t)n_trials * n_sel);
+    o_hm = take(4 * (size_t)bound), o_hg = take(4 * (size_t)bound), o_he = take(4 * (size_t)bound);
+    o_acc = take(sizeof(AdjCounts) * (size_t)n_sel);
+    o_slots = take(sizeof(SlotCounts) * (size_t)std::max<int64_t>(total_slots, 1));
+    o_ents = take(8);
+    o_words = yx ? take(sizeof(uint32_t) * (size_t)n_trials) : 0;
+  };
+  lay_out();
   char* scratch = nullptr;
-  ARA_TRY(dmalloc_async((void**)&scratch, off, s));
+  if (dmalloc_async((void**)&scratch, off, s) != cudaSuccess) {
+    cudaGetLastError();
+    pair = 0;              // without room for whole pairs: rows of single entries
+    by_event = false;
+    lay_out();
+    ARA_TRY(dmalloc_async((void**)&scratch, off, s));
+  }
   uint8_t* reg_all = (uint8_t*)(scratch + o_reg);
   uint32_t* bits = (uint32_t*)(scratch + o_bits);
   uint32_t* ptr = (uint32_t*)(scratch + o_ptr);
