@@ -327,8 +327,8 @@ def run_ours(args, rank, ws, local):
     # One step: the YLT of the layer and its PML / TVaR, queued stream-ordered; each step's
     # results and device status are copied to pinned host slots without a host wait, so the
     # host queues step k+1 while step k runs (one synchronisation at the end).  The selection
-    # runs on a second stream behind an event.  Its blocks, like the stream kernel's, fill an SM's
-    # registers and it is cooperative, so it starts once every SM is free: the next step's fold
+    # runs on a second stream behind an event.  It is cooperative and does not fit beside the
+    # stream kernel, so it starts once that has left every SM: the next step's fold
     # (the first thing its ara_run_ylt queues, right behind the stream kernel) runs first and
     # hides the event's latency, and the selection then runs before that step's stream kernel.
     # The YLT is double-buffered so that the next step's stream kernel does not overwrite the
@@ -780,7 +780,7 @@ def measure_batched(rank: int, reps: int = 5):
     alg = 4 * n_occ + 8 * n_occ + 8 * walked + 8 * (yet.n_trials + 1) + 8 * pf.n_layers * yet.n_trials
     peak, peak_kind = measured_peaks()
     stream_ms = info["tuned_ms"]
-    roof = {"bound": "l1 / l2 gathers and shared-memory atomics (not hbm)",
+    roof = {"bound": "l1 / l2 gathers and shared-memory sums (not hbm)",
             "alg_bytes_per_launch": alg, "entries_walked": walked, "table_entries": n_entries,
             "table_mb": round(8 * n_entries / 1e6, 1), "stream_ms": round(stream_ms, 4),
             "achieved_gbs": round(alg / (stream_ms / 1e3) / 1e9, 1), "peak_gbs": peak,

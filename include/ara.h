@@ -536,8 +536,9 @@ ARA_API ara_status ara_risk_metrics(const double* d_ylt, int64_t n_trials, int32
  *                in when a device-side wait runs out (the other outputs are then undefined)
  * Scratch comes from the library's memory pool in stream order and is released in stream order.  Argument
  * errors are returned at once (ARA_EINVAL, ARA_ENOMEM, ARA_ECUDA) and nothing is queued.
- * Scheduling: the selection's blocks, like those of the default stream kernel, each fill an SM's
- * registers, and the selection starts only once every SM is free.  When it runs on another
+ * Scheduling: a block of the default stream kernel fills an SM's registers and a block of the
+ * selection half of them; the selection of up to 32 rows starts only once every SM has room
+ * for its blocks.  When it runs on another
  * stream than the next ara_run_ylt, order it before that run's stream kernel, e.g.
  * ara_prepare_ylt on the run's stream, a wait on an event recorded after this call, then
  * ara_run_ylt with ARA_RUN_PREPARED: otherwise the next stream kernel may take every SM first and
@@ -607,7 +608,8 @@ ARA_API ara_status ara_set_stream_shape(int32_t index);
  *                          multiple of 16, <= 4096; 0 = normal): every wait then runs out,
  *                          which exercises the timeout path without any fault.
  *   ARA_DBG_SKIP_BARRIER_ARRIVAL  1: the selection's blocks do not arrive at its grid
- *                          barriers, so every barrier wait runs out (0 = normal).
+ *                          barriers (the cooperative form of up to 32 rows of more than
+ *                          4,096 values), so every barrier wait runs out (0 = normal).
  *   ARA_DBG_ADJOINT_PER_LAYER  1: ara_adjoint of several layers takes one histogram pass per
  *                          layer instead of one pass for all (0 = normal); same results.
  * ARA_EINVAL for an unknown key or value. */
