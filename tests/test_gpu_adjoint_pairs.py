@@ -46,3 +46,27 @@ def test_pairs_equal_the_other_passes(n_layers, nnz, ascending):
     for b in others:
         assert all(torch.equal(a[k], b[k]) for k in ("elt", "layer", "loss")) and np.array_equal(a["ties"], b["ties"])
     pf.close()
+
+
+def test_longest_yets_count_single_entries():
+    """A YET of 2^32 occurrences and more keeps one 32-bit add per entry; here its trials cover the first few."""
+    g = np.random.default_rng(3)
+    C, n_elts, trials, n_layers = 5_000, 12, 300, 20
+    ids = [g.choice(C, size=3_000, replace=False).astype(np.int32) for _ in range(n_elts)]
+    loss = [np.exp(11.0 + 2.0 * g.standard_normal(3_000)) for _ in ids]
+    layers = [sorted(g.choice(n_elts, size=3, replace=False).tolist()) for _ in range(n_layers)]
+    z = np.zeros(n_layers)
+    pf = ara.Portfolio(C, ids, loss, np.full(n_elts, 1e4), np.full(n_elts, 1.5e6), layers, z + 1e4, z + 2e6,
+                       g.uniform(0.0, 1e6, n_layers), z + 1e13)
+    off = torch.arange(trials + 1, dtype=torch.int64, device="cuda") * 200
+    ev = torch.from_numpy(g.integers(0, C, trials * 200, dtype=np.int32)).cuda()
+    reg = torch.empty((n_layers, trials), dtype=torch.uint8, device="cuda")
+    ylt = pf.run_ylt(off, ev, regimes=reg)
+    pf.check()
+    a = pf.adjoint(off, ev, ylt, reg, 0.98)
+    assert float(a["loss"].abs().sum()) > 0
+    longest = torch.empty(1 << 32, dtype=torch.int32, device="cuda")
+    longest[: ev.numel()] = ev
+    b = pf.adjoint(off, longest, ylt, reg, 0.98)
+    assert all(torch.equal(a[k], b[k]) for k in ("elt", "layer", "loss")) and np.array_equal(a["ties"], b["ties"])
+    pf.close()
