@@ -473,7 +473,8 @@ struct AdjbHistParams {
 // (206 G/s, the same for 4, 8 and 16 bytes).  With PAIR two neighbouring counts take one 64-bit add
 // (the low count cannot carry: an event has fewer than 2^32 occurrences), and the descriptor's
 // narrower slots spare most loads of ent: 16 layers over 2e8 occurrences (1.4 entries per event)
-// 1.69 -> 1.43 ms.  One 32-bit add per entry is for YETs of 2^32 occurrences and more.
+// 1.69 -> 1.43 ms.  One 32-bit add per entry is for YETs of 2^32 occurrences and more, and for calls
+// without room for rows of whole pairs.
 template <bool PAIR>
 __global__ void __launch_bounds__(ADJB_WARPS * 32) k_adjb_hist(AdjbHistParams p) {
   __shared__ uint8_t cls_s[ADJB_WARPS][ADJB_MAX_SEL + 1];
