@@ -738,7 +738,7 @@ static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, in
 static ara_status run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets,
                           int64_t n_events, const int32_t* d_ids, int32_t n_sel,
                           const int32_t* layer_sel, double* d_ylt, uint8_t* d_regimes, int32_t flags,
-                          bool rows_ok, void* stream) {
+                          int64_t likely_events, void* stream) {
   if (!pf || n_trials < 0 || n_events < 0 || n_trials > ((int64_t)1 << 40)) return ARA_EINVAL;
   std::vector<int32_t> sel;
   ara_status st = check_selection(*pf, n_sel, layer_sel, sel);
@@ -756,7 +756,7 @@ static ara_status run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_
   // An ordinary run of several layers may take the event-major rows.  They need scratch, so a run
   // that is being captured stays with the per-layer kernels.
   bool rows = false;
-  if (rows_ok && flags == 0 && rows_faster(*pf, sel, n_trials, n_events)) {
+  if (flags == 0 && rows_faster(*pf, sel, n_trials, likely_events)) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     rows = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
   }
@@ -804,7 +804,7 @@ ara_status ara_run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_off
                        int32_t n_sel, const int32_t* layer_sel, double* d_ylt, uint8_t* d_regimes,
                        int32_t flags, void* stream) {
   (void)d_timestamps;
-  return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, n_sel, layer_sel, d_ylt, d_regimes, flags, true, stream);
+  return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, n_sel, layer_sel, d_ylt, d_regimes, flags, n_events, stream);
 }
 
 }  // extern "C"
@@ -1061,8 +1061,9 @@ ara_status ara_run_ylt_host(ara_portfolio* pf, int64_t n_trials, const int64_t* 
 }  // extern "C"
 
 namespace ara {
-ara_status run_ylt_per_layer(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets, int64_t n_events,
-                             const int32_t* d_ids, double* d_ylt, uint8_t* d_regimes, int32_t flags, void* stream) {
-  return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, 0, nullptr, d_ylt, d_regimes, flags, false, stream);
+ara_status run_ylt_slice(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets, int64_t n_events,
+                         int64_t likely_events, const int32_t* d_ids, double* d_ylt, uint8_t* d_regimes, int32_t flags,
+                         void* stream) {
+  return run_ylt(pf, n_trials, d_offsets, n_events, d_ids, 0, nullptr, d_ylt, d_regimes, flags, likely_events, stream);
 }
 }  // namespace ara

@@ -386,10 +386,11 @@ struct ara_portfolio : public ara::Portfolio {};
 struct ara_yet_index : public ara::YetIndex {};
 
 namespace ara {
-// ara_run_ylt of every layer that stays with the per-layer kernels (the server: its workers' short
-// kernels share the device better between the passes of others).
-ara_status run_ylt_per_layer(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets, int64_t n_events,
-                             const int32_t* d_ids, double* d_ylt, uint8_t* d_regimes, int32_t flags, void* stream);
+// ara_run_ylt of every layer over a slice of a YET: likely_events (about how many of the n_events
+// occurrences the slice's trials hold) decides between the per-layer streams and the rows.
+ara_status run_ylt_slice(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets, int64_t n_events,
+                         int64_t likely_events, const int32_t* d_ids, double* d_ylt, uint8_t* d_regimes, int32_t flags,
+                         void* stream);
 }  // namespace ara
 
 namespace ara {
