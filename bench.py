@@ -820,7 +820,7 @@ def measure_serving(rank: int, n_requests: int = 200, workers: int = 1, saturati
     per second, well above what any mode serves, so every makespan is set by the server and not
     by the last arrival), and compared with the same queries run one at a time (one worker, no
     merging; the batched path for requests of 4 or more layers, as in the served mode) and with
-    sequential plain runs (one at a time, every layer by the single-layer path).  The server's
+    sequential plain runs (one at a time, every request a plain run of its layers).  The server's
     adjoint requests read an event-major index of the resident YET, built when each server is set
     up, in every arm but the sequential plain runs and one served arm without it.  Latencies are
     then taken at 2x and 0.5x of the served mode's measured capacity.  Results must be identical
