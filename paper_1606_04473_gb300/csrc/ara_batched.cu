@@ -195,6 +195,8 @@ struct ara_plan {
   int64_t req_t0[BT_MAX_REQ] = {0, 0, 0, 0}, req_t1[BT_MAX_REQ] = {0, 0, 0, 0};
   double* req_ylt[BT_MAX_REQ] = {nullptr, nullptr, nullptr, nullptr};
   uint8_t* req_reg[BT_MAX_REQ] = {nullptr, nullptr, nullptr, nullptr};
+  // Whether a trial may lie outside a request's window (its rows hold the window's trials only).
+  bool windowed() const { return n_req > 1 || req_t0[0] != 0 || req_t1[0] != n_trials; }
   // The rows (d_rows: their descriptors), from the event-major records (by_event) or the folds.
   bool by_event = false;
   RowTable rt;
@@ -271,6 +273,7 @@ ara_status bt_stream(ara_plan& P, cudaStream_t s) {
   r.part = P.part;
   r.ns = (int32_t)P.sel.size();
   r.n_req = P.n_req;
+  r.windowed = P.windowed();
   r.layers = P.pf->d_layers;
   r.queue = P.d_queue;
   r.err = P.pf->d_err;
@@ -360,7 +363,7 @@ ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
   const int64_t C = pf.catalogue;
   for (P.by_event = rows_usable(pf, P.sel);; P.by_event = false) {
     P.rt = RowTable{};
-    P.rt.K = P.by_event && P.n_req == 1 ? rows_k(pf, P.sel) : 0;
+    P.rt.K = P.by_event && !P.windowed() ? rows_k(pf, P.sel) : 0;
     const RowSizes z = rows_sizes(pf, P.sel, P.rt.K, P.n_trials);
     P.rt.first_shift = z.first_shift;
     P.sched = rows_schedule(pf, (int)P.sel.size(), P.rt.K, z.likely_bytes, z.likely_entries,

@@ -281,10 +281,11 @@ struct RowsStream {
   uint32_t e_lo, e_n;               // events of this pass
   int32_t ns;
   int32_t n_req;
+  bool windowed;                    // requests with trial windows: several, or one short of every trial
   const LayerConst* layers;
   unsigned long long* queue;
   uint32_t* err;
-  int64_t t0[4], t1[4];             // requests as in GroupArgs (one: all trials)
+  int64_t t0[4], t1[4];             // requests as in GroupArgs
   double* ylt[4];
   uint8_t* regimes[4];
   int32_t first[5];                 // first slot of each request; unused ones past every slot

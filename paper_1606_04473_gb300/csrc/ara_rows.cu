@@ -653,6 +653,8 @@ k_rows_stream(RowsStream p) {
 // PASSES: the pass reads every ID but keeps only the events in [e_lo, e_hi), whose rows stay in L2
 // (compacted into a queue of 128 IDs per warp so that every round is full); the trial's exact
 // sums go through `part` from one pass to the next.
+//
+// MULTI: requests with trial windows (RowsStream::windowed); otherwise one request over every trial.
 template <int NC, bool MULTI, bool PASSES>
 __global__ void __launch_bounds__(RW_WARPS * 32, RW_MIN_BLOCKS)
 k_rows_join(RowsStream p) {
@@ -1021,7 +1023,7 @@ static ara_status launch_join(const Portfolio& pf, RowsStream p, RowSchedule& sc
 }
 
 static ara_status launch_rows_join(const Portfolio& pf, const RowsStream& p, RowSchedule& sched, cudaStream_t s) {
-  const bool m = p.n_req > 1;
+  const bool m = p.windowed;
   switch (sched.nc) {
     case 32:
     case 16: return m ? launch_join<16, true>(pf, p, sched, s) : launch_join<16, false>(pf, p, sched, s);
@@ -1055,8 +1057,10 @@ static ara_status launch_stream_nc(const Portfolio& pf, const RowsStream& p, Row
   }
 }
 
-// K > 0 holds one request's rows; merged requests always have their rows end to end.
+// K > 0 holds the rows of one request over every trial; requests with windows always have their rows
+// end to end, because the stream of rows in place writes every trial to d_ylt[0].
 ara_status launch_rows_stream(Portfolio& pf, const RowsStream& p, int K, RowSchedule& sched, cudaStream_t s) {
+  if (K > 0 && p.windowed) return ARA_EINVAL;
   switch (K) {
     case 1: return launch_stream_nc<1>(pf, p, sched, s);
     case 2: return launch_stream_nc<2>(pf, p, sched, s);

@@ -209,3 +209,30 @@ def test_fold_by_event_equals_fold_by_tiles(C, n_elts, nnz, f32):
         assert torch.equal(a["elt"], b["elt"].flip(1)) and k == a["elt"].shape[1]
         pf.check()
         pf.close()
+
+
+# every row form of FORMS, and windows at both ends of the trials, inside them and of one trial
+@pytest.mark.parametrize("form", [0, 1, 2, 3, 4, 6])
+@pytest.mark.parametrize("window", [(0, 1), (0, 40), (7, 52), "last"])
+def test_one_request_with_a_window_writes_its_own_trials_only(form, window):
+    """One request over a part of the trials: rows of the window's length, equal to a run of the slice,
+    and nothing before or after them."""
+    import ctypes
+    C, n_elts, nnz, n_layers, (lo, hi), f32, trials, events = FORMS[form]
+    pf, off, ids = make(form, C, n_elts, nnz, own(np.random.default_rng(form), n_layers, n_elts, lo, hi), f32,
+                        trials, events)
+    t0, t1 = window if window != "last" else (trials - 1, trials)
+    n, pad = n_layers * (t1 - t0), n_layers * trials
+    y = torch.full((n + 2 * pad,), -7.0, dtype=torch.float64, device="cuda")
+    r = torch.full((n + 2 * pad,), 77, dtype=torch.uint8, device="cuda")
+    one = lambda v: (ctypes.c_int64 * 1)(v)
+    st = ara.lib().ara_run_ylt_requests(
+        pf._h, trials, off.data_ptr(), ids.numel(), ids.data_ptr(), 1, (ctypes.c_int32 * 2)(0, n_layers), one(t0),
+        one(t1), (ctypes.c_void_p * 1)(y.data_ptr() + 8 * pad), (ctypes.c_void_p * 1)(r.data_ptr() + pad),
+        torch.cuda.current_stream().cuda_stream)
+    assert st == ara.ARA_OK
+    pf.check()
+    ref, reg_ref = singles(pf, off[t0:t1 + 1], ids, list(range(n_layers)))
+    assert torch.equal(y[pad:pad + n].view(n_layers, -1), ref) and torch.equal(r[pad:pad + n].view(n_layers, -1), reg_ref)
+    assert bool((y[:pad] == -7.0).all() & (y[pad + n:] == -7.0).all() & (r[:pad] == 77).all() & (r[pad + n:] == 77).all())
+    pf.close()
