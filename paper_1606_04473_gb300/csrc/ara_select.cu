@@ -33,19 +33,13 @@
 #include <cooperative_groups.h>
 
 #include "ara_internal.cuh"
+#include "ara_select_plan.h"
 
 namespace ara {
 
 constexpr int SEL_MAX_T = 16;
-constexpr int SEL_THREADS = 512;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
-constexpr int SEL_SAMPLE = 1024;                 // sampled keys per row
-constexpr int SEL_CLASSES = 2 * SEL_SAMPLE + 1;
-constexpr int SEL_SMALL = 4096;                  // rows up to this length are sorted whole
 constexpr int SEL_PICK = 4096;                   // list keys the pick keeps in shared memory
-// Rows of one request up to which the cooperative launch is the faster (16 rows of 200,000 values, 3
-// targets: 60 us against 95 us in clusters; 64 rows: 177 and 119).
-constexpr int SEL_GRID_ROWS = 32;
 constexpr unsigned SFULL = 0xffffffffu;
 
 struct SelTargets {
@@ -54,14 +48,6 @@ struct SelTargets {
   int64_t rank[SEL_MAX_T];     // 1-based rank from the top
 };
 
-struct SelState {
-  uint64_t key;                // the selected key (known at once when its class is a tie)
-  uint64_t lo, hi;             // the open interval it lies in otherwise (0 and ~0 at the ends: closed)
-  int32_t tie;                 // 1: the class is a splitter's own
-  int32_t list;                // the target whose list holds the interval (the first with that class)
-  int64_t before;              // keys above the class
-  int64_t in_class;            // keys in the class
-};
 __device__ __forceinline__ bool in_interval(uint64_t k, uint64_t lo, uint64_t hi) {
   return (k > lo || (lo == 0ull && k == 0ull)) && (k < hi || (hi == ~0ull && k == ~0ull));
 }
@@ -91,67 +77,6 @@ struct SelScratch {
   double* user_tvar;           // [n_layers][n_t - n_rp]
   double* user_mean;           // [n_layers]
 };
-
-// Sampled keys of a row: sorting them costs every block 2 us for 256 and 9 us for 1,024, and the
-// intervals they leave are picked from in about 4 us per 4,096 keys.
-__host__ __device__ inline int32_t sel_sample(int64_t n) { return n <= (1 << 19) ? 256 : SEL_SAMPLE; }
-
-// Room for the keys of one open interval between neighbouring samples: the interval that holds a
-// given rank has 2 / sample of the keys on average and more than 16 / sample with probability 2e-6 (a
-// list that would overflow is not used: its target is picked from the row itself).
-static int64_t list_cap(int64_t n) { return std::min<int64_t>(n, 16 * (n / sel_sample(n)) + 4096); }
-
-// A request's launch plan and scratch.  cap: keys per list; rounds: 2 when cap is short of list_cap
-// (the allocation-free call on long rows): overfull intervals are split again before the pick.
-struct SelPlan {
-  int64_t n = 0, cap = 0;
-  int32_t n_layers = 0, n_t = 0, blocks = 1, rounds = 1;
-  bool cluster = false;             // one cluster of `blocks` blocks per row
-  bool small = false;               // one block per row, sorted whole
-  int n_sms = 1;
-  size_t off[13];
-  size_t zero_bytes = 0, bytes = 0;
-};
-// beside: the caller's kernels share the device with other streams' (the server)
-static SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int64_t cap, bool beside = false) {
-  SelPlan y;
-  y.n = n;
-  y.cap = cap;
-  y.n_layers = n_layers;
-  y.n_t = n_t;
-  y.small = n <= SEL_SMALL;
-  y.n_sms = std::max(1, n_sms);
-  y.rounds = !y.small && cap < list_cap(n) ? 2 : 1;
-  const int64_t slots = 2ll * std::max(1, n_sms);           // blocks that run at once
-  y.cluster = !y.small && y.rounds == 1 && n <= (4 << 20) && (beside || n_layers > SEL_GRID_ROWS);
-  if (y.cluster) {                                          // all rows' clusters at once, if they can be
-    y.blocks = 16;
-    while (y.blocks > 1 && ((int64_t)n_layers * y.blocks > slots || n < 2048ll * y.blocks)) y.blocks /= 2;
-  } else if (!y.small) {
-    y.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, std::max<int64_t>(1, n_sms / n_layers)));
-  }
-  const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1), two = y.rounds > 1 ? lt : 0;
-  const size_t grid = y.small || y.cluster ? 0 : 1, lists = y.small ? 0 : 1;
-  size_t b = 0;
-  int i = 0;
-  auto t = [&](size_t k) { b = (b + 15) / 16 * 16; y.off[i++] = b; b += k; };
-  t(4 * grid * L * SEL_CLASSES);
-  t(4 * grid * lt);
-  t(4 * grid * L);
-  t(4);
-  t(4 * two * SEL_CLASSES);
-  t(4 * two);
-  y.zero_bytes = (b + 15) / 16 * 16;
-  t(sizeof(SelState) * lt);
-  t(8 * lists * lt * (size_t)cap);
-  t(8 * grid * lt * (size_t)y.blocks);
-  t(8 * grid * L * (size_t)y.blocks);
-  t(8 * (lt + L));
-  t(8 * lt);
-  t(8 * lt);
-  y.bytes = (b + 255) / 256 * 256;
-  return y;
-}
 
 static SelScratch carve(void* base, const SelPlan& y) {
   char* p = (char*)base;
@@ -1317,26 +1242,17 @@ extern "C" ara_status ara_risk_metrics_static(const double* d_ylt, int64_t n_tri
                       8 * lt, 8 * (size_t)n_layers, 8 * (size_t)n_layers})
     need = (need + 255) / 256 * 256 + part;
   if ((need + 255) / 256 * 256 > ARA_STATIC_SELECT_BYTES) return ARA_ERANGE;
-  // As many layers at a time as the array holds; where even one layer's lists do not fit, shorter
-  // lists and a second round.
-  const int64_t cap = list_cap(n_trials);
-  int32_t per = n_layers;
-  auto plan = [&](int64_t c) {
-    return sel_plan(n_trials, per, tg.n_t, sms, c);
-  };
-  while (per > 1 && plan(cap).bytes > ARA_STATIC_SELECT_BYTES) per = (per + 1) / 2;
-  SelPlan y = plan(cap);
-  for (int64_t c = cap / 2; y.bytes > ARA_STATIC_SELECT_BYTES && c >= SEL_SAMPLE; c /= 2) y = plan(c);
-  if (y.bytes > ARA_STATIC_SELECT_BYTES) return ARA_ERANGE;
+  SelGroups g;
+  if (!sel_groups(n_trials, n_layers, tg.n_t, sms, ARA_STATIC_SELECT_BYTES, g)) return ARA_ERANGE;
   void* scratch = nullptr;
   if ((st = static_scratch(&scratch)) != ARA_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
   uint32_t timed_out = 0;
   const size_t row = sizeof(double) * (size_t)tg.n_t;
-  for (int32_t l0 = 0; l0 < n_layers && st == ARA_OK && e == cudaSuccess && !timed_out; l0 += per) {
-    const int32_t nl = std::min(per, n_layers - l0);
-    if (nl < per) y = sel_plan(n_trials, nl, tg.n_t, sms, y.cap);
+  for (int32_t l0 = 0; l0 < n_layers && st == ARA_OK && e == cudaSuccess && !timed_out; l0 += g.per) {
+    const SelPlan& y = n_layers - l0 >= g.per ? g.first : g.last;
+    const int32_t nl = y.n_layers;
     SelScratch sc;
     st = launch_select(d_ylt + (int64_t)l0 * n_trials, y, tg, scratch, h_mean != nullptr, s, &sc);
     if (st != ARA_OK) break;

@@ -1,0 +1,121 @@
+// Launch plans of the PML / TVaR selection (ara_select.cu): its forms, block counts and scratch layout.
+// Host arithmetic only, apart from the constants the kernels share.
+#pragma once
+
+#include <stddef.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#ifdef __CUDACC__
+#define ARA_HD __host__ __device__
+#else
+#define ARA_HD
+#endif
+
+namespace ara {
+
+constexpr int SEL_THREADS = 512;
+constexpr int SEL_SAMPLE = 1024;                 // sampled keys per row
+constexpr int SEL_CLASSES = 2 * SEL_SAMPLE + 1;
+constexpr int SEL_SMALL = 4096;                  // rows up to this length are sorted whole
+// Rows of one request up to which the cooperative launch is the faster (16 rows of 200,000 values, 3
+// targets: 60 us against 95 us in clusters; 64 rows: 177 and 119).
+constexpr int SEL_GRID_ROWS = 32;
+
+struct SelState {
+  uint64_t key;                // the selected key (known at once when its class is a tie)
+  uint64_t lo, hi;             // the open interval it lies in otherwise (0 and ~0 at the ends: closed)
+  int32_t tie;                 // 1: the class is a splitter's own
+  int32_t list;                // the target whose list holds the interval (the first with that class)
+  int64_t before;              // keys above the class
+  int64_t in_class;            // keys in the class
+};
+
+// Sampled keys of a row: sorting them costs every block 2 us for 256 and 9 us for 1,024, and the
+// intervals they leave are picked from in about 4 us per 4,096 keys.
+ARA_HD inline int32_t sel_sample(int64_t n) { return n <= (1 << 19) ? 256 : SEL_SAMPLE; }
+
+// Room for the keys of one open interval between neighbouring samples: the interval that holds a
+// given rank has 2 / sample of the keys on average and more than 16 / sample with probability 2e-6 (a
+// list that would overflow is not used: its target is picked from the row itself).
+inline int64_t list_cap(int64_t n) { return std::min<int64_t>(n, 16 * (n / sel_sample(n)) + 4096); }
+
+// A request's launch plan and scratch.  cap: keys per list; rounds: 2 when cap is short of list_cap
+// (the allocation-free call on long rows): overfull intervals are split again before the pick.
+struct SelPlan {
+  int64_t n = 0, cap = 0;
+  int32_t n_layers = 0, n_t = 0, blocks = 1, rounds = 1;
+  bool cluster = false;             // one cluster of `blocks` blocks per row
+  bool small = false;               // one block per row, sorted whole
+  int n_sms = 1;
+  size_t off[13];
+  size_t zero_bytes = 0, bytes = 0;
+};
+// beside: the caller's kernels share the device with other streams' (the server)
+inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int64_t cap, bool beside = false) {
+  SelPlan y;
+  y.n = n;
+  y.cap = cap;
+  y.n_layers = n_layers;
+  y.n_t = n_t;
+  y.small = n <= SEL_SMALL;
+  y.n_sms = std::max(1, n_sms);
+  y.rounds = !y.small && cap < list_cap(n) ? 2 : 1;
+  const int64_t slots = 2ll * std::max(1, n_sms);           // blocks that run at once
+  y.cluster = !y.small && y.rounds == 1 && n <= (4 << 20) && (beside || n_layers > SEL_GRID_ROWS);
+  if (y.cluster) {                                          // all rows' clusters at once, if they can be
+    y.blocks = 16;
+    while (y.blocks > 1 && ((int64_t)n_layers * y.blocks > slots || n < 2048ll * y.blocks)) y.blocks /= 2;
+  } else if (!y.small) {
+    y.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, std::max<int64_t>(1, n_sms / n_layers)));
+  }
+  const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1), two = y.rounds > 1 ? lt : 0;
+  const size_t grid = y.small || y.cluster ? 0 : 1, lists = y.small ? 0 : 1;
+  size_t b = 0;
+  int i = 0;
+  auto t = [&](size_t k) { b = (b + 15) / 16 * 16; y.off[i++] = b; b += k; };
+  t(4 * grid * L * SEL_CLASSES);
+  t(4 * grid * lt);
+  t(4 * grid * L);
+  t(4);
+  t(4 * two * SEL_CLASSES);
+  t(4 * two);
+  y.zero_bytes = (b + 15) / 16 * 16;
+  t(sizeof(SelState) * lt);
+  t(8 * lists * lt * (size_t)cap);
+  t(8 * grid * lt * (size_t)y.blocks);
+  t(8 * grid * L * (size_t)y.blocks);
+  t(8 * (lt + L));
+  t(8 * lt);
+  t(8 * lt);
+  y.bytes = (b + 255) / 256 * 256;
+  return y;
+}
+
+// The rows of a request in groups whose scratch fits `limit` bytes each: groups of `per` rows (plan
+// `first`) and a last one of what is left (plan `last`).  Where even one row's lists do not fit, shorter
+// lists and a second round.  The last group can need more than the others although it has fewer rows
+// (33 rows run as clusters, 32 as one cooperative launch with class counts), so both are checked.
+struct SelGroups {
+  int32_t per = 1;
+  SelPlan first, last;
+};
+inline bool sel_groups(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, size_t limit, SelGroups& g) {
+  int64_t cap = list_cap(n);
+  auto fits = [&](int32_t per) {
+    g.per = per;
+    g.first = sel_plan(n, per, n_t, n_sms, cap);
+    g.last = n_layers % per ? sel_plan(n, n_layers % per, n_t, n_sms, cap) : g.first;
+    return g.first.bytes <= limit && g.last.bytes <= limit;
+  };
+  int32_t per = n_layers;
+  while (!fits(per) && per > 1) per = (per + 1) / 2;
+  while (!fits(per)) {
+    cap /= 2;
+    if (cap < SEL_SAMPLE) return false;
+  }
+  return true;
+}
+
+}  // namespace ara

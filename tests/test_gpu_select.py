@@ -78,3 +78,10 @@ def test_allocation_free_call_splits_overfull_lists():
 def test_short_rows_at_the_widths_of_the_sort(n):
     levels = [p for p in LEVELS if count(n * (1.0 - p)) >= 1]
     check(rows(n + 1, 5, n), levels=levels)
+
+
+@pytest.mark.parametrize("n,rps,levels", [(57_935, [100.0], [0.99]), (19_052, [100.0, 10.0], [0.99])])
+def test_allocation_free_call_in_uneven_groups(n, rps, levels):
+    """65 rows: a first group of 33 (a cluster each) would fit the array, its remainder of 32 (one cooperative
+    launch, which needs class counts) would not."""
+    check(rows(n, 65, n), rps, levels, ara.risk_metrics_static)
