@@ -1212,8 +1212,9 @@ static ara_status adjoint_common(ara_portfolio* pf_, const YetIndex* yx, int64_t
   while (cw(shift) * 4 > bm_budget) ++shift;
   const int smem = (int)(cw(shift) * 4);
   ara_status out_st = ARA_OK;
+  // the most that any catalogue asks for (see allow_shared; the kernel has static shared memory too)
   if (cudaFuncSetAttribute((const void*)k_adj_hist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           std::max(smem, 48 * 1024)) != cudaSuccess)
+                           (int)std::max<int64_t>(bm_budget, 48 * 1024)) != cudaSuccess)
     out_st = ARA_ECUDA;
 
   int64_t elt_slot0 = 0, loss_base0 = 0;

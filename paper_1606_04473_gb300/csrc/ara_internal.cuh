@@ -309,6 +309,10 @@ ara_status launch_rows_build(Portfolio& pf, const std::vector<int32_t>& sel, con
 ara_status launch_rows_stream(Portfolio& pf, const RowsStream& p, int K, RowSchedule& sched, cudaStream_t s);
 
 ara_status build_dense(Portfolio& pf, cudaStream_t s);
+// Lets launches of a kernel without static shared memory ask for all that a block may have.  Always
+// the same value: the attribute belongs to the function, which calls from other threads launch with
+// other sizes, and a launch that asks for more than the attribute says fails.
+ara_status allow_shared(const Portfolio& pf, const void* fn);
 // Compiled shapes (warps per block, ring stages) of the bulk-staged YET stream kernel.
 int32_t n_bulk_shapes();
 void set_bulk_shape(int32_t i);

@@ -996,7 +996,8 @@ ara_status launch_adjoint_rows(const Portfolio& pf, const std::vector<int32_t>& 
 // Blocks per SM of a stream kernel with this much shared memory; ARA_ERANGE when it does not fit.
 static ara_status rows_occupancy(const Portfolio& pf, const void* fn, int smem, int* per_sm) {
   if (smem > pf.max_smem_block) return ARA_ERANGE;
-  ARA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const ara_status st = allow_shared(pf, fn);
+  if (st != ARA_OK) return st;
   ARA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, RW_WARPS * 32, smem));
   return *per_sm < 1 ? ARA_ERANGE : ARA_OK;
 }

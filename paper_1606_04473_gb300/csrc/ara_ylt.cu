@@ -939,8 +939,8 @@ static int bitmap_shift(int64_t catalogue, int64_t max_bytes) {
   return s;
 }
 
-static ara_status set_smem(const void* fn, int bytes) {
-  ARA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+ara_status allow_shared(const Portfolio& pf, const void* fn) {
+  ARA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pf.max_smem_block));
   return ARA_OK;
 }
 
@@ -1031,7 +1031,7 @@ static ara_status launch_folded_one(Portfolio& pf, StreamParams& sp, cudaStream_
   const auto fn = k_ylt_folded<FILTER, Acc, U>;
   const int smem = FILTER ? (int)(sp.smem_words * 4) : 0;
   if (smem > 48 * 1024) {
-    ara_status st = set_smem((const void*)fn, smem);
+    ara_status st = allow_shared(pf, (const void*)fn);
     if (st != ARA_OK) return st;
   }
   LaunchScope ls(ARA_K_YLT, s);
@@ -1063,7 +1063,7 @@ static ara_status launch_bulk_shape(Portfolio& pf, StreamParams& sp, cudaStream_
   const int64_t bm_bytes = FILTER ? ((sp.smem_words * 4 + 127) / 128) * 128 : 0;
   using Sh = BulkShape<WARPS, STAGES, CHUNK>;
   const int smem = (int)(bm_bytes + Sh::ring_bytes + Sh::bar_bytes);
-  ara_status st = set_smem((const void*)fn, smem);
+  ara_status st = allow_shared(pf, (const void*)fn);
   if (st != ARA_OK) return st;
   LaunchScope ls(ARA_K_YLT, s);
   fn<<<pf.n_sms, WARPS * 32, smem, s>>>(sp);
