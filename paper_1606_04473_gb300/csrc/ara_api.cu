@@ -719,7 +719,7 @@ ara_status ara_prepare_ylt(ara_portfolio* pf, int32_t n_sel, const int32_t* laye
 // layer.  At 2e8 occurrences of 2 M events the line lies at 4-5 layers (4 layers: 1.07 ms layer by
 // layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
 static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, int64_t n_trials, int64_t events) {
-  if (sel.size() < 2 || !rows_usable(pf, sel)) return false;
+  if (sel.size() < 2 || !batched_fits(pf, sel.size()) || !rows_usable(pf, sel)) return false;
   const int K = rows_k(pf, sel);
   const RowSizes z = rows_sizes(pf, sel, K, n_trials);
   const double C = (double)pf.catalogue, L = (double)sel.size(), ev = (double)events, tr = (double)n_trials;

@@ -306,6 +306,11 @@ namespace {
 ara_status run_plan_async(ara_plan& P, cudaStream_t s);
 }  // namespace
 
+bool batched_fits(const Portfolio& pf, size_t n_sel) {
+  return n_sel <= (size_t)BT_MAX_LAYERS && n_sel <= (size_t)pf.n_layers &&
+         (int64_t)n_sel * pf.catalogue < ((int64_t)1 << 32);
+}
+
 // The batched path as one asynchronous call (no graph, default schedule): scratch comes from the
 // stream-ordered allocator, the table is sized by a host-known bound (every non-zero entry of
 // layer i is an event of one of its ELTs), and nothing waits on the host.
@@ -357,9 +362,7 @@ namespace {
 // of its ELTs), its scratch from the stream-ordered allocator; nothing waits on the host.
 ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
   Portfolio& pf = *P.pf;
-  if ((int)P.sel.size() > BT_MAX_LAYERS || (int)P.sel.size() > pf.n_layers ||
-      (int64_t)P.sel.size() * pf.catalogue >= ((int64_t)1 << 32))
-    return ARA_ERANGE;
+  if (!batched_fits(pf, P.sel.size())) return ARA_ERANGE;
   const int64_t C = pf.catalogue;
   for (P.by_event = rows_usable(pf, P.sel);; P.by_event = false) {
     P.rt = RowTable{};
@@ -443,8 +446,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
     }
   }
   if (P->sel.empty()) { bt_free(P); return ARA_EINVAL; }
-  if ((int)P->sel.size() > BT_MAX_LAYERS || (int)P->sel.size() > pf->n_layers ||
-      (int64_t)P->sel.size() * pf->catalogue >= ((int64_t)1 << 32)) {   // 32-bit row pointers
+  if (!batched_fits(*pf, P->sel.size())) {
     bt_free(P);
     return ARA_ERANGE;
   }

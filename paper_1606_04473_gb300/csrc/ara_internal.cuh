@@ -212,6 +212,9 @@ struct FoldOutHost {
 ara_status launch_fold_to(Portfolio& pf, int32_t n_sel, const int32_t* sel_host,
                           const FoldOutHost& o, cudaStream_t s, bool counted = true);
 ara_status launch_ylt(Portfolio& pf, const YltArgs& a, cudaStream_t s);
+// Whether a batched pass takes this many layers (slots of one byte, 32-bit row pointers over the folds
+// of every layer); a larger request gets ARA_ERANGE.
+bool batched_fits(const Portfolio& pf, size_t n_sel);
 ara_status run_batched_async(Portfolio& pf, const YltArgs& a, cudaStream_t s);
 // One pass of the batched stream for several requests at once (serving): request r owns the
 // portfolio's layers (= slots) [slot_first[r], slot_first[r + 1]) and the trials [t0[r], t1[r])

@@ -211,6 +211,32 @@ def test_fold_by_event_equals_fold_by_tiles(C, n_elts, nnz, f32):
         pf.close()
 
 
+def test_largest_portfolios_run_layer_by_layer():
+    """32 layers over 2^27 events, one step past what a batched pass takes: the ordinary run goes layer by
+    layer, also where the rows would be the faster way."""
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 40 GB of device memory")
+    C, n_layers, n = 1 << 27, 32, 64
+    g = np.random.default_rng(6)
+    ids = [np.sort(g.choice(C, size=5_000, replace=False)).astype(np.int32) for _ in range(4)]
+    ids[0][0], ids[1][-1] = 0, C - 1
+    loss = [np.full(5_000, 1e5 * (j + 1)) for j in range(4)]
+    z = np.zeros(n_layers)
+    pf = ara.Portfolio(C, ids, loss, np.zeros(4), np.full(4, np.inf), own(g, n_layers, 4, 1, 3), z + 1e4, z + 3e5,
+                       z, z + 1e9)
+    hits = np.concatenate(ids)
+    yet = torch.from_numpy(g.choice(hits, size=n * 50)).cuda()
+    off = torch.arange(n + 1, dtype=torch.int64, device="cuda") * 50
+    y = pf.run_ylt(off, yet)
+    pf.check()
+    ref, _ = singles(pf, off, yet, [0, 17, 31])
+    assert torch.equal(y[[0, 17, 31]], ref) and bool((y > 0).any(1).all())
+    with pytest.raises(ara.AraError) as e:
+        pf.run_ylt(off, yet, flags=ara.ARA_RUN_BATCHED)
+    assert e.value.status == ara.ARA_ERANGE
+    pf.close()
+
+
 # every row form of FORMS, and windows at both ends of the trials, inside them and of one trial
 @pytest.mark.parametrize("form", [0, 1, 2, 3, 4, 6])
 @pytest.mark.parametrize("window", [(0, 1), (0, 40), (7, 52), "last"])
