@@ -114,7 +114,21 @@ static cudaMemPool_t library_pool(int dev) {
   return g_pools[dev];
 }
 
+static std::atomic<int64_t> g_budget{-1};   // bytes left; -1: no limit
+
+void set_memory_budget(int64_t bytes) { g_budget.store(bytes > 0 ? bytes : -1); }
+
+bool take_budget(size_t bytes) {
+  int64_t left = g_budget.load(std::memory_order_relaxed);
+  while (left >= 0) {
+    if ((uint64_t)left < bytes) return false;
+    if (g_budget.compare_exchange_weak(left, left - (int64_t)bytes)) return true;
+  }
+  return true;
+}
+
 cudaError_t dmalloc_async(void** ptr, size_t bytes, cudaStream_t s) {
+  if (!take_budget(bytes)) return cudaErrorMemoryAllocation;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -278,7 +292,7 @@ static void free_portfolio(ara_portfolio* p) {
 template <typename T>
 static ara_status upload(T** dst, const T* src, size_t n) {
   if (n == 0) return ARA_OK;
-  ARA_TRY(cudaMalloc((void**)dst, n * sizeof(T)));
+  ARA_TRY(dmalloc(dst, n * sizeof(T)));
   ARA_TRY(cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice));
   return ARA_OK;
 }
@@ -328,6 +342,10 @@ ara_status ara_debug_set(int32_t key, int64_t value) {
     case ARA_DBG_ADJOINT_PER_LAYER:
       if (value != 0 && value != 1) return ARA_EINVAL;
       set_adjoint_per_layer((int32_t)value);
+      return ARA_OK;
+    case ARA_DBG_MEMORY_BUDGET:
+      if (value < 0) return ARA_EINVAL;
+      set_memory_budget(value);
       return ARA_OK;
     default:
       return ARA_EINVAL;
@@ -515,16 +533,16 @@ ara_status ara_create_portfolio(int64_t C, int32_t n_elts, const int64_t* rec_of
   p->bm_words = ((C + 31) / 32 + 3) / 4 * 4;
   p->cbits_stride = (((C + 1) / 2 + 31) / 32 + 3) / 4 * 4;   // coarsest needed: 1 bit per 2 events
   if (n_layers > 0) {
-    if (cudaMalloc(&p->d_q, sizeof(uint64_t) * (size_t)n_layers * C) != cudaSuccess) return fail(ARA_ENOMEM);
-    if (cudaMalloc(&p->d_bits, 4 * (size_t)n_layers * p->bm_words) != cudaSuccess) return fail(ARA_ENOMEM);
+    if (dmalloc(&p->d_q, sizeof(uint64_t) * (size_t)n_layers * C) != cudaSuccess) return fail(ARA_ENOMEM);
+    if (dmalloc(&p->d_bits, 4 * (size_t)n_layers * p->bm_words) != cudaSuccess) return fail(ARA_ENOMEM);
     if (cudaMemset(p->d_bits, 0, 4 * (size_t)n_layers * p->bm_words) != cudaSuccess) return fail(ARA_ECUDA);
-    if (cudaMalloc(&p->d_cbits, 4 * (size_t)n_layers * p->cbits_stride) != cudaSuccess) return fail(ARA_ENOMEM);
+    if (dmalloc(&p->d_cbits, 4 * (size_t)n_layers * p->cbits_stride) != cudaSuccess) return fail(ARA_ENOMEM);
   }
-  if (cudaMalloc(&p->d_err, sizeof(uint32_t)) != cudaSuccess) return fail(ARA_ENOMEM);
+  if (dmalloc(&p->d_err, sizeof(uint32_t)) != cudaSuccess) return fail(ARA_ENOMEM);
   if (cudaMemset(p->d_err, 0, sizeof(uint32_t)) != cudaSuccess) return fail(ARA_ECUDA);
   if (flags & ARA_DENSE_TABLES) {
     const size_t esz = f32 ? sizeof(float) : sizeof(double);
-    if (cudaMalloc(&p->d_dense, esz * (size_t)std::max(n_elts, 1) * C) != cudaSuccess) return fail(ARA_ENOMEM);
+    if (dmalloc(&p->d_dense, esz * (size_t)std::max(n_elts, 1) * C) != cudaSuccess) return fail(ARA_ENOMEM);
     if ((st = build_dense(*p, 0)) != ARA_OK) return fail(st);
   }
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(ARA_ECUDA);
@@ -693,9 +711,9 @@ ara_status ara_prepare_ylt(ara_portfolio* pf, int32_t n_sel, const int32_t* laye
   if (slot == 1 && !pf->d_q_alt) {   // the second workspace, allocated on first use
     const size_t nl = (size_t)std::max(pf->n_layers, 1), C = (size_t)pf->catalogue;
     ARA_TRY(cudaStreamSynchronize(s));
-    if (cudaMalloc(&pf->d_q_alt, sizeof(uint64_t) * nl * C) != cudaSuccess ||
-        cudaMalloc(&pf->d_bits_alt, sizeof(uint32_t) * nl * (size_t)pf->bm_words) != cudaSuccess ||
-        cudaMalloc(&pf->d_cbits_alt, sizeof(uint32_t) * nl * (size_t)pf->cbits_stride) != cudaSuccess) {
+    if (dmalloc(&pf->d_q_alt, sizeof(uint64_t) * nl * C) != cudaSuccess ||
+        dmalloc(&pf->d_bits_alt, sizeof(uint32_t) * nl * (size_t)pf->bm_words) != cudaSuccess ||
+        dmalloc(&pf->d_cbits_alt, sizeof(uint32_t) * nl * (size_t)pf->cbits_stride) != cudaSuccess) {
       cudaGetLastError();
       if (pf->d_q_alt) cudaFree(pf->d_q_alt);
       if (pf->d_bits_alt) cudaFree(pf->d_bits_alt);
@@ -776,7 +794,7 @@ static ara_status run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_
   a.flags = flags;
   if (flags & ARA_RUN_BATCHED) return run_batched_async(*pf, a, s);
   if (rows) {
-    st = run_batched_async(*pf, a, s);
+    st = run_batched_async(*pf, a, s, true);
     if (st == ARA_OK) {
       pf->fold0_missing.resize((size_t)pf->n_layers, 0);
       for (int32_t l : sel) pf->fold0_missing[(size_t)l] = 1;
@@ -844,7 +862,7 @@ static ara_status ensure_stage(Portfolio& pf, int64_t events, int64_t trials, in
     for (int i = 0; i < 2; ++i) {
       if (pf.d_stage_ids[i]) cudaFree(pf.d_stage_ids[i]);
       pf.d_stage_ids[i] = nullptr;
-      ARA_TRY(cudaMalloc(&pf.d_stage_ids[i], sizeof(int32_t) * (size_t)std::max<int64_t>(events, 4)));
+      ARA_TRY(dmalloc(&pf.d_stage_ids[i], sizeof(int32_t) * (size_t)std::max<int64_t>(events, 4)));
     }
     pf.stage_events = events;
   }
@@ -852,14 +870,14 @@ static ara_status ensure_stage(Portfolio& pf, int64_t events, int64_t trials, in
     for (int i = 0; i < 2; ++i) {
       if (pf.d_stage_off[i]) cudaFree(pf.d_stage_off[i]);
       pf.d_stage_off[i] = nullptr;
-      ARA_TRY(cudaMalloc(&pf.d_stage_off[i], sizeof(int64_t) * (size_t)(trials + 1)));
+      ARA_TRY(dmalloc(&pf.d_stage_off[i], sizeof(int64_t) * (size_t)(trials + 1)));
     }
     pf.stage_trials = trials;
   }
   if (ylt_elems > pf.ylt_full_elems) {
     if (pf.d_ylt_full) cudaFree(pf.d_ylt_full);
     pf.d_ylt_full = nullptr;
-    ARA_TRY(cudaMalloc(&pf.d_ylt_full, sizeof(double) * (size_t)ylt_elems));
+    ARA_TRY(dmalloc(&pf.d_ylt_full, sizeof(double) * (size_t)ylt_elems));
     pf.ylt_full_elems = ylt_elems;
   }
   return ARA_OK;
@@ -1008,7 +1026,7 @@ ara_status ara_run_ylt_host(ara_portfolio* pf, int64_t n_trials, const int64_t* 
     pf->d_res = nullptr;
     pf->h_res = nullptr;
     pf->res_elems = 0;
-    ARA_TRY(cudaMalloc((void**)&pf->d_res, sizeof(double) * (size_t)res_elems));
+    ARA_TRY(dmalloc(&pf->d_res, sizeof(double) * (size_t)res_elems));
     ARA_TRY(cudaMallocHost((void**)&pf->h_res, sizeof(double) * (size_t)res_elems));
     pf->res_elems = res_elems;
   }
@@ -1029,7 +1047,7 @@ ara_status ara_run_ylt_host(ara_portfolio* pf, int64_t n_trials, const int64_t* 
       if (pf->d_sel_scratch) cudaFree(pf->d_sel_scratch);
       pf->d_sel_scratch = nullptr;
       pf->sel_scratch_bytes = 0;
-      ARA_TRY(cudaMalloc(&pf->d_sel_scratch, need));
+      ARA_TRY(dmalloc(&pf->d_sel_scratch, need));
       pf->sel_scratch_bytes = need;
       st = queue(&need);
     }

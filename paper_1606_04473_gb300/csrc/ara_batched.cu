@@ -199,6 +199,7 @@ struct ara_plan {
   bool windowed() const { return n_req > 1 || req_t0[0] != 0 || req_t1[0] != n_trials; }
   // The rows (d_rows: their descriptors), from the event-major records (by_event) or the folds.
   bool by_event = false;
+  bool own_tables = false;           // never the folds (see run_batched_async)
   RowTable rt;
   RowSchedule sched;
   ulonglong2* part = nullptr;        // sums between passes (sched.passes > 1)
@@ -314,7 +315,7 @@ bool batched_fits(const Portfolio& pf, size_t n_sel) {
 // The batched path as one asynchronous call (no graph, default schedule): scratch comes from the
 // stream-ordered allocator, the table is sized by a host-known bound (every non-zero entry of
 // layer i is an event of one of its ELTs), and nothing waits on the host.
-ara_status run_batched_async(Portfolio& pf, const YltArgs& a, cudaStream_t s) {
+ara_status run_batched_async(Portfolio& pf, const YltArgs& a, cudaStream_t s, bool own_tables) {
   ara_plan P;
   P.pf = &pf;
   P.n_trials = a.n_trials;
@@ -325,6 +326,7 @@ ara_status run_batched_async(Portfolio& pf, const YltArgs& a, cudaStream_t s) {
   P.d_ylt = a.ylt;
   P.d_reg = a.regimes;
   if (a.id_base != 0 || a.row_stride != a.n_trials) return ARA_EINVAL;
+  P.own_tables = own_tables;
   single_request(P);
   return run_plan_async(P, s);
 }
@@ -383,7 +385,7 @@ ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
     char* buf = nullptr;
     if (dmalloc_async((void**)&buf, off, s) != cudaSuccess) {
       cudaGetLastError();
-      if (P.by_event) continue;      // the general way needs less
+      if (P.by_event && !P.own_tables) continue;      // the general way needs less
       return ARA_ENOMEM;
     }
     if (P.rt.K == 0) P.d_rows = (uint64_t*)(buf + o_rows);
@@ -463,11 +465,11 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
   P->rt.K = P->by_event ? rows_k(*pf, P->sel) : 0;
   const RowSizes z = rows_sizes(*pf, P->sel, P->rt.K, n_trials);
   P->rt.first_shift = z.first_shift;
-  if ((P->rt.K > 0 && cudaMalloc(&P->rt.table, 8 * (size_t)P->rt.K * (size_t)C) != cudaSuccess) ||
-      cudaMalloc(&P->d_rows, 8 * (size_t)C) != cudaSuccess || cudaMalloc(&P->d_total, 8) != cudaSuccess ||
-      cudaMalloc(&P->d_queue, sizeof(unsigned long long)) != cudaSuccess ||
-      (!P->by_event && (cudaMalloc(&P->d_ptr, 4 * (size_t)(C + 1)) != cudaSuccess ||
-                        cudaMalloc(&P->d_bsum, 4 * (size_t)P->n_blocks) != cudaSuccess)))
+  if ((P->rt.K > 0 && dmalloc(&P->rt.table, 8 * (size_t)P->rt.K * (size_t)C) != cudaSuccess) ||
+      dmalloc(&P->d_rows, 8 * (size_t)C) != cudaSuccess || dmalloc(&P->d_total, 8) != cudaSuccess ||
+      dmalloc(&P->d_queue, sizeof(unsigned long long)) != cudaSuccess ||
+      (!P->by_event && (dmalloc(&P->d_ptr, 4 * (size_t)(C + 1)) != cudaSuccess ||
+                        dmalloc(&P->d_bsum, 4 * (size_t)P->n_blocks) != cudaSuccess)))
     return fail(ARA_ENOMEM);
   P->rt.counters = P->d_total;
   P->rt.desc = P->d_rows;
@@ -479,7 +481,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
   if (cudaMemcpyAsync(total, P->d_total, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return fail(ARA_ECUDA);
-  if (cudaMalloc(&P->rt.ovf, 16 * (size_t)std::max<uint32_t>(total[0], 1)) != cudaSuccess) return fail(ARA_ENOMEM);
+  if (dmalloc(&P->rt.ovf, 16 * (size_t)std::max<uint32_t>(total[0], 1)) != cudaSuccess) return fail(ARA_ENOMEM);
   P->rt.ovf_pairs = total[0];
   if ((st = bt_prep(*P, s, true, nullptr)) != ARA_OK) return fail(st);
   const int64_t table_bytes = 8 * C * std::max(P->rt.K, 1) + 16 * (int64_t)total[0];
@@ -489,7 +491,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
   const bool tune = (flags & ARA_PLAN_AUTOTUNE) != 0;
   // room for the sums between passes: where the rule takes several, or where they are tried
   const bool try_passes = tune && P->rt.K == 0 && table_bytes > RW_PASS_BYTES / 2;
-  if ((P->sched.passes > 1 || try_passes) && cudaMalloc(&P->part, part_bytes) != cudaSuccess) {
+  if ((P->sched.passes > 1 || try_passes) && dmalloc(&P->part, part_bytes) != cudaSuccess) {
     cudaGetLastError();
     P->part = nullptr;
     P->sched.passes = 1;

@@ -30,6 +30,14 @@ void note_cuda_error(cudaError_t e, const char* what, const char* file, int line
 // pool's behaviour, which made every synchronous call map its scratch again).  Free with
 // cudaFreeAsync.  ara_release_memory() returns the idle part to the system.
 cudaError_t dmalloc_async(void** ptr, size_t bytes, cudaStream_t s);
+// cudaMalloc and cudaMallocAsync of the library within the test hook's budget (set_memory_budget, in
+// bytes from now on; 0: no limit).
+bool take_budget(size_t bytes);
+void set_memory_budget(int64_t bytes);
+template <typename T>
+cudaError_t dmalloc(T** ptr, size_t bytes) {
+  return take_budget(bytes) ? cudaMalloc((void**)ptr, bytes) : cudaErrorMemoryAllocation;
+}
 // A small block of pinned host memory, mapped into the device's address space, for the results of a
 // synchronous call: kernels write into it or one copy fills it without staging, where a copy to
 // pageable memory costs the call about 10 us each.  From a bounded list shared by all threads (p is
@@ -215,7 +223,9 @@ ara_status launch_ylt(Portfolio& pf, const YltArgs& a, cudaStream_t s);
 // Whether a batched pass takes this many layers (slots of one byte, 32-bit row pointers over the folds
 // of every layer); a larger request gets ARA_ERANGE.
 bool batched_fits(const Portfolio& pf, size_t n_sel);
-ara_status run_batched_async(Portfolio& pf, const YltArgs& a, cudaStream_t s);
+// own_tables: with its scratch alone, or ARA_ENOMEM (the general way folds by slot into the portfolio's
+// workspace of slot 0, over other layers' tables).
+ara_status run_batched_async(Portfolio& pf, const YltArgs& a, cudaStream_t s, bool own_tables = false);
 // One pass of the batched stream for several requests at once (serving): request r owns the
 // portfolio's layers (= slots) [slot_first[r], slot_first[r + 1]) and the trials [t0[r], t1[r])
 // of a union range of trials; every trial of the union is read once and walks only the table

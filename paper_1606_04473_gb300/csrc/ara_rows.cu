@@ -156,7 +156,7 @@ ara_status build_event_index(Portfolio& pf, cudaStream_t s) {
   const size_t o_elt = ((size_t)(pf.catalogue + 1) * 4 + 255) / 256 * 256;
   const size_t o_loss = o_elt + ((size_t)pf.n_records * 4 + 255) / 256 * 256;
   char* buf = nullptr;
-  if (cudaMalloc((void**)&buf, o_loss + (size_t)pf.n_records * esz) != cudaSuccess) {
+  if (dmalloc(&buf, o_loss + (size_t)pf.n_records * esz) != cudaSuccess) {
     cudaGetLastError();
     return ARA_OK;
   }

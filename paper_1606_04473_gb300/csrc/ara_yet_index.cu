@@ -133,8 +133,8 @@ extern "C" ara_status ara_yet_index_create(ara_portfolio* pf_, int64_t n_trials,
   cudaError_t e;
   if ((e = dmalloc_async((void**)&d_cnt, sizeof(uint32_t) * (size_t)(H * C), s)) != cudaSuccess ||
       (e = dmalloc_async((void**)&d_err, sizeof(uint32_t), s)) != cudaSuccess ||
-      (e = cudaMalloc((void**)&yx->d_len, sizeof(uint32_t) * (size_t)(H * G))) != cudaSuccess ||
-      (e = cudaMalloc((void**)&yx->d_base, sizeof(int64_t) * (size_t)(H * G))) != cudaSuccess)
+      (e = dmalloc(&yx->d_len, sizeof(uint32_t) * (size_t)(H * G))) != cudaSuccess ||
+      (e = dmalloc(&yx->d_base, sizeof(int64_t) * (size_t)(H * G))) != cudaSuccess)
     return fail(cuda_status(e));
   const unsigned grid = (unsigned)std::max(1, pf->n_sms * 8);
   if ((e = cudaMemsetAsync(d_cnt, 0, sizeof(uint32_t) * (size_t)(H * C), s)) != cudaSuccess ||
@@ -158,7 +158,7 @@ extern "C" ara_status ara_yet_index_create(ara_portfolio* pf_, int64_t n_trials,
     n_ent += (int64_t)len[i] * 32;
   }
   yx->n_ent = n_ent;
-  if ((e = cudaMalloc((void**)&yx->d_ent, sizeof(uint16_t) * (size_t)std::max<int64_t>(n_ent, 1))) != cudaSuccess)
+  if ((e = dmalloc(&yx->d_ent, sizeof(uint16_t) * (size_t)std::max<int64_t>(n_ent, 1))) != cudaSuccess)
     return fail(cuda_status(e));
   if (cudaMemcpyAsync(yx->d_base, base.data(), sizeof(int64_t) * base.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemsetAsync(yx->d_ent, 0xC0, sizeof(uint16_t) * (size_t)n_ent, s) != cudaSuccess ||

@@ -211,6 +211,31 @@ def test_fold_by_event_equals_fold_by_tiles(C, n_elts, nnz, f32):
         pf.close()
 
 
+def test_without_room_for_the_rows_prepared_folds_stay():
+    """An ordinary run whose rows do not fit the memory goes layer by layer, through its own layers' tables
+    only: a fold prepared in slot 0 for other layers is still there.  (The general way of a batched run
+    needs less scratch than rows in place, here 1.8 MB against 2.4, but uses the tables by slot.)"""
+    pf, off, ids = make(11, 50_000, 18, 6_000, [[l] for l in range(18)], True, 900, 200.0)
+    sel = list(range(2, 18))
+    ref, _ = singles(pf, off, ids, list(range(18)))
+    pf.prepare_ylt(layers=[0, 1], slot=0)
+    for budget in (2_100_000, 1):
+        ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, budget)
+        try:
+            n0 = ara.launch_count()
+            y = pf.run_ylt(off, ids, layers=sel)
+            assert ara.launch_count() - n0 >= len(sel)
+        finally:
+            ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+        assert torch.equal(y, ref[sel])
+        z = pf.run_ylt(off, ids, layers=[0, 1], flags=ara.ARA_RUN_PREPARED)
+        assert torch.equal(z, ref[[0, 1]])
+    n0 = ara.launch_count()
+    assert torch.equal(pf.run_ylt(off, ids, layers=sel), ref[sel]) and ara.launch_count() - n0 <= 3   # with room: rows
+    pf.check()
+    pf.close()
+
+
 def test_largest_portfolios_run_layer_by_layer():
     """32 layers over 2^27 events, one step past what a batched pass takes: the ordinary run goes layer by
     layer, also where the rows would be the faster way."""
