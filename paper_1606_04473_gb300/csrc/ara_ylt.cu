@@ -1020,8 +1020,13 @@ ara_status launch_fold(Portfolio& pf, int32_t n_sel, const int32_t* sel_host, in
   o.q_stride = pf.catalogue;
   o.bits_stride = pf.bm_words;
   o.f64_table = (flags & ARA_RUN_F64_SUM) ? 1 : 0;
-  if (slot == 0 && !pf.fold0_missing.empty())
-    for (int32_t i = 0; i < n_sel; ++i) pf.fold0_missing[(size_t)sel_host[i]] = 0;
+  if (slot == 0 && !pf.fold0_missing.empty()) {
+    // a captured fold has not run, and may not before the next prepared run: its layers stay missing
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    ARA_TRY(cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone)
+      for (int32_t i = 0; i < n_sel; ++i) pf.fold0_missing[(size_t)sel_host[i]] = 0;
+  }
   return launch_fold_to(pf, n_sel, sel_host, o, s);
 }
 

@@ -211,6 +211,35 @@ def test_fold_by_event_equals_fold_by_tiles(C, n_elts, nnz, f32):
         pf.close()
 
 
+@pytest.mark.parametrize("captured", ["prepared", "plain"])
+def test_a_captured_fold_does_not_count_before_its_replay(captured):
+    """After an ordinary run by rows the folds of its layers are missing from slot 0.  A prepared (or an
+    ordinary) run that is only captured records the fold; an eager prepared run before the first replay
+    still finds it missing and folds itself."""
+    g = np.random.default_rng(12)
+    pf, off, ids = make(13, 20_000, 30, 2_000, own(g, 12, 30, 3, 12), True, 500, 200.0)
+    sel = list(range(12))
+    ref, _ = singles(pf, off, ids, sel)
+    # slot 0 holds other values for these layers (sums in FP64, not the fixed point of an ordinary run)
+    pf.run_ylt(off, ids, layers=sel[::-1], flags=ara.ARA_RUN_F64_SUM)
+    n0 = ara.launch_count()
+    assert torch.equal(pf.run_ylt(off, ids, layers=sel), ref) and ara.launch_count() - n0 <= 3
+    s = torch.cuda.Stream()
+    out = torch.zeros_like(ref)
+    graph = torch.cuda.CUDAGraph()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=s):
+        pf.run_ylt(off, ids, layers=sel, out=out, flags=ara.ARA_RUN_PREPARED if captured == "prepared" else 0, stream=s)
+    assert torch.equal(pf.run_ylt(off, ids, layers=sel, flags=ara.ARA_RUN_PREPARED), ref)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+    pf.check()
+    pf.close()
+
+
 def test_without_room_for_the_rows_prepared_folds_stay():
     """An ordinary run whose rows do not fit the memory goes layer by layer, through its own layers' tables
     only: a fold prepared in slot 0 for other layers is still there.  (The general way of a batched run
