@@ -529,7 +529,6 @@ ara_status ara_create_portfolio(int64_t C, int32_t n_elts, const int64_t* rec_of
     const std::vector<uint64_t> mem = layer_members(*p);
     if ((st = upload(&p->d_mem, mem.data(), mem.size())) != ARA_OK) return fail(st);
   }
-  if ((st = build_event_index(*p, 0)) != ARA_OK) return fail(st);
   p->bm_words = ((C + 31) / 32 + 3) / 4 * 4;
   p->cbits_stride = (((C + 1) / 2 + 31) / 32 + 3) / 4 * 4;   // coarsest needed: 1 bit per 2 events
   if (n_layers > 0) {
@@ -545,6 +544,8 @@ ara_status ara_create_portfolio(int64_t C, int32_t n_elts, const int64_t* rec_of
     if (dmalloc(&p->d_dense, esz * (size_t)std::max(n_elts, 1) * C) != cudaSuccess) return fail(ARA_ENOMEM);
     if ((st = build_dense(*p, 0)) != ARA_OK) return fail(st);
   }
+  // last, because the portfolio can do without it: what it needs goes first
+  if ((st = build_event_index(*p, 0)) != ARA_OK) return fail(st);
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(ARA_ECUDA);
   *out = p;
   return ARA_OK;

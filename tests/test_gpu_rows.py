@@ -240,6 +240,27 @@ def test_a_captured_fold_does_not_count_before_its_replay(captured):
     pf.close()
 
 
+def test_a_portfolio_without_room_for_its_event_index():
+    """Room for the portfolio (13 MB here) but not for the records event by event too (5 MB): it is made all
+    the same, and works through the per-layer folds."""
+    args = (15, 100_000, 20, 20_000, [[2 * l, 2 * l + 1] for l in range(8)], False, 500, 200.0)
+    pf, off, ids = make(*args)
+    ref, reg_ref = singles(pf, off, ids, list(range(8)))
+    pf.close()
+    ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 14_200_000)
+    try:
+        pf, off, ids = make(*args)
+    finally:
+        ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+    y, reg = singles(pf, off, ids, list(range(8)))
+    assert torch.equal(y, ref) and torch.equal(reg, reg_ref)
+    n0 = ara.launch_count()
+    assert torch.equal(pf.run_ylt(off, ids), ref) and ara.launch_count() - n0 >= 8      # no rows without the index
+    assert torch.equal(pf.run_ylt(off, ids, flags=ara.ARA_RUN_BATCHED), ref)
+    pf.check()
+    pf.close()
+
+
 def test_without_room_for_the_rows_prepared_folds_stay():
     """An ordinary run whose rows do not fit the memory goes layer by layer, through its own layers' tables
     only: a fold prepared in slot 0 for other layers is still there.  (The general way of a batched run
