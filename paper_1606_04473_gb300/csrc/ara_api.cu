@@ -1035,11 +1035,12 @@ ara_status ara_run_ylt_host(ara_portfolio* pf, int64_t n_trials, const int64_t* 
   ARA_TRY(cudaMemsetAsync(d_words, 0, 2 * sizeof(uint32_t), s));
   if (metrics) {
     // the selection's scratch is kept with the portfolio, so repeated calls allocate nothing
+    size_t limit = SIZE_MAX;
     auto queue = [&](size_t* need) {
       return risk_metrics_queue(pf->d_ylt_full, n_trials, nsel, n_rp, rps, n_tvar, levels,
                                 n_rp > 0 ? pf->d_res : nullptr, n_tvar > 0 ? pf->d_res + n_pml : nullptr,
                                 h_mean ? pf->d_res + n_pml + n_tv : nullptr, d_words,
-                                pf->d_sel_scratch, pf->sel_scratch_bytes, need, s);
+                                pf->d_sel_scratch, pf->sel_scratch_bytes, limit, need, s);
     };
     size_t need = 0;
     st = queue(&need);
@@ -1048,9 +1049,18 @@ ara_status ara_run_ylt_host(ara_portfolio* pf, int64_t n_trials, const int64_t* 
       if (pf->d_sel_scratch) cudaFree(pf->d_sel_scratch);
       pf->d_sel_scratch = nullptr;
       pf->sel_scratch_bytes = 0;
-      ARA_TRY(dmalloc(&pf->d_sel_scratch, need));
-      pf->sel_scratch_bytes = need;
-      st = queue(&need);
+      // with less memory, fewer rows at a time and shorter lists
+      while (dmalloc(&pf->d_sel_scratch, need) != cudaSuccess) {
+        cudaGetLastError();
+        const size_t tried = need;
+        limit = tried - tried / 4;
+        if ((st = queue(&need)) != ARA_ERANGE) break;
+        if (need >= tried) { st = ARA_ENOMEM; break; }
+      }
+      if (pf->d_sel_scratch) {
+        pf->sel_scratch_bytes = need;
+        st = queue(&need);
+      }
     }
     if (st != ARA_OK) {
       cudaStreamSynchronize(pf->copy_stream);

@@ -360,12 +360,12 @@ struct SelectResult {
 ara_status select_one_rank(const double* d_ylt, int64_t n, int32_t n_layers, int64_t m, int n_sms,
                            cudaStream_t s, SelectResult* out, uint32_t* err);
 void free_select_result(SelectResult& r, cudaStream_t s);
-// The stream-ordered risk metrics with caller-owned scratch: ARA_ERANGE (and *need) when the
-// scratch is too small.
+// The stream-ordered risk metrics with caller-owned scratch, planned within `limit` bytes where that is
+// possible: ARA_ERANGE (and *need) when the scratch is too small.
 ara_status risk_metrics_queue(const double* d_ylt, int64_t n_trials, int32_t n_layers, int32_t n_rp,
                               const double* rps, int32_t n_tvar, const double* levels,
                               double* d_pml, double* d_tvar, double* d_mean, uint32_t* d_status,
-                              void* scratch, size_t scratch_bytes, size_t* need, cudaStream_t s);
+                              void* scratch, size_t scratch_bytes, size_t limit, size_t* need, cudaStream_t s);
 // PML / TVaR of n_layers device YLT rows into host arrays (synchronises s); scratch from the
 // stream-ordered allocator.  beside: blocks that run beside other streams' kernels, no cooperative
 // launch (the server).

@@ -52,18 +52,19 @@ __device__ __forceinline__ bool in_interval(uint64_t k, uint64_t lo, uint64_t hi
   return (k > lo || (lo == 0ull && k == 0ull)) && (k < hi || (hi == ~0ull && k == ~0ull));
 }
 
-// Scratch (one allocation; the first part, up to state, is zero-filled before the launch):
+// Scratch (one allocation; the first part, up to state, is zero-filled before the launch).  Layers count
+// from the first one of a launch group; G of them share the working parts at a time.
 struct SelScratch {
-  uint32_t* count;             // [n_layers][SEL_CLASSES] class totals
-  uint32_t* n_list;            // [n_layers][n_t] keys in each list
-  uint32_t* bar;               // [n_layers] grid-barrier counters
   uint32_t* err;               // [1]
-  uint32_t* count2;            // second round: [n_layers][n_t][SEL_CLASSES], else null
-  uint32_t* n_list2;           // second round: [n_layers][n_t]
+  uint32_t* count;             // [G][SEL_CLASSES] class totals
+  uint32_t* n_list;            // [G][n_t] keys in each list
+  uint32_t* bar;               // [G] grid-barrier counters
+  uint32_t* count2;            // second round: [G][n_t][SEL_CLASSES], else null
+  uint32_t* n_list2;           // second round: [G][n_t]
   SelState* state;             // [n_layers][n_t]
-  uint64_t* list;              // [n_layers][n_t][cap]
-  double* psum;                  // [n_layers][n_t][blocks] block partials of the tail sums
-  double* pmean;                 // [n_layers][blocks] block partials of the row sum
+  uint64_t* list;              // [G][n_t][cap]
+  double* psum;                // [G][n_t][blocks] block partials of the tail sums
+  double* pmean;               // [G][blocks] block partials of the row sum
   // results, contiguous: out, mean
   double* out;                 // [n_layers][n_t] PML / TVaR
   double* mean;                // [n_layers]
@@ -81,10 +82,10 @@ struct SelScratch {
 static SelScratch carve(void* base, const SelPlan& y) {
   char* p = (char*)base;
   SelScratch s{};
-  s.count = (uint32_t*)(p + y.off[0]);
-  s.n_list = (uint32_t*)(p + y.off[1]);
-  s.bar = (uint32_t*)(p + y.off[2]);
-  s.err = (uint32_t*)(p + y.off[3]);
+  s.err = (uint32_t*)(p + y.off[0]);
+  s.count = (uint32_t*)(p + y.off[1]);
+  s.n_list = (uint32_t*)(p + y.off[2]);
+  s.bar = (uint32_t*)(p + y.off[3]);
   s.count2 = y.rounds > 1 ? (uint32_t*)(p + y.off[4]) : nullptr;
   s.n_list2 = (uint32_t*)(p + y.off[5]);
   s.state = (SelState*)(p + y.off[6]);
@@ -976,7 +977,70 @@ static ara_status sel_prepare_kernels() {
 }
 
 size_t select_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_t, int n_sms) {
-  return sel_plan(n, n_layers, n_t, n_sms, list_cap(n), true).bytes;
+  return sel_plan_within(n, n_layers, n_t, n_sms, true, SEL_SCRATCH).bytes;
+}
+
+// Plan and stream-ordered scratch of a request; with less memory, fewer rows at a time and shorter lists.
+static ara_status take_scratch(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, bool beside, cudaStream_t s,
+                               SelPlan* y, void** scratch) {
+  *y = sel_plan_within(n, n_layers, n_t, n_sms, beside, SEL_SCRATCH);
+  while (true) {
+    const cudaError_t e = dmalloc_async(scratch, y->bytes, s);
+    if (e == cudaSuccess) return ARA_OK;
+    if (e != cudaErrorMemoryAllocation) ARA_TRY(e);
+    cudaGetLastError();
+    const SelPlan less = sel_plan_within(n, n_layers, n_t, n_sms, beside, y->bytes - y->bytes / 4);
+    if (less.bytes >= y->bytes) ARA_TRY(e);
+    *y = less;
+  }
+}
+
+// One group of a request: `rows` rows of `d_ylt`, results to `sc` (counted from the group's first row).
+static ara_status launch_group(const double* d_ylt, const SelPlan& y, const SelTargets& tg, int32_t rows,
+                               const SelScratch& sc, int want_mean, cudaStream_t s) {
+  const int64_t n = y.n;
+  if (y.small) {
+    int pad = 64;
+    while (pad < n) pad <<= 1;
+    LaunchScope ls(ARA_K_SELECT, s);
+    const auto fn = pad <= 1024 ? k_sel_small<2> : pad <= 2048 ? k_sel_small<4> : k_sel_small<8>;
+    fn<<<(unsigned)rows, SEL_THREADS, (size_t)pad * 8, s>>>(d_ylt, (int32_t)n, pad, tg, sc, want_mean);
+    ARA_TRY(cudaGetLastError());
+    return ARA_OK;
+  }
+  const int skip = debug_skip_arrival();
+  if (y.cluster) {
+    for (int32_t l0 = 0; l0 < rows; l0 += 32768) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)y.blocks, (unsigned)std::min<int32_t>(32768, rows - l0));
+      cfg.blockDim = dim3(SEL_THREADS);
+      cfg.dynamicSmemBytes = SEL_SMEM;
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)y.blocks;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      LaunchScope ls(ARA_K_SELECT, s);
+      ARA_TRY(cudaLaunchKernelEx(&cfg, k_sel_cluster, d_ylt, n, l0, tg, sc, want_mean, skip));
+    }
+    return ARA_OK;
+  }
+  const int32_t per = y.at_once();
+  for (int32_t l0 = 0; l0 < rows; l0 += per) {
+    const dim3 grid((unsigned)y.blocks, (unsigned)std::min(per, rows - l0));
+    uint64_t limit = wait_limit_ns();
+    int64_t nn = n;
+    SelTargets t2 = tg;
+    SelScratch s2 = sc;
+    int wm = want_mean, sk = skip;
+    void* args[] = {(void*)&d_ylt, &nn, &l0, &t2, &s2, &wm, &limit, &sk};
+    LaunchScope ls(ARA_K_SELECT, s);
+    ARA_TRY(cudaLaunchCooperativeKernel((const void*)k_sel_grid, grid, dim3(SEL_THREADS), args, (size_t)SEL_SMEM, s));
+  }
+  return ARA_OK;
 }
 
 // Launch the whole selection into `scratch` (laid out by `y`, its first part zero-filled here);
@@ -991,52 +1055,27 @@ ara_status launch_select(const double* d_ylt, const SelPlan& y, const SelTargets
   sc.user_pml = user_pml;
   sc.user_tvar = user_tvar;
   sc.user_mean = user_mean;
-  const int64_t n = y.n;
   const ara_status ready = sel_prepare_kernels();
   if (ready != ARA_OK) return ready;
-  // (without counts in global memory only the error word needs clearing, and the host's is clear)
-  if (!host_err || !(y.small || y.cluster)) ARA_TRY(cudaMemsetAsync(scratch, 0, y.zero_bytes, s));
-  if (y.small) {
-    int pad = 64;
-    while (pad < n) pad <<= 1;
-    LaunchScope ls(ARA_K_SELECT, s);
-    const auto fn = pad <= 1024 ? k_sel_small<2> : pad <= 2048 ? k_sel_small<4> : k_sel_small<8>;
-    fn<<<(unsigned)y.n_layers, SEL_THREADS, (size_t)pad * 8, s>>>(d_ylt, (int32_t)n, pad, tg, sc, want_mean);
-    ARA_TRY(cudaGetLastError());
-    *out = sc;
-    return ARA_OK;
-  }
-  const int skip = debug_skip_arrival();
-  if (y.cluster) {
-    for (int32_t l0 = 0; l0 < y.n_layers; l0 += 32768) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)y.blocks, (unsigned)std::min<int32_t>(32768, y.n_layers - l0));
-      cfg.blockDim = dim3(SEL_THREADS);
-      cfg.dynamicSmemBytes = SEL_SMEM;
-      cfg.stream = s;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = (unsigned)y.blocks;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      LaunchScope ls(ARA_K_SELECT, s);
-      ARA_TRY(cudaLaunchKernelEx(&cfg, k_sel_cluster, d_ylt, n, l0, tg, sc, want_mean, skip));
+  const bool counts = !(y.small || y.cluster);    // class counts in global memory, cleared for every group
+  for (int32_t g0 = 0; g0 < y.n_layers; g0 += y.per) {
+    // (without counts only the error word needs clearing, and the host's is clear)
+    if (g0 == 0 ? counts || !host_err : counts) {
+      const size_t z = g0 == 0 ? 0 : y.off[1];
+      ARA_TRY(cudaMemsetAsync((char*)scratch + z, 0, y.zero_bytes - z, s));
     }
-    *out = sc;
-    return ARA_OK;
-  }
-  const int32_t per = std::max(1, y.n_sms / y.blocks);      // rows whose blocks run at once
-  for (int32_t l0 = 0; l0 < y.n_layers; l0 += per) {
-    const dim3 grid((unsigned)y.blocks, (unsigned)std::min(per, y.n_layers - l0));
-    uint64_t limit = wait_limit_ns();
-    int64_t nn = n;
-    SelTargets t2 = tg;
-    int wm = want_mean, sk = skip;
-    void* args[] = {(void*)&d_ylt, &nn, &l0, &t2, &sc, &wm, &limit, &sk};
-    LaunchScope ls(ARA_K_SELECT, s);
-    ARA_TRY(cudaLaunchCooperativeKernel((const void*)k_sel_grid, grid, dim3(SEL_THREADS), args, (size_t)SEL_SMEM, s));
+    SelScratch g = sc;
+    const int64_t l = g0, lt = l * y.n_t;
+    g.state += lt;
+    g.out += lt;
+    g.mean += l;
+    g.gt += lt;
+    g.eq += lt;
+    if (g.user_pml) g.user_pml += l * tg.n_rp;
+    if (g.user_tvar) g.user_tvar += l * (y.n_t - tg.n_rp);
+    if (g.user_mean) g.user_mean += l;
+    const ara_status st = launch_group(d_ylt + l * y.n, y, tg, std::min(y.per, y.n_layers - g0), g, want_mean, s);
+    if (st != ARA_OK) return st;
   }
   *out = sc;
   return ARA_OK;
@@ -1054,11 +1093,12 @@ ara_status select_one_rank(const double* d_ylt, int64_t n, int32_t n_layers, int
   tg.n_t = 1;
   tg.n_rp = 1;               // the key and its counts, no tail sum
   tg.rank[0] = m;
-  const SelPlan y = sel_plan(n, n_layers, 1, n_sms, list_cap(n));
+  SelPlan y;
   void* scratch = nullptr;
-  ARA_TRY(dmalloc_async(&scratch, y.bytes, s));
+  ara_status st = take_scratch(n, n_layers, 1, n_sms, false, s, &y, &scratch);
+  if (st != ARA_OK) return st;
   SelScratch sc;
-  ara_status st = launch_select(d_ylt, y, tg, scratch, 0, s, &sc, err);
+  st = launch_select(d_ylt, y, tg, scratch, 0, s, &sc, err);
   if (st != ARA_OK) {
     cudaFreeAsync(scratch, s);
     return st;
@@ -1090,9 +1130,9 @@ ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const SelPlan y = sel_plan(n_trials, n_layers, tg.n_t, sms, list_cap(n_trials), beside);
+  SelPlan y;
   void* scratch = nullptr;
-  ARA_TRY(dmalloc_async(&scratch, y.bytes, s));
+  if ((st = take_scratch(n_trials, n_layers, tg.n_t, sms, beside, s, &y, &scratch)) != ARA_OK) return st;
   SelScratch sc;
   const size_t L = (size_t)n_layers, n_pml = L * n_rp, n_tv = L * n_tvar;
   PinnedSlot slot;
@@ -1137,12 +1177,13 @@ ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_
 }  // namespace ara
 
 namespace ara {
-// ara_risk_metrics_async with caller-owned scratch (the host pipeline keeps one per portfolio):
-// ARA_ERANGE with *need set when scratch_bytes is too small, nothing queued.
+// ara_risk_metrics_async with caller-owned scratch (the host pipeline keeps one per portfolio), within
+// `limit` bytes where a plan fits them: ARA_ERANGE with *need set when scratch_bytes is too small, nothing
+// queued.
 ara_status risk_metrics_queue(const double* d_ylt, int64_t n_trials, int32_t n_layers, int32_t n_rp,
                               const double* rps, int32_t n_tvar, const double* levels,
                               double* d_pml, double* d_tvar, double* d_mean, uint32_t* d_status,
-                              void* scratch, size_t scratch_bytes, size_t* need, cudaStream_t s) {
+                              void* scratch, size_t scratch_bytes, size_t limit, size_t* need, cudaStream_t s) {
   SelTargets tg;
   if (!d_ylt || n_layers < 1 || !d_status || !need) return ARA_EINVAL;
   if ((n_rp > 0 && !d_pml) || (n_tvar > 0 && !d_tvar)) return ARA_EINVAL;
@@ -1153,7 +1194,7 @@ ara_status risk_metrics_queue(const double* d_ylt, int64_t n_trials, int32_t n_l
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const SelPlan y = sel_plan(n_trials, n_layers, tg.n_t, sms, list_cap(n_trials));
+  const SelPlan y = sel_plan_within(n_trials, n_layers, tg.n_t, sms, false, std::min(limit, SEL_SCRATCH));
   *need = y.bytes;
   if (!scratch || scratch_bytes < *need) return ARA_ERANGE;
   SelScratch sc;
@@ -1180,9 +1221,9 @@ extern "C" ara_status ara_risk_metrics_async(const double* d_ylt, int64_t n_tria
   int dev = 0, sms = 0;
   ARA_TRY(cudaGetDevice(&dev));
   ARA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const SelPlan y = sel_plan(n_trials, n_layers, tg.n_t, sms, list_cap(n_trials));
+  SelPlan y;
   void* scratch = nullptr;
-  if (dmalloc_async(&scratch, y.bytes, s) != cudaSuccess) return ARA_ENOMEM;
+  if ((st = take_scratch(n_trials, n_layers, tg.n_t, sms, false, s, &y, &scratch)) != ARA_OK) return st;
   ara_status r = ARA_OK;
   SelScratch sc;
   if (cudaMemsetAsync(d_status, 0, sizeof(uint32_t), s) != cudaSuccess) r = ARA_ECUDA;

@@ -41,51 +41,60 @@ ARA_HD inline int32_t sel_sample(int64_t n) { return n <= (1 << 19) ? 256 : SEL_
 // list that would overflow is not used: its target is picked from the row itself).
 inline int64_t list_cap(int64_t n) { return std::min<int64_t>(n, 16 * (n / sel_sample(n)) + 4096); }
 
-// A request's launch plan and scratch.  cap: keys per list; rounds: 2 when cap is short of list_cap
-// (the allocation-free call on long rows): overfull intervals are split again before the pick.
+// A request's launch plan and scratch.  The form and the blocks of a row (on which the order of the TVaR and
+// mean sums depends) follow from the request; how many rows share the lists at a time (per: groups run
+// one after the other) and how long the lists are follow from the memory, and change no result.
 struct SelPlan {
-  int64_t n = 0, cap = 0;
-  int32_t n_layers = 0, n_t = 0, blocks = 1, rounds = 1;
+  int64_t n = 0, cap = 0;           // cap: keys per list
+  int32_t n_layers = 0, n_t = 0, blocks = 1;
+  int32_t per = 1;                  // rows per group
+  int32_t rounds = 1;               // 2: lists may overflow, overfull intervals are split again before the pick
   bool cluster = false;             // one cluster of `blocks` blocks per row
   bool small = false;               // one block per row, sorted whole
   int n_sms = 1;
   size_t off[13];
   size_t zero_bytes = 0, bytes = 0;
+  int32_t at_once() const { return std::max(1, (cluster ? 2 * n_sms : n_sms) / blocks); }   // rows that run at once
 };
-// beside: the caller's kernels share the device with other streams' (the server)
-inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int64_t cap, bool beside = false) {
+// per: 0 for all rows in one group.  beside: the caller's kernels share the device with other streams'
+// (the server).  A row in a cluster whose list overflows is picked from the row itself, without a
+// second round.
+inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int64_t cap, bool beside = false,
+                        int32_t per = 0) {
   SelPlan y;
   y.n = n;
   y.cap = cap;
   y.n_layers = n_layers;
   y.n_t = n_t;
+  y.per = per > 0 ? std::min(per, n_layers) : n_layers;
   y.small = n <= SEL_SMALL;
   y.n_sms = std::max(1, n_sms);
-  y.rounds = !y.small && cap < list_cap(n) ? 2 : 1;
-  const int64_t slots = 2ll * std::max(1, n_sms);           // blocks that run at once
-  y.cluster = !y.small && y.rounds == 1 && n <= (4 << 20) && (beside || n_layers > SEL_GRID_ROWS);
+  const int64_t slots = 2ll * y.n_sms;                      // blocks that run at once
+  y.cluster = !y.small && n <= (4 << 20) && (beside || n_layers > SEL_GRID_ROWS);
+  y.rounds = !y.small && !y.cluster && cap < list_cap(n) ? 2 : 1;
   if (y.cluster) {                                          // all rows' clusters at once, if they can be
     y.blocks = 16;
     while (y.blocks > 1 && ((int64_t)n_layers * y.blocks > slots || n < 2048ll * y.blocks)) y.blocks /= 2;
   } else if (!y.small) {
     y.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, std::max<int64_t>(1, n_sms / n_layers)));
   }
-  const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1), two = y.rounds > 1 ? lt : 0;
+  const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1);
+  const size_t G = (size_t)y.per, gt = G * (size_t)n_t, two = y.rounds > 1 ? gt : 0;   // of a group
   const size_t grid = y.small || y.cluster ? 0 : 1, lists = y.small ? 0 : 1;
   size_t b = 0;
   int i = 0;
   auto t = [&](size_t k) { b = (b + 15) / 16 * 16; y.off[i++] = b; b += k; };
-  t(4 * grid * L * SEL_CLASSES);
-  t(4 * grid * lt);
-  t(4 * grid * L);
   t(4);
+  t(4 * grid * G * SEL_CLASSES);
+  t(4 * grid * gt);
+  t(4 * grid * G);
   t(4 * two * SEL_CLASSES);
   t(4 * two);
   y.zero_bytes = (b + 15) / 16 * 16;
   t(sizeof(SelState) * lt);
-  t(8 * lists * lt * (size_t)cap);
-  t(8 * grid * lt * (size_t)y.blocks);
-  t(8 * grid * L * (size_t)y.blocks);
+  t(8 * lists * gt * (size_t)cap);
+  t(8 * grid * gt * (size_t)y.blocks);
+  t(8 * grid * G * (size_t)y.blocks);
   t(8 * (lt + L));
   t(8 * lt);
   t(8 * lt);
@@ -93,8 +102,29 @@ inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int
   return y;
 }
 
-// The rows of a request in groups whose scratch fits `limit` bytes each: groups of `per` rows (plan
-// `first`) and a last one of what is left (plan `last`).  Where even one row's lists do not fit, shorter
+// A request's plan within `limit` bytes: all rows in one group, else groups (whole waves of rows while
+// they hold one), else shorter lists; the smallest plan where nothing fits.  Lists hold 16 n / sample +
+// 4,096 keys for each row and target: 1,000 rows of 200,000 values with 16 targets take 2.1 GB at once (3.2
+// ms; in 4 groups of a wave, 650 MB, 3.6 ms; in 14 groups of a quarter of a wave 9.5).
+constexpr size_t SEL_SCRATCH = (size_t)4 << 30;
+inline SelPlan sel_plan_within(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, bool beside, size_t limit) {
+  int64_t cap = list_cap(n);
+  SelPlan y = sel_plan(n, n_layers, n_t, n_sms, cap, beside);
+  if (y.small) return y;                                    // no working parts to share
+  for (int32_t per = n_layers; y.bytes > limit && per > 1;) {
+    per = (per + 1) / 2;
+    if (per > y.at_once()) per -= per % y.at_once();
+    y = sel_plan(n, n_layers, n_t, n_sms, cap, beside, per);
+  }
+  while (y.bytes > limit && cap > SEL_SAMPLE) {
+    cap = std::max<int64_t>(cap / 2, SEL_SAMPLE);
+    y = sel_plan(n, n_layers, n_t, n_sms, cap, beside, 1);
+  }
+  return y;
+}
+
+// The rows of the allocation-free call, as requests of their own whose scratch fits `limit` bytes each (few
+// rows at a time get more blocks each): `per` rows (plan `first`) and a last one of what is left (`last`).  Where even one row's lists do not fit, shorter
 // lists and a second round.  The last group can need more than the others although it has fewer rows
 // (33 rows run as clusters, 32 as one cooperative launch with class counts), so both are checked.
 struct SelGroups {

@@ -85,3 +85,64 @@ def test_allocation_free_call_in_uneven_groups(n, rps, levels):
     """65 rows: a first group of 33 (a cluster each) would fit the array, its remainder of 32 (one cooperative
     launch, which needs class counts) would not."""
     check(rows(n, 65, n), rps, levels, ara.risk_metrics_static)
+
+
+@pytest.mark.parametrize("n_rows,n", [(40, 70_001), (6, 600_000), (1, 1_000_003), (300, 5_000)])
+def test_with_little_memory_the_same_bits(n_rows, n):
+    """With 8 KiB for each row and target (and for a single row the least that two rounds need), the rows
+    run in groups with short lists, in clusters or in the cooperative form: every result the same."""
+    import ctypes
+    d = torch.from_numpy(rows(n, n_rows, n)).cuda()
+    want = ara.risk_metrics(d, RPS, LEVELS, want_mean=True)
+    nt = len(RPS) + len(LEVELS)
+    out = [torch.full((n_rows, k), -1.0, dtype=torch.float64, device="cuda") for k in (len(RPS), len(LEVELS), 1)]
+    status = torch.full((1,), 9, dtype=torch.int32, device="cuda")
+    arr = lambda v: (ctypes.c_double * len(v))(*v)
+    for budget in (8192 * max(n_rows, 4) * nt, 8192 * max(n_rows // 4, 4) * nt):
+        for call in ("wait", "queue"):
+            ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, budget)
+            try:
+                if call == "wait":
+                    got = ara.risk_metrics(d, RPS, LEVELS, want_mean=True)
+                else:
+                    st = ara.lib().ara_risk_metrics_async(
+                        d.data_ptr(), n, n_rows, len(RPS), arr(RPS), len(LEVELS), arr(LEVELS), out[0].data_ptr(),
+                        out[1].data_ptr(), out[2].data_ptr(), status.data_ptr(), torch.cuda.current_stream().cuda_stream)
+                    assert st == ara.ARA_OK
+                    got = [o.cpu().numpy() for o in out]
+                    assert int(status) == 0
+            finally:
+                ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+            assert all(np.array_equal(a.reshape(b.shape), b) for a, b in zip(got, want))
+    # the row sum alone has no lists
+    ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 40_000 + 200 * n_rows)
+    try:
+        got = ara.risk_metrics(d, [], [], want_mean=True)
+    finally:
+        ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+    assert np.array_equal(got[2], want[2])
+
+
+def test_host_run_with_little_memory():
+    """The selection of a run from host memory keeps its scratch with the portfolio: the same metrics
+    where only short lists fit."""
+    g = np.random.default_rng(2)
+    n = 30_000
+    off = np.arange(n + 1, dtype=np.int64) * 4
+    ids = g.integers(0, 1000, 4 * n, dtype=np.int32)
+    made = lambda: ara.Portfolio(1000, [np.arange(1000, dtype=np.int32)], [np.exp(g2.normal(10, 1, 1000))], [0.0], [np.inf],
+                                 [[0]] * 3, [0.0] * 3, [1e9] * 3, [0.0, 1e4, 2e4], [1e12] * 3)
+    g2 = np.random.default_rng(3)
+    a = made()
+    want = a.run_ylt_host(off, ids, return_periods=RPS, tvar_levels=LEVELS, want_mean=True)
+    g2 = np.random.default_rng(3)
+    b = made()
+    # staging, offsets, rows and results, and 200 KB of the 1.2 MB of lists
+    ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 2 * (4 * ids.size + 8 * off.size) + 8 * 3 * n + 4096 + 200_000)
+    try:
+        got = b.run_ylt_host(off, ids, return_periods=RPS, tvar_levels=LEVELS, want_mean=True)
+    finally:
+        ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+    assert all(np.array_equal(x, y) for x, y in zip(got, want))
+    a.close()
+    b.close()
