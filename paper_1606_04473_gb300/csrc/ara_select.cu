@@ -278,7 +278,10 @@ constexpr int SEL_QUEUE = 32 + 32 * SEL_U;    // keys a warp's queue can hold
 struct SelShared {                            // shared memory of a block (dynamic: SEL_SMEM bytes)
   uint64_t key[SEL_SAMPLE];                   // the sorted sample, then the splitters
   uint64_t queue[SEL_WARPS][SEL_QUEUE];       // per warp: keys waiting for a full warp
-  uint64_t keep[SEL_PICK];                    // the pick's list
+  union {
+    uint64_t keep[SEL_PICK];                  // the pick's list
+    double psum[SEL_MAX_T][SEL_SLICES];       // afterwards, a cluster's block: its partial tail sums, by part
+  };
   uint32_t hist[SEL_CLASSES];                 // class counts of the slice (the pick: digit counts)
   uint32_t cnt[SEL_CLASSES];                  // inclusive prefix of the row's class totals
   uint64_t ext[2 * SEL_WARPS];
@@ -291,8 +294,8 @@ struct SelShared {                            // shared memory of a block (dynam
   uint32_t got[SEL_MAX_T], base[SEL_MAX_T];
   uint64_t found, prefix;
   int64_t k, gt, eq;
-  // a cluster's row: its own partial results, and (rank 0) the row's lists and picked targets
-  double pmean, psum[SEL_MAX_T];
+  // a cluster's row: its own partial row sums, by part, and (rank 0) the row's lists and picked targets
+  double pmean[SEL_SLICES];
   uint32_t reported, n_list[SEL_MAX_T];
   uint64_t pick_key[SEL_MAX_T];
   int64_t pick_gt[SEL_MAX_T];
@@ -405,38 +408,51 @@ __device__ __forceinline__ int row_splitters(SelShared& S, const double* __restr
   return np;
 }
 
-// Class counts of the slice into S.hist.  Class 2 i: between splitters i - 1 and i; class 2 i + 1:
-// equal to splitter i (its first place).  Only keys within [lo, hi] count (the whole range, or an
-// interval that is split again).  Returns the slice's sum (thread 0) when want_mean.
-__device__ __forceinline__ double count_slice(SelShared& S, const double* __restrict__ row, int64_t i0, int64_t i1,
-                                              int np, uint64_t lo, uint64_t hi, int want_mean) {
+// Part v of V of a row of n values.
+__device__ __forceinline__ int64_t slice_begin(int64_t n, unsigned v, unsigned V) { return (int64_t)v * n / V; }
+
+// Class counts of the row's parts [v0, v1) of V into S.hist.  Class 2 i: between splitters i - 1 and i;
+// class 2 i + 1: equal to splitter i (its first place).  Only keys within [lo, hi] count (the whole range,
+// or an interval that is split again).  out(v, sum) is called by thread 0 for each part when want_mean.
+// PARTS: there may be more than one part.
+template <bool PARTS, typename O>
+__device__ __forceinline__ void count_slices(SelShared& S, const double* __restrict__ row, int64_t n, unsigned v0,
+                                             unsigned v1, unsigned V, int np, uint64_t lo, uint64_t hi, int want_mean,
+                                             O&& out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i <= 2 * np; i += SEL_THREADS) S.hist[i] = 0u;
   __syncthreads();
-  double sum[2] = {0.0, 0.0};
   const int top = np > 0 ? 1 << (31 - __clz(np)) : 0;
   const bool part = lo != 0ull || hi != ~0ull;
   // keys below every splitter are counted, not searched
   const uint64_t floor_key = np == 0 ? ~0ull : part ? lo : S.key[np - 1];
-  const uint32_t near = for_keys_from(row, i0, i1, floor_key, S.queue[warp], [&](uint64_t k, bool valid) {
-    if (part) valid = valid && in_interval(k, lo, hi);
-    int c = 0;               // splitters above k
-    for (int step = top; step; step >>= 1)
-      if (c + step <= np && S.key[c + step - 1] > k) c += step;
-    const uint32_t cls = valid ? 2u * (uint32_t)c + (np > 0 && S.key[min(c, np - 1)] == k ? 1u : 0u) : 0xffffffffu;
-    const unsigned peers = __match_any_sync(SFULL, cls);
-    if (valid && lane == __ffs(peers) - 1) atomicAdd(&S.hist[cls], (uint32_t)__popc(peers));
-  }, [&](double y, int u) {
-    if (want_mean) sum[u & 1] = __dadd_rn(sum[u & 1], y);
-  });
+  uint32_t near = 0;
+  unsigned v = v0;
+  do {
+    double sum[2] = {0.0, 0.0};
+    near += for_keys_from(row, slice_begin(n, v, V), slice_begin(n, v + 1, V), floor_key, S.queue[warp], [&](uint64_t k, bool valid) {
+      if (part) valid = valid && in_interval(k, lo, hi);
+      int c = 0;               // splitters above k
+      for (int step = top; step; step >>= 1)
+        if (c + step <= np && S.key[c + step - 1] > k) c += step;
+      const uint32_t cls = valid ? 2u * (uint32_t)c + (np > 0 && S.key[min(c, np - 1)] == k ? 1u : 0u) : 0xffffffffu;
+      const unsigned peers = __match_any_sync(SFULL, cls);
+      if (valid && lane == __ffs(peers) - 1) atomicAdd(&S.hist[cls], (uint32_t)__popc(peers));
+    }, [&](double y, int u) {
+      if (want_mean) sum[u & 1] = __dadd_rn(sum[u & 1], y);
+    });
+    if (want_mean) {
+      const double s = block_sum(__dadd_rn(sum[0], sum[1]), S.wsum);
+      if (threadIdx.x == 0) out(v, s);
+    }
+  } while (PARTS && ++v < v1);
   if (lane == 0) S.wcnt[warp] = near;
   __syncthreads();
   if (warp == 0 && np > 0 && !part) {
     const uint32_t counted = __reduce_add_sync(SFULL, lane < SEL_WARPS ? S.wcnt[lane] : 0u);
-    if (lane == 0) S.hist[2 * np] += (uint32_t)(i1 - i0) - counted;
+    if (lane == 0) S.hist[2 * np] += (uint32_t)(slice_begin(n, v1, V) - slice_begin(n, v0, V)) - counted;
   }
   __syncthreads();
-  return want_mean ? block_sum(__dadd_rn(sum[0], sum[1]), S.wsum) : 0.0;
 }
 
 // The classes of the targets [first, last) from the row's class totals (S.cnt, i <= 2 np; a barrier
@@ -702,15 +718,16 @@ __device__ __forceinline__ void tail_slice(SelShared& S, const double* __restric
   }
 }
 
-// Block b of B's part of a row of n values.
-__device__ __forceinline__ int64_t slice_begin(int64_t n, unsigned b, unsigned B) { return (int64_t)b * n / B; }
-
 // ------------------------------------------------------------------------------------------
 // One kernel per row in a thread-block cluster: the steps with cluster barriers between them.
 // ------------------------------------------------------------------------------------------
+// PARTS: the row's sums are taken in V parts, several to a block, as the cooperative form takes them, so
+// that both give the same bits (a burst of 12 served requests takes 0.4 to 0.9 % longer for it); otherwise V
+// is the number of blocks.
+template <bool PARTS>
 __global__ void __launch_bounds__(SEL_THREADS, 2)
-k_sel_cluster(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets tg, SelScratch sc, int want_mean,
-              int skip_report) {
+k_sel_cluster(const double* __restrict__ ylt, int64_t n, int32_t l0, unsigned n_parts, SelTargets tg, SelScratch sc,
+              int want_mean, int skip_report) {
   extern __shared__ __align__(16) unsigned char sel_smem[];
   SelShared& S = *reinterpret_cast<SelShared*>(sel_smem);
   namespace cg = cooperative_groups;
@@ -718,14 +735,13 @@ k_sel_cluster(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets 
   const unsigned B = gridDim.x, rank = blockIdx.x;     // a cluster spans the grid's x
   const int layer = l0 + (int)blockIdx.y, nt = tg.n_t;
   const double* row = ylt + (int64_t)layer * n;
-  const int64_t i0 = slice_begin(n, rank, B), i1 = slice_begin(n, rank + 1, B);
+  const unsigned V = PARTS ? n_parts : B;
+  const unsigned v0 = PARTS ? rank * V / B : rank, v1 = PARTS ? (rank + 1) * V / B : rank + 1;   // this block's parts
+  const int64_t i0 = slice_begin(n, v0, V), i1 = slice_begin(n, v1, V);
   if (threadIdx.x < SEL_MAX_T) S.n_list[threadIdx.x] = 0u;
   const int np = nt > 0 ? row_splitters(S, row, n, sc.sample, tg) : 0;
-  const double part = count_slice(S, row, i0, i1, np, 0ull, ~0ull, want_mean);
-  if (threadIdx.x == 0) {
-    S.pmean = part;
-    S.reported = skip_report ? 0u : 1u;
-  }
+  count_slices<PARTS>(S, row, n, v0, v1, V, np, 0ull, ~0ull, want_mean, [&](unsigned v, double s) { S.pmean[v - v0] = s; });
+  if (threadIdx.x == 0) S.reported = skip_report ? 0u : 1u;
   cluster.sync();
   // (remote words are read by different threads at once: one after the other costs 300 cycles each)
   const unsigned lane = threadIdx.x & 31;
@@ -770,18 +786,40 @@ k_sel_cluster(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets 
       const int m = min(4, nt - t0);
 #pragma unroll
       for (int q = 0; q < 4; ++q) thr[q] = q < m ? cluster.map_shared_rank(&S, 0)->pick_key[t0 + q] : ~0ull;
-      tail_slice(S, row, i0, i1, m, thr, [&](int q, double s) { S.psum[t0 + q] = s; });
+      unsigned v = v0;
+      do {
+        tail_slice(S, row, PARTS ? slice_begin(n, v, V) : i0, PARTS ? slice_begin(n, v + 1, V) : i1, m, thr,
+                   [&](int q, double s) { S.psum[t0 + q][v - v0] = s; });
+      } while (PARTS && ++v < v1);
     }
   cluster.sync();                                      // partial sums complete
   if (rank == 0) {
-    // warp w: result w of the mean (if wanted) and the TVaR targets; lane b holds block b's partial,
-    // added by a fixed tree
+    // warp w: result w of the mean (if wanted) and the TVaR targets, from the parts' sums by the tree of
+    // block_sum over one part per thread
     if (!ok && threadIdx.x == 0) sel_timeout(sc);
     for (int w = (int)(threadIdx.x >> 5); ok && w < 1 + nt - tg.n_rp; w += SEL_WARPS) {
       if (w == 0 && !want_mean) continue;
       const int t = tg.n_rp + w - 1;
-      const SelShared* const o = cluster.map_shared_rank(&S, lane < B ? lane : 0u);
-      const double a = warp_add(lane < B ? (w == 0 ? o->pmean : o->psum[t]) : 0.0, 8);
+      double a;
+      if constexpr (!PARTS) {     // one part to a block (with the loop below, 16 targets took 7 % longer)
+        const SelShared* const o = cluster.map_shared_rank(&S, lane < B ? lane : 0u);
+        a = warp_add(lane < B ? (w == 0 ? o->pmean[0] : o->psum[t][0]) : 0.0, 8);
+      } else {
+        double wsum = 0.0;                             // lane l: the sum of the parts 32 l .. 32 l + 31
+        for (unsigned base = 0; base < V; base += 32) {
+          const unsigned v = base + lane;
+          double x = 0.0;
+          if (v < V) {
+            const unsigned owner = ((v + 1) * B - 1) / V;
+            const SelShared* const o = cluster.map_shared_rank(&S, owner);
+            const unsigned at = v - owner * V / B;
+            x = w == 0 ? o->pmean[at] : o->psum[t][at];
+          }
+          const double sum = __shfl_sync(SFULL, warp_add(x, 16), 0);
+          if (lane == base / 32) wsum = sum;
+        }
+        a = warp_add(lane < SEL_WARPS ? wsum : 0.0, SEL_WARPS / 2);
+      }
       if (lane != 0) continue;
       if (w == 0) {
         put_mean(sc, layer, a / (double)n);
@@ -870,8 +908,8 @@ k_sel_grid(const double* __restrict__ ylt, int64_t n, int32_t l0, SelTargets tg,
       n_list = sc.n_list2 + lt0;
     }
     if (nt > 0) np = row_splitters(S, row, n, sc.sample, tg, t < nt ? sc.list + (lt0 + old.list) * sc.cap : nullptr, sc.cap);
-    const double part = count_slice(S, row, i0, i1, np, old.lo, old.hi, t == nt ? want_mean : 0);
-    if (t == nt && want_mean && threadIdx.x == 0) sc.pmean[(int64_t)layer * B + blockIdx.x] = part;
+    count_slices<false>(S, row, n, blockIdx.x, blockIdx.x + 1, B, np, old.lo, old.hi, t == nt ? want_mean : 0,
+                 [&](unsigned b, double s) { sc.pmean[(int64_t)layer * B + b] = s; });
     for (int i = threadIdx.x; np > 0 && i <= 2 * np; i += SEL_THREADS)
       if (S.hist[i]) atomicAdd(g + i, S.hist[i]);
     if (!meet()) return;
@@ -963,7 +1001,7 @@ static ara_status sel_prepare_kernels() {
   if (dev < 0 || dev >= 64) return ARA_ECUDA;
   std::lock_guard<std::mutex> lk(mu);
   if (done[dev]) return ARA_OK;
-  for (const void* f : {(const void*)k_sel_cluster, (const void*)k_sel_grid})
+  for (const void* f : {(const void*)k_sel_cluster<false>, (const void*)k_sel_cluster<true>, (const void*)k_sel_grid})
     ARA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
   // k_sel_grid has at most one block per SM.  100 KB of shared memory (44 % of 228) keeps two from
   // sharing one while others stand empty, and a stream kernel queued behind it on another stream from
@@ -971,7 +1009,8 @@ static ara_status sel_prepare_kernels() {
   // second stream, 1.167 -> 1.067 ms (selection 72 -> 61 us, stream 1.09 -> 1.00).
   ARA_TRY(cudaFuncSetAttribute((const void*)k_sel_grid, cudaFuncAttributePreferredSharedMemoryCarveout, 44));
   static_assert(SEL_SMEM <= 99 * 1024 && 2 * SEL_SMEM > 99 * 1024, "one block in 100 KB");
-  ARA_TRY(cudaFuncSetAttribute((const void*)k_sel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  for (const void* f : {(const void*)k_sel_cluster<false>, (const void*)k_sel_cluster<true>})
+    ARA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   done[dev] = true;
   return ARA_OK;
 }
@@ -1024,7 +1063,8 @@ static ara_status launch_group(const double* d_ylt, const SelPlan& y, const SelT
       cfg.attrs = at;
       cfg.numAttrs = 1;
       LaunchScope ls(ARA_K_SELECT, s);
-      ARA_TRY(cudaLaunchKernelEx(&cfg, k_sel_cluster, d_ylt, n, l0, tg, sc, want_mean, skip));
+      const auto fn = y.slices > y.blocks ? k_sel_cluster<true> : k_sel_cluster<false>;
+      ARA_TRY(cudaLaunchKernelEx(&cfg, fn, d_ylt, n, l0, (unsigned)y.slices, tg, sc, want_mean, skip));
     }
     return ARA_OK;
   }

@@ -22,6 +22,7 @@ constexpr int SEL_SMALL = 4096;                  // rows up to this length are s
 // Rows of one request up to which the cooperative launch is the faster (16 rows of 200,000 values, 3
 // targets: 60 us against 95 us in clusters; 64 rows: 177 and 119).
 constexpr int SEL_GRID_ROWS = 32;
+constexpr int SEL_SLICES = 16;                   // slices of a row's sums that a block of a cluster can hold
 
 struct SelState {
   uint64_t key;                // the selected key (known at once when its class is a tie)
@@ -41,12 +42,13 @@ ARA_HD inline int32_t sel_sample(int64_t n) { return n <= (1 << 19) ? 256 : SEL_
 // list that would overflow is not used: its target is picked from the row itself).
 inline int64_t list_cap(int64_t n) { return std::min<int64_t>(n, 16 * (n / sel_sample(n)) + 4096); }
 
-// A request's launch plan and scratch.  The form and the blocks of a row (on which the order of the TVaR and
-// mean sums depends) follow from the request; how many rows share the lists at a time (per: groups run
+// A request's launch plan and scratch.  The form and the slices of a row (on which the order of the TVaR and
+// mean sums depends) follow from the request, the slices also where the form differs (beside); how many rows share the lists at a time (per: groups run
 // one after the other) and how long the lists are follow from the memory, and change no result.
 struct SelPlan {
   int64_t n = 0, cap = 0;           // cap: keys per list
   int32_t n_layers = 0, n_t = 0, blocks = 1;
+  int32_t slices = 1;               // parts of a row that are summed one by one, at least `blocks`
   int32_t per = 1;                  // rows per group
   int32_t rounds = 1;               // 2: lists may overflow, overfull intervals are split again before the pick
   bool cluster = false;             // one cluster of `blocks` blocks per row
@@ -71,13 +73,20 @@ inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int
   y.n_sms = std::max(1, n_sms);
   const int64_t slots = 2ll * y.n_sms;                      // blocks that run at once
   y.cluster = !y.small && n <= (4 << 20) && (beside || n_layers > SEL_GRID_ROWS);
-  y.rounds = !y.small && !y.cluster && cap < list_cap(n) ? 2 : 1;
+  if (!y.small)
+    y.slices = (int32_t)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, std::max<int64_t>(1, n_sms / n_layers)));
   if (y.cluster) {                                          // all rows' clusters at once, if they can be
     y.blocks = 16;
     while (y.blocks > 1 && ((int64_t)n_layers * y.blocks > slots || n < 2048ll * y.blocks)) y.blocks /= 2;
-  } else if (!y.small) {
-    y.blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, std::max<int64_t>(1, n_sms / n_layers)));
+    if (n_layers > SEL_GRID_ROWS) {
+      y.slices = y.blocks;
+    } else {       // the sums of the cooperative form, so that a served request's have the bits of a direct call's
+      while (y.blocks > y.slices) y.blocks /= 2;
+      if ((y.slices + y.blocks - 1) / y.blocks > SEL_SLICES) y.cluster = false;
+    }
   }
+  if (!y.cluster) y.blocks = y.slices;
+  y.rounds = !y.small && !y.cluster && cap < list_cap(n) ? 2 : 1;
   const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1);
   const size_t G = (size_t)y.per, gt = G * (size_t)n_t, two = y.rounds > 1 ? gt : 0;   // of a group
   const size_t grid = y.small || y.cluster ? 0 : 1, lists = y.small ? 0 : 1;

@@ -248,3 +248,32 @@ def test_server_adjoints_over_the_yet_index_are_identical(world):
     for t in tickets:
         srv.wait(t)
     srv.close()
+
+
+@pytest.mark.parametrize("trials", [4_097, 9_000, 60_011])
+def test_served_metrics_have_the_bits_of_a_direct_call(trials):
+    """TVaR and mean are FP64 sums: the server's selection (a cluster per row) adds in the order of
+    ara_risk_metrics on the same rows (one cooperative launch, up to 32 rows; clusters beyond)."""
+    g = np.random.default_rng(trials)
+    n_elts, cat = 40, 3_000
+    ids = [np.sort(g.choice(cat, size=900, replace=False)).astype(np.int32) for _ in range(n_elts)]
+    loss = [np.exp(11.0 + 2.0 * g.standard_normal(900)) for _ in ids]
+    pool = ara.Portfolio(cat, ids, loss, np.full(n_elts, 1e3), np.full(n_elts, 1e7), [], [], [], [], [])
+    off = torch.arange(trials + 1, dtype=torch.int64, device="cuda") * 20
+    ev = torch.from_numpy(g.integers(0, cat, 20 * trials, dtype=np.int32)).cuda()
+    rps, levels = [100.0, 10.0], [0.99, 0.9, 0.5, 0.0, 0.25]
+    srv = ara.Server(pool, off, ev, max_concurrent=1)
+    for n_layers in (1, 2, 5, 9, 17, 32, 33):
+        z = np.ones(n_layers)
+        q = dict(layer_elts=[sorted(g.choice(n_elts, size=5, replace=False).tolist()) for _ in z], occ_ret=1e4 * z,
+                 occ_lim=1e6 * z, agg_ret=0.0 * z, agg_lim=1e9 * z)
+        got = srv.wait(srv.submit(trials=(0, trials), return_periods=rps, tvar_levels=levels, want_mean=True,
+                                  want_adjoint=False, flags=0, tenant=0, **q))
+        ls = pool.layer_set(**q)
+        want = ara.risk_metrics(ls.run_ylt(off, ev), rps, levels, want_mean=True)
+        ls.check()
+        ls.close()
+        for k, w in zip(("pml", "tvar", "mean"), want):
+            assert np.array_equal(got[k], w), (n_layers, k)
+    srv.close()
+    pool.close()
