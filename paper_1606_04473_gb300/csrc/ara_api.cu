@@ -86,16 +86,39 @@ void timing_add_host(int k, double ms) {
   g_count[k] += 1;
 }
 
+uint64_t context_id() {
+  using Fn = CUresult (*)(CUcontext, unsigned long long*);
+  static const Fn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return (Fn)f;
+  }();
+  unsigned long long id = 0;
+  int dev = 0;
+  if (!fn) return 0;
+  if (fn(nullptr, &id) == CUDA_SUCCESS) return id;
+  // this thread has no context yet
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return 0;
+  return fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
 namespace {
 constexpr int kMaxPoolDevices = 64;
 std::mutex g_pool_mu;
-cudaMemPool_t g_pools[kMaxPoolDevices];
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  uint64_t ctx = 0;                 // the context it was made in
+} g_pools[kMaxPoolDevices];
 }  // namespace
 
 static cudaMemPool_t library_pool(int dev) {
   if (dev < 0 || dev >= kMaxPoolDevices) return nullptr;
+  const uint64_t ctx = context_id();
   std::lock_guard<std::mutex> lk(g_pool_mu);
-  if (!g_pools[dev]) {
+  if (!g_pools[dev].pool || g_pools[dev].ctx != ctx) {
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
     props.allocType = cudaMemAllocationTypePinned;
@@ -109,9 +132,10 @@ static cudaMemPool_t library_pool(int dev) {
     }
     uint64_t keep = UINT64_MAX;   // keep freed memory until ara_release_memory
     cudaMemPoolSetAttribute(mp, cudaMemPoolAttrReleaseThreshold, &keep);
-    g_pools[dev] = mp;
+    g_pools[dev].pool = mp;
+    g_pools[dev].ctx = ctx;
   }
-  return g_pools[dev];
+  return g_pools[dev].pool;
 }
 
 static std::atomic<int64_t> g_budget{-1};   // bytes left; -1: no limit
@@ -139,18 +163,29 @@ cudaError_t dmalloc_async(void** ptr, size_t bytes, cudaStream_t s) {
 
 namespace {
 constexpr int kMaxPinnedSlots = 64;
+struct PinnedBlock {
+  void* p;
+  uint64_t ctx;                     // the context it was made in: gone when its device has another
+  int dev;
+};
 std::mutex g_pin_mu;
-std::vector<void*> g_pin_idle;
+std::vector<PinnedBlock> g_pin_idle;
 int g_pin_total = 0;
 }  // namespace
 
-PinnedSlot::PinnedSlot() : p(nullptr) {
+PinnedSlot::PinnedSlot() : p(nullptr), ctx(context_id()), dev(0) {
+  if (ctx == 0 || cudaGetDevice(&dev) != cudaSuccess) return;
   {
     std::lock_guard<std::mutex> lk(g_pin_mu);
-    if (!g_pin_idle.empty()) {
-      p = g_pin_idle.back();
-      g_pin_idle.pop_back();
-      return;
+    for (size_t i = g_pin_idle.size(); i-- > 0;) {
+      const PinnedBlock b = g_pin_idle[i];
+      if (b.dev != dev) continue;
+      g_pin_idle.erase(g_pin_idle.begin() + (ptrdiff_t)i);
+      if (b.ctx == ctx) {
+        p = b.p;
+        return;
+      }
+      --g_pin_total;
     }
     if (g_pin_total >= kMaxPinnedSlots) return;
     ++g_pin_total;
@@ -166,7 +201,7 @@ PinnedSlot::PinnedSlot() : p(nullptr) {
 PinnedSlot::~PinnedSlot() {
   if (!p) return;
   std::lock_guard<std::mutex> lk(g_pin_mu);
-  g_pin_idle.push_back(p);
+  g_pin_idle.push_back(PinnedBlock{p, ctx, dev});
 }
 
 int64_t pool_idle_bytes(int dev) {
@@ -174,7 +209,7 @@ int64_t pool_idle_bytes(int dev) {
   cudaMemPool_t mp;
   {
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    mp = g_pools[dev];
+    mp = g_pools[dev].pool;
   }
   if (!mp) return 0;
   uint64_t reserved = 0, used = 0;
@@ -359,16 +394,24 @@ ara_status ara_set_stream_shape(int32_t index) {
 }
 
 ara_status ara_release_memory(void) {
+  std::vector<PinnedBlock> idle;
   {
     std::lock_guard<std::mutex> lk(g_pin_mu);
-    for (void* q : g_pin_idle) cudaFreeHost(q);
-    g_pin_total -= (int)g_pin_idle.size();
-    g_pin_idle.clear();
+    idle.swap(g_pin_idle);
+    g_pin_total -= (int)idle.size();
+  }
+  for (const PinnedBlock& b : idle) {
+    DeviceGuard g(b.dev);
+    if (context_id() == b.ctx) cudaFreeHost(b.p);
   }
   std::lock_guard<std::mutex> lk(g_pool_mu);
   ara_status st = ARA_OK;
-  for (int d = 0; d < kMaxPoolDevices; ++d)
-    if (g_pools[d] && cudaMemPoolTrimTo(g_pools[d], 0) != cudaSuccess) st = ARA_ECUDA;
+  for (int d = 0; d < kMaxPoolDevices; ++d) {
+    if (!g_pools[d].pool) continue;
+    DeviceGuard g(d);
+    if (context_id() != g_pools[d].ctx) g_pools[d].pool = nullptr;
+    else if (cudaMemPoolTrimTo(g_pools[d].pool, 0) != cudaSuccess) st = ARA_ECUDA;
+  }
   return st;
 }
 

@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libara.so.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -38,6 +39,10 @@ template <typename T>
 cudaError_t dmalloc(T** ptr, size_t bytes) {
   return take_budget(bytes) ? cudaMalloc((void**)ptr, bytes) : cudaErrorMemoryAllocation;
 }
+// The current device's context: an ID that no other context of the process gets, also after
+// cudaDeviceReset (0: unknown).  What the library keeps for the life of the process and the context
+// owns (memory pools, pinned blocks, function attributes) is kept with it and made again in another.
+uint64_t context_id();
 // A small block of pinned host memory, mapped into the device's address space, for the results of a
 // synchronous call: kernels write into it or one copy fills it without staging, where a copy to
 // pageable memory costs the call about 10 us each.  From a bounded list shared by all threads (p is
@@ -45,6 +50,8 @@ cudaError_t dmalloc(T** ptr, size_t bytes) {
 struct PinnedSlot {
   static constexpr size_t kBytes = 16384;
   void* p;
+  uint64_t ctx;
+  int dev;
   PinnedSlot();
   ~PinnedSlot();
   PinnedSlot(const PinnedSlot&) = delete;

@@ -992,15 +992,16 @@ ara_status validate_metrics(int64_t n, int32_t n_rp, const double* rps, int32_t 
   return select_targets(n, n_rp, rps, n_tvar, levels, tg);
 }
 
-// Shared-memory and cluster attributes of the kernels, set once per device.
+// Shared-memory and cluster attributes of the kernels, set once per context.
 static ara_status sel_prepare_kernels() {
   static std::mutex mu;
-  static bool done[64] = {false};
+  static uint64_t done[64] = {0};
   int dev = 0;
   ARA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return ARA_ECUDA;
+  const uint64_t ctx = context_id();
   std::lock_guard<std::mutex> lk(mu);
-  if (done[dev]) return ARA_OK;
+  if (ctx != 0 && done[dev] == ctx) return ARA_OK;
   for (const void* f : {(const void*)k_sel_cluster<false>, (const void*)k_sel_cluster<true>, (const void*)k_sel_grid})
     ARA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
   // k_sel_grid has at most one block per SM.  100 KB of shared memory (44 % of 228) keeps two from
@@ -1011,7 +1012,7 @@ static ara_status sel_prepare_kernels() {
   static_assert(SEL_SMEM <= 99 * 1024 && 2 * SEL_SMEM > 99 * 1024, "one block in 100 KB");
   for (const void* f : {(const void*)k_sel_cluster<false>, (const void*)k_sel_cluster<true>})
     ARA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  done[dev] = true;
+  done[dev] = ctx;
   return ARA_OK;
 }
 
