@@ -838,7 +838,12 @@ static ara_status run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_
   a.flags = flags;
   if (flags & ARA_RUN_BATCHED) return run_batched_async(*pf, a, s);
   if (rows) {
+    // Scratch is not taken from a pool while any thread captures in the global mode, unless this thread says
+    // that its calls have nothing to do with that capture: `s` is not captured.
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    ARA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
     st = run_batched_async(*pf, a, s, true);
+    ARA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
     if (st == ARA_OK) {
       pf->fold0_missing.resize((size_t)pf->n_layers, 0);
       for (int32_t l : sel) pf->fold0_missing[(size_t)l] = 1;

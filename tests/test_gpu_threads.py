@@ -97,6 +97,52 @@ def test_two_portfolios_from_two_threads(kind, a, b):
     assert not failed
 
 
+@pytest.mark.parametrize("where", ["another thread", "the capturing thread"])
+def test_an_ordinary_run_beside_a_capture(where):
+    """A run of several layers (by rows, with scratch from the pool) on a stream of its own neither fails nor
+    spoils the capture that is going on in the process, in any mode."""
+    w = world(5, 20_000, 16, 900, 16)
+    pf, off, ids = w
+    side, s = torch.cuda.Stream(), torch.cuda.Stream()
+    want = run(w, None, "plain")
+    out = torch.zeros_like(want)
+    x = torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    ara.lib().ara_release_memory()
+    for mode in ("global", "thread_local", "relaxed"):
+        out.zero_()
+        torch.cuda.synchronize()
+        graph, failed = torch.cuda.CUDAGraph(), []
+
+        def work():
+            try:
+                n0 = ara.launch_count()
+                pf.run_ylt(off, ids, out=out, stream=side)
+                if ara.launch_count() - n0 > 3:
+                    failed.append("not by rows")
+            except ara.AraError as e:
+                failed.append(str(e))
+
+        with torch.cuda.graph(graph, stream=s, capture_error_mode=mode):
+            x += 1
+            if where == "another thread":
+                t = threading.Thread(target=work)
+                t.start()
+                t.join()
+            else:
+                work()
+            x += 1
+        assert not failed
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        x.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert bool((x == 2).all())
+    pf.check()
+    pf.close()
+
+
 def test_a_wide_plan_outlives_the_making_of_a_narrow_one():
     wide, narrow = world(3, 20_000, 16, 900, 16), world(4, 20_000, 3, 4_500, 3)
     want = run(wide, None, "plain")
