@@ -18,7 +18,7 @@
 #include <atomic>
 #include <vector>
 
-#include "ara_internal.cuh"
+#include "ara_device.cuh"
 
 namespace ara {
 
@@ -36,11 +36,6 @@ struct AdjCounts {          // per layer
 struct SlotCounts {          // per ELT slot
   unsigned long long rl[2][3];    // [R (interior) / L (above)][mean, gt, eq]
 };
-
-__device__ __forceinline__ uint64_t adj_key(double y) {
-  const uint64_t b = (uint64_t)__double_as_longlong(y);
-  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
 
 template <typename T>
 __device__ __forceinline__ T warp_sum_int(T v) {
@@ -141,7 +136,7 @@ __global__ void __launch_bounds__(1024, 1) k_adj_hist(AdjHistParams p) {
     const uint8_t rg = tl < p.n_trials ? p.regimes[tl] : 0;
     bool above = false, equal = false;
     if (rg != 0) {
-      const uint64_t key = adj_key(p.ylt[tl]);
+      const uint64_t key = key_of(p.ylt[tl]);
       above = key > thr;
       equal = key == thr;
     }
@@ -434,7 +429,7 @@ k_adjb_class(int64_t n_trials, int32_t n_sel, const uint8_t* __restrict__ regime
     const uint8_t rg = rg_row[t];
     uint8_t c = 0;
     if (rg != 0) {
-      const uint64_t key = adj_key(y_row[t]);
+      const uint64_t key = key_of(y_row[t]);
       const bool above = key > thr, equal = key == thr;
       const int o = rg == 1 ? 0 : 3;
       v[o] += 1;

@@ -72,6 +72,18 @@ __device__ __forceinline__ uint64_t fixed_rn(double o, int fb) {
   return q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull);
 }
 
+// Order-preserving map of an IEEE double to an unsigned 64-bit key (total order: a NaN above +inf or below
+// -inf, by its sign).  Flipped bits, by a mask that depends on the sign: setting and clearing the sign bit
+// of a double becomes a floating-point operation, which does not keep a NaN's bits.
+__device__ __forceinline__ uint64_t key_of(double y) {
+  const long long b = __double_as_longlong(y);
+  return (uint64_t)(b ^ ((b >> 63) | (long long)0x8000000000000000ull));
+}
+__device__ __forceinline__ double value_of(uint64_t k) {
+  const long long b = (long long)k;
+  return __longlong_as_double(b ^ ((~b >> 63) | (long long)0x8000000000000000ull));
+}
+
 struct U128 {
   uint64_t lo, hi;
 };

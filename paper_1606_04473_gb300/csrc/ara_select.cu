@@ -32,7 +32,7 @@
 
 #include <cooperative_groups.h>
 
-#include "ara_internal.cuh"
+#include "ara_device.cuh"
 #include "ara_select_plan.h"
 
 namespace ara {
@@ -99,16 +99,6 @@ static SelScratch carve(void* base, const SelPlan& y) {
   s.cap = y.cap;
   s.sample = sel_sample(y.n);
   return s;
-}
-
-// Order-preserving map of an IEEE double to an unsigned 64-bit key (total order).
-__device__ __forceinline__ uint64_t key_of(double y) {
-  const uint64_t b = (uint64_t)__double_as_longlong(y);
-  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double value_of(uint64_t k) {
-  const uint64_t b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
-  return __longlong_as_double((long long)b);
 }
 
 // Bitonic sort of m shared-memory keys (a power of two: 512 E, or for E = 2 any from 64), descending,

@@ -146,3 +146,45 @@ def test_host_run_with_little_memory():
     assert all(np.array_equal(x, y) for x, y in zip(got, want))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n_rows,n", [(6, 1000), (6, 9_001), (40, 9_001), (6, 600_000)])
+def test_special_values(n_rows, n):
+    """Infinities, NaN, zeros of both signs and the type's extremes: in the order of the bits (a NaN above
+    +inf or below -inf, by its sign); sums as IEEE gives them."""
+    g = np.random.default_rng(n)
+    big = np.finfo(np.float64).max
+    special = np.array([np.inf, -np.inf, np.nan, -np.nan, 0.0, -0.0, big, -big, 5e-324, -5e-324])
+    special = np.append(special, np.frombuffer(b"\xff" * 8 + b"\xff" * 7 + b"\x7f", dtype=np.float64))
+    y = g.lognormal(3.0, 2.0, (n_rows, n))
+    for i in range(n_rows):
+        k = i % 6
+        if k == 0:
+            y[i, g.choice(n, 40, replace=False)] = np.inf
+        elif k == 1:
+            y[i, g.choice(n, n // 3, replace=False)] = -np.inf
+        elif k == 2:
+            y[i, g.choice(n, n // 2, replace=False)] = np.nan
+        elif k == 3:
+            y[i] = special[g.integers(0, special.size, n)]
+        elif k == 4:
+            y[i] = np.where(g.random(n) < 0.5, 0.0, -0.0)
+        else:
+            y[i] = np.inf
+    levels = [p for p in LEVELS if count(n * (1.0 - p)) >= 1]
+    pml, tvar, mean = ara.risk_metrics(torch.from_numpy(y).cuda(), RPS, levels, want_mean=True)
+    b = y.view(np.uint64)
+    key = np.where(b >> np.uint64(63), ~b, b | np.uint64(1 << 63))
+    order = np.argsort(key, axis=1)[:, ::-1]
+    s = np.take_along_axis(y, order, axis=1)
+    same = lambda x, w: np.array_equal(x.view(np.uint64), w.view(np.uint64))
+    with np.errstate(all="ignore"):
+        for i, r in enumerate(RPS):
+            assert same(np.ascontiguousarray(pml[:, i]), np.ascontiguousarray(s[:, count(n / r) - 1]))
+        for i, p in enumerate(levels):
+            m = count(n * (1.0 - p))
+            want = s[:, :m].astype(np.longdouble).sum(1) / m
+            rows = [r for r in range(n_rows) if r % 6 != 3]      # sums near the largest double may overflow on the way
+            np.testing.assert_allclose(tvar[rows, i], want[rows].astype(np.float64), rtol=1e-13)
+        want = (y.astype(np.longdouble).sum(1) / n).astype(np.float64)
+        np.testing.assert_allclose(mean[rows], want[rows], rtol=1e-13)
