@@ -70,3 +70,46 @@ def test_longest_yets_count_single_entries():
     b = pf.adjoint(off, longest, ylt, reg, 0.98)
     assert all(torch.equal(a[k], b[k]) for k in ("elt", "layer", "loss")) and np.array_equal(a["ties"], b["ties"])
     pf.close()
+
+
+@pytest.mark.parametrize("ascending", [True, False])
+def test_with_less_memory_single_entries(ascending):
+    """Without room for rows of whole pairs (13 bytes for each event more) the histogram counts single
+    entries, from the folds: the same gradients down to the least memory the call runs in."""
+    g = np.random.default_rng(9)
+    C, n_elts, trials, n_layers = 60_000, 12, 700, 6
+    ids = [g.choice(C, size=20_000, replace=False).astype(np.int32) for _ in range(n_elts)]
+    loss = [np.exp(11.0 + 2.0 * g.standard_normal(20_000)) for _ in ids]
+    layers = [sorted(g.choice(n_elts, size=4, replace=False).tolist(), reverse=not ascending) for _ in range(n_layers)]
+    z = np.zeros(n_layers)
+    pf = ara.Portfolio(C, ids, loss, np.full(n_elts, 1e4), np.full(n_elts, 1.5e6), layers, z + 1e4, z + 2e6, z + 1e5,
+                       z + 1e13)
+    off = torch.arange(trials + 1, dtype=torch.int64, device="cuda") * 200
+    ev = torch.from_numpy(g.integers(0, C, trials * 200, dtype=np.int32)).cuda()
+    reg = torch.empty((n_layers, trials), dtype=torch.uint8, device="cuda")
+    ylt = pf.run_ylt(off, ev, regimes=reg)
+    want = pf.adjoint(off, ev, ylt, reg, 0.98)
+
+    def within(budget):
+        ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, budget)
+        try:
+            return pf.adjoint(off, ev, ylt, reg, 0.98)
+        except ara.AraError as e:
+            assert e.status == ara.ARA_ENOMEM
+            return None
+        finally:
+            ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+
+    lo, hi = 1, 64 << 20                       # the least budget, to 1 KB
+    while hi - lo > 1024:
+        mid = (lo + hi) // 2
+        got = within(mid)
+        if got is None:
+            lo = mid
+        else:
+            hi = mid
+            assert all(torch.equal(got[k], want[k]) for k in ("elt", "layer", "loss"))
+            assert np.array_equal(got["ties"], want["ties"])
+    entries = sum(20_000 * len(l) for l in layers)
+    assert hi < 13 * (entries + C) + n_layers * C + 12 * C + (2 << 20)
+    pf.close()
