@@ -202,8 +202,8 @@ k_fold(int64_t catalogue, const int64_t* __restrict__ tile_rec, int64_t n_tiles,
 // in the tile; the tile is written coalesced.  The listed events fill whole warps, which matters
 // because an FP64 instruction costs 16 clocks of the SM's pipe however few lanes need it.
 // Bound by its chain of dependent loads (record range, record, terms).  Measured (us, by tiles of the
-// records of every ELT in turn / this): 30 ELTs x 10,000 records over 200,000 events, FP64: 71 / 16;
-// 15 x 20,000 over 1 M, FP64: 22 / 13, over 2 M, FP32: 17 / 18; 4 x 1,000 over 10,000: 19 / 5.
+// records of every ELT in turn / this): 30 ELTs x 10,000 records over 200,000 events, FP64: 71 / 12;
+// 15 x 20,000 over 1 M, FP64: 22 / 13, over 2 M, FP32: 17 / 18; 4 x 1,000 over 10,000: 19 / 4.4.
 // ------------------------------------------------------------------------------------------
 struct FoldByEvent {
   int64_t catalogue;
@@ -285,14 +285,21 @@ k_fold_events(FoldByEvent p, SelList sel, FoldOut out) {
   }
 }
 
+// Tiles of 256 events while those of a layer run at once (6 blocks per SM): a block's time is its longest
+// events', and small tiles spread them.  Beyond, tiles of 512, or of 1,024 where less than a third of the
+// events have a record and listing them is most of the work.  Measured (us a layer, FP64, tiles of 256 / 512 /
+// 1,024 / 2,048 events), 1.5 records per event: 199,000 events 8.9 / 9.2 / 12.4 / 18.2, 400,000 14.0 / 15.9 / 15.9 /
+// 21.4, 1 M 29.0 / 30.8 / 35.2 / 36.4, 1 M and 4 layers 103.8 / 102.0 / 106.5 / 121.5; 0.5: 1 M 14.4 / 12.4 / 14.1;
+// 0.25: 199,000 4.1 / 4.4 / 4.7 / 5.9, 250,000 5.8 / 4.7 / 4.7 / 6.2, 1 M 12.0 / 10.5 / 9.5 / 9.5.
 template <typename LossT>
-static void launch_fold_events(const FoldByEvent& p, const SelList& sl, const FoldOut& out, cudaStream_t s) {
-  const int64_t C = p.catalogue;
+static void launch_fold_events(const FoldByEvent& p, const SelList& sl, const FoldOut& out, int64_t n_records,
+                               int n_sms, cudaStream_t s) {
+  const int64_t C = p.catalogue, at_once = 6ll * n_sms;
   auto grid = [&](int T) { return dim3((unsigned)((C + T - 1) / T), sl.n); };
-  // small catalogues in small tiles, so that every SM has some
-  if (C >= 1000000) k_fold_events<LossT, 2048><<<grid(2048), FOLDE_THREADS, 0, s>>>(p, sl, out);
-  else if (C >= 200000) k_fold_events<LossT, 1024><<<grid(1024), FOLDE_THREADS, 0, s>>>(p, sl, out);
-  else k_fold_events<LossT, 256><<<grid(256), FOLDE_THREADS, 0, s>>>(p, sl, out);
+  if (C <= 256 * at_once) k_fold_events<LossT, 256><<<grid(256), FOLDE_THREADS, 0, s>>>(p, sl, out);
+  else if (C <= 512 * at_once || 3 * n_records >= C)
+    k_fold_events<LossT, 512><<<grid(512), FOLDE_THREADS, 0, s>>>(p, sl, out);
+  else k_fold_events<LossT, 1024><<<grid(1024), FOLDE_THREADS, 0, s>>>(p, sl, out);
 }
 
 // Whether these layers fold from the event-major records: ascending ELT lists, their records at
@@ -995,8 +1002,8 @@ ara_status launch_fold_to(Portfolio& pf, int32_t n_sel, const int32_t* sel_host,
       }
       const FoldByEvent p{pf.catalogue, pf.d_ev_ptr, pf.d_ev_elt, pf.d_ev_loss, all ? nullptr : pf.d_mem,
                           pf.d_elt_ret, pf.d_elt_lim, pf.d_layers};
-      if (pf.d_rec_loss32) launch_fold_events<float>(p, sl, ob, s);
-      else launch_fold_events<double>(p, sl, ob, s);
+      if (pf.d_rec_loss32) launch_fold_events<float>(p, sl, ob, pf.n_records, pf.n_sms, s);
+      else launch_fold_events<double>(p, sl, ob, pf.n_records, pf.n_sms, s);
     } else if (pf.d_rec_loss32)
       k_fold<float><<<grid, FOLD_THREADS, 0, s>>>(pf.catalogue, pf.d_tile_rec, pf.n_tiles, pf.d_rec_ids,
                                                   pf.d_rec_loss32, pf.d_elt_ret, pf.d_elt_lim,

@@ -337,3 +337,10 @@ def test_one_request_with_a_window_writes_its_own_trials_only(form, window):
     assert torch.equal(y[pad:pad + n].view(n_layers, -1), ref) and torch.equal(r[pad:pad + n].view(n_layers, -1), reg_ref)
     assert bool((y[:pad] == -7.0).all() & (y[pad + n:] == -7.0).all() & (r[:pad] == 77).all() & (r[pad + n:] == 77).all())
     pf.close()
+
+
+# the fold's tiles beyond those that run at once: 512 events (by size, and with enough records), 1,024 (few records)
+@pytest.mark.parametrize("C,n_elts,nnz,f32", [(300_001, 6, 9_000, True), (999_999, 10, 60_000, False),
+                                              (600_007, 8, 20_000, True), (1_300_000, 12, 30_000, False)])
+def test_fold_by_event_in_larger_tiles(C, n_elts, nnz, f32):
+    test_fold_by_event_equals_fold_by_tiles(C, n_elts, nnz, f32)
