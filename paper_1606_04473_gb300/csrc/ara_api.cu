@@ -783,7 +783,7 @@ ara_status ara_prepare_ylt(ara_portfolio* pf, int32_t n_sel, const int32_t* laye
 static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, int64_t n_trials, int64_t events) {
   if (sel.size() < 2 || !batched_fits(pf, sel.size()) || !rows_usable(pf, sel)) return false;
   const int K = rows_k(pf, sel);
-  const RowSizes z = rows_sizes(pf, sel, K, n_trials);
+  const RowSizes z = rows_sizes(pf, sel, K);
   const double C = (double)pf.catalogue, L = (double)sel.size(), ev = (double)events, tr = (double)n_trials;
   double rec = 0.0;
   for (int32_t l : sel)

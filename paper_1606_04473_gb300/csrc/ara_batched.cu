@@ -369,10 +369,9 @@ ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
   for (P.by_event = rows_usable(pf, P.sel);; P.by_event = false) {
     P.rt = RowTable{};
     P.rt.K = P.by_event && !P.windowed() ? rows_k(pf, P.sel) : 0;
-    const RowSizes z = rows_sizes(pf, P.sel, P.rt.K, P.n_trials);
+    const RowSizes z = rows_sizes(pf, P.sel, P.rt.K);
     P.rt.first_shift = z.first_shift;
-    P.sched = rows_schedule(pf, (int)P.sel.size(), P.rt.K, z.likely_bytes, z.likely_entries,
-                            P.n_trials, P.n_events);
+    P.sched = rows_schedule((int)P.sel.size(), P.rt.K, z.likely_bytes, z.likely_entries, P.n_trials, P.n_events);
     P.n_blocks = (C + BT_SCAN_BLOCK - 1) / BT_SCAN_BLOCK;
     size_t off = 0;
     auto take = [&](size_t n) { size_t o = (off + 255) / 256 * 256; off = o + n; return o; };
@@ -463,7 +462,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
   };
   P->by_event = rows_usable(*pf, P->sel);
   P->rt.K = P->by_event ? rows_k(*pf, P->sel) : 0;
-  const RowSizes z = rows_sizes(*pf, P->sel, P->rt.K, n_trials);
+  const RowSizes z = rows_sizes(*pf, P->sel, P->rt.K);
   P->rt.first_shift = z.first_shift;
   if ((P->rt.K > 0 && dmalloc(&P->rt.table, 8 * (size_t)P->rt.K * (size_t)C) != cudaSuccess) ||
       dmalloc(&P->d_rows, 8 * (size_t)C) != cudaSuccess || dmalloc(&P->d_total, 8) != cudaSuccess ||
@@ -485,8 +484,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
   P->rt.ovf_pairs = total[0];
   if ((st = bt_prep(*P, s, true, nullptr)) != ARA_OK) return fail(st);
   const int64_t table_bytes = 8 * C * std::max(P->rt.K, 1) + 16 * (int64_t)total[0];
-  P->sched = rows_schedule(*pf, (int)P->sel.size(), P->rt.K, table_bytes, (double)total[1] / (double)C,
-                           n_trials, n_events);
+  P->sched = rows_schedule((int)P->sel.size(), P->rt.K, table_bytes, (double)total[1] / (double)C, n_trials, n_events);
   const size_t part_bytes = 16 * (size_t)n_trials * P->sel.size();
   const bool tune = (flags & ARA_PLAN_AUTOTUNE) != 0;
   // room for the sums between passes: where the rule takes several, or where they are tried
@@ -506,6 +504,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
     for (int nc : {4, 8, 16, 32})
       for (int passes : {1, 2, 3}) {
         if (nc > 2 * rule.nc || 2 * nc < rule.nc) continue;
+        if (nc == 32 && P->rt.K == 0) continue;   // rows end to end have 16 columns at most
         if (passes > 1 && !(try_passes && P->part)) continue;
         P->sched = RowSchedule{nc, passes, 0};
         float ms = 0.f, tot = 0.f;

@@ -313,11 +313,9 @@ struct RowsStream {
 };
 ara_status build_event_index(Portfolio& pf, cudaStream_t s);
 bool rows_usable(const Portfolio& pf, const std::vector<int32_t>& sel);
-int64_t rows_bound(const Portfolio& pf, const std::vector<int32_t>& sel);
 int rows_k(const Portfolio& pf, const std::vector<int32_t>& sel);
-RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K, int64_t n_trials);
-RowSchedule rows_schedule(const Portfolio& pf, int ns, int K, int64_t table_bytes, double entries,
-                          int64_t n_trials, int64_t n_events);
+RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K);
+RowSchedule rows_schedule(int ns, int K, int64_t table_bytes, double entries, int64_t n_trials, int64_t n_events);
 // Slots within an adjoint row descriptor (ara_adjoint.cu).
 struct AdjbSlots {
   uint32_t width, n, mask;          // bits per slot, slots held, the width's mask

@@ -860,7 +860,7 @@ bool rows_usable(const Portfolio& pf, const std::vector<int32_t>& sel) {
     if (seen[(size_t)l] || !pf.layer_asc[(size_t)l]) return false;
     seen[(size_t)l] = 1;
   }
-  return rows_sizes(pf, sel, 0, 1).pairs < (int64_t)UINT32_MAX;
+  return rows_sizes(pf, sel, 0).pairs < (int64_t)UINT32_MAX;
 }
 
 // Entries per event: an upper bound (every record of the layers) and a guess that counts an event
@@ -896,8 +896,7 @@ int rows_k(const Portfolio& pf, const std::vector<int32_t>& sel) {
   return 8 * (int64_t)K * pf.catalogue <= (80ll << 20) ? K : 0;
 }
 
-RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K, int64_t n_trials) {
-  (void)n_trials;
+RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K) {
   RowSizes z;
   int64_t bound;
   row_entries(pf, sel, &bound, &z.likely_entries);
@@ -917,9 +916,7 @@ RowSizes rows_sizes(const Portfolio& pf, const std::vector<int32_t>& sel, int K,
 // Passes: parts of the catalogue whose rows stay in L2 (118 MB of rows, 64 layers: 4.83 ms in one
 // pass, 4.27 in two, 4.61 in three; 179 MB, 100 layers, 4 columns: 3.73 and 4.22; 283 MB, 150
 // layers, 4 columns: 4.58 and 4.05).
-RowSchedule rows_schedule(const Portfolio& pf, int ns, int K, int64_t table_bytes, double entries,
-                          int64_t n_trials, int64_t n_events) {
-  (void)pf;
+RowSchedule rows_schedule(int ns, int K, int64_t table_bytes, double entries, int64_t n_trials, int64_t n_events) {
   RowSchedule r;
   const int extra = 16 * ns + (K > 0 ? 640 : 128);
   r.nc = 4;
@@ -1026,7 +1023,6 @@ static ara_status launch_join(const Portfolio& pf, RowsStream p, RowSchedule& sc
 static ara_status launch_rows_join(const Portfolio& pf, const RowsStream& p, RowSchedule& sched, cudaStream_t s) {
   const bool m = p.windowed;
   switch (sched.nc) {
-    case 32:
     case 16: return m ? launch_join<16, true>(pf, p, sched, s) : launch_join<16, false>(pf, p, sched, s);
     case 8: return m ? launch_join<8, true>(pf, p, sched, s) : launch_join<8, false>(pf, p, sched, s);
     default: return m ? launch_join<4, true>(pf, p, sched, s) : launch_join<4, false>(pf, p, sched, s);
