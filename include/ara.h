@@ -515,8 +515,8 @@ ARA_API ara_status ara_adjoint_indexed(ara_portfolio* pf, const ara_yet_index* y
  *   h_mean        host [n_layers] or NULL: the mean year loss (1/N) sum_t y_t of each row
  * n_rp + n_tvar <= 16 (at least one metric requested), n_trials >= 1.  Allocates its scratch
  * in stream order on `stream`, from the library's memory pool: about 48 KiB for each row and metric at
- * 30,000 trials, 131 at 200,000 and 156 at 1,000,000, at most 4 GiB; with less memory fewer rows at a time
- * and shorter lists (down to about 16 KiB for each metric), the same results.  The selection of up to 32 rows
+ * 30,000 trials, 131 at 200,000 and 156 at 1,000,000, at most 4 GiB; with less memory an eighth of that,
+ * then fewer rows at a time (down to about 16 KiB for each metric of one), the same results.  The selection of up to 32 rows
  * (of more than 4,096 values) is one cooperative launch whose blocks meet at device-side barriers,
  * each wait bounded like the bulk copies' (ara_debug_set ARA_DBG_WAIT_LIMIT_NS).
  * Errors: ARA_EINVAL, ARA_ENOMEM, ARA_ECUDA, ARA_ETIMEOUT (a barrier wait ran out).
@@ -565,6 +565,9 @@ ARA_API ara_status ara_risk_metrics_async(const double* d_ylt, int64_t n_trials,
  * the process exits).  Arguments, results and errors are those of ara_risk_metrics, plus:
  *   - a request whose scratch (about 8 KiB per layer per requested PML/TVaR level) does not
  *     fit in the array returns ARA_ERANGE and launches nothing;
+ *   - rows whose lists do not fit the array together (about 8 KiB for each row and metric up to
+ *     65,000 trials, 25 at 200,000, 122 at 1,000,000) go in parts, whose TVaR and means may differ
+ *     from ara_risk_metrics' in the last bits (sums in another order);
  *   - every call looks up the array's device address on the current device (a cheap host
  *     query), so the address stays right after the device's context is torn down and
  *     recreated (cudaDeviceReset reloads the library's module, possibly elsewhere);

@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -52,10 +53,10 @@ __device__ __forceinline__ bool in_interval(uint64_t k, uint64_t lo, uint64_t hi
   return (k > lo || (lo == 0ull && k == 0ull)) && (k < hi || (hi == ~0ull && k == ~0ull));
 }
 
-// Scratch (one allocation; the first part, up to state, is zero-filled before the launch).  Layers count
+// Scratch (one allocation; the part from err up to state is zero-filled before the launch).  Layers count
 // from the first one of a launch group; G of them share the working parts at a time.
 struct SelScratch {
-  uint32_t* err;               // [1]
+  uint32_t* err;               // [1], behind the results
   uint32_t* count;             // [G][SEL_CLASSES] class totals
   uint32_t* n_list;            // [G][n_t] keys in each list
   uint32_t* bar;               // [G] grid-barrier counters
@@ -65,7 +66,7 @@ struct SelScratch {
   uint64_t* list;              // [G][n_t][cap]
   double* psum;                // [G][n_t][blocks] block partials of the tail sums
   double* pmean;               // [G][blocks] block partials of the row sum
-  // results, contiguous: out, mean
+  // results, contiguous: out, mean, err
   double* out;                 // [n_layers][n_t] PML / TVaR
   double* mean;                // [n_layers]
   unsigned long long* gt;      // [n_layers][n_t] #{y > key}
@@ -82,22 +83,22 @@ struct SelScratch {
 static SelScratch carve(void* base, const SelPlan& y) {
   char* p = (char*)base;
   SelScratch s{};
-  s.err = (uint32_t*)(p + y.off[0]);
-  s.count = (uint32_t*)(p + y.off[1]);
-  s.n_list = (uint32_t*)(p + y.off[2]);
-  s.bar = (uint32_t*)(p + y.off[3]);
-  s.count2 = y.rounds > 1 ? (uint32_t*)(p + y.off[4]) : nullptr;
-  s.n_list2 = (uint32_t*)(p + y.off[5]);
-  s.state = (SelState*)(p + y.off[6]);
-  s.list = (uint64_t*)(p + y.off[7]);
-  s.psum = (double*)(p + y.off[8]);
-  s.pmean = (double*)(p + y.off[9]);
-  s.out = (double*)(p + y.off[10]);
+  s.out = (double*)(p + y.off[0]);
   s.mean = s.out + (size_t)y.n_layers * y.n_t;
+  s.err = (uint32_t*)(p + y.off[1]);
+  s.count = (uint32_t*)(p + y.off[2]);
+  s.n_list = (uint32_t*)(p + y.off[3]);
+  s.bar = (uint32_t*)(p + y.off[4]);
+  s.count2 = y.rounds > 1 ? (uint32_t*)(p + y.off[5]) : nullptr;
+  s.n_list2 = (uint32_t*)(p + y.off[6]);
+  s.state = (SelState*)(p + y.off[7]);
+  s.list = (uint64_t*)(p + y.off[8]);
+  s.psum = (double*)(p + y.off[9]);
+  s.pmean = (double*)(p + y.off[10]);
   s.gt = (unsigned long long*)(p + y.off[11]);
   s.eq = (unsigned long long*)(p + y.off[12]);
-  s.cap = y.cap;
-  s.sample = sel_sample(y.n);
+  s.cap = y.lists.cap;
+  s.sample = y.lists.sample;
   return s;
 }
 
@@ -1092,8 +1093,8 @@ ara_status launch_select(const double* d_ylt, const SelPlan& y, const SelTargets
   for (int32_t g0 = 0; g0 < y.n_layers; g0 += y.per) {
     // (without counts only the error word needs clearing, and the host's is clear)
     if (g0 == 0 ? counts || !host_err : counts) {
-      const size_t z = g0 == 0 ? 0 : y.off[1];
-      ARA_TRY(cudaMemsetAsync((char*)scratch + z, 0, y.zero_bytes - z, s));
+      const size_t z = y.off[g0 == 0 ? 1 : 2];
+      ARA_TRY(cudaMemsetAsync((char*)scratch + z, 0, y.zero_end - z, s));
     }
     SelScratch g = sc;
     const int64_t l = g0, lt = l * y.n_t;
@@ -1147,6 +1148,21 @@ void free_select_result(SelectResult& r, cudaStream_t s) {
   r.scratch = nullptr;
 }
 
+// The host copy of a request's results (out, mean, err) into the caller's arrays.
+static ara_status split_results(const double* out, int32_t n_layers, const SelTargets& tg, double* h_pml,
+                                double* h_tvar, double* h_mean) {
+  const size_t L = (size_t)n_layers, nt = (size_t)tg.n_t, n_rp = (size_t)tg.n_rp;
+  uint32_t timed_out = 0;
+  memcpy(&timed_out, out + L * nt + L, sizeof(timed_out));
+  if (timed_out) return ARA_ETIMEOUT;
+  for (size_t l = 0; l < L; ++l) {
+    for (size_t i = 0; i < n_rp; ++i) h_pml[l * n_rp + i] = out[l * nt + i];
+    for (size_t i = n_rp; i < nt; ++i) h_tvar[l * (nt - n_rp) + i - n_rp] = out[l * nt + i];
+    if (h_mean) h_mean[l] = out[L * nt + l];
+  }
+  return ARA_OK;
+}
+
 ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_layers,
                                int32_t n_rp, const double* rps, int32_t n_tvar,
                                const double* levels, double* h_pml, double* h_tvar,
@@ -1184,25 +1200,14 @@ ara_status risk_metrics_device(const double* d_ylt, int64_t n_trials, int32_t n_
     return ARA_OK;
   }
   st = launch_select(d_ylt, y, tg, scratch, h_mean != nullptr, s, &sc);
-  std::vector<double> out(L * tg.n_t + L);
-  uint32_t timed_out = 0;
-  if (st == ARA_OK) {
-    cudaError_t e = cudaMemcpyAsync(out.data(), sc.out, sizeof(double) * out.size(),   // and the means
-                                    cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&timed_out, sc.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) st = ARA_ECUDA;
-  }
+  std::vector<double> out(L * tg.n_t + L + 1);   // metrics, means and the error word
+  if (st == ARA_OK &&
+      cudaMemcpyAsync(out.data(), sc.out, 8 * (out.size() - 1) + 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    st = ARA_ECUDA;
   cudaFreeAsync(scratch, s);
   if (cudaStreamSynchronize(s) != cudaSuccess && st == ARA_OK) st = ARA_ECUDA;
   if (st != ARA_OK) return st;
-  if (timed_out) return ARA_ETIMEOUT;
-  for (int32_t l = 0; l < n_layers; ++l) {
-    for (int i = 0; i < n_rp; ++i) h_pml[(size_t)l * n_rp + i] = out[(size_t)l * tg.n_t + i];
-    for (int i = 0; i < n_tvar; ++i) h_tvar[(size_t)l * n_tvar + i] = out[(size_t)l * tg.n_t + n_rp + i];
-    if (h_mean) h_mean[l] = out[L * tg.n_t + l];
-  }
-  return ARA_OK;
+  return split_results(out.data(), n_layers, tg, h_pml, h_tvar, h_mean);
 }
 
 }  // namespace ara
@@ -1319,37 +1324,27 @@ extern "C" ara_status ara_risk_metrics_static(const double* d_ylt, int64_t n_tri
   void* scratch = nullptr;
   if ((st = static_scratch(&scratch)) != ARA_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = cudaSuccess;
-  uint32_t timed_out = 0;
-  const size_t row = sizeof(double) * (size_t)tg.n_t;
-  for (int32_t l0 = 0; l0 < n_layers && st == ARA_OK && e == cudaSuccess && !timed_out; l0 += g.per) {
+  std::vector<double> out((size_t)g.per * (tg.n_t + 1) + 1);
+  for (int32_t l0 = 0; l0 < n_layers && st == ARA_OK; l0 += g.per) {
     const SelPlan& y = n_layers - l0 >= g.per ? g.first : g.last;
-    const int32_t nl = y.n_layers;
     SelScratch sc;
     st = launch_select(d_ylt + (int64_t)l0 * n_trials, y, tg, scratch, h_mean != nullptr, s, &sc);
-    if (st != ARA_OK) break;
-    if (n_rp > 0)
-      e = cudaMemcpy2DAsync(h_pml + (size_t)l0 * n_rp, sizeof(double) * n_rp, sc.out, row, sizeof(double) * n_rp,
-                            (size_t)nl, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && n_tvar > 0)
-      e = cudaMemcpy2DAsync(h_tvar + (size_t)l0 * n_tvar, sizeof(double) * n_tvar, sc.out + n_rp, row,
-                            sizeof(double) * n_tvar, (size_t)nl, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && h_mean)
-      e = cudaMemcpyAsync(h_mean + l0, sc.mean, sizeof(double) * nl, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&timed_out, sc.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-    // the next layers reuse the array, and the status decides whether they run
-    if (l0 + nl < n_layers && e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaError_t e = cudaSuccess;
+    if (st == ARA_OK) {
+      e = cudaMemcpyAsync(out.data(), sc.out, 8 * (size_t)y.n_layers * (tg.n_t + 1) + 4, cudaMemcpyDeviceToHost, s);
+      if (e != cudaSuccess) note_cuda_error(e, "static risk metrics: result copy", __FILE__, __LINE__);
+    }
+    // Always wait for the stream before returning (and before the array is used again), so that no copy
+    // queued here can land anywhere after the call has returned.
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && es != cudaSuccess) {
+      note_cuda_error(es, "cudaStreamSynchronize", __FILE__, __LINE__);
+      e = es;
+    }
+    if (st == ARA_OK && e != cudaSuccess) st = ARA_ECUDA;
+    if (st == ARA_OK)
+      st = split_results(out.data(), y.n_layers, tg, h_pml ? h_pml + (size_t)l0 * n_rp : nullptr,
+                         h_tvar ? h_tvar + (size_t)l0 * n_tvar : nullptr, h_mean ? h_mean + l0 : nullptr);
   }
-  // Always wait for the stream before returning, so that no copy queued here can land in the
-  // caller's buffers after the call has returned.
-  if (e != cudaSuccess) note_cuda_error(e, "static risk metrics: result copy", __FILE__, __LINE__);
-  const cudaError_t es = cudaStreamSynchronize(s);
-  if (e == cudaSuccess && es != cudaSuccess) {
-    note_cuda_error(es, "cudaStreamSynchronize", __FILE__, __LINE__);
-    e = es;
-  }
-  if (st != ARA_OK) return st;
-  if (e != cudaSuccess) return ARA_ECUDA;
-  return timed_out ? ARA_ETIMEOUT : ARA_OK;
+  return st;
 }

@@ -7,12 +7,6 @@
 
 #include <algorithm>
 
-#ifdef __CUDACC__
-#define ARA_HD __host__ __device__
-#else
-#define ARA_HD
-#endif
-
 namespace ara {
 
 constexpr int SEL_THREADS = 512;
@@ -33,39 +27,52 @@ struct SelState {
   int64_t in_class;            // keys in the class
 };
 
-// Sampled keys of a row: sorting them costs every block 2 us for 256 and 9 us for 1,024, and the
-// intervals they leave are picked from in about 4 us per 4,096 keys.
-ARA_HD inline int32_t sel_sample(int64_t n) { return n <= (1 << 19) ? 256 : SEL_SAMPLE; }
+// Sampled keys of a row, and room for the keys of one open interval between neighbouring samples: the
+// interval that holds a given rank has 2 / sample of the keys on average and more than 16 / sample with
+// probability 2e-6 (a list that would overflow is not used: its target is picked from the row itself).
+// Sorting the sample costs every block longer the larger it is, and the intervals it leaves are picked from
+// in about 4 us per 4,096 keys: 256 keys up to 2^19 values, and lists that rarely overflow at any length.
+struct SelLists {
+  int32_t sample;
+  int64_t cap;                      // keys per list
+};
+inline SelLists roomy_lists(int64_t n) {
+  const int32_t sample = n <= (1 << 19) ? 256 : SEL_SAMPLE;
+  return SelLists{sample, std::min<int64_t>(n, 16 * (n / sample) + 4096)};
+}
+// The same chance of an overflow in up to eight times less room.
+inline SelLists tight_lists(int64_t n) {
+  return SelLists{SEL_SAMPLE, std::min<int64_t>(n, std::max<int64_t>(16 * (n / SEL_SAMPLE), SEL_SAMPLE))};
+}
 
-// Room for the keys of one open interval between neighbouring samples: the interval that holds a
-// given rank has 2 / sample of the keys on average and more than 16 / sample with probability 2e-6 (a
-// list that would overflow is not used: its target is picked from the row itself).
-inline int64_t list_cap(int64_t n) { return std::min<int64_t>(n, 16 * (n / sel_sample(n)) + 4096); }
-
-// A request's launch plan and scratch.  The form and the slices of a row (on which the order of the TVaR and
-// mean sums depends) follow from the request, the slices also where the form differs (beside); how many rows share the lists at a time (per: groups run
-// one after the other) and how long the lists are follow from the memory, and change no result.
+// A request's launch plan and scratch.  The form and the parts of a row that are summed one by one (on which
+// the order of the TVaR and mean sums depends) follow from the request, the parts also where the form differs
+// (beside).  How many rows share the lists at a time and how long the lists are follow from the memory, and
+// change no result.
 struct SelPlan {
-  int64_t n = 0, cap = 0;           // cap: keys per list
+  int64_t n = 0;
+  SelLists lists{0, 0};
   int32_t n_layers = 0, n_t = 0, blocks = 1;
-  int32_t slices = 1;               // parts of a row that are summed one by one, at least `blocks`
-  int32_t per = 1;                  // rows per group
-  int32_t rounds = 1;               // 2: lists may overflow, overfull intervals are split again before the pick
+  int32_t slices = 1;               // parts of a row's sums, at least `blocks`
+  int32_t per = 1;                  // rows per group; the groups run one after the other
+  int32_t rounds = 1;               // 2: lists may well overflow, overfull intervals are split again before the pick
   bool cluster = false;             // one cluster of `blocks` blocks per row
   bool small = false;               // one block per row, sorted whole
   int n_sms = 1;
+  // out and mean, err, then count, n_list, bar, count2, n_list2 (from err on cleared before the launch; err
+  // only before the first group), state, list, psum, pmean, gt, eq
   size_t off[13];
-  size_t zero_bytes = 0, bytes = 0;
+  size_t zero_end = 0, bytes = 0;
   int32_t at_once() const { return std::max(1, (cluster ? 2 * n_sms : n_sms) / blocks); }   // rows that run at once
 };
 // per: 0 for all rows in one group.  beside: the caller's kernels share the device with other streams'
 // (the server).  A row in a cluster whose list overflows is picked from the row itself, without a
 // second round.
-inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int64_t cap, bool beside = false,
+inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, SelLists lists, bool beside = false,
                         int32_t per = 0) {
   SelPlan y;
   y.n = n;
-  y.cap = cap;
+  y.lists = lists;
   y.n_layers = n_layers;
   y.n_t = n_t;
   y.per = per > 0 ? std::min(per, n_layers) : n_layers;
@@ -86,73 +93,77 @@ inline SelPlan sel_plan(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, int
     }
   }
   if (!y.cluster) y.blocks = y.slices;
-  y.rounds = !y.small && !y.cluster && cap < list_cap(n) ? 2 : 1;
-  const size_t L = (size_t)n_layers, lt = L * (size_t)std::max(n_t, 1);
+  y.rounds = !y.small && !y.cluster && lists.cap < std::min<int64_t>(n, 16 * (n / lists.sample)) ? 2 : 1;
+  const size_t L = (size_t)n_layers, lt = L * (size_t)n_t;
   const size_t G = (size_t)y.per, gt = G * (size_t)n_t, two = y.rounds > 1 ? gt : 0;   // of a group
-  const size_t grid = y.small || y.cluster ? 0 : 1, lists = y.small ? 0 : 1;
+  const size_t grid = y.small || y.cluster ? 0 : 1, listed = y.small ? 0 : 1;
   size_t b = 0;
   int i = 0;
-  auto t = [&](size_t k) { b = (b + 15) / 16 * 16; y.off[i++] = b; b += k; };
-  t(4);
-  t(4 * grid * G * SEL_CLASSES);
+  auto t = [&](size_t k, size_t align = 16) { b = (b + align - 1) / align * align; y.off[i++] = b; b += k; };
+  t(8 * (lt + L));
+  t(4, 8);                                                  // right behind the results: one copy takes both
+  t(4 * grid * (n_t > 0 ? G : 0) * SEL_CLASSES);
   t(4 * grid * gt);
   t(4 * grid * G);
   t(4 * two * SEL_CLASSES);
   t(4 * two);
-  y.zero_bytes = (b + 15) / 16 * 16;
+  y.zero_end = (b + 15) / 16 * 16;
   t(sizeof(SelState) * lt);
-  t(8 * lists * gt * (size_t)cap);
+  t(8 * listed * gt * (size_t)lists.cap);
   t(8 * grid * gt * (size_t)y.blocks);
   t(8 * grid * G * (size_t)y.blocks);
-  t(8 * (lt + L));
   t(8 * lt);
   t(8 * lt);
   y.bytes = (b + 255) / 256 * 256;
   return y;
 }
 
-// A request's plan within `limit` bytes: all rows in one group, else groups (whole waves of rows while
-// they hold one), else shorter lists; the smallest plan where nothing fits.  Lists hold 16 n / sample +
-// 4,096 keys for each row and target: 1,000 rows of 200,000 values with 16 targets take 2.1 GB at once (3.2
-// ms; in 4 groups of a wave, 650 MB, 3.6 ms; in 14 groups of a quarter of a wave 9.5).
+// A request's plan within `limit` bytes: roomy lists, else tight ones, else groups of rows (whole waves while
+// they hold one), else shorter lists; the smallest plan where nothing fits.  1,000 rows of 200,000 values with
+// 16 targets take 2.1 GB with roomy lists.
 constexpr size_t SEL_SCRATCH = (size_t)4 << 30;
 inline SelPlan sel_plan_within(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, bool beside, size_t limit) {
-  int64_t cap = list_cap(n);
-  SelPlan y = sel_plan(n, n_layers, n_t, n_sms, cap, beside);
-  if (y.small) return y;                                    // no working parts to share
+  SelPlan y = sel_plan(n, n_layers, n_t, n_sms, roomy_lists(n), beside);
+  if (y.bytes <= limit || y.small || n_t == 0) return y;
+  SelLists lists = tight_lists(n);
+  y = sel_plan(n, n_layers, n_t, n_sms, lists, beside);
   for (int32_t per = n_layers; y.bytes > limit && per > 1;) {
     per = (per + 1) / 2;
     if (per > y.at_once()) per -= per % y.at_once();
-    y = sel_plan(n, n_layers, n_t, n_sms, cap, beside, per);
+    y = sel_plan(n, n_layers, n_t, n_sms, lists, beside, per);
   }
-  while (y.bytes > limit && cap > SEL_SAMPLE) {
-    cap = std::max<int64_t>(cap / 2, SEL_SAMPLE);
-    y = sel_plan(n, n_layers, n_t, n_sms, cap, beside, 1);
+  while (y.bytes > limit && lists.cap > SEL_SAMPLE) {
+    lists.cap = std::max<int64_t>(lists.cap / 2, SEL_SAMPLE);
+    y = sel_plan(n, n_layers, n_t, n_sms, lists, beside, 1);
   }
   return y;
 }
 
-// The rows of the allocation-free call, as requests of their own whose scratch fits `limit` bytes each (few
-// rows at a time get more blocks each): `per` rows (plan `first`) and a last one of what is left (`last`).  Where even one row's lists do not fit, shorter
-// lists and a second round.  The last group can need more than the others although it has fewer rows
-// (33 rows run as clusters, 32 as one cooperative launch with class counts), so both are checked.
+// The allocation-free call within `limit` bytes: the request's own plan (roomy or tight lists) where it fits.
+// Else its rows go as requests of their own, `per` at a time (plan `first`) and a last one of what is left
+// (`last`), because fewer rows get more blocks each: in groups of one plan, 16 rows of 4.3 M values would run
+// on 9 blocks at a time.  Where even one row's lists do not fit, shorter lists and a second round.  The last
+// request can need more than the others although it has fewer rows (33 rows run as clusters, 32 as one
+// cooperative launch with class counts), so both are checked.
 struct SelGroups {
   int32_t per = 1;
   SelPlan first, last;
 };
 inline bool sel_groups(int64_t n, int32_t n_layers, int32_t n_t, int n_sms, size_t limit, SelGroups& g) {
-  int64_t cap = list_cap(n);
+  SelLists lists = roomy_lists(n);
   auto fits = [&](int32_t per) {
     g.per = per;
-    g.first = sel_plan(n, per, n_t, n_sms, cap);
-    g.last = n_layers % per ? sel_plan(n, n_layers % per, n_t, n_sms, cap) : g.first;
+    g.first = sel_plan(n, per, n_t, n_sms, lists);
+    g.last = n_layers % per ? sel_plan(n, n_layers % per, n_t, n_sms, lists) : g.first;
     return g.first.bytes <= limit && g.last.bytes <= limit;
   };
+  if (fits(n_layers)) return true;
+  lists = tight_lists(n);
   int32_t per = n_layers;
   while (!fits(per) && per > 1) per = (per + 1) / 2;
   while (!fits(per)) {
-    cap /= 2;
-    if (cap < SEL_SAMPLE) return false;
+    if (lists.cap <= SEL_SAMPLE) return false;
+    lists.cap = std::max<int64_t>(lists.cap / 2, SEL_SAMPLE);
   }
   return true;
 }

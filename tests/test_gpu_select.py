@@ -188,3 +188,14 @@ def test_special_values(n_rows, n):
             np.testing.assert_allclose(tvar[rows, i], want[rows].astype(np.float64), rtol=1e-13)
         want = (y.astype(np.longdouble).sum(1) / n).astype(np.float64)
         np.testing.assert_allclose(mean[rows], want[rows], rtol=1e-13)
+
+
+@pytest.mark.parametrize("n_rows,n", [(40, 100_000), (33, 5_000), (8, 4_097), (24, 300_001), (100, 9_000)])
+def test_allocation_free_call_has_the_bits_of_the_allocating_one(n_rows, n):
+    """Where the request fits the fixed array with tight lists, it runs in one go in the same form."""
+    d = torch.from_numpy(rows(n, n_rows, n)).cuda()
+    rps, levels = [100.0, 250.0], [0.99]
+    n0 = ara.launch_count()
+    got = ara.risk_metrics_static(d, rps, levels, want_mean=True)
+    assert ara.launch_count() - n0 == 1
+    assert all(np.array_equal(a, b) for a, b in zip(got, ara.risk_metrics(d, rps, levels, want_mean=True)))

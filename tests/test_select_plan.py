@@ -25,10 +25,10 @@ int main() {
           uneven += left != 0;
           if (g.per < 1 || g.per > L || g.first.n_layers != g.per || g.last.n_layers != (left ? left : g.per)) ++bad;
           for (const SelPlan* y : {&g.first, &g.last}) {
-            if (y->bytes > limit || y->zero_bytes > y->bytes || y->n != n || y->n_t != t) ++bad;
-            for (int i = 0; i < 12; ++i) bad += y->off[i] > y->off[i + 1] || y->off[i] % 16;
+            if (y->bytes > limit || y->zero_end > y->off[7] || y->n != n || y->n_t != t) ++bad;
+            for (int i = 0; i < 12; ++i) bad += y->off[i] > y->off[i + 1] || y->off[i] % 8;
             if (y->off[12] + 8ull * y->n_layers * t > y->bytes) ++bad;
-            if (!y->small && y->off[7] + 8ull * y->n_layers * t * y->cap > y->off[8]) ++bad;
+            if (!y->small && y->off[8] + 8ull * y->n_layers * t * y->lists.cap > y->off[9]) ++bad;
           }
         }
   printf("%ld %ld\n", bad, uneven);
@@ -49,21 +49,21 @@ int main() {
     for (int L : {1, 2, 6, 32, 33, 64, 100, 152, 304, 1000, 100000})
       for (int t = 0; t <= 16; ++t)
         for (int beside = 0; beside < 2; ++beside) {
-          const SelPlan all = sel_plan(n, L, t, 152, list_cap(n), beside);
+          const SelPlan all = sel_plan(n, L, t, 152, roomy_lists(n), beside);
           size_t before = 0;
           for (size_t limit : limits) {
             const SelPlan y = sel_plan_within(n, L, t, 152, beside, limit);
             // the results' order of addition follows from the request alone
             bad += y.blocks != all.blocks || y.cluster != all.cluster || y.small != all.small;
             bad += y.bytes > all.bytes + 8 * 16 * SEL_CLASSES + 4096 || y.bytes < before || y.per < 1 || y.per > L;
-            if (limit >= all.bytes) bad += y.per != L || y.cap != all.cap || y.rounds != all.rounds;
+            if (limit >= all.bytes) bad += y.per != L || y.lists.cap != all.lists.cap || y.rounds != all.rounds;
             if (y.bytes <= limit && y.per > y.at_once() && y.per < L) bad += y.per % y.at_once() != 0;
             // never much more than 8 KiB for each row and target and the results
             if (limit == 0) bad += y.bytes > 17000ull * (t + 1) + 100ull * L * (t + 1) + 8ull * 152 * (t + 1) + 4096;
-            for (int i = 0; i < 12; ++i) bad += y.off[i] > y.off[i + 1] || y.off[i] % 16;
-            if (!y.small && y.off[7] + 8ull * y.per * t * y.cap > y.off[8]) ++bad;
+            for (int i = 0; i < 12; ++i) bad += y.off[i] > y.off[i + 1] || y.off[i] % 8;
+            if (!y.small && y.off[8] + 8ull * y.per * t * y.lists.cap > y.off[9]) ++bad;
             grouped += y.per < L;
-            shorter += y.cap < all.cap;
+            shorter += y.lists.cap < all.lists.cap;
             before = y.bytes;
           }
         }
