@@ -9,9 +9,9 @@
 //   1. q_i(e) = round(C(sum_j C(x_j(e); R_j, L_j); OccR_i, OccL_i) * 2^f_i) and the hit bitmap
 //      of every selected layer i, in one launch of the single-layer fold kernel (slot i of the
 //      fold workspace; only the non-zero q are stored).
-//   2. per-event counts of non-zero q, read from the bitmaps, and the exclusive scan of their
-//      16-byte pairs.
-//   3. the rows, end to end: slot << 56 | q in slot order (q < 2^55; q is read only where the bitmap
+//   2. per-event counts of non-zero q, read from the bitmaps, and the exclusive scan of the 16-byte
+//      pairs that they take (in place: beyond the row's place).
+//   3. the rows, in place or end to end as from the records: slot << 56 | q in slot order (q < 2^55; q is read only where the bitmap
 //      bit is set), padded to whole pairs with an entry of the spare slot.  The event's row
 //      descriptor holds its first entry and, per request of a merged serving pass (slots are
 //      grouped by request), the number of its entries in one byte each (a row has at most 255
@@ -75,13 +75,18 @@ __device__ __forceinline__ uint32_t bt_count(const uint32_t* __restrict__ bits, 
 __global__ void __launch_bounds__(BT_SCAN_BLOCK)
 k_bt_scan_blocks(const uint32_t* __restrict__ bits, int64_t bits_stride, int32_t n_sel, int64_t n,
                  uint32_t* __restrict__ ptr, uint32_t* __restrict__ block_sums,
-                 uint32_t* __restrict__ entries) {
+                 uint32_t* __restrict__ entries, uint32_t K) {
   const int64_t e = (int64_t)blockIdx.x * BT_SCAN_BLOCK + threadIdx.x;
   uint32_t v = e < n ? bt_count(bits, bits_stride, n_sel, e) : 0u;
   if (entries) {   // rows in pairs of entries: the scan counts pairs, *entries gets the entries
+    __shared__ uint32_t sum;     // one atomic per block (one per warp took 28 us for 2 M events)
+    if (threadIdx.x == 0) sum = 0u;
+    __syncthreads();
     const uint32_t c = __reduce_add_sync(0xffffffffu, v);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(entries, c);
-    v = (v + 1u) >> 1;
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sum, c);
+    __syncthreads();
+    if (threadIdx.x == 0 && sum) atomicAdd(entries, sum);
+    v = row_pairs(v, K);
   }
   uint32_t tot;
   const uint32_t ex = block_excl_scan(v, &tot);
@@ -120,7 +125,7 @@ ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t 
                              cudaStream_t s) {
   const int64_t n_blocks = (n + BT_SCAN_BLOCK - 1) / BT_SCAN_BLOCK;
   k_bt_scan_blocks<<<(unsigned)n_blocks, BT_SCAN_BLOCK, 0, s>>>(bits, bits_stride, n_sel, n, ptr,
-                                                              block_sums, entries);
+                                                              block_sums, entries, 0u);
   k_bt_scan_sums<<<1, BT_SCAN_BLOCK, 0, s>>>(block_sums, n_blocks, total);
   k_bt_scan_add<<<(unsigned)((n + 1 + 255) / 256), 256, 0, s>>>(ptr, n, block_sums, total);
   ARA_TRY(cudaGetLastError());
@@ -140,19 +145,14 @@ __device__ __forceinline__ uint32_t bt_req_of_slot(const BtReqSlots& rs, int i) 
   return (uint32_t)(i >= rs.first[1]) + (uint32_t)(i >= rs.first[2]) + (uint32_t)(i >= rs.first[3]);
 }
 
-__global__ void __launch_bounds__(256)
-k_bt_fill(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restrict__ bits,
-          int64_t bits_stride, int64_t catalogue, const uint32_t* __restrict__ ptr,
-          uint64_t* __restrict__ entries, uint64_t* __restrict__ rows, BtReqSlots rs, int first_shift) {
+// Event e's entries in slot order, put(slot, entry) each, while more().
+template <typename M, typename F>
+__device__ __forceinline__ void bt_row(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restrict__ bits,
+                                       int64_t bits_stride, int64_t catalogue, int64_t e, M&& more, F&& put) {
   constexpr int U = 8;   // slots per step: their bitmap words and table entries load together
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= catalogue) return;
-  uint64_t pos = 2ull * ptr[e];
-  const uint64_t end = 2ull * ptr[e + 1];
-  uint32_t lens = 0;   // entries of request r in byte r (one 8-byte descriptor per occurrence)
   const uint32_t* b = bits + (e >> 5);
   const int sh = (int)(e & 31);
-  for (int i0 = 0; i0 < n_sel && pos < end; i0 += U) {
+  for (int i0 = 0; i0 < n_sel && more(); i0 += U) {
     bool hit[U];
     uint64_t v[U];
 #pragma unroll
@@ -162,16 +162,63 @@ k_bt_fill(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restr
     for (int u = 0; u < U; ++u) v[u] = hit[u] ? __ldg(q + (int64_t)(i0 + u) * catalogue + e) : 0ull;
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (hit[u]) {
-        if (pos < end) {
-          entries[pos] = ((uint64_t)(i0 + u) << 56) | v[u];
-          lens += 1u << (8 * bt_req_of_slot(rs, i0 + u));
-        }
-        ++pos;
-      }
+      if (hit[u]) put(i0 + u, ((uint64_t)(i0 + u) << 56) | v[u]);
   }
+}
+
+// End to end.
+__global__ void __launch_bounds__(256)
+k_bt_fill(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restrict__ bits,
+          int64_t bits_stride, int64_t catalogue, const uint32_t* __restrict__ ptr,
+          uint64_t* __restrict__ entries, uint64_t* __restrict__ rows, BtReqSlots rs, int first_shift) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= catalogue) return;
+  uint64_t pos = 2ull * ptr[e];
+  const uint64_t end = 2ull * ptr[e + 1];
+  uint32_t lens = 0;   // entries of request r in byte r (one 8-byte descriptor per occurrence)
+  bt_row(n_sel, q, bits, bits_stride, catalogue, e, [&] { return pos < end; }, [&](int i, uint64_t v) {
+    if (pos < end) {
+      entries[pos] = v;
+      lens += 1u << (8 * bt_req_of_slot(rs, i));
+    }
+    ++pos;
+  });
   if (pos < end) entries[pos] = (uint64_t)n_sel << 56;   // padding: adds 0 to the spare slot
   rows[e] = (uint64_t)(ptr[e] << first_shift) | ((uint64_t)lens << 32);
+}
+
+// In place (one request): the row at table + K e in the form of k_rows_build, a longer one with a
+// continuation in its last place and the rest in ovf.
+__global__ void __launch_bounds__(256)
+k_bt_fill_place(int32_t n_sel, const uint64_t* __restrict__ q, const uint32_t* __restrict__ bits,
+                int64_t bits_stride, int64_t catalogue, const uint32_t* __restrict__ ptr, uint32_t K,
+                uint64_t* __restrict__ table, uint64_t* __restrict__ ovf, uint64_t* __restrict__ rows) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= catalogue) return;
+  const uint32_t first = ptr[e], room = 2u * (ptr[e + 1] - first);   // entries outside the row's place
+  uint64_t* const ov = ovf + 2ull * first;
+  uint64_t* const row = table + (int64_t)K * e;
+  const uint32_t inl = room ? K - 1u : K;         // entries at most in the place
+  const uint64_t spare = (uint64_t)n_sel << 56;
+  uint64_t held = 0;                              // first of a 16-byte pair
+  auto put = [&](uint32_t i, uint64_t v) {
+    if (K == 1u) row[0] = v;
+    else if (i & 1u) reinterpret_cast<ulonglong2*>(row)[i >> 1] = make_ulonglong2(held, v);
+    else held = v;
+  };
+  uint32_t n = 0;
+  bt_row(n_sel, q, bits, bits_stride, catalogue, e, [&] { return n < inl + room; }, [&](int, uint64_t v) {
+    if (n < inl) put(n, v);
+    else if (n < inl + room) ov[n - inl] = v;
+    ++n;
+  });
+  if (room) {
+    if (n - inl < room) ov[n - inl] = spare;
+    put(K - 1u, ((uint64_t)(n - inl) << 56) | RW_CONT | first);
+  } else {
+    for (uint32_t k = n; k < K; ++k) put(k, spare);
+  }
+  if (rows) rows[e] = (uint64_t)(K * e) | ((uint64_t)n << 32);
 }
 
 }  // namespace ara
@@ -226,6 +273,14 @@ void single_request(ara_plan& P) {
   P.req_reg[0] = P.d_reg;
 }
 
+// Entries in place per event: the rule of the rows, and from the folds up to 2 (launches of plans with ELTs
+// in descending order, us, end to end / in place: 50,000 trials x 1,000 over 2 M events, 1 layer 468 / 308, 4
+// layers 528 / 410, 8 layers 586 / 509 (2 places); 100,000 trials, 16 layers 1,123 / 1,317 (4 places)).
+int plan_k(const ara_plan& P) {
+  const int K = rows_k(*P.pf, P.sel);
+  return P.by_event || K <= 2 ? K : 0;
+}
+
 ara_status bt_prep(ara_plan& P, cudaStream_t s, bool fill, int* n_kernels) {
   Portfolio& pf = *P.pf;
   if (P.by_event) {
@@ -245,14 +300,19 @@ ara_status bt_prep(ara_plan& P, cudaStream_t s, bool fill, int* n_kernels) {
   if (st != ARA_OK) return st;
   ARA_TRY(cudaMemsetAsync(P.d_total, 0, 2 * sizeof(uint32_t), s));
   k_bt_scan_blocks<<<(unsigned)P.n_blocks, BT_SCAN_BLOCK, 0, s>>>(pf.d_bits, pf.bm_words, n_sel, C,
-                                                                  P.d_ptr, P.d_bsum, P.d_total + 1);
+                                                                  P.d_ptr, P.d_bsum, P.d_total + 1,
+                                                                  (uint32_t)P.rt.K);
   k_bt_scan_sums<<<1, BT_SCAN_BLOCK, 0, s>>>(P.d_bsum, P.n_blocks, P.d_total);
   k_bt_scan_add<<<(unsigned)((C + 1 + 255) / 256), 256, 0, s>>>(P.d_ptr, C, P.d_bsum, P.d_total);
   int k = 4;
   if (fill) {
-    k_bt_fill<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(n_sel, pf.d_q, pf.d_bits, pf.bm_words, C,
-                                                          P.d_ptr, P.rt.ovf, P.d_rows, P.rs,
-                                                          P.rt.first_shift);
+    const unsigned blocks = (unsigned)((C + 255) / 256);
+    if (P.rt.K > 0)
+      k_bt_fill_place<<<blocks, 256, 0, s>>>(n_sel, pf.d_q, pf.d_bits, pf.bm_words, C, P.d_ptr, (uint32_t)P.rt.K,
+                                             P.rt.table, P.rt.ovf, P.d_rows);
+    else
+      k_bt_fill<<<blocks, 256, 0, s>>>(n_sel, pf.d_q, pf.d_bits, pf.bm_words, C, P.d_ptr, P.rt.ovf, P.d_rows, P.rs,
+                                       P.rt.first_shift);
     ++k;
   }
   ARA_TRY(cudaGetLastError());
@@ -366,10 +426,11 @@ ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
   Portfolio& pf = *P.pf;
   if (!batched_fits(pf, P.sel.size())) return ARA_ERANGE;
   const int64_t C = pf.catalogue;
-  for (P.by_event = rows_usable(pf, P.sel);; P.by_event = false) {
+  P.by_event = rows_usable(pf, P.sel);
+  for (int K = P.windowed() ? 0 : plan_k(P);; K = 0) {
     P.rt = RowTable{};
-    P.rt.K = P.by_event && !P.windowed() ? rows_k(pf, P.sel) : 0;
-    const RowSizes z = rows_sizes(pf, P.sel, P.rt.K);
+    P.rt.K = K;
+    const RowSizes z = rows_sizes(pf, P.sel, K);
     P.rt.first_shift = z.first_shift;
     P.sched = rows_schedule((int)P.sel.size(), P.rt.K, z.likely_bytes, z.likely_entries, P.n_trials, P.n_events);
     P.n_blocks = (C + BT_SCAN_BLOCK - 1) / BT_SCAN_BLOCK;
@@ -384,8 +445,9 @@ ara_status run_plan_async(ara_plan& P, cudaStream_t s) {
     char* buf = nullptr;
     if (dmalloc_async((void**)&buf, off, s) != cudaSuccess) {
       cudaGetLastError();
-      if (P.by_event && !P.own_tables) continue;      // the general way needs less
-      return ARA_ENOMEM;
+      if (P.own_tables || (!P.by_event && K == 0)) return ARA_ENOMEM;
+      P.by_event = false;            // the general way, end to end, needs least
+      continue;
     }
     if (P.rt.K == 0) P.d_rows = (uint64_t*)(buf + o_rows);
     else P.rt.table = (uint64_t*)(buf + o_tab);
@@ -461,7 +523,7 @@ ara_status ara_plan_batched(ara_portfolio* pf_, int64_t n_trials, const int64_t*
     return st;
   };
   P->by_event = rows_usable(*pf, P->sel);
-  P->rt.K = P->by_event ? rows_k(*pf, P->sel) : 0;
+  P->rt.K = plan_k(*P);
   const RowSizes z = rows_sizes(*pf, P->sel, P->rt.K);
   P->rt.first_shift = z.first_shift;
   if ((P->rt.K > 0 && dmalloc(&P->rt.table, 8 * (size_t)P->rt.K * (size_t)C) != cudaSuccess) ||

@@ -84,6 +84,11 @@ __device__ __forceinline__ double value_of(uint64_t k) {
   return __longlong_as_double(b ^ ((~b >> 63) | (long long)0x8000000000000000ull));
 }
 
+// 16-byte pairs that a row of n entries takes outside its place of K entries (K = 0: it has none).
+__device__ __forceinline__ uint32_t row_pairs(uint32_t n, uint32_t K) {
+  return K == 0u ? (n + 1u) >> 1 : n > K ? (n - K + 2u) >> 1 : 0u;
+}
+
 struct U128 {
   uint64_t lo, hi;
 };

@@ -260,6 +260,7 @@ ara_status launch_event_scan(const uint32_t* bits, int64_t bits_stride, int32_t 
 ara_status report_device_errors(Portfolio& pf, uint32_t err, cudaStream_t s);
 // Event-major rows and their stream (ara_rows.cu).
 constexpr int RW_MAX_LAYERS = 255;
+constexpr uint64_t RW_CONT = 1ull << 55;       // entry flag: a continuation, not a loss (ara_rows.cu)
 constexpr int RW_BUILD_THREADS = 128;
 constexpr int RW_BUILD_SUMS = 2560;            // sums a block of the build holds at a time (20 KB)
 constexpr int64_t RW_MAX_CATALOGUE = (int64_t)1 << 27;

@@ -30,7 +30,6 @@ namespace ara {
 __device__ __forceinline__ void red_u64(unsigned long long* a, unsigned long long q) {
   asm volatile("red.shared.add.u64 [%0], %1;" :: "r"((uint32_t)__cvta_generic_to_shared(a)), "l"(q) : "memory");
 }
-constexpr uint64_t RW_CONT = 1ull << 55;          // entry flag: a continuation, not a loss
 constexpr uint64_t RW_Q = (1ull << 55) - 1;
 
 // ------------------------------------------------------------------------------------------
@@ -328,7 +327,7 @@ k_rows_build(RowsBuild p) {
     }
     // room for the rows (K = 0) or their overflow, one atomic per block
     const uint32_t more = p.K == 0 ? n : n > (uint32_t)p.K ? n - (uint32_t)p.K + 1u : 0u;
-    const uint32_t need = (more + 1u) >> 1;
+    const uint32_t need = row_pairs(n, (uint32_t)p.K);
     uint32_t pairs, cnt;
     uint32_t at = rb_scan(need, part, &pairs);
     rb_scan(n, part, &cnt);

@@ -110,6 +110,32 @@ def test_layers_in_any_elt_order_take_the_general_way():
     pf.close()
 
 
+@pytest.mark.parametrize("form", [0, 1, 2, 3, 5, 7])
+def test_rows_of_layers_in_descending_elt_order(form):
+    """The general way in every form of the rows, in place with and without overflow and end to end."""
+    C, n_elts, nnz, n_layers, (lo, hi), f32, trials, events = FORMS[form]
+    layers = [l[::-1] for l in own(np.random.default_rng(form), n_layers, n_elts, max(lo, 2), hi)] + [[]]
+    pf, off, ids = make(form, C, n_elts, nnz, layers, f32, trials, events)
+    sel = [0] + list(range(n_layers + 1))[1:][::-1]
+    ref, reg_ref = singles(pf, off, ids, sel)
+    for autotune in (False, True):
+        reg = torch.full((len(sel), trials), 9, dtype=torch.uint8, device="cuda")
+        plan = ara.BatchedPlan(pf, off, ids, layers=sel, regimes=reg, autotune=autotune)
+        assert torch.equal(plan.launch(), ref) and torch.equal(reg, reg_ref)
+        rows, n_entries = plan.table()
+        assert int(((rows >> 32) & 0xff).sum()) == n_entries
+        plan.close()
+    for budget in (0, 20 * C + 8 * sum(nnz * len(l) for l in layers) + 8 * C + 4096):   # and end to end without room
+        ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, budget)
+        try:
+            a = pf.run_ylt(off, ids, layers=sel, flags=ara.ARA_RUN_BATCHED)
+        finally:
+            ara.debug_set(ara.ARA_DBG_MEMORY_BUDGET, 0)
+        assert torch.equal(a, ref)
+    pf.check()
+    pf.close()
+
+
 @pytest.mark.parametrize("shape", [(2_000_000, 60, 20_000, 70, 4, 18), (1_500_000, 80, 30_000, 120, 3, 20)])
 def test_tables_beyond_l2_run_in_several_passes(shape):
     """Tables large enough for several passes over the YET (8 and 4 columns): sums carried from
