@@ -772,28 +772,56 @@ ara_status ara_prepare_ylt(ara_portfolio* pf, int32_t n_sel, const int32_t* laye
   return launch_coarsen(*pf, (int32_t)sel.size(), sel.data(), flags, s, slot);
 }
 
+// Pairs of entries that an occurrence of rows in place of K entries reads beyond them, on average: layers
+// hit an event together as far as they share ELTs, so an event with any of the selection's ELTs
+// (probability p) is taken to have entries / p of them, binomially spread over the layers.
+static double rows_overflow(const Portfolio& pf, const std::vector<int32_t>& sel, int K, double entries) {
+  if (K == 0) return 0.0;
+  std::vector<uint8_t> seen((size_t)pf.n_elts, 0);
+  double lambda = 0.0;
+  for (int32_t l : sel)
+    for (int k = pf.layer_off[(size_t)l]; k < pf.layer_off[(size_t)l + 1]; ++k) {
+      const size_t j = (size_t)pf.layer_elts[(size_t)k];
+      if (!seen[j]) lambda += (double)(pf.rec_off[j + 1] - pf.rec_off[j]) / (double)pf.catalogue;
+      seen[j] = 1;
+    }
+  const int L = (int)sel.size();
+  const double p = 1.0 - std::exp(-lambda), q = std::min(p > 0.0 ? entries / p / L : 0.0, 0.999);
+  double pn = std::pow(1.0 - q, L), pairs = 0.0;             // pn: probability of n entries
+  for (int n = 0; n < L; ++n) {
+    pn *= (double)(L - n) / (double)(n + 1) * q / (1.0 - q);
+    if (n + 1 > K) pairs += pn * (double)((n + 1 - K + 2) / 2);
+  }
+  return p * pairs;
+}
+
 // Whether an ordinary run of several layers is faster over event-major rows (one pass for all
-// layers, the same results) than layer by layer.  Both costs in microseconds, fitted to runs of
-// 2-250 layers over 1e4-2.5e6 events, 5e4-1e9 occurrences: the per-layer stream takes 1.0 ps per
-// occurrence, 0.17 ns per trial and 8 us per layer, its folds 6 ps per event and layer and 20 ps
-// per record; the rows 20 ps per event and 18 ps per record to build, then 5.5 ps per occurrence and
-// 0.7 (rows in place) or 2.2 (rows end to end) per entry of its event, and 0.035 ns per trial and
-// layer.  At 2e8 occurrences of 2 M events the line lies at 4-5 layers (4 layers: 1.07 ms layer by
-// layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
+// layers, the same results) than layer by layer.  Both costs in microseconds, linear in what the kernels
+// do, fitted (least squares of the relative error, no negative terms) to both ways' times in 400 random
+// portfolios: 2-40 layers of 1-20 of 4-200 ELTs (shared or their own) of 300-30,000 records over 5,000-2.5 M
+// events, 500-400,000 trials of 20-1,500 occurrences.  Layer by layer: a stream's start, its
+// occurrences, trials and hits, and the fold of its table and its walk of the portfolio's records; rows: their
+// build (events, the layers' records), then occurrences, entries, pairs beyond a row's place, trials.  Half
+// of the predictions lie within 10 % (layers) and 12 % (rows), nine of ten within 33 and 55 %.  On 400 other
+// portfolios of the same ranges the choice costs 1.1 % over the sum of the faster ways: 8 go by rows more than
+// 5 % slower (at worst 1.44 times; the rule before, without hits and overflow: 23 of its 400, 1.65 times), 22
+// stay layer by layer more than 5 % slower (3.7).  At 2e8 occurrences of 2 M events the line lies at 4-5
+// layers (4 layers: 1.07 ms layer by layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
 static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, int64_t n_trials, int64_t events) {
   if (sel.size() < 2 || !batched_fits(pf, sel.size()) || !rows_usable(pf, sel)) return false;
   const int K = rows_k(pf, sel);
-  const RowSizes z = rows_sizes(pf, sel, K);
-  const double C = (double)pf.catalogue, L = (double)sel.size(), ev = (double)events, tr = (double)n_trials;
+  const double C = 1e-6 * (double)pf.catalogue, L = (double)sel.size(), ev = 1e-6 * (double)events,
+               tr = 1e-3 * (double)n_trials, entries = rows_sizes(pf, sel, K).likely_entries;
   double rec = 0.0;
   for (int32_t l : sel)
     for (int k = pf.layer_off[(size_t)l]; k < pf.layer_off[(size_t)l + 1]; ++k) {
       const size_t j = (size_t)pf.layer_elts[(size_t)k];
-      rec += (double)(pf.rec_off[j + 1] - pf.rec_off[j]);
+      rec += 1e-6 * (double)(pf.rec_off[j + 1] - pf.rec_off[j]);
     }
-  const double layers = L * (8.0 + 1e-6 * ev + 0.17e-3 * tr + 6e-6 * C) + 20e-6 * rec;
-  const double rows = 16.0 + 20e-6 * C + 18e-6 * rec + 1e-6 * ev * (5.5 + (K ? 0.7 : 2.2) * z.likely_entries) +
-                      0.035e-3 * tr * L;
+  const double layers = 9.1 + L * (7.0 + 0.61 * ev + 0.144 * tr + 5.0 * C + 1.31e-6 * (double)pf.n_records) +
+                        4.85 * ev * entries;
+  const double rows = 29.0 + 14.8 * C + 21.7 * rec + (0.355 + 0.008 * L) * tr +
+                      ev * (3.89 + (K ? 1.77 : 2.1) * entries + 14.4 * rows_overflow(pf, sel, K, entries));
   return rows < 0.92 * layers;
 }
 

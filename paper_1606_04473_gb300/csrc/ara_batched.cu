@@ -274,8 +274,8 @@ void single_request(ara_plan& P) {
 }
 
 // Entries in place per event: the rule of the rows, and from the folds up to 2 (launches of plans with ELTs
-// in descending order, us, end to end / in place: 50,000 trials x 1,000 over 2 M events, 1 layer 468 / 308, 4
-// layers 528 / 410, 8 layers 586 / 509 (2 places); 100,000 trials, 16 layers 1,123 / 1,317 (4 places)).
+// in descending order, us, end to end / in place: 50,000 trials x 1,000 over 2 M events, 1 layer 464 / 307, 4
+// layers 524 / 407, 8 layers 584 / 506 (2 places); 100,000 trials, 16 layers 1,118 / 1,299 (4 places)).
 int plan_k(const ara_plan& P) {
   const int K = rows_k(*P.pf, P.sel);
   return P.by_event || K <= 2 ? K : 0;
