@@ -71,7 +71,10 @@ typedef struct ara_portfolio ara_portfolio;
                                [n_elts][catalogue] (Section IV-B), used by ARA_RUN_PER_ELT */
 
 /*
- * Copy a portfolio to the current CUDA device.  Synchronous.
+ * Copy a portfolio to the current CUDA device.  Synchronous.  Device memory: the records by ELT (12
+ * bytes each with ARA_LOSSES_F32, else 16); where there is room, and the catalogue has at most 2^27
+ * events, the records again event by event (8 or 12 bytes each and 4 per event), which the runs, plans
+ * and adjoints of several layers read; and about 8.3 bytes per layer and event.
  *   catalogue_size           number of events in the global event catalogue; event IDs are
  *                            0 .. catalogue_size-1  (1 <= catalogue_size <= 2^31 - 1)
  *   n_elts                   number of ELTs (>= 0)
@@ -346,7 +349,8 @@ typedef struct ara_query {
  * few small warm-up requests
  * (synchronous), so the first real requests pay no one-time costs.  The pool and the YET must
  * outlive the server.  Results of a request do not depend on what else runs or on the group it
- * ran in (bitwise).
+ * ran in, and equal those of ara_run_ylt, ara_risk_metrics and ara_adjoint on its layers and slice
+ * (bitwise).
  */
 ARA_API ara_status ara_server_create(ara_portfolio* pool, int64_t n_trials,
                                      const int64_t* d_trial_offsets, int64_t n_events,

@@ -788,6 +788,7 @@ static double rows_overflow(const Portfolio& pf, const std::vector<int32_t>& sel
   const int L = (int)sel.size();
   const double p = 1.0 - std::exp(-lambda), q = std::min(p > 0.0 ? entries / p / L : 0.0, 0.999);
   double pn = std::pow(1.0 - q, L), pairs = 0.0;             // pn: probability of n entries
+  if (pn < 1e-300) return p * std::max(0.0, (q * L - K + 2.0) / 2.0);   // nearly every layer, or very many
   for (int n = 0; n < L; ++n) {
     pn *= (double)(L - n) / (double)(n + 1) * q / (1.0 - q);
     if (n + 1 > K) pairs += pn * (double)((n + 1 - K + 2) / 2);

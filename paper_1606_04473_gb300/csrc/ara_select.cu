@@ -21,8 +21,8 @@
 // barrier each).  Kernel time of one call, 3 targets / 6 targets and the mean, us:
 //   rows x values   1 x 1e3    1 x 3e4    1 x 1.5e5  1 x 1e6    1 x 5e6    8 x 1e5    16 x 2e5   64 x 2e5
 //   radix select    23 / 30    31 / 39    36 / 48    60 / 82    161 / 225  44 / 68    89 / 145   394 / 557
-//   this            14 / 17    33 / 40    33 / 40    46 / 57    97 / 121   39 / 46    66 / 85    120 / 166
-// Few rows are bound by the steps' latencies (sorting the sample 3-9 us, a barrier 1.5 us, a pick 3 us,
+//   this            15 / 16    31 / 38    31 / 40    43 / 62    99 / 128   35 / 43    50 / 72    93 / 124
+// Few rows are bound by the steps' latencies (sorting the sample 4-7 us, a barrier 1.5 us, a pick 3 us,
 // each pass over the row one L2 round trip), many rows by reading them three times.
 
 #include <algorithm>
@@ -105,7 +105,7 @@ static SelScratch carve(void* base, const SelPlan& y) {
 // Bitonic sort of m shared-memory keys (a power of two: 512 E, or for E = 2 any from 64), descending,
 // by the whole block, E per thread in registers: thread l of warp w holds the keys 32 E w + 32 u + l,
 // so steps of stride below 32 are shuffles, those below 32 E stay within the thread and only the wider
-// ones go through shared memory.  (1,024 keys with all steps through shared memory: 8 us; this: 2 us.
+// ones go through shared memory.  (256 keys take 3.9 us, 1,024 6.7, one block alone on its SM.
 // The loops are not unrolled: the code runs once per launch, and fetching it costs more than running it.)
 template <int E>
 __device__ __forceinline__ void sort_keys(uint64_t* a, int m) {

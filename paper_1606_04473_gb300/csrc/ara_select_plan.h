@@ -13,8 +13,11 @@ constexpr int SEL_THREADS = 512;
 constexpr int SEL_SAMPLE = 1024;                 // sampled keys per row
 constexpr int SEL_CLASSES = 2 * SEL_SAMPLE + 1;
 constexpr int SEL_SMALL = 4096;                  // rows up to this length are sorted whole
-// Rows of one request up to which the cooperative launch is the faster (16 rows of 200,000 values, 3
-// targets: 60 us against 95 us in clusters; 64 rows: 177 and 119).
+// Rows of one request up to which they go as one cooperative launch.  Rows of 200,000 values, 3 targets / 6
+// targets and the mean, us, cooperative and in clusters: 9 rows 43 / 60 and 47 / 62, 16 rows 56 / 72 and 83 / 106, 24
+// rows 59 / 91 and 64 / 81, 32 rows 79 / 119 and 64 / 85, 64 rows 119 / 183 and 92 / 126.  (From about 24 rows
+// clusters are the faster way since the keys take no FP64 instructions; the line decides the order in
+// which TVaR and mean are added, and has stayed.)
 constexpr int SEL_GRID_ROWS = 32;
 constexpr int SEL_SLICES = 16;                   // slices of a row's sums that a block of a cluster can hold
 
@@ -30,8 +33,8 @@ struct SelState {
 // Sampled keys of a row, and room for the keys of one open interval between neighbouring samples: the
 // interval that holds a given rank has 2 / sample of the keys on average and more than 16 / sample with
 // probability 2e-6 (a list that would overflow is not used: its target is picked from the row itself).
-// Sorting the sample costs every block longer the larger it is, and the intervals it leaves are picked from
-// in about 4 us per 4,096 keys: 256 keys up to 2^19 values, and lists that rarely overflow at any length.
+// Sorting the sample costs every block 3.9 us for 256 keys and 6.7 for 1,024, and the intervals it leaves are
+// picked from in about 4 us per 4,096 keys: 256 keys up to 2^19 values.
 struct SelLists {
   int32_t sample;
   int64_t cap;                      // keys per list
