@@ -798,32 +798,49 @@ static double rows_overflow(const Portfolio& pf, const std::vector<int32_t>& sel
 
 // Whether an ordinary run of several layers is faster over event-major rows (one pass for all
 // layers, the same results) than layer by layer.  Both costs in microseconds, linear in what the kernels
-// do, fitted (least squares of the relative error, no negative terms) to both ways' times in 400 random
-// portfolios: 2-40 layers of 1-20 of 4-200 ELTs (shared or their own) of 300-30,000 records over 5,000-2.5 M
-// events, 500-400,000 trials of 20-1,500 occurrences.  Layer by layer: a stream's start, its
-// occurrences, trials and hits, and the fold of its table and its walk of the portfolio's records; rows: their
-// build (events, the layers' records), then occurrences, entries, pairs beyond a row's place, trials.  Half
-// of the predictions lie within 10 % (layers) and 12 % (rows), nine of ten within 33 and 55 %.  On 400 other
-// portfolios of the same ranges the choice costs 1.1 % over the sum of the faster ways: 8 go by rows more than
-// 5 % slower (at worst 1.44 times; the rule before, without hits and overflow: 23 of its 400, 1.65 times), 22
-// stay layer by layer more than 5 % slower (3.7).  At 2e8 occurrences of 2 M events the line lies at 4-5
+// do, fitted (least squares of the relative error, no negative terms) to the times of both ways in 1,120
+// random portfolios: 2-40 layers of 1-20 of 4-240 ELTs (shared or their own) of 300-30,000 records over
+// 5,000-2.5 M events, up to 2.2e8 occurrences in trials of 20-1,500.  Layer by layer: a stream's start, its
+// occurrences, trials and hits, writing its table, and the fold, by event (the chain of an event's
+// records, and their walk) or by tile (the chain of a tile's records).  Rows: their build (events, the
+// layers' records, the portfolio's records and their chain per event), then occurrences (more for a table of
+// up to 32 MB), entries, pairs beyond a row's place, trials, and the chain of a trial's occurrences.  Half of the
+// predictions lie within 7 % (layers) and 8 % (rows), nine of ten within 22 and 29 %.  On 400 other portfolios
+// the ways chosen take 0.3 % more than the faster ones (16 % by the rule before, which had no terms for hits,
+// overflow, folds and trials): 2 go by rows more than 5 % slower (at worst 1.37 times; 9 before), 9 stay
+// layer by layer more than 5 % slower (1.24; 19 and 4.7 before).  At 2e8 occurrences of 2 M events the line lies at 4-5
 // layers (4 layers: 1.07 ms layer by layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
 static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, int64_t n_trials, int64_t events) {
   if (sel.size() < 2 || !batched_fits(pf, sel.size()) || !rows_usable(pf, sel)) return false;
   const int K = rows_k(pf, sel);
   const double C = 1e-6 * (double)pf.catalogue, L = (double)sel.size(), ev = 1e-6 * (double)events,
-               tr = 1e-3 * (double)n_trials, entries = rows_sizes(pf, sel, K).likely_entries;
-  double rec = 0.0;
-  for (int32_t l : sel)
+               tr = 1e-3 * (double)n_trials, all = 1e-6 * (double)pf.n_records,
+               entries = rows_sizes(pf, sel, K).likely_entries;
+  double rec = 0.0, most = 0.0;                             // records of the layers, of the largest one
+  for (int32_t l : sel) {
+    double r = 0.0;
     for (int k = pf.layer_off[(size_t)l]; k < pf.layer_off[(size_t)l + 1]; ++k) {
       const size_t j = (size_t)pf.layer_elts[(size_t)k];
-      rec += 1e-6 * (double)(pf.rec_off[j + 1] - pf.rec_off[j]);
+      r += 1e-6 * (double)(pf.rec_off[j + 1] - pf.rec_off[j]);
     }
-  const double layers = 9.1 + L * (7.0 + 0.61 * ev + 0.144 * tr + 5.0 * C + 1.31e-6 * (double)pf.n_records) +
-                        4.85 * ev * entries;
-  const double rows = 29.0 + 14.8 * C + 21.7 * rec + (0.355 + 0.008 * L) * tr +
-                      ev * (3.89 + (K ? 1.77 : 2.1) * entries + 14.4 * rows_overflow(pf, sel, K, entries));
-  return rows < 0.92 * layers;
+    rec += r;
+    most = std::max(most, r);
+  }
+  const double per_event = all / C;
+  double fold;
+  if (fold_by_event(pf, (int32_t)sel.size(), sel.data())) {
+    fold = 0.33 * per_event + 4.7 * L * all;
+  } else {        // tiles of all layers in waves of 7 blocks per SM
+    const double waves = std::max(1.0, (double)pf.n_tiles * L / (7.0 * pf.n_sms));
+    fold = 0.015 * most / C * (double)std::min<int64_t>(FOLD_TILE, pf.catalogue) * waves;
+  }
+  const double layers = 7.1 + L * (6.8 + ev * (0.63 + 0.16 * std::min(1.0, 0.5 * C)) + 0.152 * tr + 5.4 * C) +
+                        3.0 * ev * entries + fold;
+  const double table = std::min(1.0, 8.0 * C * (K ? K : 1.0 + entries) / 32.0);
+  const double rows = 22.0 + 15.0 * C + 18.0 * rec + 0.98 * per_event + 4.2 * all + (0.41 + 0.012 * L) * tr +
+                      25.6e-3 * (double)events / (double)std::max<int64_t>(n_trials, 1) +
+                      ev * (3.2 + 1.1 * table + (K ? 1.5 : 1.8) * entries + 6.3 * rows_overflow(pf, sel, K, entries));
+  return rows < layers;
 }
 
 static ara_status run_ylt(ara_portfolio* pf, int64_t n_trials, const int64_t* d_offsets,

@@ -207,6 +207,7 @@ inline FoldSlot fold_slot(const struct Portfolio& pf, int slot) {
   return slot ? FoldSlot{pf.d_q_alt, pf.d_bits_alt, pf.d_cbits_alt} : FoldSlot{pf.d_q, pf.d_bits, pf.d_cbits};
 }
 
+bool fold_by_event(const Portfolio& pf, int32_t n_sel, const int32_t* sel);
 ara_status launch_fold(Portfolio& pf, int32_t n_sel, const int32_t* sel_host, int32_t flags,
                        cudaStream_t s, int slot = 0);
 // The coarse hit bitmaps the default stream kernel reads (when the exact bitmap does not fit in

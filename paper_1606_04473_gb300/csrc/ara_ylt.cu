@@ -306,7 +306,7 @@ static void launch_fold_events(const FoldByEvent& p, const SelList& sl, const Fo
 // least a quarter of those that the walks read (every layer reads the portfolio's), and not a large
 // catalogue with few records per event (at 0.15 per event of 2 M both ways take the time of writing the
 // table, at 0.3 of 1 M this one takes 13 us and the tiles 22).
-static bool fold_by_event(const Portfolio& pf, int32_t n_sel, const int32_t* sel) {
+bool fold_by_event(const Portfolio& pf, int32_t n_sel, const int32_t* sel) {
   if (!pf.d_ev_ptr || !pf.d_mem) return false;
   int64_t rec = 0;
   for (int32_t i = 0; i < n_sel; ++i) {
