@@ -805,10 +805,10 @@ static double rows_overflow(const Portfolio& pf, const std::vector<int32_t>& sel
 // records, and their walk) or by tile (the chain of a tile's records).  Rows: their build (events, the
 // layers' records, the portfolio's records and their chain per event), then occurrences (more for a table of
 // up to 32 MB), entries, pairs beyond a row's place, trials, and the chain of a trial's occurrences.  Half of the
-// predictions lie within 7 % (layers) and 8 % (rows), nine of ten within 22 and 29 %.  On 400 other portfolios
-// the ways chosen take 0.3 % more than the faster ones (16 % by the rule before, which had no terms for hits,
-// overflow, folds and trials): 2 go by rows more than 5 % slower (at worst 1.37 times; 9 before), 9 stay
-// layer by layer more than 5 % slower (1.24; 19 and 4.7 before).  At 2e8 occurrences of 2 M events the line lies at 4-5
+// predictions lie within 7 % (layers) and 8 % (rows), nine of ten within 22 and 29 %.  On 560 other portfolios,
+// 160 of them of 1e7 occurrences and more, 5 go by rows more than 5 % slower (at worst 1.26 times) and 10 stay layer
+// by layer more than 5 % slower (2.2 times); without the terms for hits, overflow, folds, trials and large
+// tables 19 (1.65) and 22 (4.1).  At 2e8 occurrences of 2 M events the line lies at 4-5
 // layers (4 layers: 1.07 ms layer by layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
 static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, int64_t n_trials, int64_t events) {
   if (sel.size() < 2 || !batched_fits(pf, sel.size()) || !rows_usable(pf, sel)) return false;
