@@ -798,15 +798,15 @@ static double rows_overflow(const Portfolio& pf, const std::vector<int32_t>& sel
 
 // Whether an ordinary run of several layers is faster over event-major rows (one pass for all
 // layers, the same results) than layer by layer.  Both costs in microseconds, linear in what the kernels
-// do, fitted (least squares of the relative error, no negative terms) to the times of both ways in 1,120
+// do, fitted (least squares of the relative error, no negative terms) to the times of both ways in 1,520
 // random portfolios: 2-40 layers of 1-20 of 4-240 ELTs (shared or their own) of 300-30,000 records over
 // 5,000-2.5 M events, up to 2.2e8 occurrences in trials of 20-1,500.  Layer by layer: a stream's start, its
-// occurrences, trials and hits, writing its table, and the fold, by event (the chain of an event's
-// records, and their walk) or by tile (the chain of a tile's records).  Rows: their build (events, the
+// occurrences, trials and hits, writing its table, and the fold, by event (the walk of the portfolio's
+// records) or by tile (the chain of a tile's records).  Rows: their build (events, the
 // layers' records, the portfolio's records and their chain per event), then occurrences (more for a table of
 // up to 32 MB), entries, pairs beyond a row's place, trials, and the chain of a trial's occurrences.  Half of the
-// predictions lie within 7 % (layers) and 8 % (rows), nine of ten within 22 and 29 %.  On 560 other portfolios,
-// 160 of them of 1e7 occurrences and more, 5 go by rows more than 5 % slower (at worst 1.26 times) and 10 stay layer
+// predictions lie within 7 % (layers) and 8 % (rows), nine of ten within 23 and 29 %.  On 560 other portfolios,
+// 160 of them of 1e7 occurrences and more, 7 go by rows more than 5 % slower (at worst 1.26 times) and 7 stay layer
 // by layer more than 5 % slower (2.2 times); without the terms for hits, overflow, folds, trials and large
 // tables 19 (1.65) and 22 (4.1).  At 2e8 occurrences of 2 M events the line lies at 4-5
 // layers (4 layers: 1.07 ms layer by layer, 1.22 by rows; 8: 2.20 and 1.40; 16: 3.66 and 1.46).
@@ -826,20 +826,19 @@ static bool rows_faster(const Portfolio& pf, const std::vector<int32_t>& sel, in
     rec += r;
     most = std::max(most, r);
   }
-  const double per_event = all / C;
   double fold;
   if (fold_by_event(pf, (int32_t)sel.size(), sel.data())) {
-    fold = 0.33 * per_event + 4.7 * L * all;
+    fold = 12.0 * L * all;
   } else {        // tiles of all layers in waves of 7 blocks per SM
     const double waves = std::max(1.0, (double)pf.n_tiles * L / (7.0 * pf.n_sms));
     fold = 0.015 * most / C * (double)std::min<int64_t>(FOLD_TILE, pf.catalogue) * waves;
   }
-  const double layers = 7.1 + L * (6.8 + ev * (0.63 + 0.16 * std::min(1.0, 0.5 * C)) + 0.152 * tr + 5.4 * C) +
-                        3.0 * ev * entries + fold;
+  const double layers = 7.2 + L * (6.5 + ev * (0.65 + 0.135 * std::min(1.0, 0.5 * C)) + 0.149 * tr + 5.55 * C) +
+                        3.2 * ev * entries + fold;
   const double table = std::min(1.0, 8.0 * C * (K ? K : 1.0 + entries) / 32.0);
-  const double rows = 22.0 + 15.0 * C + 18.0 * rec + 0.98 * per_event + 4.2 * all + (0.41 + 0.012 * L) * tr +
-                      25.6e-3 * (double)events / (double)std::max<int64_t>(n_trials, 1) +
-                      ev * (3.2 + 1.1 * table + (K ? 1.5 : 1.8) * entries + 6.3 * rows_overflow(pf, sel, K, entries));
+  const double rows = 22.0 + 15.9 * C + 18.6 * rec + 0.94 * all / C + 4.0 * all + (0.4 + 0.012 * L) * tr +
+                      23.8e-3 * (double)events / (double)std::max<int64_t>(n_trials, 1) +
+                      ev * (3.2 + 0.97 * table + (K ? 1.53 : 1.87) * entries + 6.7 * rows_overflow(pf, sel, K, entries));
   return rows < layers;
 }
 
